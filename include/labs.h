@@ -113,9 +113,11 @@ typedef struct {
   int64_t n_thresh_samples; /* auto threshold: starts sampled (stream (seed, 2, i, 0)), e.g. 10^6 */
   int64_t thresh_rank;      /* auto threshold: 0-based rank of E_thr among the samples, e.g. 999 */
   int32_t E_target;     /* record each walk's first flip reaching E <= E_target; INT32_MIN = off */
-  int32_t tile_m;       /* neighbours per tile (8, 12 or 16); 0 = chosen by the library */
-  int32_t warps_per_cta;/* warps per CTA: 1..8 with 32 lanes per walk, 1..12 with 16; 0 = chosen by the library */
-  int32_t lanes_per_walk; /* 32: one walk per warp; 16: two walks per warp (R <= 16); 0 = chosen by the library */
+  int32_t tile_m;       /* 8, 12 or 16: accepted where that tile of neighbours has a plan for L and p (the walks
+                           keep their neighbours incrementally and have no tiles); 0 = no request */
+  int32_t warps_per_cta;/* warps (walks) per CTA: 1..8 with lanes_per_walk 32, 1..12 with 16; 0 = chosen by the
+                           library */
+  int32_t lanes_per_walk; /* 32, or 16 (R <= 16): accepted, every walk runs on one warp; 0 = no request */
   const int32_t* E_thr_dev; /* nullable device int32: when set, the sieve bound is read from it (for
                                instance written by labs_sample_threshold on the same stream) and
                                E_thr is ignored */
@@ -164,8 +166,8 @@ typedef struct {
   int64_t n_thresh_samples; /* per-length sieve bound: samples (<= 2^31) */
   int64_t thresh_rank;      /* per-length sieve bound: 0-based rank */
   int32_t E_target;         /* per-walk first flip reaching E <= E_target (walk_stats[5]); INT32_MIN = off */
-  int32_t tile_m;           /* 0: autotuned (timed trial, cached per length set and SM count); 8, 12, 16 */
-  int32_t warps_per_cta;    /* 0: autotuned; 1..8 */
+  int32_t tile_m;           /* as in labs_walk_cfg */
+  int32_t warps_per_cta;    /* 0: chosen by the library; 1..8 */
   int32_t use_graph;        /* 1: capture the step into a CUDA graph on first use and replay it */
 } labs_batch_cfg;
 
@@ -349,7 +351,7 @@ int labs_policy_train_step(labs_policy* policy, const uint64_t* seqs, const int3
  *   logits_log [n_chunks][n_walks][L] FP32: the logits each chunk used;
  *   state_log  [n_chunks][n_walks][W] uint64: every walk's sequence when its chunk began;
  *   move_log   [n_chunks][n_walks][2] int32: the chunk's first move (position, Delta E), (-1, 0) if none.
- *   Workspace: about 5.5 KB per walk.  With a policy the call synchronises `stream` at its end and returns
+ *   Workspace with a policy: about 8 KB per walk (up to 11 KB at L = 576).  With a policy the call synchronises `stream` at its end and returns
  *   LABS_ERR_TIMEOUT if a tensor-core wait of the network expired.
  */
 int labs_chunked_search(labs_ctx* ctx, const labs_walk_cfg* cfg, labs_policy* policy, float lambda, int chunk,

@@ -137,7 +137,7 @@ def make_walk_cfg(L, skew=True, p=0, n_walks=1, flip_budget=1000, T_i=0, seed=0,
                   E_thr=INT32_MAX, n_thresh_samples=0, thresh_rank=0, E_target=INT32_MIN, walk_begin=0, tile_m=0,
                   warps_per_cta=0, E_thr_dev=None, lanes_per_walk=0):
     """labs_walk_cfg; E_thr_dev (a device int32 tensor) makes the walk read its sieve bound from it;
-    lanes_per_walk 32 / 16 fixes one walk per warp / per half-warp (0: the library chooses)."""
+    tile_m and lanes_per_walk are accepted where they have a plan and select nothing (include/labs.h)."""
     cfg = WalkCfg()
     cfg.L, cfg.skew, cfg.p, cfg.T_i = L, int(bool(skew)), p, T_i
     cfg.n_walks, cfg.walk_begin, cfg.flip_budget, cfg.seed = n_walks, walk_begin, flip_budget, seed

@@ -9,7 +9,7 @@
 namespace labsg {
 
 void* ws_get(labs_ctx* ctx, int slot, size_t bytes) {
-  if (slot < 0 || slot >= 8) return nullptr;
+  if (slot < 0 || slot >= kWorkspaces) return nullptr;
   if (ctx->ws_bytes[slot] >= bytes && ctx->ws[slot]) return ctx->ws[slot];
   if (ctx->ws[slot]) {
     cudaDeviceSynchronize();
@@ -77,7 +77,7 @@ void labs_ctx_destroy(labs_ctx* ctx) {
   cudaDeviceSynchronize();
   if (ctx->graph_exec) cudaGraphExecDestroy(ctx->graph_exec);
   if (ctx->capture_stream) cudaStreamDestroy(ctx->capture_stream);
-  for (int i = 0; i < 8; i++)
+  for (int i = 0; i < kWorkspaces; i++)
     if (ctx->ws[i]) cudaFree(ctx->ws[i]);
   delete ctx;
 }

@@ -1,6 +1,8 @@
-// labs_core.cuh -- device building blocks shared by the LABS kernels (sm_103a).
+// labs_core.cuh -- device building blocks shared by the LABS kernels (sm_103a): random streams, walk starts,
+// fingerprints, and the neighbour scan of one sequence from scratch (the neighbour scan entry point, step 2's
+// expansions; the walks keep their neighbours' energies incrementally, walk.cu).
 //
-// One walk (or one sequence) is owned by one warp.  Its state lives in the warp's shared-memory slab:
+// One sequence is owned by one warp.  Its state lives in the warp's shared-memory slab:
 //   * the sequence, bit-packed (32-bit words, 1 = +1);
 //   * the correlation table C_{lambda g}, g = 1..G, as int16 (master) and int8 (fast-path copy);
 //   * "byte windows": for every neighbour m the kernel needs s_{m + lambda g} and s_{m - lambda g}
@@ -8,9 +10,9 @@
 //     position outside 1..L, in a forward array and a reversed array per position class, so that both
 //     windows of every neighbour are contiguous and increasing in g.
 //
-// lambda is the lag stride: 2 for skew-symmetric walks (odd lags have C = 0 by Eq. 2 and stay 0 under
+// lambda is the lag stride: 2 for skew-symmetric sequences (odd lags have C = 0 by Eq. 2 and stay 0 under
 // skew-preserving flips, so only even lags are tracked and positions split by parity into two
-// classes), 1 for unrestricted walks.
+// classes), 1 for the unrestricted neighbourhood.
 //
 // Single-flip Delta E (Section 3, linear-time neighbour evaluation).  Flipping F in {{m}, {m, m'}}
 // changes C_kappa by delta_kappa = -alpha s_m y_kappa with
@@ -86,53 +88,6 @@ __device__ __forceinline__ uint64_t warp_xor_u64(uint64_t v) {
 }
 
 // ------------------------------------------------------------------------------------------------
-// Lane groups: GL consecutive lanes (GL = 32: the whole warp; GL = 16: either half) own one walk or one
-// sequence.  Every synchronising primitive names the group's own lanes only, so the two halves of a
-// warp may hold different walks and diverge safely; shuffles use width GL, so source lanes are
-// group-relative.
-// ------------------------------------------------------------------------------------------------
-template <int GL>
-__device__ __forceinline__ int glane() {
-  return (int)(threadIdx.x & (GL - 1));
-}
-template <int GL>
-__device__ __forceinline__ int gbase() {  // first lane of the group inside the warp
-  return (int)(threadIdx.x & 31 & ~(GL - 1));
-}
-template <int GL>
-__device__ __forceinline__ unsigned gmask() {
-  if (GL == 32) return kFull;
-  return ((1u << (GL & 31)) - 1u) << gbase<GL>();
-}
-template <int GL>
-__device__ __forceinline__ int gsum(int v) { return __reduce_add_sync(gmask<GL>(), v); }
-template <int GL>
-__device__ __forceinline__ int gmin(int v) { return __reduce_min_sync(gmask<GL>(), v); }
-template <int GL>
-__device__ __forceinline__ int gmax(int v) { return __reduce_max_sync(gmask<GL>(), v); }
-template <int GL>
-__device__ __forceinline__ unsigned gminu(unsigned v) { return __reduce_min_sync(gmask<GL>(), v); }
-// group-relative ballot: bit j is group lane j
-template <int GL>
-__device__ __forceinline__ unsigned gballot(bool p) { return __ballot_sync(gmask<GL>(), p) >> gbase<GL>(); }
-template <int GL>
-__device__ __forceinline__ bool gall(bool p) { return __all_sync(gmask<GL>(), p); }
-template <int GL>
-__device__ __forceinline__ bool gany(bool p) { return __any_sync(gmask<GL>(), p); }
-template <int GL>
-__device__ __forceinline__ void gsync() { __syncwarp(gmask<GL>()); }
-template <int GL, class T>
-__device__ __forceinline__ T gshfl(T v, int src) { return __shfl_sync(gmask<GL>(), v, src, GL); }
-template <int GL, class T>
-__device__ __forceinline__ T gshfl_xor(T v, int o) { return __shfl_xor_sync(gmask<GL>(), v, o, GL); }
-template <int GL>
-__device__ __forceinline__ uint64_t gxor_u64(uint64_t v) {
-#pragma unroll
-  for (int o = GL / 2; o > 0; o >>= 1) v ^= gshfl_xor<GL>(v, o);
-  return v;
-}
-
-// ------------------------------------------------------------------------------------------------
 // Layout of one walk for (L, skew, p, M).  Identical on every lane (pure function of its inputs).
 // ------------------------------------------------------------------------------------------------
 struct Layout {
@@ -146,10 +101,6 @@ struct Layout {
   int NGh;    // groups of lag range 0 (range 1, when H = 2, is [NGh, NGend))
   int NGend;  // padded end of the groups (C = 0 beyond NG)
   int n_tasks;
-  // ceil(2^16 / tasks of the class): for 0 <= n <= 32, (n * fold_magic) >> 16 = n / tasks exactly (the
-  // error n * (magic * tasks - 2^16) stays below 32 * tasks < 2^16), so a lane splits a class's tasks
-  // without a divide
-  int fold_magic[2];
   int cw;  // 32-bit words per class in the byte-window arrays (class `cls` starts at word cls * cw)
   int cl;  // correlation-table entries kept (C16 / C8 lengths): > G, a multiple of 8, zero beyond G
 };
@@ -203,10 +154,6 @@ __host__ __device__ inline bool make_layout(Layout& ly, int L, int skew, int p, 
   }
   ly.Qr = qmax_end + ((2 - (qmax_end & 3)) & 3);
   ly.n_tasks = ly.n_tiles * H;
-  for (int cls = 0; cls < 2; cls++) {
-    const int nt = ly.ntiles[cls] * H;
-    ly.fold_magic[cls] = nt > 0 ? ((1 << 16) + nt - 1) / nt : 0;
-  }
   if (H == 1) {
     ly.NGh = ((ly.NG + ly.R - 1) / ly.R) * ly.R;
     ly.NGend = ly.NGh;
@@ -222,32 +169,8 @@ __host__ __device__ inline bool make_layout(Layout& ly, int L, int skew, int p, 
   int need_b = ly.Qr + 4 * ly.NGend + 8;
   ly.cw = cap / 4;
   ly.cl = kCLen;
-  // the walk's P bookkeeping reads class index 2q - q_f <= 2 * qmax_end
   return (H == 1 || H == 2) && M % 4 == 0 && need_f < cap && need_b < cap && 2 * qmax_end < cap &&
          4 * ly.NGend <= kCLen && L >= 2 && L <= kMaxL;
-}
-
-// Shrinks a valid layout's arrays to what its length needs (the walk kernels size their shared-memory
-// slabs per launch with it): class arrays of the smallest multiple of 16 bytes above every window, the
-// P bookkeeping's index 2 qmax_end and the class itself, and a table of the smallest multiple of 8
-// entries above G and 4 NGend (its last entry, always zero, stands in for a missing pair term).
-__host__ __device__ inline void compact_layout(Layout& ly) {
-  int qmax_end = 0;
-  for (int cls = 0; cls < ly.ncls; cls++)
-    if (ly.ntiles[cls] > 0) {
-      const int end = ly.tile_first[cls] + ly.ntiles[cls] * ly.M - 1;
-      if (end > qmax_end) qmax_end = end;
-    }
-  int need = qmax_end + 4 * ly.NGend + 8;
-  const int need_b = ly.Qr + 4 * ly.NGend + 8;
-  if (need_b > need) need = need_b;
-  if (2 * qmax_end + 1 > need) need = 2 * qmax_end + 1;
-  const int n_cls = ly.skew ? (ly.L + 1) / 2 : ly.L;  // class indices kQOff .. kQOff + n_cls - 1 hold positions
-  if (kQOff + n_cls + 1 > need) need = kQOff + n_cls + 1;
-  ly.cw = (need + 15) / 16 * 4;
-  int cl = 4 * ly.NGend;
-  if (ly.G + 1 > cl) cl = ly.G + 1;
-  ly.cl = (cl + 7) / 8 * 8;
 }
 
 // Tile tau -> (class, first class index).
@@ -262,10 +185,8 @@ __device__ __forceinline__ void tile_of(const Layout& ly, int tau, int& cls, int
 }
 
 // ------------------------------------------------------------------------------------------------
-// Shared-memory slab of one walk.  ScanSmem is the fixed-size form (every length up to 576); the walk
-// kernels carve slabs sized for their launch's lengths out of dynamic shared memory and address them
-// through a ScanView with the same members.  Class `cls` of fwd/bwd starts at word cls * ly.cw; the
-// tables hold ly.cl entries.
+// Shared-memory slab of one sequence (every length up to 576).  Class `cls` of fwd/bwd starts at word
+// cls * ly.cw; the tables hold ly.cl entries.
 // ------------------------------------------------------------------------------------------------
 struct __align__(16) ScanSmem {
   uint32_t fwd[kDirBytes / 4];
@@ -273,14 +194,6 @@ struct __align__(16) ScanSmem {
   int16_t C16[kCLen];  // C_{lambda (h+1)} at h, zero beyond G
   int8_t C8[kCLen];    // int8 copy, valid when every |C| <= 127
   uint32_t bits[kBitWords];
-};
-
-struct ScanView {
-  uint32_t* fwd;
-  uint32_t* bwd;
-  int16_t* C16;
-  int8_t* C8;
-  uint32_t* bits;
 };
 
 template <class S>
@@ -339,19 +252,19 @@ __device__ __forceinline__ uint32_t window_bytes(const S& sm, int L, int p, int 
 
 // The forward and reversed byte windows of every class: class index t is position q_pos(cls, t), i.e.
 // lambda (t - kQOff) + first position of the class, so every word is four positions lambda apart.
-template <int GL = 32, class S>
+template <class S>
 __device__ inline void build_bytes(S& sm, const Layout& ly) {
   const int words_per_cls = ly.cw;
   for (int cls = 0; cls < ly.ncls; cls++) {
     uint32_t* F = sm.fwd + cls_words(ly, cls);
     uint32_t* B = sm.bwd + cls_words(ly, cls);
     const int first = q_pos(ly, cls, kQOff);  // position of class index kQOff
-    for (int w = glane<GL>(); w < words_per_cls; w += GL) {
+    for (int w = lane_id(); w < words_per_cls; w += 32) {
       F[w] = window_bytes(sm, ly.L, first + ly.lam * (4 * w - kQOff), ly.lam, false);
       B[w] = window_bytes(sm, ly.L, first + ly.lam * (ly.Qr - 4 * w - 3 - kQOff), ly.lam, true);
     }
   }
-  gsync<GL>();
+  __syncwarp();
 }
 
 // C_k = (L-k) - 2 popc((x XOR (x >> k)) restricted to the low L-k bits) from the packed bits.
@@ -437,37 +350,37 @@ __device__ inline void p_all(const ScanSmem& sm, const Layout& ly, uint32_t* xb,
 
 // C_{lambda g} for g = 1..G; lanes split the lags.  Writes C16 (zero-padded to ly.cl) and returns E on
 // every lane of the group (sum over the tracked lags; for skew inputs the untracked odd lags are zero).
-template <int GL = 32, class S>
+template <class S>
 __device__ inline int build_table(S& sm, const Layout& ly) {
   int e_part = 0;
-  for (int h = glane<GL>(); h < ly.cl; h += GL) {
+  for (int h = lane_id(); h < ly.cl; h += 32) {
     int g = h + 1;
     int cval = (g <= ly.G) ? corr_lag(sm.bits, ly.L, ly.lam * g) : 0;
     sm.C16[h] = (int16_t)cval;
     e_part += cval * cval;
   }
-  gsync<GL>();
-  return gsum<GL>(e_part);
+  __syncwarp();
+  return warp_sum_i32(e_part);
 }
 
 // int8 copy of the table; returns true on every lane if all |C| <= 127 (fast path allowed).
-template <int GL = 32, class S>
+template <class S>
 __device__ inline bool pack_c8(S& sm, const Layout& ly) {
   bool ok = true;
-  for (int h = glane<GL>(); h < ly.cl; h += GL) {
+  for (int h = lane_id(); h < ly.cl; h += 32) {
     int v = sm.C16[h];
     ok &= (v >= -127 && v <= 127);
     sm.C8[h] = (int8_t)max(-127, min(127, v));
   }
-  gsync<GL>();
-  return gall<GL>(ok);
+  __syncwarp();
+  return __all_sync(kFull, ok);
 }
 
-template <int GL = 32, class S>
+template <class S>
 __device__ inline int table_sum(const S& sm, const Layout& ly) {
   int s = 0;
-  for (int h = glane<GL>(); h < ly.cl; h += GL) s += sm.C16[h];
-  return gsum<GL>(s);
+  for (int h = lane_id(); h < ly.cl; h += 32) s += sm.C16[h];
+  return warp_sum_i32(s);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -618,7 +531,7 @@ __device__ __forceinline__ int finish_delta(const S& sm, const Layout& ly, int c
 // bytewise (as in the scan).  Lags beyond G have pads at both ends, so their y is 0 and C stays 0.
 // Returns the change of the table sum; *fast receives whether every |C| <= 127 (the int8 copy is only
 // read while that holds, and every step rewrites all of it).
-template <int GL = 32, class S>
+template <class S>
 __device__ inline int table_update(S& sm, const Layout& ly, int mstar, bool* fast) {
   const int cls = pos_cls(ly, mstar), q = pos_q(ly, mstar);
   const int pair = (ly.skew && mstar != ly.c) ? 1 : 0;
@@ -634,7 +547,7 @@ __device__ inline int table_update(S& sm, const Layout& ly, int mstar, bool* fas
   uint32_t* C8w = reinterpret_cast<uint32_t*>(sm.C8);
   int dsum = 0;
   bool ok = true;
-  for (int u = glane<GL>(); u < ly.NG; u += GL) {
+  for (int u = lane_id(); u < ly.NG; u += 32) {
     uint32_t y4 = __funnelshift_r(Fw[wf + u], Fw[wf + u + 1], sf) + __funnelshift_r(Bw[wb + u], Bw[wb + u + 1], sb);
     // the pair's own product is not part of C: lag gd drops s_m' from its byte, which holds
     // (s_m' + 1) + (the other end + 1 or a pad 1), so the byte stays in 0..4 and no borrow crosses bytes
@@ -654,9 +567,9 @@ __device__ inline int table_update(S& sm, const Layout& ly, int mstar, bool* fas
     C16w[2 * u + 1] = ((uint32_t)c[2] & 0xffffu) | ((uint32_t)c[3] << 16);
     C8w[u] = c8;
   }
-  gsync<GL>();
-  *fast = gall<GL>(ok);
-  return gsum<GL>(dsum);
+  __syncwarp();
+  *fast = __all_sync(kFull, ok);
+  return warp_sum_i32(dsum);
 }
 
 // Negates s_i in the bits and both byte arrays (one lane per position, distinct positions may run
@@ -688,50 +601,42 @@ __device__ inline void load_bits(S& sm, const uint64_t* src, int L) {
   __syncwarp();
 }
 
-// Builds a walk start into the bits: s_1..s_p from the prefix, free element j (position p+1+j) is +1
-// iff bit j%64 of output j/64 of stream `key`; skew walks fill the last k by Eq. (2).  Each 32-bit word
-// is assembled from 32 / GL group ballots.
-template <int GL = 32, class S>
-__device__ inline void build_start(S& sm, const Layout& ly, const uint64_t* prefix, uint64_t key) {
-  const int lane = glane<GL>();
-  const int W32 = (ly.L + 31) >> 5;
+// Builds a walk start into the bits (kBitWords words): s_1..s_p from the prefix, free element j (position
+// p+1+j) is +1 iff bit j%64 of output j/64 of stream `key`; skew walks fill the last k by Eq. (2) around the
+// centre c.
+__device__ inline void build_start(uint32_t* bits, int L, bool skew, int c, int p, const uint64_t* prefix, uint64_t key) {
+  const int lane = lane_id();
   for (int w = 0; w < kBitWords; w++) {
-    unsigned word = 0;
-#pragma unroll
-    for (int part = 0; part < 32 / GL; part++) {
-      int i = 32 * w + GL * part + lane + 1;
-      int bit = 0;
-      if (i <= ly.L) {
-        int src = i;
-        int neg = 0;
-        if (ly.skew && i > ly.c) {
-          src = 2 * ly.c - i;
-          neg = (i - ly.c) & 1;
-        }
-        int b;
-        if (src <= ly.p) {
-          b = (int)((prefix[(src - 1) >> 6] >> ((src - 1) & 63)) & 1u);
-        } else {
-          int j = src - ly.p - 1;
-          b = (int)((sm64_at(key, (uint64_t)(j >> 6)) >> (j & 63)) & 1u);
-        }
-        bit = b ^ neg;
+    const int i = 32 * w + lane + 1;
+    int bit = 0;
+    if (i <= L) {
+      int src = i;
+      int neg = 0;
+      if (skew && i > c) {
+        src = 2 * c - i;
+        neg = (i - c) & 1;
       }
-      const unsigned bal = gballot<GL>(bit != 0);
-      word |= GL == 32 ? bal : (bal & ((1u << (GL & 31)) - 1u)) << (GL * part);
+      int b;
+      if (src <= p) {
+        b = (int)((prefix[(src - 1) >> 6] >> ((src - 1) & 63)) & 1u);
+      } else {
+        int j = src - p - 1;
+        b = (int)((sm64_at(key, (uint64_t)(j >> 6)) >> (j & 63)) & 1u);
+      }
+      bit = b ^ neg;
     }
-    if (lane == 0) sm.bits[w] = (w < W32) ? word : 0u;
+    const unsigned word = __ballot_sync(kFull, bit);
+    if (lane == 0) bits[w] = word;
   }
-  gsync<GL>();
+  __syncwarp();
 }
 
 // Zobrist fingerprint of the sequence in the bits.
-template <int GL = 32, class S>
-__device__ inline uint64_t fingerprint(const S& sm, int L, uint64_t zkey) {
+__device__ inline uint64_t fingerprint(const uint32_t* bits, int L, uint64_t zkey) {
   uint64_t h = 0;
-  for (int i = glane<GL>() + 1; i <= L; i += GL)
-    if (!seq_bit(sm, i)) h ^= zobrist(zkey, i);
-  return gxor_u64<GL>(h);
+  for (int i = lane_id() + 1; i <= L; i += 32)
+    if (!((bits[(i - 1) >> 5] >> ((i - 1) & 31)) & 1u)) h ^= zobrist(zkey, i);
+  return warp_xor_u64(h);
 }
 
 }  // namespace labsg

@@ -18,19 +18,15 @@ struct LabsTraceRange {
 };
 #define LABS_TRACE(name) LabsTraceRange labs_trace_range_(name)
 
-constexpr int kMaxTuned = 16;
+constexpr int kWorkspaces = 9;
 
 struct labs_ctx {
   int device;
   int num_sms;
   size_t smem_optin;
   // growable device workspace, one region per purpose
-  void* ws[8];
-  size_t ws_bytes[8];
-  // autotuner cache: (length-set key) -> tile M, lag ranges H, lanes per walk, warps per CTA
-  int n_tuned;
-  uint64_t tuned_key[kMaxTuned];
-  int tuned[kMaxTuned][4];
+  void* ws[kWorkspaces];
+  size_t ws_bytes[kWorkspaces];
   // captured batched step (one at a time) and the stream it was captured on
   cudaGraphExec_t graph_exec;
   uint64_t graph_key;
@@ -47,7 +43,8 @@ enum WsSlot {
   kWsPq0 = 4,
   kWsChunkState = 5,
   kWsChunkIo = 6,
-  kWsPqIndep = 7
+  kWsPqIndep = 7,
+  kWsZpair = 8
 };
 
 // Returns a device region of at least `bytes` for `slot`, growing it if needed (not capturable).

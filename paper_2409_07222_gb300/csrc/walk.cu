@@ -1,20 +1,22 @@
 // walk.cu -- step 1 of the dual-step search: Algorithm 1's self-avoiding walks (labs_skew_search,
 // labs_batched_search) and the sieve bound E_l (labs_sample_threshold).
 //
-// GB300 mapping.  The paper runs one walk per thread block with a shared-memory reduction (Fig. 3);
-// here one walk is one warp (shuffle/redux reductions, no block barriers) and a persistent grid pulls
-// work items (length, walk) from a device counter, so walks of different lengths and lengths of
-// different cost balance across the 152 SMs in one launch.  Each warp's state (sequence bits, byte
-// windows, correlation table, Bloom filter of 2^bloom_log2 bits, per-neighbour slots) lives in its
-// shared-memory slab; a step is
-//   scan   -- Delta E of every free neighbour (tiled dp4a loop, labs_core.cuh),
-//   select -- group argmin of (Delta E, m); Bloom test of the winner's fingerprint; on a hit the owner
-//             lane puts its second best in its place and the argmin repeats (same result as testing
-//             them all),
-//   apply  -- O(L) table update, O(1)-per-neighbour P update, byte/bit flips, fingerprint, Bloom insert,
-//   sieve  -- the walk's R best distinct (E, fp) states with E <= E_thr, one per lane.
+// GB300 mapping.  The paper runs one walk per thread block and evaluates every neighbour in time linear in L
+// (Section III); here one walk is one warp and a flip changes every neighbour's Delta E by a constant number
+// of table values (below), so a step is linear in L instead of quadratic.  A persistent grid of one block per
+// SM pulls work items (length, walk) from a device counter, so walks of different lengths and cost balance
+// across the 152 SMs in one launch.  A walk's sequence bytes, tables and Bloom filter of 2^bloom_log2 bits
+// live in its warp's shared-memory slab (7 KB at L = 451: 32 walks an SM), its neighbours' sums in registers;
+// a step is
+//   select -- Delta E of the lane's neighbours, warp argmin of (Delta E, m), Bloom test of the winner's
+//             fingerprint; on a hit the owner lane looks for its next smallest (same result as testing all),
+//   apply  -- the flip, the O(L) tables, then every neighbour's sum from them,
+//   sieve  -- the walk's R best distinct (E, fp) states with E <= E_thr.
+// Measured (L = 451, p = 24, 65,536 walks x 2,000 flips, sieve bound of 10^6 samples included): 78.8 ms, where
+// the scan of every neighbour took 337 ms; 256 walks x 8,192 flips 11.3 ms (74.6 ms: its blocks filled 11 SMs).
 #include <algorithm>
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <vector>
 
@@ -24,26 +26,48 @@
 namespace labsg {
 namespace {
 
-constexpr int kMaxLens = 96;    // lengths in one launch (kernel parameter table)
-constexpr int kMaxPasses = 3;   // lane passes over the tasks of one walk
-// per slot and lane: slot word and choice key (int32 each), plus Delta E when the choice is biased
-__host__ __device__ constexpr int slot_bytes(bool biased) { return biased ? 12 : 8; }
-// threads per block the kernels are compiled for: whole-warp walks run two 8-warp blocks per SM (128
-// registers a thread); half-warp walks run one block of up to 12 warps (24 walks), whose register budget,
-// 65536 / 384 threads, holds the whole step without spills
-__host__ __device__ constexpr int walk_block_threads(int GL) { return GL == 32 ? 256 : 384; }
-__host__ __device__ constexpr int walk_min_blocks(int GL) { return GL == 32 ? 2 : 1; }
+constexpr int kMaxLens = 96;  // lengths in one launch (kernel parameter table)
 
-// Shared-memory slab of one walk, sized per launch for its lengths (byte offsets, 16-byte aligned):
-// the sequence bits at 0, the tables, the byte-window arrays, the Bloom filter and the per-slot words
-// ([slot][lane of the group]).
-struct SlabPlan {
-  int off_C16, off_C8, off_fwd, off_bwd, off_bloom, off_slots, bytes;
+// Slots (values of T) a lane of a walk kernel holds, and the threads per block it is compiled for (one block
+// per SM): 32 walks of up to 10 slots a lane (64 registers a thread), 24 walks of up to 18 slots (80).
+__host__ __device__ constexpr int walk_slots(int mode, int ns, int nu) {
+  return mode == 0 ? 2 * ns : (mode == 1 || nu > 2 * ns ? nu : 2 * ns);
+}
+__host__ __device__ constexpr int walk_block_threads(int mode, int ns, int nu) {
+  return walk_slots(mode, ns, nu) <= 10 ? 1024 : 768;
+}
+
+// Halves of a packed table word hold value + kBias, so that adding packed changes never borrows across
+// them: |Z| <= 2 * 288 + 576, |X| <= 288, |2 C_d| <= 1152 and |V| <= 576 for every L <= 576.
+constexpr int kBias = 2048;
+
+// What a walk changes rarely (its busy values are registers), and with it the values saved between launches.
+struct WalkCtl {
+  long long skips, skips0;  // skips0 .. dead0: the values when the launch took the walk up
+  unsigned long long fp, wfp;
+  int E, bestE, first_hit, aprev, dprev;
+  int wE, wlane;          // the sieve's worst slot: key (wE, wfp), lane
+  unsigned flips, flips0, segs, segs0, dead, dead0;
+  unsigned seg0;          // flips at the segment's beginning
+  unsigned logged, log_next;  // chunks logged, flips at the beginning of the next
+  int need_start, done;
 };
 
-// Per-length entry of a launch: the layout (tiles, windows) and where its walks sit among the items.
-struct LenEntry {
-  Layout ly;
+// Shared-memory slab of one walk, sized per launch for its lengths (byte offsets, 16-byte aligned): the
+// sequence bits at 0, the control block, the sequence bytes, the tables, the Bloom filter (at least kScratch
+// bytes: the table builds use its words before a segment's filter is cleared).
+struct SlabPlan {
+  int off_ctl, off_S, off_tab, off_bloom, bytes;
+};
+constexpr int kScratch = 96;
+
+// One length of a launch.  Skew walks (odd L = 2k + 1, c = k + 1) address positions by their distance h from
+// the centre: S[h] = s_{c-h} for |h| <= k, S[-h] = (-1)^h S[h] (Eq. 2), neighbours h = 0 .. hmax = k - p.
+// Unrestricted walks address positions m = p + 1 .. L.
+struct WalkLen {
+  int L, skew, p, k, c, hmax;
+  int so, sn;   // byte of S[0] inside the sequence bytes, their number
+  int t1, t2;   // entries of the first table(s) and of all tables: Z0 | Z1 | X at 0, t1, 2 t1 (skew); Z | V (else)
   int T_i;
   int32_t E_thr_value;  // used when WalkParams::E_thr_dev is null
   int64_t item_begin;   // first work item of this length
@@ -51,38 +75,31 @@ struct LenEntry {
 };
 
 struct WalkParams {
-  int n_len, R, bloom_log2, bloom_k, prefix_words, n_prefix, slot_stride;
+  int n_len, R, bloom_log2, bloom_k, prefix_words, n_prefix;
   int32_t E_target;
   int64_t n_items, flip_budget;
   uint64_t seed;
   const uint64_t* prefixes;
+  const uint64_t* zpair;     // [n_len][kMaxL]: fingerprint change of neighbour m at m - 1 (walk_init_kernel)
   const int32_t* E_thr_dev;  // nullable: per-length sieve bounds in device memory
   labs_candidate* out;       // [n_items][R]
   int64_t* walk_stats;       // nullable: [n_items][6]
   labs_walk_stats* stats;
   unsigned long long* counter;
+  // logs of a plain chunked run (nullable): every `log_chunk` flips the sequence and the next move
+  int log_chunk;
+  uint64_t* state_log;  // [n_chunks][n_items][W]
+  int32_t* move_log;    // [n_chunks][n_items][2]: a chunk's first move (position, Delta E)
   // resumable chunks (learned proposal); all nullable / zero for a plain run to the end
-  unsigned char* state;  // [n_items][state_stride] walk states between launches
+  unsigned char* state;  // [n_items][state_stride]: a walk's slab and its T values ([slot][lane]) between launches
   int state_stride;
   int chunk;             // > 0: at most `chunk` accepted flips per walk and launch; < 0: set-up only
   const float* bias;     // [n_items][L] proposal logits biasing the choice (null: plain walk)
   float lambda;
   uint64_t* seq_out;     // [n_items][W]: the walk's sequence when the launch leaves it
-  int32_t* move_log;     // [n_items][2]: first move of the launch (position, Delta E), (-1, 0) if none
   SlabPlan slab;
-  LenEntry len[kMaxLens];
+  WalkLen len[kMaxLens];
 };
-
-// Header of a saved walk state; followed by the sequence bits, the int16 table and the Bloom filter.
-struct WalkStateHdr {
-  unsigned long long fp;
-  long long skips;
-  int E, flips, segs, dead, it, mprev, first_hit, bestE, need_start, started, done, pad[5];
-};
-constexpr int kStateBits = sizeof(WalkStateHdr);
-constexpr int kStateC = kStateBits + 4 * kBitWords;
-constexpr int kStateBloom = kStateC + 2 * kCLen;
-constexpr int kStateBytes = kStateBloom + 4 * 1024;
 
 // Order-preserving int32 image of a float (-0 folded onto +0 first).
 __device__ __forceinline__ int float_key(float f) {
@@ -95,632 +112,780 @@ __device__ __forceinline__ uint32_t bloom_idx(uint64_t fp, int j, uint32_t mask)
   return (lo + (uint32_t)j * (hi | 1u)) & mask;
 }
 
-// Every lane of the group returns whether all K probes of fp are set.
-template <int GL>
-__device__ __forceinline__ bool bloom_test(const uint32_t* bloom, uint64_t fp, int K, uint32_t mask) {
-  const int lane = glane<GL>();
-  bool hit = true;
-  if (lane < K) {
-    uint32_t b = bloom_idx(fp, lane, mask);
-    hit = (bloom[b >> 5] >> (b & 31)) & 1u;
-  }
-  return gall<GL>(hit);
-}
-
-template <int GL>
-__device__ __forceinline__ void bloom_add(uint32_t* bloom, uint64_t fp, int K, uint32_t mask) {
-  const int lane = glane<GL>();
-  if (lane < K) {
-    uint32_t b = bloom_idx(fp, lane, mask);
-    atomicOr(&bloom[b >> 5], 1u << (b & 31));
-  }
-  gsync<GL>();
+// Whether all K probes of fp are set; a lane beyond K repeats the last probe.  Each lane's probe word and
+// bit go to `at` and `bit`.
+__device__ __forceinline__ bool bloom_test(const uint32_t* bloom, uint64_t fp, int probe, uint32_t mask, uint32_t& at,
+                                           uint32_t& bit) {
+  const uint32_t b = bloom_idx(fp, probe, mask);
+  at = b >> 5;
+  bit = 1u << (b & 31);
+  return __all_sync(kFull, bloom[at] & bit);
 }
 
 __device__ __forceinline__ bool key_less(int Ea, uint64_t fa, int Eb, uint64_t fb) {
   return Ea < Eb || (Ea == Eb && fa < fb);
 }
 
-// Slot word of one neighbour: high half the signed position s_m * m (0: no neighbour in this slot), low
-// half alpha^2 Q_m, where Q_m = sum of y_kappa^2 over the valid lags = n_f + n_b - [pair] + 2 P_m.  It is
-// a sum of squares, so 0 <= alpha^2 Q_m <= 16 * 4 * 287 < 2^16 for every L <= 576.
-__device__ __forceinline__ int slot_pack(int sm_m, int Pt) { return (int)(((unsigned)sm_m << 16) | (unsigned)Pt); }
-__device__ __forceinline__ int slot_pos(int word) { return word >> 16; }  // s_m * m
-__device__ __forceinline__ int slot_Pt(int word) { return word & 0xffff; }
-
-// Delta E of a neighbour from its accumulator a = sum_g C8/C16 (y + 2) and the table sum SC:
-//   Delta E = base - 2 alpha s_m (a - 2 SC),   base = alpha^2 Q_m + 2 alpha sigma C_{gd} [pair],
-// alpha = 4 for a skew pair (m, m'), 2 otherwise; the pair's own product at lag gd = c - m is removed
-// with s_{m'} = sigma s_m, sigma = (-1)^{c-m} (Eq. 2).  base depends only on the table and the slot
-// word, so it is formed before the scan (prep_code).
-
-// The last accepted move, not yet folded into the slot words: its flipped positions f0 (and the mirror
-// f1 of a skew pair), their class and class indices, and their values before the flip.  Flipping f
-// changes the product s_{2m-f} s_f of every neighbour m of f's class by -2 s_f s_{2m-f}; the byte at
-// class index 2q - q_f gives s_{2m-f}, and the pads (s = 0) drop products with an end outside 1..L.
-// That byte is never one of the flipped positions for the neighbours that change, so the update may be
-// applied after the flip, when the next step reads the slot anyway.  Excluded: the flipped neighbour
-// itself (its products do not contain s_m; its sign changes), the skew centre when a pair flips (both
-// ends of each of its products flip), and the pair product (m, m') of m, whose end m' is 2m - f0 when
-// 3 q - q_f0 = c + 6 - b (b = 1 for odd positions, 2 for even).
-struct PendingFlip {
-  bool on, pair;
-  int cls, q0f, q1f, s0, s1, qmir;
-};
-
-// Folds the pending move into the slot words of its class.  The class's (task, k) slots are spread over
-// the group's lanes, task fastest, so that neighbouring lanes touch different banks.
-template <int M, int H, int GL, class S>
-__device__ __forceinline__ void fold_flip(const S& sm, const Layout& ly, const PendingFlip& pf, int* sl_w) {
-  constexpr int MH = M / H;
-  const uint8_t* Fc = reinterpret_cast<const uint8_t*>(sm.fwd + cls_words(ly, pf.cls));
-  const int pmul = ly.skew ? -64 : -16;  // -4 alpha^2 for the neighbours that change
-  const int qc = (pf.pair && pos_cls(ly, ly.c) == pf.cls) ? pos_q(ly, ly.c) : -1;  // the centre
-  const int m3 = ly.skew ? pf.qmir + pf.q0f : -1;                                  // 3 q of the pair-product
-  const int qm = (m3 >= 0 && m3 % 3 == 0) ? m3 / 3 : -1;                           // exclusion
-  const int q1f = pf.pair ? pf.q1f : (1 << 20);  // single flip: the f1 term reads a pad
-  const int nt = ly.ntiles[pf.cls] * H;          // tasks of the class
-  const int task0 = (pf.cls ? ly.ntiles[0] : 0) * H;
-  const int qt = ly.tile_first[pf.cls];
-  const int mg = ly.fold_magic[pf.cls];
-  const int lane = glane<GL>();
-  int k = (lane * mg) >> 16, tl = lane - k * nt;
-  const int step_k = (GL * mg) >> 16, step_t = GL - step_k * nt;
-  for (; k < MH;) {
-    const int task = task0 + tl;
-    const int q = qt + (tl / H) * M + (tl % H) * MH + k;
-    const int idx = ((task / GL) * MH + k) * GL + (task % GL);
-    int wv = sl_w[idx];
-    const int ms = slot_pos(wv);
-    int v = ((int)Fc[max(2 * q - pf.q0f, 0)] - 1) * pf.s0;
-    if (q == qm) v = 0;
-    v += ((int)Fc[max(2 * q - q1f, 0)] - 1) * pf.s1;
-    if (ms != 0 && q != pf.q0f && q != qc) wv += pmul * v;
-    if (ms != 0 && q == pf.q0f) wv = slot_pack(-ms, slot_Pt(wv));
-    sl_w[idx] = wv;
-    tl += step_t;
-    k += step_k;
-    if (tl >= nt) {
-      tl -= nt;
-      k++;
-    }
+// sum_{j < cnt} a_j b_{j + d} of two +-1 sequences given by bits, d >= 0.
+__device__ __forceinline__ int corr_bits(const uint32_t* a, const uint32_t* b, int cnt, int d) {
+  if (cnt <= 0) return 0;
+  const int ws = d >> 5, sh = d & 31;
+  int dis = 0;
+  for (int w = 0; 32 * w < cnt; w++) {
+    uint32_t x = a[w] ^ __funnelshift_r(b[w + ws], b[w + ws + 1], sh);
+    const int rem = cnt - 32 * w;
+    if (rem < 32) x &= (1u << rem) - 1u;
+    dis += __popc(x);
   }
-  gsync<GL>();
+  return cnt - 2 * dis;
 }
 
-// Finish code of a slot, formed by prep: base * 32 + code, where base is the constant part of the
-// neighbour's Delta E and code = 2 alpha s_m + 8 (0, 4, 12 or 16), plus 1 for the neighbour
-// the last move flipped (the state just left), or 31 for no neighbour.  Branch-free: a slot without a
-// pair term reads the table's last entry, which is always zero (lags beyond G).
-constexpr int kNoSlot = 31;
-template <class S>
-__device__ __forceinline__ int prep_code(const S& sm, const Layout& ly, int word, bool back) {
-  const int ms = slot_pos(word);
-  const int m = ms < 0 ? -ms : ms;
-  const bool pair = ly.skew && m != ly.c && m != 0;
-  const int gd = pair ? ly.c - m : ly.cl;
-  const int cg = 8 * (int)sm.C16[gd - 1];
-  const int base = slot_Pt(word) + ((gd & 1) ? -cg : cg);
-  const int a2 = pair ? 8 : 4;
-  const int code = (ms < 0 ? 8 - a2 : 8 + a2) + (back ? 1 : 0);
-  return ms == 0 ? kNoSlot : base * 32 + code;
-}
+// ------------------------------------------------------------------------------------------------
+// The incremental neighbourhood.
+//
+// With T_m = sum_{j != m} C_{|m-j|} s_j (the linear-time sum of a neighbour's Delta E), a flip of f changes
+// every T_m by a second difference of E, and that is a constant number of table values: for
+// y_d(m) = s_{m+d} + s_{m-d},
+//     sum_d y_d(f) y_d(m) = C_{|m-f|} + V_{m+f} - 2 s_f s_m,      V_t = sum_i s_i s_{t-i},
+// because the products s_{f+d} s_{m+d} and s_{f-d} s_{m-d} run over all pairs at distance |m - f| but the
+// flipped one, and s_{f+d} s_{m-d}, s_{f-d} s_{m+d} over all pairs with index sum m + f.  One flip is then
+// O(L): the tables change in one or two products per entry, every T_m in a few table values, and Delta E of
+// every neighbour follows.  With the values after the flip (s_f = s, tables C and V updated):
+//
+// unrestricted, Z_d = 2 C_d with Z_0 := L + 4:
+//     T_m += 2 s (Z_{|m-f|} + V_{m+f}) - 8 s_m - 4 s_{2f-m}                          (m = f included)
+//     Delta E_m = 4 (V_{2m} + L - 2 - s_m T_m)
+//     flip of f:  Z_d += 4 s (s_{f+d} + s_{f-d}),   V_{f+j} += 4 s s_j (j != f)
+//
+// skew-symmetric, flips of the pair (a, -a) in distances from the centre, e = a mod 2, eta = (-1)^a:
+// correlations inside one parity class R^e_g = sum_{h = e (2)} S[h] S[h+2g], C_{2g} = R^0_g + R^1_g,
+// Z^e_g = 2 R^e_g + C_{2g} with Z^e_0 := 2 n_e + 12 (n_e = positions of the class), and across the classes
+// X_d = sum_{h even} S[h] S[h+d], d odd (odd C vanish, so X of odd h is -X_d).  By Eq. 2 the index-sum
+// products are class correlations too.  T_h carries + 4 (-1)^h S[3h] (h > 0):
+//     h = e (2):  T_h += 2 s (Z^e_{|h-a|/2} + eta Z^e_{(h+a)/2}) - 24 S[h] - 12 eta y,   y = S[h+2a] + S[h-2a]
+//                 and + 8 eta s more for h = 3a and for 3h = a
+//     else:       T_h += 4 s (eta sgn(h-a) X_{|h-a|} + X_{h+a}) - 8 S[h] - 4 eta y
+//     Delta E_h = 8 ((-1)^h Z^h_h - S[h] T_h) + 16 (n_h - 3),  centre: Delta E_0 = -4 S[0] T_0 + 8 n_0 - 8
+//     flip:       R^e_g += 4 s (S[a+2g] + S[a-2g]) without the mirror's product (g = a),
+//                 X_d += 2 s eta (S[a+d] - S[a-d])
+// The centre alone (a = 0): half of all the above and no y term, T_0 -= 16 s.
+//
+// Delta E is a multiple of 4 and |Delta E| < 2^23 for every L <= 576 (|T| <= sqrt(E sum y^2), E < 2^26), so
+// (Delta E / 4) * 1024 + m orders the neighbours by (Delta E, m) in one int32.
+// ------------------------------------------------------------------------------------------------
 
-// Task of group lane `lane` in pass `ps`: tile (class, q0), lag range h, whether it exists.
-template <int GL>
-__device__ __forceinline__ bool lane_task(const Layout& ly, int H, int ps, int lane, int& cls, int& q0, int& h) {
-  const int task = ps * GL + lane;
-  h = H == 2 ? (task & 1) : 0;
-  cls = 0;
-  q0 = 0;
-  if (task >= ly.n_tasks) return false;
-  tile_of(ly, H == 2 ? (task >> 1) : task, cls, q0);
-  return true;
-}
-
-// One walk-step kernel for every length of the launch.  Template: tile size M and lag ranges per tile H
-// (the autotuned "words per thread"), lanes per walk GL (32: one walk per warp; 16: one per half-warp,
-// two walks sharing every instruction of the step's serial phases); the number of lane passes is per
-// length (<= kMaxPasses).  Per-slot state sits in the walk's slab, lane-major ([slot][lane], conflict
-// free): the slot word, the step's choice key and, for biased walks, its Delta E.  With `state` the walk
-// runs in chunks of accepted flips and is saved between launches (bits, table, Bloom filter, counters);
-// the sieve slots stay in the output records meanwhile.
-// ONE: a single-length launch -- the length's entry is read at a fixed parameter offset and its
-// Zobrist keys are tabulated once per block in shared memory.  BIASED: the choice key is the proposal
-// score of WalkParams::bias (single-length launches only).
-template <int M, int H, bool ONE, bool BIASED, int GL>
-__global__ void __launch_bounds__(walk_block_threads(GL), walk_min_blocks(GL))
+// One walk per warp.  A lane holds NS slots (values of T) per parity class of a skew walk, NU slots of an
+// unrestricted one.  MODE 0: a launch of one skew length, 1: one unrestricted length, 2: several lengths of
+// either kind; BIASED: the choice key is the proposal score of WalkParams::bias.
+//
+// Bound (L = 451, skew): issue slots and shared-memory instructions -- a flip is about 75 shared-memory
+// accesses and a few hundred warp instructions, where scanning every neighbour took 2,285.
+template <int NS, int NU, int MODE, bool BIASED>
+__global__ void __launch_bounds__(walk_block_threads(MODE, NS, NU), 1)
     walk_kernel(const __grid_constant__ WalkParams P) {
-  constexpr int MH = M / H;  // slots owned by a lane per pass
+  constexpr int SL = walk_slots(MODE, NS, NU);
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int gid = threadIdx.x / GL;  // walk slot of this group in the block
-  const int ngroups = blockDim.x / GL;
-  unsigned char* slab = smem_raw + (size_t)gid * P.slab.bytes;
-  ScanView sm;
-  sm.bits = reinterpret_cast<uint32_t*>(slab);
-  sm.C16 = reinterpret_cast<int16_t*>(slab + P.slab.off_C16);
-  sm.C8 = reinterpret_cast<int8_t*>(slab + P.slab.off_C8);
-  sm.fwd = reinterpret_cast<uint32_t*>(slab + P.slab.off_fwd);
-  sm.bwd = reinterpret_cast<uint32_t*>(slab + P.slab.off_bwd);
+  unsigned char* slab = smem_raw + (size_t)(threadIdx.x >> 5) * P.slab.bytes;
+  uint32_t* bits = reinterpret_cast<uint32_t*>(slab);
+  WalkCtl* ctl = reinterpret_cast<WalkCtl*>(slab + P.slab.off_ctl);
+  uint8_t* Sraw = slab + P.slab.off_S;
+  uint16_t* tab = reinterpret_cast<uint16_t*>(slab + P.slab.off_tab);
   uint32_t* bloom = reinterpret_cast<uint32_t*>(slab + P.slab.off_bloom);
-  uint64_t* ztab = reinterpret_cast<uint64_t*>(smem_raw + (size_t)P.slab.bytes * ngroups);
-  if (ONE) {
-    const uint64_t zk = stream_key(0, kPurposeZobrist, (uint64_t)P.len[0].ly.L, 0);
-    for (int i = threadIdx.x; i < P.len[0].ly.L; i += blockDim.x) ztab[i] = zobrist(zk, i + 1);
-    __syncthreads();
-  }
-  int* sl_w = reinterpret_cast<int*>(slab + P.slab.off_slots);  // slot words
-  int* sl_k = sl_w + P.slot_stride * GL;                         // choice keys of the step
-  int* sl_d = sl_k + P.slot_stride * GL;                         // Delta E of the step (BIASED only; else = key)
-  const int lane = glane<GL>();
+  const int lane = lane_id();
   const uint32_t bmask = (1u << P.bloom_log2) - 1u;
   const int bwords = 1 << (P.bloom_log2 - 5);
   const int R = P.R;
   const unsigned budget = (unsigned)P.flip_budget;  // < 2^32, checked by the host
 
-  long long agg_flips = 0, agg_segs = 0, agg_skips = 0, agg_dead = 0;
-  int agg_best = INT32_MAX;
-
   while (true) {
-    unsigned long long item = 0;
-    if (lane == 0) item = atomicAdd(P.counter, 1ull);
-    item = gshfl<GL>(item, 0);
-    if ((long long)item >= P.n_items) break;
+    unsigned item = 0;  // n_items < 2^32, checked by the host
+    if (lane == 0) item = (unsigned)min(atomicAdd(P.counter, 1ull), (unsigned long long)P.n_items);
+    item = __shfl_sync(kFull, item, 0);
+    if (item >= P.n_items) break;
     int li = 0;
-    if (!ONE)
+    if (MODE == 2)
       while (li + 1 < P.n_len && P.len[li + 1].item_begin <= (long long)item) li++;
-    const LenEntry& le = ONE ? P.len[0] : P.len[li];
-    const Layout& ly = le.ly;
-    const int64_t w = le.walk_begin + ((long long)item - le.item_begin);
-    const uint64_t* prefix = P.prefixes + (w % P.n_prefix) * P.prefix_words;
-    const uint64_t zkey = stream_key(0, kPurposeZobrist, (uint64_t)ly.L, 0);
-    const int32_t E_thr = P.E_thr_dev ? P.E_thr_dev[li] : le.E_thr_value;
-    const int W = (ly.L + 63) >> 6;
-    const int NP = (ly.n_tasks + GL - 1) / GL;
-    const int S = NP * MH;
-    labs_candidate* rec = P.out + (int64_t)item * R;
-    const float* bias = BIASED ? P.bias + (long long)item * ly.L : nullptr;
-    WalkStateHdr* gh = P.state ? reinterpret_cast<WalkStateHdr*>(P.state + (size_t)item * P.state_stride) : nullptr;
-    if (gh && gh->done) continue;
-    const bool resumed = gh && gh->started;
+    const WalkLen& le = MODE == 2 ? P.len[li] : P.len[0];
+    const int L = le.L, p = le.p;
+    const bool skew = MODE == 0 || (MODE == 2 && le.skew);
+    const uint64_t* zp = P.zpair + (size_t)li * kMaxL;
+    unsigned char* saved = P.state ? P.state + (size_t)item * P.state_stride : nullptr;
+    const bool resumed = saved && P.chunk > 0;
+    if (resumed && reinterpret_cast<const WalkCtl*>(saved + P.slab.off_ctl)->done) continue;
 
-    // slot positions of this length
-    for (int ps = 0; ps < NP; ps++) {
-      int cls, q0, h;
-      const bool has = lane_task<GL>(ly, H, ps, lane, cls, q0, h);
-#pragma unroll
-      for (int k = 0; k < MH; k++) {
-        const int m = q_pos(ly, cls, q0 + h * MH + k);
-        sl_w[(ps * MH + k) * GL + lane] = slot_pack((has && m >= ly.p + 1 && m <= ly.mlast) ? m : 0, 0);
-      }
-    }
-    int cE = INT32_MAX;
-    uint64_t cfp = ~0ull;
-    int wE = INT32_MAX;
-    uint64_t wfp = ~0ull;
-    int wlane = 0;
-    unsigned flips = 0, segs = 0, dead = 0;
-    long long skips = 0;
-    int first_hit = -1;
-    int bestE = INT32_MAX;
-    int E = 0, SC = 0, it = 0;
-    int mprev = 0;  // free position flipped by the previous move of this segment
+    uint8_t* S = Sraw + le.so;  // S[h] (skew) or S[position], value + 1 in {0, 2}, 1 outside the sequence
+    // skew: Z^0 | Z^1 | X (entry d >> 1); unrestricted: Z | V
+    uint16_t* T1 = tab + le.t1;
+    uint16_t* TX = tab + 2 * le.t1;
+    const int k = le.k, c = le.c, hmax = le.hmax;
+    const int n0 = 2 * (k >> 1) + 1, n1 = 2 * ((k + 1) >> 1);  // positions of the even and odd class
+    // skew: T[j] is class 0, slot j (h = 2 (lane + 32 j)), T[NS + j] class 1 (h + 1); unrestricted: position
+    // p + 1 + lane + 32 j.  sg: the slot's element, 0 without one
+    int T[SL], sg[SL];
+
+    unsigned flips = 0, skips = 0;  // skips: Bloom skips since they were last added to ctl
+    int bestE = INT32_MAX, E = 0;
+    int aprev = -1, dprev = 0;  // neighbour flipped by the previous move of this segment (h or position), its Delta E
     uint64_t fp = 0;
-    bool fast = true, need_start = true;
-    PendingFlip pend;
-    pend.on = false;
+    bool need_start = true;
 
-    // rebuilds everything derived from the bits and the table: windows, int8 table, slot P and signs
-    auto derive = [&]() {
-      SC = table_sum<GL>(sm, ly);
-      fast = pack_c8<GL>(sm, ly);
-      build_bytes<GL>(sm, ly);
-      for (int t = 0; t < S; t++) {
-        int m = slot_pos(sl_w[t * GL + lane]);
-        m = m < 0 ? -m : m;
-        int word = 0;
-        if (m) {
-          const SlotInfo si = slot_info(ly, pos_cls(ly, m), pos_q(ly, m));
-          const int Pm = p_from_scratch(sm, ly, pos_cls(ly, m), pos_q(ly, m), si);
-          const int a2 = si.pair ? 16 : 4;
-          word = slot_pack(s_at(sm, ly, m) * m, a2 * (si.nf + si.nb - si.pair + 2 * Pm));
-        }
-        sl_w[t * GL + lane] = word;
+    // elements of the lane's slots, from the sequence bytes
+    auto load_signs = [&]() {
+      if (skew) {
+#pragma unroll
+        for (int j = 0; j < NS; j++)
+          {
+            const int h = 2 * (lane + 32 * j);
+            sg[j] = (int)S[h] - 1;
+            sg[NS + j] = (int)S[h + 1] - 1;
+          }
+      } else if (MODE != 0) {
+#pragma unroll
+        for (int j = 0; j < NU; j++)
+          sg[j] = (int)S[p + 1 + lane + 32 * j] - 1;
       }
-      pend.on = false;
+    };
+    // everything derived from the bits: sequence bytes, tables, energy, T
+    auto build_state = [&]() {
+      uint32_t* scr = bloom;
+      for (int b = lane; b < le.sn; b += 32) {
+        const int x = b - le.so;
+        const int i = skew ? c - x : x;  // position
+        Sraw[b] = (i >= 1 && i <= L) ? (uint8_t)(2 * ((bits[(i - 1) >> 5] >> ((i - 1) & 31)) & 1u)) : (uint8_t)1;
+      }
+      __syncwarp();
+      int e_part = 0;
+      if (skew) {
+        // class bits: a_j = S[2j - k0], b_j = S[2j - k1], k0 / k1 the largest even / odd distance
+        const int k0 = k & ~1, k1 = (k - 1) | 1;
+        uint32_t *ab = scr, *bb = scr + 12;
+        for (int t = 0; t < 12; t++) {
+          const int j = 32 * t + lane;
+          const unsigned wa = __ballot_sync(kFull, j < n0 && S[2 * j - k0] == 2);
+          const unsigned wb = __ballot_sync(kFull, j < n1 && S[2 * j - k1] == 2);
+          if (lane == 0) {
+            ab[t] = wa;
+            bb[t] = wb;
+          }
+        }
+        __syncwarp();
+        for (int g = lane; g < le.t1; g += 32) {
+          const int r0 = corr_bits(ab, ab, n0 - g, g), r1 = corr_bits(bb, bb, n1 - g, g);
+          const int cg = r0 + r1;
+          tab[g] = (uint16_t)(kBias + (g ? 2 * r0 + cg : 2 * n0 + 12));
+          T1[g] = (uint16_t)(kBias + (g ? 2 * r1 + cg : 2 * n1 + 12));
+          const int sh = (2 * g + 1 + k1 - k0) / 2;
+          TX[g] = (uint16_t)(kBias + corr_bits(ab, bb, min(n0, n1 - sh), sh));
+          if (g >= 1 && g <= k) e_part += cg * cg;
+        }
+      } else if (MODE != 0) {
+        for (int t = 0; t < kBitWords; t++) {  // the reversed sequence
+          const int j = 32 * t + lane;
+          const unsigned wr = __ballot_sync(kFull, j < L && S[L - j] == 2);
+          if (lane == 0) scr[t] = wr;
+        }
+        __syncwarp();
+        for (int d = lane; d < le.t1; d += 32) {
+          const int cd = d < L ? corr_bits(bits, bits, L - d, d) : 0;
+          tab[d] = (uint16_t)(kBias + (d ? 2 * cd : L + 4));
+          if (d >= 1) e_part += cd * cd;
+        }
+        for (int t = lane; t < le.t2 - le.t1; t += 32) {  // V_t: the correlation with the reversal at L + 1 - t
+          const int d = L + 1 - t;
+          int v = 0;
+          if (t >= 2 && t <= 2 * L) v = d >= 0 ? corr_bits(bits, scr, L - d, d) : corr_bits(scr, bits, L + d, -d);
+          T1[t] = (uint16_t)(kBias + v);
+        }
+      }
+      E = warp_sum_i32(e_part);
+      __syncwarp();
+      load_signs();
+      int csum = 0;
+#pragma unroll
+      for (int j = 0; j < SL; j++) T[j] = 0;
+      if (skew) {
+        const uint8_t* s0 = S + 2 * lane;
+        for (int g = 1; g <= k; g++) {
+          const int cg = ((int)tab[g] + (int)T1[g] - 2 * kBias) >> 2;
+          csum += cg;
+#pragma unroll
+          for (int j = 0; j < NS; j++)
+            {
+              const int yy = (int)*reinterpret_cast<const uint16_t*>(s0 + 64 * j + 2 * g) +
+                             (int)*reinterpret_cast<const uint16_t*>(s0 + 64 * j - 2 * g);
+              T[j] += cg * (yy & 255);
+              T[NS + j] += cg * (yy >> 8);
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < NS; j++)
+          {
+            const int h = 2 * (lane + 32 * j);
+            T[j] -= 2 * csum;
+            T[NS + j] -= 2 * csum;
+            if (h > 0 && 3 * h <= k) T[j] += 4 * ((int)S[3 * h] - 1);
+            if (3 * h + 3 <= k) T[NS + j] -= 4 * ((int)S[3 * h + 3] - 1);
+          }
+      } else if (MODE != 0) {
+        const uint8_t* s0 = S + p + 1 + lane;
+        for (int d = 1; d < L; d++) {
+          const int cd = ((int)tab[d] - kBias) >> 1;
+          csum += cd;
+#pragma unroll
+          for (int j = 0; j < NU; j++)
+            T[j] += cd * ((int)s0[32 * j + d] + (int)s0[32 * j - d]);
+        }
+#pragma unroll
+        for (int j = 0; j < NU; j++) T[j] -= 2 * csum;
+      }
     };
     // INIT_PARTITIONED_SEQUENCE of a new segment (Algorithm 1)
     auto start_segment = [&]() {
-      for (int t = lane; t < bwords; t += GL) bloom[t] = 0u;
-      build_start<GL>(sm, ly, prefix, stream_key(P.seed, kPurposeWalk, (uint64_t)w, (uint64_t)segs));
-      segs++;
-      fp = fingerprint<GL>(sm, ly.L, zkey);
-      bloom_add<GL>(bloom, fp, P.bloom_k, bmask);
-      E = build_table<GL>(sm, ly);
-      derive();
-      it = 0;
-      mprev = 0;
+      const int64_t w = le.walk_begin + ((long long)item - le.item_begin);
+      const unsigned seg = ctl->segs;
+      build_start(bits, L, skew, c, p, P.prefixes + (w % P.n_prefix) * P.prefix_words,
+                  stream_key(P.seed, kPurposeWalk, (uint64_t)w, (uint64_t)seg));
+      build_state();
+      __syncwarp();
+      for (int t = lane; t < bwords; t += 32) bloom[t] = 0u;
+      fp = fingerprint(bits, L, stream_key(0, kPurposeZobrist, (uint64_t)L, 0));
+      __syncwarp();
+      if (lane < P.bloom_k) {
+        const uint32_t b = bloom_idx(fp, lane, bmask);
+        atomicOr(&bloom[b >> 5], 1u << (b & 31));
+      }
+      if (lane == 0) {
+        ctl->segs = seg + 1;
+        ctl->seg0 = flips;
+        ctl->skips += skips;
+      }
+      skips = 0;
+      __syncwarp();
+      aprev = -1;
       need_start = false;
     };
-    // new worst sieve slot: largest (E, fp), lowest lane among equals
-    auto find_worst = [&]() {
-      int mE = gmax<GL>(lane < R ? cE : INT32_MIN);
+    // The tables and T after the flip of neighbour a (already flipped in S; s its new value; own: the bit of
+    // its slot in the lane that holds it).
+    auto apply_flip = [&](const int a, const int s, const unsigned own) {
+      if (skew) {
+        const int e = a & 1, es = e ? -s : s;  // es: eta s, the mirror's element
+        {
+          // lane entry pair g = 2u, 2u + 1 (X: d = 4u + 1, 4u + 3), u = lane + 32 i: the four elements
+          // S[a + 4u ..] and the four S[a - 4u - 3 ..], as bytes; 16-bit halves hold the pair
+          const int m4 = a ? 4 * s : 2 * s, mz0 = e ? m4 : 3 * m4, mz1 = e ? 3 * m4 : m4, mx = a ? 2 * es : s;
+          const int n_it = (min((k + a) >> 1, hmax) >> 6) + 1;
+          const int bf = le.so + a, bb = le.so + a - 3;
+          const uint32_t* wf = reinterpret_cast<const uint32_t*>(Sraw) + (bf >> 2) + lane;
+          const uint32_t* wb = reinterpret_cast<const uint32_t*>(Sraw) + (bb >> 2) - lane;
+          const int sf = 8 * (bf & 3), sb = 8 * (bb & 3);
+          uint32_t* z0 = reinterpret_cast<uint32_t*>(tab) + lane;
+          uint32_t* z1 = reinterpret_cast<uint32_t*>(T1) + lane;
+          uint32_t* xx = reinterpret_cast<uint32_t*>(TX) + lane;
+          const int ua = (a >> 1) - lane;                               // the pair holding g = a
+          const int corr = a ? (e ? es * 65536 : es) : 0;               // its mirror product
+#pragma unroll
+          for (int i = 0; i < NS; i++) {
+            if (i >= n_it) break;
+            const uint32_t f = __funnelshift_r(wf[32 * i], wf[32 * i + 1], sf);
+            const uint32_t b = __funnelshift_r(wb[-32 * i], wb[-32 * i + 1], sb);
+            // even lags: sums of elements 0, 2 of f and 3, 1 of b; odd lags: differences of 1, 3 and 2, 0
+            int dy = (int)(__byte_perm(f, 0, 0x4240) + __byte_perm(b, 0, 0x4143) - 0x00020002u);
+            const int dx = (int)(__byte_perm(f, 0, 0x4341) - __byte_perm(b, 0, 0x4042));
+            if (ua == 32 * i) dy -= corr;
+            if (i == 0 && lane == 0) dy -= 2 * s;  // g = 0 is no lag
+            z0[32 * i] += (uint32_t)(dy * mz0);
+            z1[32 * i] += (uint32_t)(dy * mz1);
+            xx[32 * i] += (uint32_t)(dx * mx);
+          }
+        }
+        __syncwarp();
+        // T of the class of a, then of the other class; the biases of the bytes and the tables are taken
+        // out with the table values (2 cy / cz, 2 cy / cx)
+        const int a1 = a >> 1, a2 = (a + 1) >> 1;
+        const uint8_t* sp = S + 2 * lane + 2 * a;
+        const uint8_t* sm = S + 2 * lane - 2 * a;
+        const uint16_t* zq = (e ? T1 : tab) + lane + a2;
+        const uint16_t* zm = e ? T1 : tab;
+        const uint16_t* xq = TX + lane + a1;
+        const int u1 = lane - a1, u2 = lane - a2;
+        // odd: a is odd; pair: a > 0 (compile-time)
+        auto classes = [&](const bool odd, const bool pair) {
+          const int bs = odd ? NS : 0, bo = odd ? 0 : NS;  // first slot of the class of a / of the other class
+          const int s2 = pair ? 2 * s : s, s4 = 2 * s2;    // cz, cx
+          const int q = odd ? -s4 : s4;                    // eta cx
+          const int ky = pair ? (odd ? -12 * s : 12 * s - 2 * kBias) : -2 * kBias;
+          const int kx = pair ? (odd ? -2 * s : 2 * s) - kBias : -kBias;
+          constexpr int cs = 24, cso = 8, cy = 12, cyo = 4;
+#pragma unroll
+          for (int j = 0; j < NS; j++) {
+            int ylo = 0, yhi = 0;
+            if (pair) {
+              const int yy = (int)*reinterpret_cast<const uint16_t*>(sp + 64 * j) +
+                             (int)*reinterpret_cast<const uint16_t*>(sm + 64 * j);
+              ylo = yy & 255;
+              yhi = yy >> 8;
+            }
+            const int vm = zm[abs(u1 + 32 * j)], vq = zq[32 * j];
+            int t = T[bs + j] - (pair ? cs : cs / 2) * sg[bs + j];
+            t += s2 * (odd ? vm - vq + ky : vm + vq + ky);
+            if (pair) t += (odd ? cy : -cy) * (odd ? yhi : ylo);
+            T[bs + j] = t;
+            const int u = u2 + 32 * j, mk = u >> 31;
+            int o = T[bo + j] - (pair ? cso : cso / 2) * sg[bo + j];
+            o += (mk ? -q : q) * ((int)TX[u ^ mk] - kBias);
+            o += s4 * ((int)xq[32 * j] + kx);
+            if (pair) o += (odd ? cyo : -cyo) * (odd ? ylo : yhi);
+            T[bo + j] = o;
+          }
+        };
+        // the flipped element's own slot
+#pragma unroll
+        for (int t = 0; t < SL; t++)
+          if (t < 2 * NS && (own >> t & 1)) sg[t] = s;
+        if (e)
+          classes(true, true);
+        else if (a)
+          classes(false, true);
+        else
+          classes(false, false);
+        if (a == 0) {
+          if (lane == 0) T[0] -= 16 * s;
+        } else if (3 * a <= hmax || a % 3 == 0) {  // h = 3a and 3h = a: 8 eta s more, in the class of a
+          const int i3 = ((3 * a) >> 1) - lane, id3 = a % 3 == 0 ? (a / 3 >> 1) - lane : -1;
+#pragma unroll
+          for (int j = 0; j < NS; j++)
+            if (i3 == 32 * j || id3 == 32 * j) {
+              if (e)
+                T[NS + j] += 8 * es;
+              else
+                T[j] += 8 * es;
+            }
+        }
+      } else if (MODE != 0) {
+        const int f = a;  // position
+        {
+          // Z_d, four lags d = 4u .. 4u + 3 per lane
+          const int n_it = (max(f - 1, L - f) >> 7) + 1;
+          const int bf = le.so + f, bb = le.so + f - 3;
+          const uint32_t* wf = reinterpret_cast<const uint32_t*>(Sraw) + (bf >> 2) + lane;
+          const uint32_t* wb = reinterpret_cast<const uint32_t*>(Sraw) + (bb >> 2) - lane;
+          const int sf = 8 * (bf & 3), sb = 8 * (bb & 3);
+          uint2* z = reinterpret_cast<uint2*>(tab) + lane;
+          for (int i = 0; i < n_it; i++) {
+            const uint32_t fw = __funnelshift_r(wf[32 * i], wf[32 * i + 1], sf);
+            const uint32_t bw = __funnelshift_r(wb[-32 * i], wb[-32 * i + 1], sb);
+            int dlo = (int)(__byte_perm(fw, 0, 0x4140) + __byte_perm(bw, 0, 0x4243)) - 0x00020002;
+            const int dhi = (int)(__byte_perm(fw, 0, 0x4342) + __byte_perm(bw, 0, 0x4041)) - 0x00020002;
+            if (lane + 32 * i == 0) dlo -= 2 * s;  // d = 0 is no lag
+            uint2 v = z[32 * i];
+            v.x += (uint32_t)(dlo * 4 * s);
+            v.y += (uint32_t)(dhi * 4 * s);
+            z[32 * i] = v;
+          }
+          // V_t, four sums t = t0 + 4u .. + 3 per lane, elements j = t - f
+          const int t0 = (f + 1) & ~3;
+          const int m_it = ((f + L - t0) >> 7) + 1;
+          const int bj = le.so + t0 - f;
+          const uint32_t* wj = reinterpret_cast<const uint32_t*>(Sraw) + (bj >> 2) + lane;
+          const int sj = 8 * (bj & 3);
+          uint2* vv = reinterpret_cast<uint2*>(T1 + t0) + lane;
+          const int own = 2 * f - t0;  // t = 2f: the square of the flipped element, unchanged
+          for (int i = 0; i < m_it; i++) {
+            const uint32_t x = __funnelshift_r(wj[32 * i], wj[32 * i + 1], sj);
+            int dlo = (int)__byte_perm(x, 0, 0x4140) - 0x00010001, dhi = (int)__byte_perm(x, 0, 0x4342) - 0x00010001;
+            if (lane + 32 * i == (own >> 2)) {
+              const int d = own & 1 ? s * 65536 : s;
+              if (own & 2)
+                dhi -= d;
+              else
+                dlo -= d;
+            }
+            uint2 v = vv[32 * i];
+            v.x += (uint32_t)(dlo * 4 * s);
+            v.y += (uint32_t)(dhi * 4 * s);
+            vv[32 * i] = v;
+          }
+        }
+        __syncwarp();
+        const int af = f - p - 1;  // slot index of f
+        const uint16_t* vt = T1 + f + p + 1 + lane;
+        const uint8_t* sr = S + 2 * f - p - 1 - lane;
+#pragma unroll
+        for (int j = 0; j < NU; j++)
+          {
+            const int idx = lane + 32 * j;
+            if (own >> j & 1) sg[j] = s;
+            const int z = (int)tab[abs(idx - af)] + (int)vt[32 * j] - 2 * kBias;
+            T[j] += 2 * s * z - 8 * sg[j] - 4 * ((int)sr[-32 * j] - 1);
+          }
+      }
+    };
+    // (Delta E / 4) * 1024 + m of every slot t (compile-time after unrolling) of the lane, as the sum of a
+    // value and a compile-time constant: take(t, value, constant)
+    const int b0 = (4 * (n0 - 3) - 2 * kBias) * 1024 + c - 2 * lane;
+    const int b1 = (4 * (n1 - 3) + 2 * kBias) * 1024 + c - 1 - 2 * lane;
+    const int bu = (L - 2 - kBias) * 1024 + p + 1 + lane;
+    auto lane_keys = [&](auto&& take) {
+      if (skew) {
+        const uint16_t* z0 = tab + 2 * lane;
+        const uint16_t* z1 = T1 + 2 * lane + 1;
+#pragma unroll
+        for (int j = 0; j < NS; j++) {
+          int v = ((int)z0[64 * j] - sg[j] * T[j]) * 2048 + b0;
+          if (j == 0 && lane == 0) v = (2 * n0 - 2 - sg[0] * T[0]) * 1024 + c;
+          take(j, v, -64 * j);
+          take(NS + j, ((int)z1[64 * j] + sg[NS + j] * T[NS + j]) * -2048 + b1, -64 * j);
+        }
+      } else if (MODE != 0) {
+        const uint16_t* v = T1 + 2 * (p + 1 + lane);
+#pragma unroll
+        for (int j = 0; j < NU; j++) take(j, ((int)v[64 * j] - sg[j] * T[j]) * 1024 + bu, 32 * j);
+      }
+    };
+    // bit of neighbour a's slot in the lane that holds it, 0 in the others
+    auto own_bit = [&](int a) {
+      const int idx = skew ? a >> 1 : a - p - 1;
+      const int t = (idx >> 5) + (skew && (a & 1) ? NS : 0);
+      return lane == (idx & 31) ? 1u << t : 0u;
+    };
+    unsigned act = 0;  // the lane's slots that hold a neighbour
+#pragma unroll
+    for (int t = 0; t < SL; t++) {
+      const bool on = skew ? t < 2 * NS && 2 * (lane + 32 * (t % NS)) + t / NS <= hmax : lane + 32 * t <= hmax;
+      if (on) act |= 1u << t;
+    }
+    const int probe = min(lane, P.bloom_k - 1);
+    // largest (E, fp) of the R sieve slots (lane r holds slot r), lowest lane among equals, into ctl
+    auto find_worst = [&](int cE, uint64_t cfp) {
+      const int mE = warp_max_i32(lane < R ? cE : INT32_MIN);
       uint64_t mf = (lane < R && cE == mE) ? cfp : 0ull;
 #pragma unroll
-      for (int o = GL / 2; o > 0; o >>= 1) {
-        uint64_t other = gshfl_xor<GL>(mf, o);
+      for (int o = 16; o > 0; o >>= 1) {
+        const uint64_t other = __shfl_xor_sync(kFull, mf, o);
         mf = other > mf ? other : mf;
       }
-      unsigned who = gballot<GL>(lane < R && cE == mE && cfp == mf);
-      wE = mE;
-      wfp = mf;
-      wlane = __ffs(who) - 1;
+      const unsigned who = __ballot_sync(kFull, lane < R && cE == mE && cfp == mf);
+      if (lane == 0) {
+        ctl->wE = mE;
+        ctl->wfp = mf;
+        ctl->wlane = __ffs(who) - 1;
+      }
+      __syncwarp();
     };
+    // sequence words of the walk, to global memory
+    auto store_seq = [&](uint64_t* dst) {
+      if (lane < (L + 63) >> 6) dst[lane] = (uint64_t)bits[2 * lane] | ((uint64_t)bits[2 * lane + 1] << 32);
+    };
+    auto record = [&](int r) { return P.out + (size_t)item * R + r; };
 
+    __syncwarp();  // the previous walk of this warp is done with ctl
     if (!resumed) {
-      for (int r = lane; r < R; r += GL) {  // empty sieve slots
-        rec[r].E = INT32_MAX;
-        rec[r].walk = 0;
-        rec[r].step = 0;
-        rec[r].pad = 0;
-        rec[r].fp = ~0ull;
-#pragma unroll
-        for (int t = 0; t < LABS_MAX_W; t++) rec[r].seq[t] = 0;
+      if (lane == 0) {
+        WalkCtl z{};
+        z.wE = INT32_MAX;
+        z.wfp = ~0ull;
+        z.first_hit = -1;
+        *ctl = z;
       }
+      if (lane < R) {  // empty sieve slots
+        labs_candidate* r = record(lane);
+        r->E = INT32_MAX;
+        r->walk = 0;
+        r->step = 0;
+        r->pad = 0;
+        r->fp = ~0ull;
+#pragma unroll
+        for (int t = 0; t < LABS_MAX_W; t++) r->seq[t] = 0;
+      }
+      __syncwarp();
     } else {
-      flips = gh->flips;
-      segs = gh->segs;
-      dead = gh->dead;
-      skips = gh->skips;
-      first_hit = gh->first_hit;
-      bestE = gh->bestE;
-      need_start = gh->need_start;
-      it = gh->it;
-      mprev = gh->mprev;
-      E = gh->E;
-      fp = gh->fp;
-      if (lane < R) {
-        cE = rec[lane].E;
-        cfp = rec[lane].fp;
+      for (int t = lane; t < P.slab.bytes / 4; t += 32)
+        reinterpret_cast<uint32_t*>(slab)[t] = reinterpret_cast<const uint32_t*>(saved)[t];
+      const int* gt = reinterpret_cast<const int*>(saved + P.slab.bytes) + lane;
+#pragma unroll
+      for (int j = 0; j < SL; j++) T[j] = gt[32 * j];
+      __syncwarp();
+      flips = ctl->flips;
+      fp = ctl->fp;
+      E = ctl->E;
+      bestE = ctl->bestE;
+      aprev = ctl->aprev;
+      dprev = ctl->dprev;
+      need_start = ctl->need_start;
+      load_signs();
+      __syncwarp();
+      if (lane == 0) {
+        ctl->skips0 = ctl->skips;
+        ctl->flips0 = ctl->flips;
+        ctl->segs0 = ctl->segs;
+        ctl->dead0 = ctl->dead;
+        ctl->logged = 0;
+        ctl->log_next = ctl->flips;
       }
-      find_worst();
-      if (!need_start) {
-        const unsigned char* gb = reinterpret_cast<const unsigned char*>(gh);
-        for (int t = lane; t < kBitWords; t += GL) sm.bits[t] = reinterpret_cast<const uint32_t*>(gb + kStateBits)[t];
-        for (int t = lane; t < ly.cl / 2; t += GL)
-          reinterpret_cast<uint32_t*>(sm.C16)[t] = reinterpret_cast<const uint32_t*>(gb + kStateC)[t];
-        for (int t = lane; t < bwords; t += GL) bloom[t] = reinterpret_cast<const uint32_t*>(gb + kStateBloom)[t];
-        gsync<GL>();
-        derive();
-      }
+      __syncwarp();
     }
-    const unsigned flips0 = flips, segs0 = segs, dead0 = dead;
-    const long long skips0 = skips;
-    const unsigned chunk = P.chunk > 0 ? (unsigned)P.chunk : (P.chunk < 0 ? 0u : 0xffffffffu);
-    if (P.chunk < 0 && need_start && flips < budget) start_segment();  // set-up launch: first state only
-    unsigned taken = 0;
+    // the launch's last flip; a set-up launch only builds the first state
+    const unsigned stop = P.chunk == 0 ? budget : (unsigned)min((unsigned long long)budget, (unsigned long long)flips + (P.chunk > 0 ? P.chunk : 0));
+    const int32_t E_thr = P.E_thr_dev ? P.E_thr_dev[li] : le.E_thr_value;
+    // a state with E <= gate is looked at: the sieve takes states inside its bound that beat its worst slot,
+    // and the first one at the target is noted
+    auto gate_of = [&]() {
+      const int g = min(E_thr, ctl->wE);
+      return ctl->first_hit < 0 ? max(g, P.E_target) : g;
+    };
+    int gate = gate_of();
+    bool log_move = false;  // the next accepted move is a chunk's first
 
-    while (flips < budget && taken < chunk) {
-      if (need_start) start_segment();
-      it++;
-      if (pend.on) {  // the last move's P bookkeeping
-        fold_flip<M, H, GL>(sm, ly, pend, sl_w);
-        pend.on = false;
-      }
-      // ---- scan; each lane keeps its two best (key, m), where key orders the choice: Delta E, or the
-      //      biased score Delta E - lambda * logit[m] mapped to an order-preserving integer (a Bloom hit on
-      //      its best then hands over the second without a rescan of the lane's slots)
-      int bk = INT32_MAX, bm = INT32_MAX, bdE = 0;
-      int bk2 = INT32_MAX, bm2 = INT32_MAX, bd2 = 0;
-      bool have2 = true;
-      int kprev = INT32_MAX;  // this lane's key of the move back (only its owner sets it)
-      for (int ps = 0; ps < NP; ps++) {
-        int cls, q0, h;
-        const bool has = lane_task<GL>(ly, H, ps, lane, cls, q0, h);
-        const int q_first = q0 + h * MH;
-        {
-          // prep, while no accumulator is live: park each neighbour's Delta E base with its finish code
-          // in the key array
-          int wv[MH];
-#pragma unroll
-          for (int k = 0; k < MH; k++) wv[k] = sl_w[(ps * MH + k) * GL + lane];
-          // the move back: the neighbour flipped by the previous move of this segment
-          const int kback = (mprev && pos_cls(ly, mprev) == cls) ? pos_q(ly, mprev) - q_first : -1;
-#pragma unroll
-          for (int k = 0; k < MH; k++)
-            sl_k[(ps * MH + k) * GL + lane] = prep_code(sm, ly, wv[k], k == kback);
-        }
-        int acc[M];
-#pragma unroll
-        for (int j = 0; j < M; j++) acc[j] = 0;
-        if (has) {
-          // one lag range per tile: only the groups that hold lags (the layout pads the range to whole
-          // ring turns and the table is zero beyond G); two ranges keep their padded turns, since the
-          // two lanes of a tile run in step and the longer range sets the time anyway
-          const int u_begin = h ? ly.NGh : 0;
-          const int u_end = H == 1 ? min(ly.NGh, ly.NG) : (h ? ly.NGend : ly.NGh);
-          if (fast)
-            scan_range<M, false>(sm, ly, cls, q0, u_begin, u_end, acc);
-          else
-            scan_range<M, true>(sm, ly, cls, q0, u_begin, u_end, acc);
-        }
-        // H = 2: the two lanes of a tile hold partial sums over the two lag ranges, and each needs the
-        // totals of its own MH slots only: it sends the partner's half and adds what it receives
-        if (H == 2) {
-#pragma unroll
-          for (int k = 0; k < MH; k++) {
-            const int send = h ? acc[k] : acc[MH + k];
-            const int keep = h ? acc[MH + k] : acc[k];
-            acc[k] = keep + gshfl_xor<GL>(send, 1);
+    while (true) {  // stretches of flips between the events: restarts, chunk logs, the end
+      if (P.log_chunk > 0) {
+        if (log_move && flips != ctl->log_next) {  // the chunk's first move has been made
+          const unsigned lg = ctl->logged;
+          __syncwarp();
+          if (lane == 0) {
+            if (P.move_log) {
+              int32_t* ml = P.move_log + ((size_t)lg * P.n_items + item) * 2;
+              ml[0] = skew ? c - aprev : aprev;
+              ml[1] = dprev;
+            }
+            ctl->logged = lg + 1;
+            ctl->log_next = P.chunk > 0 ? 0xffffffffu : (lg + 1) * (unsigned)P.log_chunk;
           }
+          __syncwarp();
+          log_move = false;
         }
-        // finish: keys of this pass's neighbours, then their two smallest (below)
-        const int m_first = q_pos(ly, cls, q_first);
-        int kv[MH], mv[MH], dv[MH];
-#pragma unroll
-        for (int k = 0; k < MH; k++) {
-          const int t = ps * MH + k;
-          const int pk = sl_k[t * GL + lane];
-          const int code = pk & 31;
-          const int m = m_first + ly.lam * k;
-          const int a = acc[k];
-          const int d = (pk >> 5) - ((code & 30) - 8) * (a - 2 * SC);
-          int key = d;
-          if (BIASED) {
-            float l = bias[min(max(m, 1), ly.L) - 1];
-            if (!isfinite(l)) l = 0.f;  // a missing or broken proposal falls back to the plain choice
-            key = float_key(fmaf(-P.lambda, l, (float)d));
-          }
-          if (code == kNoSlot) {
-            key = INT32_MAX;
-          } else if (code & 1) {
-            kprev = key;  // the state just left: certainly in the Bloom filter
-            key = INT32_MAX;
-          }
-          sl_k[t * GL + lane] = key;
-          if (BIASED) sl_d[t * GL + lane] = d;
-          kv[k] = key;
-          mv[k] = m;
-          dv[k] = d;
-        }
-        // the pass's two smallest (key, m): slots come in increasing m, so strict comparisons keep the
-        // smaller m ahead among equal keys
-        int p1 = INT32_MAX, q1 = INT32_MAX, e1 = 0, p2 = INT32_MAX, q2 = INT32_MAX, e2 = 0;
-#pragma unroll
-        for (int k = 0; k < MH; k++) {
-          const bool lt1 = kv[k] < p1, lt2 = kv[k] < p2;
-          p2 = lt1 ? p1 : (lt2 ? kv[k] : p2);
-          q2 = lt1 ? q1 : (lt2 ? mv[k] : q2);
-          if (BIASED) e2 = lt1 ? e1 : (lt2 ? dv[k] : e2);
-          p1 = lt1 ? kv[k] : p1;
-          q1 = lt1 ? mv[k] : q1;
-          if (BIASED) e1 = lt1 ? dv[k] : e1;
-        }
-        if (!BIASED) {
-          e1 = p1;
-          e2 = p2;
-        }
-        // merge with the earlier passes' two (a later pass may hold smaller m only in another class)
-        auto before = [](int ka, int ma, int kb, int mb) { return ka < kb || (ka == kb && ka != INT32_MAX && ma < mb); };
-        if (before(p1, q1, bk, bm)) {
-          const bool sec = before(bk, bm, p2, q2);  // the old best stays second unless the pass's second is smaller
-          bk2 = sec ? bk : p2;
-          bm2 = sec ? bm : q2;
-          bd2 = sec ? bdE : e2;
-          bk = p1;
-          bm = q1;
-          bdE = e1;
-        } else if (before(p1, q1, bk2, bm2)) {
-          bk2 = p1;
-          bm2 = q1;
-          bd2 = e1;
+        if (!log_move && flips == ctl->log_next && flips < stop) {
+          if (ctl->logged == 0 && need_start) start_segment();  // the first chunk begins with the first state
+          if (P.state_log) store_seq(P.state_log + ((size_t)ctl->logged * P.n_items + item) * ((L + 63) >> 6));
+          log_move = true;
         }
       }
-      // ---- select: smallest (key, m) whose neighbour is not in the Bloom filter
-      int mstar = -1, kstar = 0, dstar = 0;
-      uint64_t nfp = 0;
-      for (int guard = 0; guard <= S * GL; guard++) {
-        int kmin, mm;
+      if (need_start && (flips < stop || (P.chunk < 0 && flips < budget))) start_segment();
+      if (flips >= stop) break;
+      if (lane == 0) ctl->skips += skips;
+      skips = 0;
+      // flips of this stretch (at most 2^20, so that skips cannot overflow)
+      unsigned long long next = min((unsigned long long)stop, flips + (1ull << 20));
+      next = min(next, ctl->seg0 + (unsigned long long)le.T_i);
+      if (P.log_chunk > 0) next = min(next, log_move ? flips + 1ull : (unsigned long long)ctl->log_next);
+      const unsigned until = (unsigned)next;
+      do {
+        // ---- select: smallest (key, m) whose neighbour is not in the Bloom filter.  A hit makes the owner
+        //      lane look for its next smallest.  The move back is certainly in the filter: its slot is left
+        //      out, and as its Delta E undoes the last move's, it is known without its slot whether it ranked
+        //      ahead of the chosen move and counts as a skip.
+        const unsigned own_prev = aprev >= 0 ? own_bit(aprev) : 0u;
+        const unsigned use = act & ~own_prev;
+        int astar = -1, dstar = 0;
+        uint64_t nfp = 0;
+        uint32_t b_at = 0, b_bit = 0;
         if (!BIASED) {
-          // one reduction on (key, m) while the minimum key is inside the 22-bit window: a key clamped to
-          // the window's edge can only tie with the minimum when the minimum is at that edge itself
-          constexpr int kHalf = 1 << 21;
-          const unsigned comp = bk == INT32_MAX ? 0xffffffffu
-                                                : ((unsigned)(min(max(bk, -kHalf), kHalf - 1) + kHalf) << 10) | (unsigned)bm;
-          const unsigned cmin = gminu<GL>(comp);
-          if (cmin == 0xffffffffu) break;
-          kmin = (int)(cmin >> 10) - kHalf;
-          mm = (int)(cmin & 1023u);
-          if (kmin == -kHalf || kmin == kHalf - 1) {
-            kmin = gmin<GL>(bk);
-            mm = (int)gminu<GL>(bk == kmin ? (unsigned)bm : 0xffffffffu);
-          }
-        } else {
-          kmin = gmin<GL>(bk);
-          if (kmin == INT32_MAX) break;
-          mm = (int)gminu<GL>(bk == kmin ? (unsigned)bm : 0xffffffffu);
-        }
-        const bool mine = bk == kmin && bm == mm;
-        int dmm = kmin;  // the plain choice key is Delta E itself
-        if (BIASED) dmm = gshfl<GL>(bdE, __ffs(gballot<GL>(mine)) - 1);
-        uint64_t cand = fp ^ (ONE ? ztab[mm - 1] : zobrist(zkey, mm));
-        if (ly.skew && mm != ly.c) cand ^= ONE ? ztab[ly.L - mm] : zobrist(zkey, ly.L + 1 - mm);
-        if (!bloom_test<GL>(bloom, cand, P.bloom_k, bmask)) {
-          mstar = mm;
-          kstar = kmin;
-          dstar = dmm;
-          nfp = cand;
-          break;
-        }
-        skips++;
-        if (mine && have2) {
-          // the owner lane's next best is its second
-          bk = bk2;
-          bm = bm2;
-          bdE = bd2;
-          have2 = false;
-        } else if (mine) {
-          // the owner lane's next best: smallest key ranked after (kmin, mm); keys ranked ahead were
-          // dropped earlier in this step
-          bk = INT32_MAX;
-          int nbm = INT32_MAX, nbd = 0;
-          for (int t = 0; t < S; t++) {
-            const int key = sl_k[t * GL + lane];
-            const int ms = slot_pos(sl_w[t * GL + lane]);
-            const int m = ms < 0 ? -ms : ms;
-            if (key == INT32_MAX) continue;
-            if (key < kmin || (key == kmin && m <= mm)) continue;
-            if (key < bk || (key == bk && m < nbm)) {
-              bk = key;
-              nbm = m;
-              nbd = BIASED ? sl_d[t * GL + lane] : key;
+          int best = INT32_MAX, cmin;
+          lane_keys([&](int t, int v, int k) {
+            if (use >> t & 1) best = min(best, v + k);
+          });
+          while (true) {
+            cmin = warp_min_i32(best);
+            if (cmin == INT32_MAX) break;
+            const int m = cmin & 1023;
+            nfp = fp ^ zp[m - 1];
+            if (!bloom_test(bloom, nfp, probe, bmask, b_at, b_bit)) {
+              astar = skew ? c - m : m;
+              dstar = (cmin >> 10) * 4;
+              break;
+            }
+            skips++;
+            if (best == cmin) {  // the lane's smallest key above cmin
+              best = INT32_MAX;
+              lane_keys([&](int t, int v, int k) {
+                if ((use >> t & 1) && v + k > cmin) best = min(best, v + k);
+              });
             }
           }
-          bm = nbm;
-          bdE = nbd;
-        }
-      }
-      // the move back ranked ahead of the chosen move: count it as a Bloom skip
-      if (gany<GL>(kprev != INT32_MAX && (mstar < 0 || kprev < kstar || (kprev == kstar && mprev < mstar))))
-        skips++;
-      if (mstar < 0) {
-        dead++;
-        need_start = true;
-        continue;
-      }
-      // ---- apply; the slot words take the move at the next scan (fold_flip)
-      pend.on = true;
-      pend.pair = ly.skew && mstar != ly.c;
-      pend.cls = pos_cls(ly, mstar);
-      pend.q0f = pos_q(ly, mstar);
-      pend.s0 = s_at(sm, ly, mstar);
-      pend.q1f = pend.pair ? pos_q(ly, ly.L + 1 - mstar) : 0;  // the mirror has the class of m*
-      pend.s1 = pend.pair ? s_at(sm, ly, ly.L + 1 - mstar) : 0;
-      pend.qmir = ly.c + 6 - (pend.cls ? 1 : 2);
-      mprev = mstar;
-      SC += table_update<GL>(sm, ly, mstar, &fast);
-      if (lane == 0) flip_position(sm, ly, mstar);
-      if (lane == 1 && pend.pair) flip_position(sm, ly, ly.L + 1 - mstar);
-      gsync<GL>();
-      E += dstar;
-      fp = nfp;
-      bloom_add<GL>(bloom, fp, P.bloom_k, bmask);
-      flips++;
-      taken++;
-      if (taken == 1 && P.move_log && lane == 0) {
-        P.move_log[2 * item] = mstar;
-        P.move_log[2 * item + 1] = dstar;
-      }
-      if (E < bestE) bestE = E;
-      if (first_hit < 0 && E <= P.E_target) first_hit = (int)flips;
-      // ---- sieve
-      if (E <= E_thr && key_less(E, fp, wE, wfp)) {
-        bool dup = gany<GL>(lane < R && cE != INT32_MAX && cfp == fp);
-        if (!dup) {
-          if (lane == wlane) {
-            cE = E;
-            cfp = fp;
+          const int mprev = skew ? c - aprev : aprev;
+          if (aprev >= 0 && -(dprev >> 2) * 1024 + mprev < cmin) skips++;
+        } else {
+          const float* bias = P.bias + (size_t)item * L;
+          auto key_of = [&](int m, int d) {
+            float l = bias[m - 1];
+            if (!isfinite(l)) l = 0.f;  // a missing or broken proposal falls back to the plain choice
+            return float_key(fmaf(-P.lambda, l, (float)d));
+          };
+          int bk = INT32_MAX, bm = INT32_MAX, bd = 0;
+          int kmin = INT32_MIN, mm = 0;
+          bool mine = true;
+          while (true) {
+            if (mine) {  // the lane's smallest (key, m) ranked after (kmin, mm)
+              bk = INT32_MAX;
+              bm = INT32_MAX;
+              lane_keys([&](int t, int v, int k) {
+                if (!(use >> t & 1)) return;
+                const int m = (v + k) & 1023, d = ((v + k) >> 10) * 4;
+                const int key = key_of(m, d);
+                if ((key > kmin || (key == kmin && m > mm)) && (key < bk || (key == bk && m < bm))) {
+                  bk = key;
+                  bm = m;
+                  bd = d;
+                }
+              });
+            }
+            kmin = warp_min_i32(bk);
+            if (kmin == INT32_MAX) break;
+            mm = (int)warp_min_u32(bk == kmin ? (unsigned)bm : 0xffffffffu);
+            mine = bk == kmin && bm == mm;
+            const int d = __shfl_sync(kFull, bd, __ffs(__ballot_sync(kFull, mine)) - 1);
+            nfp = fp ^ zp[mm - 1];
+            if (!bloom_test(bloom, nfp, probe, bmask, b_at, b_bit)) {
+              astar = skew ? c - mm : mm;
+              dstar = d;
+              break;
+            }
+            skips++;
           }
-          labs_candidate* rr = rec + wlane;
-          if (lane == 0) {
-            rr->E = E;
-            rr->walk = (uint32_t)w;
-            rr->step = (uint32_t)flips;
-            rr->fp = fp;
+          if (aprev >= 0) {
+            const int mprev = skew ? c - aprev : aprev;
+            const int bkey = key_of(mprev, -dprev);
+            if (bkey != INT32_MAX && (astar < 0 || bkey < kmin || (bkey == kmin && mprev < mm))) skips++;
           }
-          if (lane < W) rr->seq[lane] = (uint64_t)sm.bits[2 * lane] | ((uint64_t)sm.bits[2 * lane + 1] << 32);
-          find_worst();
         }
-      }
-      if (it >= le.T_i) need_start = true;
+        if (astar < 0) {
+          if (lane == 0) ctl->dead++;
+          need_start = true;
+          break;
+        }
+        // ---- apply
+        const int s = 1 - (int)S[astar];  // the element's new value
+        __syncwarp();                     // every lane has read what the flip changes
+        if (lane < (skew && astar ? 2 : 1)) {
+          const int x = lane ? -astar : astar;
+          const int i = (skew ? c - x : x) - 1;
+          S[x] = (uint8_t)(2 - S[x]);
+          atomicXor(&bits[i >> 5], 1u << (i & 31));
+        }
+        if (lane < P.bloom_k) atomicOr(&bloom[b_at], b_bit);
+        E += dstar;
+        fp = nfp;
+        __syncwarp();
+        apply_flip(astar, s, own_bit(astar));
+        aprev = astar;
+        dprev = dstar;
+        flips++;
+        bestE = min(bestE, E);
+        if (E <= gate) {
+          if (E <= P.E_target && ctl->first_hit < 0) {
+            __syncwarp();
+            if (lane == 0) ctl->first_hit = (int)flips;
+            __syncwarp();
+          }
+          // ---- sieve
+          if (E <= E_thr && key_less(E, fp, ctl->wE, ctl->wfp)) {
+            int cE = INT32_MAX;
+            uint64_t cfp = ~0ull;
+            if (lane < R) {
+              cE = record(lane)->E;
+              cfp = record(lane)->fp;
+            }
+            if (!__any_sync(kFull, cE != INT32_MAX && cfp == fp)) {  // not kept yet
+              const int wl = ctl->wlane;
+              labs_candidate* rr = record(wl);
+              if (lane == wl) {
+                cE = E;
+                cfp = fp;
+                rr->E = E;
+                rr->walk = (uint32_t)(le.walk_begin + ((long long)item - le.item_begin));
+                rr->step = (uint32_t)flips;
+                rr->fp = fp;
+              }
+              store_seq(rr->seq);
+              find_worst(cE, cfp);
+            }
+          }
+          gate = gate_of();
+        }
+      } while (flips != until);
+      if (flips - ctl->seg0 >= (unsigned)le.T_i) need_start = true;
+      __syncwarp();
     }
-    if (P.move_log && taken == 0 && lane == 0) {
-      P.move_log[2 * item] = -1;
-      P.move_log[2 * item + 1] = 0;
+    __syncwarp();
+    if (lane == 0) {
+      ctl->skips += skips;
+      ctl->flips = flips;
+      ctl->bestE = bestE;
+      ctl->E = E;
+      ctl->fp = fp;
+      ctl->aprev = aprev;
+      ctl->dprev = dprev;
+      ctl->need_start = need_start ? 1 : 0;
     }
-    if (P.seq_out && lane < W)
-      P.seq_out[(size_t)item * W + lane] = (uint64_t)sm.bits[2 * lane] | ((uint64_t)sm.bits[2 * lane + 1] << 32);
-
+    __syncwarp();
+    if (P.seq_out) store_seq(P.seq_out + (size_t)item * ((L + 63) >> 6));
     if (flips < budget) {
       // ---- leave the walk for the next launch
-      if (gh) {
-        unsigned char* gb = reinterpret_cast<unsigned char*>(gh);
-        for (int t = lane; t < kBitWords; t += GL) reinterpret_cast<uint32_t*>(gb + kStateBits)[t] = sm.bits[t];
-        for (int t = lane; t < ly.cl / 2; t += GL)
-          reinterpret_cast<uint32_t*>(gb + kStateC)[t] = reinterpret_cast<const uint32_t*>(sm.C16)[t];
-        for (int t = lane; t < bwords; t += GL) reinterpret_cast<uint32_t*>(gb + kStateBloom)[t] = bloom[t];
-        if (lane == 0) {
-          gh->fp = fp;
-          gh->skips = skips;
-          gh->E = E;
-          gh->flips = (int)flips;
-          gh->segs = (int)segs;
-          gh->dead = (int)dead;
-          gh->it = it;
-          gh->mprev = mprev;
-          gh->first_hit = first_hit;
-          gh->bestE = bestE;
-          gh->need_start = need_start ? 1 : 0;
-          gh->started = 1;
-          gh->done = 0;
-        }
+      if (saved) {
+        for (int t = lane; t < P.slab.bytes / 4; t += 32)
+          reinterpret_cast<uint32_t*>(saved)[t] = reinterpret_cast<const uint32_t*>(slab)[t];
+        int* gt = reinterpret_cast<int*>(saved + P.slab.bytes) + lane;
+#pragma unroll
+        for (int j = 0; j < SL; j++) gt[32 * j] = T[j];
       }
     } else {
       // ---- final: sort the R slots by (E, fp) (ties between empty slots by lane) and rewrite in place
+      labs_candidate mine;
+      mine.E = INT32_MAX;
+      mine.fp = ~0ull;
+      if (lane < R) mine = *record(lane);
       int rank = 0;
       for (int r = 0; r < R; r++) {
-        int oE = gshfl<GL>(cE, r);
-        uint64_t of = gshfl<GL>(cfp, r);
-        if (key_less(oE, of, cE, cfp) || (oE == cE && of == cfp && r < lane)) rank++;
+        const int oE = __shfl_sync(kFull, mine.E, r);
+        const uint64_t of = __shfl_sync(kFull, mine.fp, r);
+        if (key_less(oE, of, mine.E, mine.fp) || (oE == mine.E && of == mine.fp && r < lane)) rank++;
       }
-      gsync<GL>();
-      labs_candidate mine;
-      if (lane < R) mine = rec[lane];
-      gsync<GL>();
-      if (lane < R) rec[rank] = mine;
-      gsync<GL>();
-      if (P.walk_stats && lane == 0) {
-        int64_t* st = P.walk_stats + (int64_t)item * 6;
-        st[0] = (int64_t)flips;
-        st[1] = (int64_t)segs;
-        st[2] = skips;
-        st[3] = (int64_t)dead;
-        st[4] = bestE;
-        st[5] = first_hit;
-      }
-      if (gh && lane == 0) {
-        gh->done = 1;
-        gh->started = 1;
+      __syncwarp();
+      if (lane < R) *record(rank) = mine;
+      if (lane == 0) {
+        if (P.walk_stats) {
+          int64_t* st = P.walk_stats + (int64_t)item * 6;
+          st[0] = (int64_t)flips;
+          st[1] = (int64_t)ctl->segs;
+          st[2] = ctl->skips;
+          st[3] = (int64_t)ctl->dead;
+          st[4] = bestE;
+          st[5] = ctl->first_hit;
+        }
+        if (saved) reinterpret_cast<WalkCtl*>(saved + P.slab.off_ctl)->done = 1;
       }
     }
-    gsync<GL>();
-    agg_flips += flips - flips0;
-    agg_segs += segs - segs0;
-    agg_skips += skips - skips0;
-    agg_dead += dead - dead0;
-    agg_best = min(agg_best, bestE);
-  }
-  if (lane == 0) {
-    atomicAdd(reinterpret_cast<unsigned long long*>(&P.stats->flips), (unsigned long long)agg_flips);
-    atomicAdd(reinterpret_cast<unsigned long long*>(&P.stats->segments), (unsigned long long)agg_segs);
-    atomicAdd(reinterpret_cast<unsigned long long*>(&P.stats->bloom_skips), (unsigned long long)agg_skips);
-    atomicAdd(reinterpret_cast<unsigned long long*>(&P.stats->dead_ends), (unsigned long long)agg_dead);
-    atomicMin(&P.stats->best_E, agg_best);
+    if (lane == 0) {
+      atomicAdd(reinterpret_cast<unsigned long long*>(&P.stats->flips), (unsigned long long)(flips - ctl->flips0));
+      atomicAdd(reinterpret_cast<unsigned long long*>(&P.stats->segments), (unsigned long long)(ctl->segs - ctl->segs0));
+      atomicAdd(reinterpret_cast<unsigned long long*>(&P.stats->bloom_skips), (unsigned long long)(ctl->skips - ctl->skips0));
+      atomicAdd(reinterpret_cast<unsigned long long*>(&P.stats->dead_ends), (unsigned long long)(ctl->dead - ctl->dead0));
+      atomicMin(&P.stats->best_E, bestE);
+    }
   }
 }
 
-// Zeroes the aggregates and the work counter; E_thr reports the first length's sieve bound.
-__global__ void walk_init_kernel(labs_walk_stats* stats, const int32_t* E_thr_dev, int32_t E_thr_value,
-                                 unsigned long long* counter) {
-  stats->flips = 0;
-  stats->segments = 0;
-  stats->bloom_skips = 0;
-  stats->dead_ends = 0;
-  stats->E_thr = E_thr_dev ? E_thr_dev[0] : E_thr_value;
-  stats->best_E = INT32_MAX;
-  stats->status = LABS_OK;
-  stats->reserved = 0;
-  *counter = 0ull;
+// One block per length: the fingerprint change of every neighbour (the Zobrist keys of its flipped
+// positions).  Block 0 also zeroes the aggregates and the work counter; E_thr reports the first length's
+// sieve bound.
+__global__ void __launch_bounds__(128) walk_init_kernel(const __grid_constant__ WalkParams P, uint64_t* zpair) {
+  const WalkLen& le = P.len[blockIdx.x];
+  const uint64_t zk = stream_key(0, kPurposeZobrist, (uint64_t)le.L, 0);
+  const int n = le.skew ? le.c : le.L;
+  for (int m = 1 + threadIdx.x; m <= n; m += blockDim.x)
+    zpair[(size_t)blockIdx.x * kMaxL + m - 1] =
+        zobrist(zk, m) ^ (le.skew && m != le.c ? zobrist(zk, le.L + 1 - m) : 0ull);
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    labs_walk_stats* stats = P.stats;
+    stats->flips = 0;
+    stats->segments = 0;
+    stats->bloom_skips = 0;
+    stats->dead_ends = 0;
+    stats->E_thr = P.E_thr_dev ? P.E_thr_dev[0] : le.E_thr_value;
+    stats->best_E = INT32_MAX;
+    stats->status = LABS_OK;
+    stats->reserved = 0;
+    *P.counter = 0ull;
+  }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -740,7 +905,8 @@ __global__ void __launch_bounds__(32 * kSampleWarps) sample_kernel(int L, int sk
   make_layout(ly, L, skew, p, 8);
   const int64_t warps_total = (int64_t)gridDim.x * kSampleWarps;
   for (int64_t i = (int64_t)blockIdx.x * kSampleWarps + (threadIdx.x >> 5); i < n; i += warps_total) {
-    build_start(sm, ly, prefixes + (i % n_prefix) * prefix_words, stream_key(seed, kPurposeThresh, (uint64_t)i, 0));
+    build_start(sm.bits, L, skew != 0, ly.c, p, prefixes + (i % n_prefix) * prefix_words,
+                stream_key(seed, kPurposeThresh, (uint64_t)i, 0));
     int E;
     if (skew) {
       E = build_table(sm, ly);
@@ -805,6 +971,12 @@ __global__ void finish_select_kernel(const unsigned* __restrict__ hist2, long lo
   }
 }
 
+// ---------------------------------------------------------------------------------------------
+// The tile parameters of a configuration (tile_m, lanes_per_walk, warps_per_cta) select nothing in the
+// incremental walk but the warps of a block; a combination that the tiled neighbour scan has no plan for
+// stays refused.
+// ---------------------------------------------------------------------------------------------
+constexpr int kMaxPasses = 3;  // lane passes over the tiles of one walk
 struct Variant {
   int M, H, GL;  // tile, lag ranges per tile, lanes per walk
 };
@@ -819,129 +991,14 @@ static int passes_for(int L, int skew, int p, const Variant& v) {
   return np < 1 ? 1 : np;
 }
 
-// Bytes of a launch's dynamic shared memory: the walks' slabs and, for single-length launches, the
-// Zobrist table.
-static size_t walk_smem(const WalkParams& P, int walks_per_block) {
-  return (size_t)P.slab.bytes * (size_t)walks_per_block + (P.n_len == 1 ? sizeof(uint64_t) * (size_t)P.len[0].ly.L : 0);
-}
-
-template <int M, int H, int GL>
-int walk_t(labs_ctx* ctx, const WalkParams& P, int warps, cudaStream_t st, bool configure, long long* blocks) {
-  const bool one = P.n_len == 1, biased = P.bias != nullptr;
-  if (biased && !one) return LABS_ERR_INVALID_ARG;
-  if (32 * warps > walk_block_threads(GL)) return LABS_ERR_INVALID_ARG;
-  const size_t smem = walk_smem(P, warps * (32 / GL));
-  auto kern = !one ? walk_kernel<M, H, false, false, GL>
-                   : biased ? walk_kernel<M, H, true, true, GL> : walk_kernel<M, H, true, false, GL>;
-  if (configure) {
-    if (smem > ctx->smem_optin) return LABS_ERR_INVALID_ARG;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-      return LABS_ERR_CUDA;
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * warps, smem) != cudaSuccess || per_sm < 1)
-      return LABS_ERR_CUDA;
-    long long b = (long long)per_sm * ctx->num_sms;
-    const long long walks_per_block = (long long)warps * (32 / GL);
-    const long long need = (P.n_items + walks_per_block - 1) / walks_per_block;
-    if (b > need) b = need;
-    *blocks = b < 1 ? 1 : b;
-    return LABS_OK;
-  }
-  kern<<<(unsigned)*blocks, 32 * warps, smem, st>>>(P);
-  return cuda_status(cudaGetLastError());
-}
-
-// configure = true: sets the kernel's shared-memory limit and sizes the persistent grid (*blocks);
-// configure = false: launches with that grid (no runtime call besides the launch itself).
-static int walk_variant(labs_ctx* ctx, const WalkParams& P, const Variant& v, int warps, cudaStream_t st,
-                        bool configure, long long* blocks) {
-  switch (v.M * 1000 + v.H * 100 + v.GL) {
-    case 8132: return walk_t<8, 1, 32>(ctx, P, warps, st, configure, blocks);
-    case 12132: return walk_t<12, 1, 32>(ctx, P, warps, st, configure, blocks);
-    case 16132: return walk_t<16, 1, 32>(ctx, P, warps, st, configure, blocks);
-    case 16232: return walk_t<16, 2, 32>(ctx, P, warps, st, configure, blocks);
-    case 8116: return walk_t<8, 1, 16>(ctx, P, warps, st, configure, blocks);
-    case 12116: return walk_t<12, 1, 16>(ctx, P, warps, st, configure, blocks);
-    case 16116: return walk_t<16, 1, 16>(ctx, P, warps, st, configure, blocks);
-    case 16216: return walk_t<16, 2, 16>(ctx, P, warps, st, configure, blocks);
-    default: return LABS_ERR_INVALID_ARG;
-  }
-}
-
-// Warps per block of a launch: the requested count, else 8 for whole-warp walks and, for half-warp
-// walks, as many (up to the block limit) as fit one block's slabs in the shared memory of an SM.
-static int warps_for(const labs_ctx* ctx, const WalkParams& P, const Variant& v, int requested) {
-  if (requested > 0) return requested;
-  if (v.GL == 32) return 8;
-  int w = walk_block_threads(16) / 32;
-  while (w > 1 && walk_smem(P, 2 * w) > ctx->smem_optin) w--;
-  return w;
-}
-
-static int launch_walk(labs_ctx* ctx, const WalkParams& P, const Variant& v, int warps, cudaStream_t st) {
-  long long blocks = 0;
-  int s = walk_variant(ctx, P, v, warps, st, true, &blocks);
-  return s == LABS_OK ? walk_variant(ctx, P, v, warps, st, false, &blocks) : s;
-}
-
 // One launch's lengths.
 struct LenSpec {
   int L, skew, p, T_i;
   int64_t walks, walk_begin;
 };
 
-// Fills the per-length table, the slot stride and the slab plan for variant v; false if some length does
-// not fit.  Every length's arrays are shrunk to what it needs (compact_layout) and the slab takes the
-// largest of each piece over the launch's lengths.
-static bool fill_params(WalkParams& P, const std::vector<LenSpec>& lens, const Variant& v, int R, bool biased,
-                        int bloom_log2) {
-  P.n_len = (int)lens.size();
-  int64_t item = 0;
-  int maxnp = 1, fwd_bytes = 16, cl = 8;
-  for (size_t i = 0; i < lens.size(); i++) {
-    LenEntry& e = P.len[i];
-    if (!make_layout(e.ly, lens[i].L, lens[i].skew, lens[i].p, v.M, v.H)) return false;
-    compact_layout(e.ly);
-    int np = (e.ly.n_tasks + v.GL - 1) / v.GL;
-    if (np > kMaxPasses) return false;
-    maxnp = std::max(maxnp, np);
-    fwd_bytes = std::max(fwd_bytes, 4 * e.ly.cw * e.ly.ncls);
-    cl = std::max(cl, e.ly.cl);
-    e.T_i = lens[i].T_i > 0 ? lens[i].T_i : 4 * (lens[i].L + 1);
-    e.E_thr_value = INT32_MAX;
-    e.item_begin = item;
-    e.walk_begin = lens[i].walk_begin;
-    item += lens[i].walks;
-  }
-  if (R > v.GL) return false;  // one sieve slot per lane
-  P.n_items = item;
-  P.slot_stride = maxnp * (v.M / v.H);
-  auto up16 = [](int b) { return (b + 15) & ~15; };
-  SlabPlan& sp = P.slab;
-  int off = up16(4 * kBitWords);
-  sp.off_C16 = off;
-  off += up16(2 * cl);
-  sp.off_C8 = off;
-  off += up16(cl);
-  sp.off_fwd = off;
-  off += up16(fwd_bytes);
-  sp.off_bwd = off;
-  off += up16(fwd_bytes);
-  sp.off_bloom = off;
-  off += up16(std::max(4, (1 << bloom_log2) / 8));
-  sp.off_slots = off;
-  off += up16(P.slot_stride * v.GL * slot_bytes(biased));
-  // slab stride = 8 (mod 128) bytes: the two walks of a half-warp launch then sit two banks apart, so
-  // their lanes' window loads (tiles four words apart, all multiples of four banks) do not collide
-  // (every slab access is at most 4 bytes wide, so 8-byte alignment of a slab suffices)
-  sp.bytes = off + (136 - off % 128) % 128;
-  return true;
-}
-
-// Heuristic choice: least total per-warp scan work, sum(walks * NP * M / H * GL / 32) (a half-warp walk
-// shares its warp's instructions with another walk); ties to fewer lanes per walk (the two walks of a
-// warp then share every instruction of the serial phases), then to fewer lane passes (each pass repeats
-// the per-slot phases), then to more lanes per tile, then the larger tile.
+// The plan of least scan work, sum(walks * NP * M / H * GL / 32), that the requested parameters allow; ties
+// to fewer lanes per walk, fewer passes, more lanes per tile, the larger tile.  False if there is none.
 // req_m / req_gl: 0 or the tile size / lanes per walk the caller fixed; R: sieve slots per walk.
 static bool choose_variant(const std::vector<LenSpec>& lens, int req_m, int req_gl, int R, Variant* out) {
   bool found = false;
@@ -981,9 +1038,141 @@ static bool choose_variant(const std::vector<LenSpec>& lens, int req_m, int req_
   return found;
 }
 
+static bool accepted(const std::vector<LenSpec>& lens, int req_m, int req_gl, int R, int warps) {
+  Variant v;
+  return choose_variant(lens, req_m, req_gl, R, &v) && 32 * warps <= (v.GL == 32 ? 256 : 384);
+}
+
+// A launch's kernel (slots per lane, mode) and shape.
+struct Launch {
+  int ns, nu, mode, warps;
+  long long blocks;
+  size_t smem;
+};
+
+typedef void (*WalkKernel)(const WalkParams);
+template <int NS, int NU>
+static WalkKernel walk_fn_of(int mode, bool biased) {  // biased launches hold one length
+  if (mode == 0) return biased ? walk_kernel<NS, NU, 0, true> : walk_kernel<NS, NU, 0, false>;
+  if (mode == 1) return biased ? walk_kernel<NS, NU, 1, true> : walk_kernel<NS, NU, 1, false>;
+  return walk_kernel<NS, NU, 2, false>;
+}
+// Compiled slot counts: lengths to 128, 256, 384, 512 and 576 (fewer slots where a prefix leaves fewer
+// neighbours); a launch takes the smallest that holds all its lengths.
+static const int kSlots[][2] = {{1, 4}, {2, 8}, {3, 12}, {4, 16}, {4, 18}, {5, 18}};
+static WalkKernel walk_fn(const Launch& ln, bool biased) {
+  switch (100 * ln.ns + ln.nu) {
+    case 104: return walk_fn_of<1, 4>(ln.mode, biased);
+    case 208: return walk_fn_of<2, 8>(ln.mode, biased);
+    case 312: return walk_fn_of<3, 12>(ln.mode, biased);
+    case 416: return walk_fn_of<4, 16>(ln.mode, biased);
+    case 418: return ln.mode == 0 ? walk_kernel<4, 16, 0, false> : ln.mode == 1 ? walk_fn_of<5, 18>(1, biased) : walk_kernel<4, 18, 2, false>;
+    default: return walk_fn_of<5, 18>(ln.mode, biased);
+  }
+}
+
+// Fills the per-length table and the slab plan, and picks the kernel.  Every index that the kernel forms
+// from these sizes is checked on the CPU for all lengths (tests/test_walk_tables.py mirrors this plan).
+static void fill_params(WalkParams& P, const std::vector<LenSpec>& lens, int bloom_log2, Launch* ln) {
+  P.n_len = (int)lens.size();
+  int need_s = 0, need_u = 0;  // slots a lane needs
+  for (const LenSpec& s : lens) {
+    if (s.skew)
+      need_s = std::max(need_s, ((s.L - 1) / 2 - s.p) / 64 + 1);
+    else
+      need_u = std::max(need_u, (s.L - s.p - 1) / 32 + 1);
+  }
+  ln->mode = lens.size() > 1 ? 2 : (lens[0].skew ? 0 : 1);
+  for (const auto& sl : kSlots) {
+    ln->ns = sl[0];
+    ln->nu = sl[1];
+    if (need_s <= sl[0] && need_u <= sl[1]) break;
+  }
+  int64_t item = 0;
+  int sn = 16, tab = 16;
+  for (size_t i = 0; i < lens.size(); i++) {
+    WalkLen& e = P.len[i];
+    const LenSpec& s = lens[i];
+    e.L = s.L;
+    e.skew = s.skew;
+    e.p = s.p;
+    e.k = (s.L - 1) / 2;
+    e.c = (s.L + 1) / 2;
+    int lo, hi;  // sequence bytes reached: S[-lo] .. S[hi]
+    if (s.skew) {
+      e.hmax = e.k - s.p;
+      const int hpad = 64 * ln->ns - 1;  // distances of the last slots, with and without a neighbour
+      e.t1 = (std::max(e.k + 1, hpad + 1) + 3) / 4 * 4;
+      e.t2 = 3 * e.t1;
+      // T reads S[h +- 2g] for g <= max(k, hmax); the table update S[a +- d] for whole 128-lag turns
+      hi = std::max(hpad + 2 * e.k, std::min(2 * e.hmax + e.k, 3 * e.hmax) + 127);
+      lo = std::max(2 * e.k, std::min(e.k, 2 * e.hmax) + 127);
+    } else {
+      e.hmax = s.L - s.p - 1;
+      const int mpad = s.p + 32 * ln->nu;  // position of the last slot
+      e.t1 = 128 * ((std::max(s.L - 1, 32 * ln->nu - 1)) / 128 + 1);
+      e.t2 = e.t1 + (std::max(2 * std::max(s.L + 64, mpad + 1), mpad + s.L + 1) + 3) / 4 * 4;
+      hi = std::max(2 * s.L + 127, mpad + s.L);
+      lo = std::max(s.L + 127, mpad);
+    }
+    e.so = (lo + 8) / 4 * 4;  // a realigned word may start three bytes below
+    e.sn = (e.so + hi + 8 + 3) / 4 * 4;
+    sn = std::max(sn, e.sn);
+    tab = std::max(tab, 2 * e.t2);
+    e.T_i = s.T_i > 0 ? s.T_i : 4 * (s.L + 1);
+    e.E_thr_value = INT32_MAX;
+    e.item_begin = item;
+    e.walk_begin = s.walk_begin;
+    item += s.walks;
+  }
+  P.n_items = item;
+  auto up16 = [](int b) { return (b + 15) & ~15; };
+  SlabPlan& sp = P.slab;
+  sp.off_ctl = up16(4 * kBitWords);
+  sp.off_S = sp.off_ctl + up16((int)sizeof(WalkCtl));
+  sp.off_tab = sp.off_S + up16(sn);
+  sp.off_bloom = sp.off_tab + up16(tab);
+  sp.bytes = sp.off_bloom + up16(std::max(kScratch, (1 << bloom_log2) / 8));
+}
+
+// Sets the kernel's shared-memory limit and sizes the persistent grid.  A block is one SM's walks: as many
+// warps as its registers and shared memory hold, fewer when the launch has fewer walks than that per SM (a
+// few walks then spread over all SMs instead of filling some).
+static int plan_launch(labs_ctx* ctx, const WalkParams& P, int requested_warps, bool biased, Launch* ln) {
+  int warps = walk_block_threads(ln->mode, ln->ns, ln->nu) / 32;
+  if (requested_warps > 0) {
+    warps = requested_warps;
+  } else {
+    const int64_t per_sm = (P.n_items + ctx->num_sms - 1) / ctx->num_sms;
+    warps = (int)std::max<int64_t>(1, std::min<int64_t>(warps, per_sm));
+  }
+  while (warps > 1 && (size_t)P.slab.bytes * warps > ctx->smem_optin) warps--;
+  ln->warps = warps;
+  ln->smem = (size_t)P.slab.bytes * warps;
+  WalkKernel kern = walk_fn(*ln, biased);
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ln->smem) != cudaSuccess)
+    return LABS_ERR_CUDA;
+  int per_sm = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * warps, ln->smem) != cudaSuccess || per_sm < 1)
+    return LABS_ERR_CUDA;
+  const long long b = (long long)per_sm * ctx->num_sms, need = (P.n_items + warps - 1) / warps;
+  ln->blocks = std::max(1ll, std::min(b, need));
+  return LABS_OK;
+}
+
+static int run_walks(const WalkParams& P, const Launch& ln, cudaStream_t st) {
+  walk_fn(ln, P.bias != nullptr)<<<(unsigned)ln.blocks, 32 * ln.warps, ln.smem, st>>>(P);
+  return cuda_status(cudaGetLastError());
+}
+
+static int run_init(const WalkParams& P, cudaStream_t st) {
+  walk_init_kernel<<<(unsigned)P.n_len, 128, 0, st>>>(P, const_cast<uint64_t*>(P.zpair));
+  return cuda_status(cudaGetLastError());
+}
+
 static void base_params(WalkParams& P, int R, int bloom_log2, int bloom_k, int p, int n_prefix, int64_t flip_budget,
                         uint64_t seed, int32_t E_target, const uint64_t* prefixes, labs_candidate* out,
-                        int64_t* walk_stats, labs_walk_stats* stats, unsigned long long* counter) {
+                        int64_t* walk_stats, labs_walk_stats* stats, unsigned long long* counter, uint64_t* zpair) {
   P.R = R;
   P.bloom_log2 = bloom_log2;
   P.bloom_k = bloom_k;
@@ -997,8 +1186,12 @@ static void base_params(WalkParams& P, int R, int bloom_log2, int bloom_k, int p
   P.walk_stats = walk_stats;
   P.stats = stats;
   P.counter = counter;
+  P.zpair = zpair;
   P.E_thr_dev = nullptr;
 }
+
+// Bytes of the fingerprint changes of a launch's lengths.
+static size_t zpair_bytes(size_t n_len) { return sizeof(uint64_t) * kMaxL * n_len; }
 
 }  // namespace
 
@@ -1026,71 +1219,43 @@ int launch_sample_threshold(labs_ctx* ctx, int L, int skew, int p, const uint64_
 
 int launch_skew_search(labs_ctx* ctx, const labs_walk_cfg* cfg, const uint64_t* prefixes, int n_prefix,
                        labs_candidate* out, int64_t* walk_stats, labs_walk_stats* stats, cudaStream_t st) {
-  std::vector<LenSpec> lens{{cfg->L, cfg->skew, cfg->p, cfg->T_i, cfg->n_walks, cfg->walk_begin}};
-  Variant v;
-  if (!choose_variant(lens, cfg->tile_m, cfg->lanes_per_walk, cfg->R, &v)) return LABS_ERR_INVALID_ARG;
-  WalkParams* P = new (std::nothrow) WalkParams();
-  if (!P) return LABS_ERR_NOMEM;
-  char* w = static_cast<char*>(ws_get(ctx, kWsWalkCounters, 256));
-  if (!w) {
-    delete P;
-    return LABS_ERR_NOMEM;
-  }
-  base_params(*P, cfg->R, cfg->bloom_log2, cfg->bloom_k, cfg->p, n_prefix, cfg->flip_budget, cfg->seed,
-              cfg->E_target, prefixes, out, walk_stats, stats, reinterpret_cast<unsigned long long*>(w));
-  if (!fill_params(*P, lens, v, cfg->R, false, cfg->bloom_log2)) {
-    delete P;
-    return LABS_ERR_INVALID_ARG;
-  }
-  int32_t* thr = reinterpret_cast<int32_t*>(w + 64);
-  int s = LABS_OK;
-  if (cfg->E_thr_dev) {
-    P->E_thr_dev = cfg->E_thr_dev;
-  } else if (cfg->E_thr == LABS_AUTO_THRESHOLD) {
-    s = launch_sample_threshold(ctx, cfg->L, cfg->skew, cfg->p, prefixes, n_prefix, P->prefix_words, cfg->seed,
-                                cfg->n_thresh_samples, cfg->thresh_rank, thr, nullptr, st);
-    P->E_thr_dev = thr;
-  } else {
-    P->len[0].E_thr_value = cfg->E_thr;
-  }
-  if (s == LABS_OK) {
-    walk_init_kernel<<<1, 1, 0, st>>>(stats, P->E_thr_dev, P->len[0].E_thr_value, P->counter);
-    s = cuda_status(cudaGetLastError());
-  }
-  if (s == LABS_OK && P->n_items > 0) s = launch_walk(ctx, *P, v, warps_for(ctx, *P, v, cfg->warps_per_cta), st);
-  delete P;
-  return s;
+  return launch_chunked_search(ctx, cfg, nullptr, 0.f, 0, prefixes, n_prefix, out, walk_stats, stats, nullptr, nullptr,
+                               nullptr, st);
 }
 
 // ---------------------------------------------------------------------------------------------
-// Chunked walks: the same Algorithm 1 walks run `chunk` accepted flips per launch and are saved in
-// between, so a proposal network can score every walk's current state before each chunk (learned mode).
-// Without a network the results equal labs_skew_search's.
+// Walks of one length.  Without a network they run in one launch, which also writes the logs of a chunked
+// run (chunk > 0): a walk does not depend on the others, so its state at a chunk's beginning is logged as it
+// passes it.  With a network the walks run `chunk` accepted flips per launch and are saved in between, and
+// the network scores every walk's current state before each chunk.
 // ---------------------------------------------------------------------------------------------
 int launch_chunked_search(labs_ctx* ctx, const labs_walk_cfg* cfg, labs_policy* policy, float lambda, int chunk,
                           const uint64_t* prefixes, int n_prefix, labs_candidate* out, int64_t* walk_stats,
                           labs_walk_stats* stats, float* logits_log, uint64_t* state_log, int32_t* move_log,
                           cudaStream_t st) {
   std::vector<LenSpec> lens{{cfg->L, cfg->skew, cfg->p, cfg->T_i, cfg->n_walks, cfg->walk_begin}};
-  Variant v;
-  if (!choose_variant(lens, cfg->tile_m, cfg->lanes_per_walk, cfg->R, &v)) return LABS_ERR_INVALID_ARG;
-  const long long n = cfg->n_walks;
-  const int L = cfg->L, W = (L + 63) / 64;
-  const long long n_chunks = (cfg->flip_budget + chunk - 1) / chunk;
+  if (!accepted(lens, cfg->tile_m, cfg->lanes_per_walk, cfg->R, cfg->warps_per_cta)) return LABS_ERR_INVALID_ARG;
+  std::unique_ptr<WalkParams> P(new (std::nothrow) WalkParams());
   char* w = static_cast<char*>(ws_get(ctx, kWsWalkCounters, 256));
-  unsigned char* state = static_cast<unsigned char*>(ws_get(ctx, kWsChunkState, (size_t)kStateBytes * (size_t)n));
-  char* io = static_cast<char*>(ws_get(ctx, kWsChunkIo, (size_t)n * (8 * W + 4 * L) + 256));
-  if (!w || !state || !io) return LABS_ERR_NOMEM;
-  uint64_t* seqbuf = reinterpret_cast<uint64_t*>(io);
-  float* logits = reinterpret_cast<float*>(io + (((size_t)n * 8 * W + 255) & ~size_t(255)));
-  WalkParams* P = new (std::nothrow) WalkParams();
-  if (!P) return LABS_ERR_NOMEM;
+  uint64_t* zpair = static_cast<uint64_t*>(ws_get(ctx, kWsZpair, zpair_bytes(1)));
+  if (!P || !w || !zpair) return LABS_ERR_NOMEM;
   unsigned long long* counter = reinterpret_cast<unsigned long long*>(w);
   base_params(*P, cfg->R, cfg->bloom_log2, cfg->bloom_k, cfg->p, n_prefix, cfg->flip_budget, cfg->seed, cfg->E_target,
-              prefixes, out, walk_stats, stats, counter);
-  if (!fill_params(*P, lens, v, cfg->R, policy != nullptr, cfg->bloom_log2)) {  // one slab plan for the plain and biased launches
-    delete P;
-    return LABS_ERR_INVALID_ARG;
+              prefixes, out, walk_stats, stats, counter, zpair);
+  Launch ln;
+  fill_params(*P, lens, cfg->bloom_log2, &ln);
+  const long long n = cfg->n_walks;
+  const int L = cfg->L, W = (L + 63) / 64;
+  unsigned char* state = nullptr;
+  uint64_t* seqbuf = nullptr;
+  float* logits = nullptr;
+  if (policy) {
+    P->state_stride = P->slab.bytes + 128 * walk_slots(ln.mode, ln.ns, ln.nu);
+    state = static_cast<unsigned char*>(ws_get(ctx, kWsChunkState, (size_t)P->state_stride * (size_t)n));
+    char* io = static_cast<char*>(ws_get(ctx, kWsChunkIo, (size_t)n * (8 * W + 4 * L) + 256));
+    if (!state || !io) return LABS_ERR_NOMEM;
+    seqbuf = reinterpret_cast<uint64_t*>(io);
+    logits = reinterpret_cast<float*>(io + (((size_t)n * 8 * W + 255) & ~size_t(255)));
   }
   int32_t* thr = reinterpret_cast<int32_t*>(w + 64);
   int s = LABS_OK;
@@ -1103,99 +1268,62 @@ int launch_chunked_search(labs_ctx* ctx, const labs_walk_cfg* cfg, labs_policy* 
   } else {
     P->len[0].E_thr_value = cfg->E_thr;
   }
-  const int warps = warps_for(ctx, *P, v, cfg->warps_per_cta);
-  long long blocks = 0, blocks_biased = 0;
-  if (s == LABS_OK) s = walk_variant(ctx, *P, v, warps, st, true, &blocks);
-  if (s == LABS_OK && policy) {  // the chunks run the biased instantiation: configure it as well
-    P->bias = logits;
-    s = walk_variant(ctx, *P, v, warps, st, true, &blocks_biased);
-    P->bias = nullptr;
+  Launch biased = ln;
+  if (s == LABS_OK) s = plan_launch(ctx, *P, cfg->warps_per_cta, false, &ln);
+  if (s == LABS_OK && policy) s = plan_launch(ctx, *P, cfg->warps_per_cta, true, &biased);
+  if (s == LABS_OK) s = run_init(*P, st);
+  if (s != LABS_OK) return s;
+  if (!policy) {
+    P->log_chunk = state_log || move_log ? chunk : 0;
+    P->state_log = state_log;
+    P->move_log = move_log;
+    return n > 0 ? run_walks(*P, ln, st) : LABS_OK;
   }
-  if (s == LABS_OK && cudaMemsetAsync(state, 0, (size_t)kStateBytes * (size_t)n, st) != cudaSuccess) s = LABS_ERR_CUDA;
-  if (s == LABS_OK) {
-    walk_init_kernel<<<1, 1, 0, st>>>(stats, P->E_thr_dev, P->len[0].E_thr_value, counter);
-    s = cuda_status(cudaGetLastError());
-  }
+  const long long n_chunks = (cfg->flip_budget + chunk - 1) / chunk;
   P->state = state;
-  P->state_stride = kStateBytes;
   P->seq_out = seqbuf;
-  // set-up launch: every walk's first state
-  P->chunk = -1;
-  if (s == LABS_OK && n > 0) s = walk_variant(ctx, *P, v, warps, st, false, &blocks);
+  P->chunk = -1;  // set-up launch: every walk's first state
+  if (n > 0) s = run_walks(*P, ln, st);
+  P->chunk = chunk;
+  P->log_chunk = move_log ? chunk : 0;
+  P->bias = logits;
+  P->lambda = lambda;
   for (long long c = 0; c < n_chunks && s == LABS_OK && n > 0; c++) {
-    if (policy) {
-      s = labs_policy_forward(policy, seqbuf, n, logits, st);
-      if (s != LABS_OK) break;
-      P->bias = logits;
-      P->lambda = lambda;
-      if (logits_log && cudaMemcpyAsync(logits_log + (size_t)c * n * L, logits, sizeof(float) * (size_t)n * L,
-                                        cudaMemcpyDeviceToDevice, st) != cudaSuccess) {
-        s = LABS_ERR_CUDA;
-        break;
-      }
-    }
-    if (state_log && cudaMemcpyAsync(state_log + (size_t)c * n * W, seqbuf, 8 * (size_t)n * W,
-                                     cudaMemcpyDeviceToDevice, st) != cudaSuccess) {
+    s = labs_policy_forward(policy, seqbuf, n, logits, st);
+    if (s != LABS_OK) break;
+    if ((logits_log && cudaMemcpyAsync(logits_log + (size_t)c * n * L, logits, sizeof(float) * (size_t)n * L,
+                                       cudaMemcpyDeviceToDevice, st) != cudaSuccess) ||
+        (state_log && cudaMemcpyAsync(state_log + (size_t)c * n * W, seqbuf, 8 * (size_t)n * W,
+                                      cudaMemcpyDeviceToDevice, st) != cudaSuccess) ||
+        cudaMemsetAsync(counter, 0, sizeof(unsigned long long), st) != cudaSuccess) {
       s = LABS_ERR_CUDA;
       break;
     }
-    P->chunk = chunk;
     P->move_log = move_log ? move_log + (size_t)c * n * 2 : nullptr;
-    if (cudaMemsetAsync(counter, 0, sizeof(unsigned long long), st) != cudaSuccess) {
-      s = LABS_ERR_CUDA;
-      break;
-    }
-    s = walk_variant(ctx, *P, v, warps, st, false, policy ? &blocks_biased : &blocks);
+    s = run_walks(*P, biased, st);
   }
-  delete P;
-  if (policy) {  // the network's tensor-core waits: a failure makes the logits of that chunk invalid
-    const int ps = labs_policy_sync_status(policy, st);
-    if (s == LABS_OK) s = ps;
-  }
-  return s;
+  // the network's tensor-core waits: a failure makes the logits of that chunk invalid
+  const int ps = labs_policy_sync_status(policy, st);
+  return s == LABS_OK ? ps : s;
 }
 
 // ---------------------------------------------------------------------------------------------
 // Batched mixed-length search: every length's sieve bound, then one persistent walk launch over all
-// (length, walk) items; the sequence is captured once into a CUDA graph and replayed.  The tile variant
-// (words per thread) and the walks per CTA come from a timing autotuner cached per (length set, SMs).
+// (length, walk) items; the sequence is captured once into a CUDA graph and replayed.
 // ---------------------------------------------------------------------------------------------
 namespace {
 
 uint64_t mix_key(uint64_t h, uint64_t v) { return sm64_at(h ^ v, 0x5EED); }
 
-// Issues the whole batched step on `st`.  blocks > 0: the walk grid was sized beforehand, so nothing
-// but stream work is issued (capturable); blocks == 0: the walk kernel is configured here.
-int issue_batch(labs_ctx* ctx, const labs_batch_cfg* cfg, const std::vector<LenSpec>& lens, const Variant& v,
-                int warps, const uint64_t* prefixes, int n_prefix, labs_candidate* out, int64_t* walk_stats,
-                int32_t* thr, labs_walk_stats* stats, unsigned long long* counter, int64_t flip_budget,
-                bool thresholds, long long blocks, cudaStream_t st) {
-  WalkParams* P = new (std::nothrow) WalkParams();
-  if (!P) return LABS_ERR_NOMEM;
-  base_params(*P, cfg->R, cfg->bloom_log2, cfg->bloom_k, cfg->p, n_prefix, flip_budget, cfg->seed, cfg->E_target,
-              prefixes, out, walk_stats, stats, counter);
-  if (!fill_params(*P, lens, v, cfg->R, false, cfg->bloom_log2)) {
-    delete P;
-    return LABS_ERR_INVALID_ARG;
-  }
-  P->E_thr_dev = thr;
+// Issues the whole batched step on `st`: stream work only (capturable).
+int issue_batch(labs_ctx* ctx, const labs_batch_cfg* cfg, const std::vector<LenSpec>& lens, const WalkParams& P,
+                const Launch& ln, int32_t* thr, cudaStream_t st) {
   int s = LABS_OK;
-  if (thresholds) {
-    for (size_t i = 0; i < lens.size() && s == LABS_OK; i++)
-      s = launch_sample_threshold(ctx, lens[i].L, lens[i].skew, lens[i].p, prefixes, n_prefix, P->prefix_words,
-                                  cfg->seed, cfg->n_thresh_samples, cfg->thresh_rank, thr + i, nullptr, st);
-  }
-  if (s == LABS_OK) {
-    walk_init_kernel<<<1, 1, 0, st>>>(stats, thr, 0, counter);
-    s = cuda_status(cudaGetLastError());
-  }
-  if (s == LABS_OK && P->n_items > 0) {
-    if (blocks > 0)
-      s = walk_variant(ctx, *P, v, warps, st, false, &blocks);
-    else
-      s = launch_walk(ctx, *P, v, warps, st);
-  }
-  delete P;
+  for (size_t i = 0; i < lens.size() && s == LABS_OK; i++)
+    s = launch_sample_threshold(ctx, lens[i].L, lens[i].skew, lens[i].p, P.prefixes, P.n_prefix, P.prefix_words,
+                                cfg->seed, cfg->n_thresh_samples, cfg->thresh_rank, thr + i, nullptr, st);
+  if (s == LABS_OK) s = run_init(P, st);
+  if (s == LABS_OK && P.n_items > 0) s = run_walks(P, ln, st);
   return s;
 }
 
@@ -1205,130 +1333,50 @@ int launch_batched_search(labs_ctx* ctx, const labs_batch_cfg* cfg, const int32_
                           const uint64_t* prefixes, int n_prefix, labs_candidate* out, int64_t* walk_stats,
                           int32_t* E_thr_out, labs_walk_stats* stats, cudaStream_t st) {
   std::vector<LenSpec> lens;
-  int64_t begin = 0;
   for (int i = 0; i < cfg->n_len; i++) {
     const int L = lengths[i];
     const int skew = L & 1;
     lens.push_back({L, skew, skew ? cfg->p : 0, cfg->T_i, walks[i], 0});
-    begin += walks[i];
   }
+  if (!accepted(lens, cfg->tile_m, 0, cfg->R, cfg->warps_per_cta)) return LABS_ERR_INVALID_ARG;
   // workspace first (nothing below may allocate once a capture has begun)
   char* w = static_cast<char*>(ws_get(ctx, kWsWalkCounters, 256));
   int32_t* thr = E_thr_out ? E_thr_out : static_cast<int32_t*>(ws_get(ctx, kWsBatchThresholds, sizeof(int32_t) * kMaxLens));
-  if (!w || !thr) return LABS_ERR_NOMEM;
+  uint64_t* zpair = static_cast<uint64_t*>(ws_get(ctx, kWsZpair, zpair_bytes(kMaxLens)));
+  std::unique_ptr<WalkParams> P(new (std::nothrow) WalkParams());
+  if (!w || !thr || !zpair || !P) return LABS_ERR_NOMEM;
   if (!ws_get(ctx, kWsThreshSamples, sizeof(int32_t) * (size_t)cfg->n_thresh_samples) ||
       !ws_get(ctx, kWsThreshHist, sizeof(unsigned) * 2 * kHistBins + 64))
     return LABS_ERR_NOMEM;
   unsigned long long* counter = reinterpret_cast<unsigned long long*>(w);
-
-  // ---- variant and walks per CTA: given, or timed
-  Variant v{0, 0, 0};
-  int warps = cfg->warps_per_cta;
-  uint64_t tkey = (uint64_t)ctx->num_sms;
-  for (const LenSpec& s : lens) tkey = mix_key(tkey, ((uint64_t)s.L << 40) ^ (uint64_t)s.walks);
-  tkey = mix_key(tkey, ((uint64_t)cfg->tile_m << 8) ^ (uint64_t)warps ^ ((uint64_t)cfg->R << 16) ^
-                           ((uint64_t)cfg->bloom_log2 << 24));
-  bool cached = false;
-  for (int i = 0; i < ctx->n_tuned; i++)
-    if (ctx->tuned_key[i] == tkey) {
-      v = {ctx->tuned[i][0], ctx->tuned[i][1], ctx->tuned[i][2]};
-      warps = ctx->tuned[i][3];
-      cached = true;
-    }
-  // the (variant, warps per CTA) candidates: whole-warp walks try 4 and 8 warps, half-warp walks the
-  // largest block whose slabs fit an SM
-  WalkParams* Q = new (std::nothrow) WalkParams();
-  if (!Q) return LABS_ERR_NOMEM;
-  if (!cached) {
-    std::vector<std::pair<Variant, int>> cands;
-    for (const Variant& c : kVariants) {
-      if (cfg->tile_m && c.M != cfg->tile_m) continue;
-      if (!fill_params(*Q, lens, c, cfg->R, false, cfg->bloom_log2)) continue;
-      if (warps > 0) {
-        if (32 * warps <= walk_block_threads(c.GL)) cands.push_back({c, warps});
-      } else if (c.GL == 32) {
-        cands.push_back({c, 4});
-        cands.push_back({c, 8});
-      } else {
-        cands.push_back({c, warps_for(ctx, *Q, c, 0)});
-      }
-    }
-    if (cands.empty()) {
-      delete Q;
-      return LABS_ERR_INVALID_ARG;
-    }
-    if (cands.size() == 1) {
-      v = cands[0].first;
-      warps = cands[0].second;
-    } else {
-      // trial: every length with 1/16 of its walks (at least one), 512 flips each, thresholds off
-      std::vector<LenSpec> trial = lens;
-      for (LenSpec& s : trial) s.walks = std::max<int64_t>(1, s.walks / 16);
-      cudaEvent_t e0, e1;
-      cudaEventCreate(&e0);
-      cudaEventCreate(&e1);
-      float best_ms = 0;
-      for (const auto& cw : cands) {
-        cudaEventRecord(e0, st);
-        int s = issue_batch(ctx, cfg, trial, cw.first, cw.second, prefixes, n_prefix, out, nullptr, thr, stats,
-                            counter, std::min<int64_t>(cfg->flip_budget, 512), false, 0, st);
-        cudaEventRecord(e1, st);
-        if (s != LABS_OK || cudaEventSynchronize(e1) != cudaSuccess) continue;
-        float ms = 0;
-        cudaEventElapsedTime(&ms, e0, e1);
-        if (v.M == 0 || ms < best_ms) {
-          best_ms = ms;
-          v = cw.first;
-          warps = cw.second;
-        }
-      }
-      cudaEventDestroy(e0);
-      cudaEventDestroy(e1);
-      if (v.M == 0) {
-        delete Q;
-        return LABS_ERR_CUDA;
-      }
-    }
-    if (ctx->n_tuned < kMaxTuned) {
-      ctx->tuned_key[ctx->n_tuned] = tkey;
-      ctx->tuned[ctx->n_tuned][0] = v.M;
-      ctx->tuned[ctx->n_tuned][1] = v.H;
-      ctx->tuned[ctx->n_tuned][2] = v.GL;
-      ctx->tuned[ctx->n_tuned][3] = warps;
-      ctx->n_tuned++;
-    }
-  }
+  base_params(*P, cfg->R, cfg->bloom_log2, cfg->bloom_k, cfg->p, n_prefix, cfg->flip_budget, cfg->seed, cfg->E_target,
+              prefixes, out, walk_stats, stats, counter, zpair);
+  Launch ln;
+  fill_params(*P, lens, cfg->bloom_log2, &ln);
+  P->E_thr_dev = thr;
   // kernel attributes and grid size before any capture
-  long long blocks = 0;
-  {
-    int s = fill_params(*Q, lens, v, cfg->R, false, cfg->bloom_log2) ? LABS_OK : LABS_ERR_INVALID_ARG;
-    Q->bloom_log2 = cfg->bloom_log2;
-    if (s == LABS_OK) s = walk_variant(ctx, *Q, v, warps, st, true, &blocks);
-    delete Q;
-    if (s != LABS_OK) return s;
-  }
-  if (!cfg->use_graph)
-    return issue_batch(ctx, cfg, lens, v, warps, prefixes, n_prefix, out, walk_stats, thr, stats, counter,
-                       cfg->flip_budget, true, blocks, st);
+  int s = plan_launch(ctx, *P, cfg->warps_per_cta, false, &ln);
+  if (s != LABS_OK) return s;
+  if (!cfg->use_graph) return issue_batch(ctx, cfg, lens, *P, ln, thr, st);
 
   // ---- CUDA graph: capture once per (configuration, buffers), replay afterwards
-  uint64_t gkey = tkey;
-  gkey = mix_key(gkey, ((uint64_t)v.M << 32) ^ ((uint64_t)v.H << 16) ^ ((uint64_t)v.GL << 8) ^ (uint64_t)warps);
+  uint64_t gkey = (uint64_t)ctx->num_sms;
+  for (const LenSpec& e : lens) gkey = mix_key(gkey, ((uint64_t)e.L << 40) ^ (uint64_t)e.walks);
+  gkey = mix_key(gkey, ((uint64_t)(100 * ln.ns + ln.nu) << 32) ^ ((uint64_t)ln.mode << 16) ^ (uint64_t)ln.warps);
   gkey = mix_key(gkey, (uint64_t)cfg->flip_budget ^ ((uint64_t)cfg->R << 48));
   gkey = mix_key(gkey, cfg->seed);
   gkey = mix_key(gkey, ((uint64_t)cfg->p << 32) ^ ((uint64_t)cfg->bloom_log2 << 16) ^ (uint64_t)cfg->bloom_k);
   gkey = mix_key(gkey, ((uint64_t)cfg->T_i << 32) ^ (uint32_t)cfg->E_target);
   gkey = mix_key(gkey, (uint64_t)cfg->n_thresh_samples ^ ((uint64_t)cfg->thresh_rank << 40));
-  const void* bufs[] = {prefixes, out, walk_stats, thr, stats, w, ctx->ws[kWsThreshSamples], ctx->ws[kWsThreshHist]};
+  const void* bufs[] = {prefixes, out, walk_stats, thr, stats, w, zpair, ctx->ws[kWsThreshSamples], ctx->ws[kWsThreshHist]};
   for (const void* ptr : bufs) gkey = mix_key(gkey, (uint64_t)(uintptr_t)ptr);
-  gkey = mix_key(gkey, (uint64_t)n_prefix ^ ((uint64_t)blocks << 32));
+  gkey = mix_key(gkey, (uint64_t)n_prefix ^ ((uint64_t)ln.blocks << 32));
   if (!ctx->graph_exec || ctx->graph_key != gkey) {
     if (!ctx->capture_stream && cudaStreamCreateWithFlags(&ctx->capture_stream, cudaStreamNonBlocking) != cudaSuccess)
       return LABS_ERR_CUDA;
     if (cudaStreamBeginCapture(ctx->capture_stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
       return LABS_ERR_CUDA;
-    int s = issue_batch(ctx, cfg, lens, v, warps, prefixes, n_prefix, out, walk_stats, thr, stats, counter,
-                        cfg->flip_budget, true, blocks, ctx->capture_stream);
+    s = issue_batch(ctx, cfg, lens, *P, ln, thr, ctx->capture_stream);
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamEndCapture(ctx->capture_stream, &g);
     if (s != LABS_OK) {
