@@ -1,55 +1,96 @@
-// energy_words.cuh -- E = sum_k C_k^2 (Section 1) of one bit-packed sequence by one warp, the sequence
+// energy_words.cuh -- C_k and E = sum_k C_k^2 (Section 1) of one bit-packed sequence by one warp, the sequence
 // held in registers.
 //
-// Lane l takes the lags k = 32 j + l (j = 0 .. NW - 1): for a given j every lane's word offset is j and its
-// bit shift is l, so with NW a compile-time constant the loops over j and the words unroll, and each 32
-// products cost one funnel shift, one XOR, one popcount and one add.  C_k = (L - k) - 2 d, d counting the
-// disagreeing pairs (s_i != s_{i+k}, i < L - k): the popcounts run over whole words, and the positions
-// past L - k (where the shifted word is zero) are taken out with prefix popcounts of the words.
+// Lane l takes the lags k = 32 j + l (j = 0 .. NW - 1): for a given j every lane's word offset is j and its bit
+// shift is l, so the shifted words f_v = (s >> l) of word v are formed once and the loops over j and the words
+// unroll.  C_k = (L - k) - 2 d, d counting the disagreeing pairs (s_i != s_{i+k}, i < L - k): the words of
+// s ^ f, those at the sequence's end masked to its positions in the same instruction.
+//
+// Popcounts issue at 16 lanes per clock and SM, logic at 64, so the words of a lag are added up by carry-save
+// adders first (sum and majority, two LOP3 each): seven words become one of weight 1, one of weight 2 and one
+// of weight 4, three popcounts instead of seven for eight LOP3.  Bound: the ALU pipe (about 270 warp
+// instructions a sequence at L = 451, 136 cycles; 51 popcounts, 102 cycles; a popcount per word: 240 cycles).
+// Measured, 2^20 sequences of L = 451: 574 us (992 us with a popcount per word).
+// The tensor cores gain less: mma.sync in 8-bit types converts to f16 pairs here, and f16 issues at 1,012
+// multiply-adds per clock and SM, 160 cycles for the product whose outputs are the C_k.
 #pragma once
 
 #include "labs_core.cuh"
 
 namespace labsg {
 
-// sb: the sequence's NW 32-bit words in shared memory followed by one zero word (sb[NW] = 0), bits at and
-// above L zero, L <= 32 NW; pre: per-warp scratch of NW + 1 ints.  Returns E on every lane; C_out, when not
-// null, receives C_k at C_out[k - 1] for k = 1 .. L-1.
-template <int NW>
-__device__ __forceinline__ int energy_words(const uint32_t* sb, int L, int* pre, int32_t* C_out) {
+// Sum and carry of three bits, lane by lane: one LOP3 each (left to the compiler, the shared a ^ b becomes a
+// third).
+__device__ __forceinline__ uint32_t add3(uint32_t a, uint32_t b, uint32_t c) {
+  uint32_t d;
+  asm("lop3.b32 %0, %1, %2, %3, 0x96;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+  return d;
+}
+__device__ __forceinline__ uint32_t maj3(uint32_t a, uint32_t b, uint32_t c) {
+  uint32_t d;
+  asm("lop3.b32 %0, %1, %2, %3, 0xE8;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+  return d;
+}
+
+// Counts the ones of N words x(0) .. x(N - 1) (compile-time N and indices).
+template <int N, int FROM = 0, class X>
+__device__ __forceinline__ int count_words(X&& x) {
+  constexpr int n = N - FROM;
+  if constexpr (n <= 0) {
+    return 0;
+  } else if constexpr (n >= 7) {
+    const uint32_t a = x(FROM), b = x(FROM + 1), c = x(FROM + 2), d = x(FROM + 3), e = x(FROM + 4), f = x(FROM + 5),
+                   g = x(FROM + 6);
+    const uint32_t s1 = add3(a, b, c), c1 = maj3(a, b, c), s2 = add3(d, e, f), c2 = maj3(d, e, f), s = add3(s1, s2, g),
+                   c3 = maj3(s1, s2, g);
+    return __popc(s) + 2 * __popc(add3(c1, c2, c3)) + 4 * __popc(maj3(c1, c2, c3)) + count_words<N, FROM + 7>(x);
+  } else if constexpr (n >= 5) {
+    const uint32_t a = x(FROM), b = x(FROM + 1), c = x(FROM + 2), d = x(FROM + 3), e = x(FROM + 4);
+    const uint32_t s1 = add3(a, b, c);
+    return __popc(add3(s1, d, e)) + 2 * (__popc(maj3(a, b, c)) + __popc(maj3(s1, d, e))) + count_words<N, FROM + 5>(x);
+  } else if constexpr (n >= 3) {
+    const uint32_t a = x(FROM), b = x(FROM + 1), c = x(FROM + 2);
+    return __popc(add3(a, b, c)) + 2 * __popc(maj3(a, b, c)) + count_words<N, FROM + 3>(x);
+  } else {
+    return __popc(x(FROM)) + count_words<N, FROM + 1>(x);
+  }
+}
+
+// One lag group j of energy_words and those after it (compile-time recursion over j).
+template <int NW, int J, bool WITH_C>
+__device__ __forceinline__ void energy_lags(const uint32_t (&b)[NW], const uint32_t (&f)[NW], uint32_t m1, uint32_t m2,
+                                            int left, int& e, int32_t* C_out) {
+  if constexpr (J < NW) {
+    const int d = count_words<NW - J>([&](int w) {
+      if (w + J < NW - 2) return b[w] ^ f[w + J];
+      uint32_t x;  // (b ^ f) & m
+      asm("lop3.b32 %0, %1, %2, %3, 0x28;" : "=r"(x) : "r"(b[w]), "r"(f[w + J]), "r"(w + J == NW - 1 ? m1 : m2));
+      return x;
+    });
+    const int t = left - 32 * J;  // L - k
+    const int c = max(t, 0) - 2 * d;
+    e += c * c;
+    if (WITH_C && t >= 1 && (J > 0 || lane_id() > 0)) C_out[32 * J + lane_id() - 1] = c;
+    energy_lags<NW, J + 1, WITH_C>(b, f, m1, m2, left, e, C_out);
+  }
+}
+
+// sb: the sequence's NW 32-bit words in shared memory (16-byte aligned), bits at and above L zero,
+// 32 (NW - 1) < L <= 32 NW.  Returns E on every lane; WITH_C: C_out receives C_k at C_out[k - 1], k = 1 .. L-1.
+template <int NW, bool WITH_C = false>
+__device__ __forceinline__ int energy_words(const uint32_t* sb, int L, int32_t* C_out = nullptr) {
   const int lane = lane_id();
-  int c1 = __popc(lane < NW ? sb[lane] : 0u);  // inclusive prefix of the words' popcounts
+  uint32_t b[NW], f[NW];
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int t = __shfl_up_sync(kFull, c1, o);
-    if (lane >= o) c1 += t;
-  }
-  __syncwarp();  // an earlier call's readers of pre are done
-  if (lane < NW) pre[lane + 1] = c1;
-  if (lane == 0) pre[0] = 0;
-  __syncwarp();
-  uint32_t b[NW + 1];
+  for (int w = 0; w < NW; w++) b[w] = sb[w];
 #pragma unroll
-  for (int w = 0; w <= NW; w++) b[w] = sb[w];
+  for (int v = 0; v < NW; v++) f[v] = __funnelshift_r(b[v], v + 1 < NW ? b[v + 1] : 0u, lane);
+  // positions of the last two shifted words inside the sequence
+  auto low = [](int n) { return n >= 32 ? 0xffffffffu : (n <= 0 ? 0u : (1u << n) - 1u); };
+  const int r = L - 32 * (NW - 1) - lane;
   int e = 0;
-#pragma unroll
-  for (int j = 0; j < NW; j++) {
-    const int k = 32 * j + lane;
-    int d = 0;
-#pragma unroll
-    for (int w = 0; w + j < NW; w++) d += __popc(b[w] ^ __funnelshift_r(b[w + j], b[w + j + 1], lane));
-    if (k >= 1 && k < L) {
-      // the words cover positions [0, 32 (NW - j)); past t = L - k the shifted word is zero, so the
-      // popcount also counted the ones of s there
-      const int t = L - k;
-      const int pt = pre[t >> 5] + __popc(sb[t >> 5] & ((1u << (t & 31)) - 1u));
-      d -= pre[NW - j] - pt;
-      const int c = t - 2 * d;
-      if (C_out) C_out[k - 1] = c;
-      e += c * c;
-    }
-  }
-  return warp_sum_i32(e);
+  energy_lags<NW, 0, WITH_C>(b, f, low(r), low(r + 32), L - lane, e, C_out);
+  return warp_sum_i32(e) - L * L;  // without k = 0
 }
 
 }  // namespace labsg

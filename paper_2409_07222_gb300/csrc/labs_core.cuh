@@ -603,32 +603,44 @@ __device__ inline void load_bits(S& sm, const uint64_t* src, int L) {
 
 // Builds a walk start into the bits (kBitWords words): s_1..s_p from the prefix, free element j (position
 // p+1+j) is +1 iff bit j%64 of output j/64 of stream `key`; skew walks fill the last k by Eq. (2) around the
-// centre c.
-__device__ inline void build_start(uint32_t* bits, int L, bool skew, int c, int p, const uint64_t* prefix, uint64_t key) {
+// centre c.  Lane w forms word w: the outputs' words shifted by p, then for skew sequences the mirrored half,
+// its bits reversed and every other one negated.  scr: kBitWords + 2 words of scratch.
+__device__ inline void build_start(uint32_t* bits, uint32_t* scr, int L, bool skew, int c, int p, const uint64_t* prefix,
+                                   uint64_t key) {
   const int lane = lane_id();
-  for (int w = 0; w < kBitWords; w++) {
-    const int i = 32 * w + lane + 1;
-    int bit = 0;
-    if (i <= L) {
-      int src = i;
-      int neg = 0;
-      if (skew && i > c) {
-        src = 2 * c - i;
-        neg = (i - c) & 1;
-      }
-      int b;
-      if (src <= p) {
-        b = (int)((prefix[(src - 1) >> 6] >> ((src - 1) & 63)) & 1u);
-      } else {
-        int j = src - p - 1;
-        b = (int)((sm64_at(key, (uint64_t)(j >> 6)) >> (j & 63)) & 1u);
-      }
-      bit = b ^ neg;
-    }
-    const unsigned word = __ballot_sync(kFull, bit);
-    if (lane == 0) bits[w] = word;
+  __syncwarp();
+  if (lane < 11) {
+    const uint64_t o = lane < LABS_MAX_W ? sm64_at(key, (uint64_t)lane) : 0ull;
+    scr[2 * lane] = (uint32_t)o;
+    scr[2 * lane + 1] = (uint32_t)(o >> 32);
   }
   __syncwarp();
+  const int i0 = 32 * lane;  // 0-based position of the word's first bit
+  // the low n bits, n of any sign
+  auto low = [](int n) { return n >= 32 ? 0xffffffffu : (n <= 0 ? 0u : (1u << n) - 1u); };
+  // 32 bits of `w` from bit o on; bits in front of w are zero
+  auto window = [](const uint32_t* w, int o) {
+    if (o < 0) return o > -32 ? w[0] << -o : 0u;
+    return __funnelshift_r(w[o >> 5], w[(o >> 5) + 1], o & 31);
+  };
+  uint32_t x = 0;
+  const int n = skew ? c : L;  // positions drawn
+  if (i0 < n) {
+    x = window(scr, i0 - p);
+    if (i0 < p) x = (x & ~low(p - i0)) | ((uint32_t)(prefix[lane >> 1] >> (32 * (lane & 1))) & low(p - i0));
+    x &= low(n - i0);
+  }
+  if (lane < kBitWords) bits[lane] = x;
+  __syncwarp();
+  if (skew) {
+    const int k = c - 1;
+    uint32_t y = 0;
+    if (i0 < L && i0 + 31 > k)  // position k + j mirrors k - j, negated for odd j
+      y = (__brev(window(bits, 2 * k - i0 - 31)) ^ (k & 1 ? 0x55555555u : 0xAAAAAAAAu)) & low(L - i0) & ~low(c - i0);
+    __syncwarp();
+    if (lane < kBitWords) bits[lane] = x | y;
+    __syncwarp();
+  }
 }
 
 // Zobrist fingerprint of the sequence in the bits.

@@ -2,6 +2,7 @@
 #pragma once
 #include <cstddef>
 #include <cstdint>
+#include <type_traits>
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
@@ -51,6 +52,17 @@ enum WsSlot {
 void* ws_get(labs_ctx* ctx, int slot, size_t bytes);
 
 int policy_length(const labs_policy* P);
+
+// fn(integral_constant<int, n>) for a run-time number of 32-bit words n, 1 .. 18 (a sequence of up to 576
+// elements): the kernels that hold a sequence in registers are compiled per word count.
+template <int N = 1, class Fn>
+int by_words(int n, Fn&& fn) {
+  if constexpr (N > 2 * LABS_MAX_W) {
+    return LABS_ERR_INVALID_ARG;
+  } else {
+    return n == N ? fn(std::integral_constant<int, N>{}) : by_words<N + 1>(n, fn);
+  }
+}
 
 inline int cuda_status(cudaError_t e) { return e == cudaSuccess ? LABS_OK : LABS_ERR_CUDA; }
 

@@ -6,6 +6,8 @@
 // the sequences (one warp each: the non-zero squares k^2 mod p, k <= (p-1)/2, marked in a shared-memory
 // bitmap, then one bitmap test per position and ballots into words) and their energies as in
 // labs_energy_batch (energy_words.cuh).
+#include <algorithm>
+
 #include "energy_words.cuh"
 #include "labs_internal.h"
 
@@ -35,12 +37,10 @@ template <int NW>
 __global__ void __launch_bounds__(32 * kLegWarps) legendre_kernel(int L, const int32_t* __restrict__ params, int64_t n,
                                                                  uint64_t* __restrict__ seqs, int32_t* __restrict__ E_out,
                                                                  const __grid_constant__ PrimeBits primes) {
-  __shared__ int pre_all[kLegWarps][kBitWords + 1];
-  __shared__ uint32_t bits_all[kLegWarps][kBitWords];
+  __shared__ __align__(16) uint32_t bits_all[kLegWarps][kBitWords];
   __shared__ uint32_t qr_all[kLegWarps][kBitWords];  // bit j: j is a non-zero square mod p
   uint32_t* bits = bits_all[threadIdx.x >> 5];
   uint32_t* qr = qr_all[threadIdx.x >> 5];
-  int* pre = pre_all[threadIdx.x >> 5];
   const int lane = lane_id();
   const int W = (L + 63) >> 6;
   const int64_t warps_total = (int64_t)gridDim.x * kLegWarps;
@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(32 * kLegWarps) legendre_kernel(int L, const i
       if (j >= p) j -= p;
     }
     __syncwarp();
-    const int e = energy_words<NW>(bits, L, pre, nullptr);
+    const int e = energy_words<NW>(bits, L);
     if (seqs && lane < W) seqs[q * W + lane] = (uint64_t)bits[2 * lane] | ((uint64_t)bits[2 * lane + 1] << 32);
     if (E_out && lane == 0) E_out[q] = e;
     __syncwarp();
@@ -114,18 +114,10 @@ int launch_legendre(labs_ctx* ctx, int L, const int32_t* params, int64_t n, uint
   PrimeBits pb{};
   for (int v = 0; v < 32 * kPrimeWords; v++)
     if (is_prime(v)) pb.w[v >> 5] |= 1u << (v & 31);
-#define LABS_LEG_CASE(NWC)                                                             \
-  case NWC:                                                                          \
-    legendre_kernel<NWC><<<nb, 32 * kLegWarps, 0, st>>>(L, params, n, seqs, E_out, pb); \
-    break;
-  switch ((L + 31) >> 5) {
-    LABS_LEG_CASE(1) LABS_LEG_CASE(2) LABS_LEG_CASE(3) LABS_LEG_CASE(4) LABS_LEG_CASE(5) LABS_LEG_CASE(6)
-    LABS_LEG_CASE(7) LABS_LEG_CASE(8) LABS_LEG_CASE(9) LABS_LEG_CASE(10) LABS_LEG_CASE(11) LABS_LEG_CASE(12)
-    LABS_LEG_CASE(13) LABS_LEG_CASE(14) LABS_LEG_CASE(15) LABS_LEG_CASE(16) LABS_LEG_CASE(17) LABS_LEG_CASE(18)
-    default: return LABS_ERR_INVALID_ARG;
-  }
-#undef LABS_LEG_CASE
-  return cuda_status(cudaGetLastError());
+  return by_words((L + 31) >> 5, [&](auto nw) {
+    legendre_kernel<decltype(nw)::value><<<nb, 32 * kLegWarps, 0, st>>>(L, params, n, seqs, E_out, pb);
+    return cuda_status(cudaGetLastError());
+  });
 }
 
 }  // namespace labsg

@@ -2,11 +2,12 @@
 // neighbouring lengths (Section 3: appending or removing an element at either end gives sequences of
 // length L+1 and L-1 with comparable merit factor, which re-enter step 2; the loop of Fig. 4).
 //
-// One warp per input sequence.  Lane w owns 32-bit word w of the sequence and of each variant: an append
-// sets bit L, a prepend shifts every word up by one bit, a removal clears the last bit or shifts down by
-// one.  Each variant's energy is then the Section 1 definition evaluated as in labs_energy_batch
-// (energy_words.cuh: the variant held in registers, one popcount per 32 products).  Six variants per
-// input: about 6 (L+-1)^2/64 popcounts.
+// One warp per result.  Lane w owns 32-bit word w of the sequence: an append sets bit L, a prepend shifts
+// every word up by one bit, a removal clears the last bit or shifts down by one.  The energy is that of
+// labs_energy_batch (energy_words.cuh).  Six results per input, so that even one input fills six warps (step
+// 2's best sequence is what a search hands over).
+#include <algorithm>
+
 #include "energy_words.cuh"
 #include "labs_internal.h"
 
@@ -22,70 +23,51 @@ __device__ __forceinline__ void store_words(const uint32_t* vbits, int Lv, uint6
   if (lane < W) dst[lane] = (uint64_t)vbits[2 * lane] | ((uint64_t)vbits[2 * lane + 1] << 32);
 }
 
-// NW: 32-bit words of the longer variants (L + 1 bits), so every variant fits with a zero word after it.
-template <int NW>
+// Result v of an input: 0, 1 append +1 / -1, 2, 3 prepend +1 / -1, 4 without the last element, 5 without the
+// first.  NG, NS: 32-bit words of L + 1 and of L - 1 positions.
+template <int NG, int NS>
 __global__ void __launch_bounds__(32 * kOpWarps) operators_kernel(const uint64_t* __restrict__ seqs, int L, int64_t n,
                                                                   uint64_t* __restrict__ grow, int32_t* __restrict__ E_grow,
                                                                   uint64_t* __restrict__ shrink,
                                                                   int32_t* __restrict__ E_shrink) {
-  __shared__ uint32_t sb[kOpWarps][kBitWords];
-  __shared__ uint32_t vb[kOpWarps][kBitWords];
-  __shared__ int pre_all[kOpWarps][kBitWords + 1];
-  uint32_t* bits = sb[threadIdx.x >> 5];
+  __shared__ __align__(16) uint32_t vb[kOpWarps][kBitWords];
   uint32_t* v = vb[threadIdx.x >> 5];
-  int* pre = pre_all[threadIdx.x >> 5];
   const int lane = lane_id();
   const int W = (L + 63) >> 6, Wg = (L + 64) >> 6, Ws = (L + 62) >> 6;
   const int W32 = (L + 31) >> 5;
   const int64_t warps_total = (int64_t)gridDim.x * kOpWarps;
-  for (int64_t q = (int64_t)blockIdx.x * kOpWarps + (threadIdx.x >> 5); q < n; q += warps_total) {
-    if (lane < kBitWords) {
-      uint32_t x = 0;
-      if (lane < W32) {
-        const uint64_t w = seqs[q * W + (lane >> 1)];
-        x = (lane & 1) ? (uint32_t)(w >> 32) : (uint32_t)w;
-        const int rem = L - 32 * lane;
-        if (rem < 32) x &= (1u << rem) - 1u;
-      }
-      bits[lane] = x;
+  for (int64_t r = (int64_t)blockIdx.x * kOpWarps + (threadIdx.x >> 5); r < 6 * n; r += warps_total) {
+    const int64_t q = r / 6;
+    const int var = (int)(r - 6 * q);
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(seqs + q * W);
+    uint32_t x = 0;
+    if (lane < W32) {
+      x = src[lane];
+      const int rem = L - 32 * lane;
+      if (rem < 32) x &= (1u << rem) - 1u;
     }
+    const uint32_t below = __shfl_up_sync(kFull, x, 1), above = __shfl_down_sync(kFull, x, 1);
+    const uint32_t bit = (var & 1) ? 0u : 1u;  // value of a new element (1 = +1)
+    uint32_t w;
+    if (var < 2)
+      w = lane == (L >> 5) ? x | bit << (L & 31) : x;
+    else if (var < 4)
+      w = (x << 1) | (lane ? below >> 31 : bit);
+    else if (var == 4)
+      w = lane == ((L - 1) >> 5) ? x & ~(1u << ((L - 1) & 31)) : x;
+    else
+      w = (x >> 1) | (above << 31);
+    __syncwarp();  // the previous result's readers of v are done
+    if (lane < kBitWords) v[lane] = w;
     __syncwarp();
-    // grow: v = 0, 1 append +1 / -1 (bit L), v = 2, 3 prepend +1 / -1 (shift up, bit 0)
-    for (int var = 0; var < 4; var++) {
-      const uint32_t x = (var & 1) ? 0u : 1u;  // bit value of the new element (1 = +1)
-      if (lane < kBitWords) {
-        uint32_t w;
-        if (var < 2) {
-          w = bits[lane];
-          if (lane == (L >> 5)) w |= x << (L & 31);
-        } else {
-          w = (bits[lane] << 1) | (lane ? bits[lane - 1] >> 31 : x);
-        }
-        v[lane] = w;
-      }
-      __syncwarp();
-      const int E = energy_words<NW>(v, L + 1, pre, nullptr);
-      if (grow) store_words(v, L + 1, grow + (q * 4 + var) * Wg);
+    const int Lv = var < 4 ? L + 1 : L - 1;
+    const int E = var < 4 ? energy_words<NG>(v, Lv) : energy_words<NS>(v, Lv);
+    if (var < 4) {
+      if (grow) store_words(v, Lv, grow + (q * 4 + var) * Wg);
       if (E_grow && lane == 0) E_grow[q * 4 + var] = E;
-      __syncwarp();
-    }
-    // shrink: v = 0 drops the last element (clear bit L-1), v = 1 drops the first (shift down)
-    for (int var = 0; var < 2; var++) {
-      if (lane < kBitWords) {
-        uint32_t w;
-        if (var == 0) {
-          w = bits[lane];
-          if (lane == ((L - 1) >> 5)) w &= ~(1u << ((L - 1) & 31));
-        } else {
-          w = (bits[lane] >> 1) | (lane + 1 < kBitWords ? bits[lane + 1] << 31 : 0u);
-        }
-        v[lane] = w;
-      }
-      __syncwarp();
-      const int E = energy_words<NW>(v, L - 1, pre, nullptr);
-      if (shrink) store_words(v, L - 1, shrink + (q * 2 + var) * Ws);
-      if (E_shrink && lane == 0) E_shrink[q * 2 + var] = E;
-      __syncwarp();
+    } else {
+      if (shrink) store_words(v, Lv, shrink + (q * 2 + var - 4) * Ws);
+      if (E_shrink && lane == 0) E_shrink[q * 2 + var - 4] = E;
     }
   }
 }
@@ -95,20 +77,15 @@ __global__ void __launch_bounds__(32 * kOpWarps) operators_kernel(const uint64_t
 int launch_sequence_operators(labs_ctx* ctx, const uint64_t* seqs, int L, int64_t n, uint64_t* grow, int32_t* E_grow,
                               uint64_t* shrink, int32_t* E_shrink, cudaStream_t st) {
   if (n == 0) return LABS_OK;
-  const unsigned blocks = (unsigned)std::min<int64_t>((n + kOpWarps - 1) / kOpWarps, (int64_t)ctx->num_sms * 32);
-#define LABS_OPS_CASE(NWC)                                                                                   \
-  case NWC:                                                                                                \
-    operators_kernel<NWC><<<blocks, 32 * kOpWarps, 0, st>>>(seqs, L, n, grow, E_grow, shrink, E_shrink); \
-    break;
-  switch ((L + 32) >> 5) {  // words of L + 1 bits
-    LABS_OPS_CASE(1) LABS_OPS_CASE(2) LABS_OPS_CASE(3) LABS_OPS_CASE(4) LABS_OPS_CASE(5) LABS_OPS_CASE(6)
-    LABS_OPS_CASE(7) LABS_OPS_CASE(8) LABS_OPS_CASE(9) LABS_OPS_CASE(10) LABS_OPS_CASE(11) LABS_OPS_CASE(12)
-    LABS_OPS_CASE(13) LABS_OPS_CASE(14) LABS_OPS_CASE(15) LABS_OPS_CASE(16) LABS_OPS_CASE(17) LABS_OPS_CASE(18)
-    LABS_OPS_CASE(19)
-    default: return LABS_ERR_INVALID_ARG;
-  }
-#undef LABS_OPS_CASE
-  return cuda_status(cudaGetLastError());
+  const unsigned nb = (unsigned)std::min<int64_t>((6 * n + kOpWarps - 1) / kOpWarps, (int64_t)ctx->num_sms * 16);
+  return by_words((L + 32) >> 5, [&](auto nw) {
+    constexpr int NG = decltype(nw)::value, NL = NG > 1 ? NG - 1 : 1;
+    if ((L + 30) >> 5 == NG)
+      operators_kernel<NG, NG><<<nb, 32 * kOpWarps, 0, st>>>(seqs, L, n, grow, E_grow, shrink, E_shrink);
+    else  // L - 1 positions end one word earlier
+      operators_kernel<NG, NL><<<nb, 32 * kOpWarps, 0, st>>>(seqs, L, n, grow, E_grow, shrink, E_shrink);
+    return cuda_status(cudaGetLastError());
+  });
 }
 
 }  // namespace labsg

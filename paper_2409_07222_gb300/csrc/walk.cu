@@ -20,7 +20,7 @@
 #include <mutex>
 #include <vector>
 
-#include "labs_core.cuh"
+#include "energy_words.cuh"
 #include "labs_internal.h"
 
 namespace labsg {
@@ -343,7 +343,7 @@ __global__ void __launch_bounds__(walk_block_threads(MODE, NS, NU), 1)
     auto start_segment = [&]() {
       const int64_t w = le.walk_begin + ((long long)item - le.item_begin);
       const unsigned seg = ctl->segs;
-      build_start(bits, L, skew, c, p, P.prefixes + (w % P.n_prefix) * P.prefix_words,
+      build_start(bits, bloom, L, skew, c, p, P.prefixes + (w % P.n_prefix) * P.prefix_words,
                   stream_key(P.seed, kPurposeWalk, (uint64_t)w, (uint64_t)seg));
       build_state();
       __syncwarp();
@@ -894,54 +894,72 @@ __global__ void __launch_bounds__(128) walk_init_kernel(const __grid_constant__ 
 constexpr int kSampleWarps = 8;
 constexpr int kHistBins = 8192;
 
+// One warp per sample: the start's bits and its energy (all lags: a skew start's odd ones are zero).  The
+// energies crowd into a few of the first level's bins, so a block counts in shared memory and adds its counts
+// once (an atomic per sample would serialise on them).
+template <int NW>
 __global__ void __launch_bounds__(32 * kSampleWarps) sample_kernel(int L, int skew, int p,
                                                                     const uint64_t* __restrict__ prefixes, int n_prefix,
                                                                     int prefix_words, uint64_t seed, int64_t n,
                                                                     int32_t* __restrict__ E_out,
                                                                     unsigned* __restrict__ hist) {
-  __shared__ ScanSmem slabs[kSampleWarps];
-  ScanSmem& sm = slabs[threadIdx.x >> 5];
-  Layout ly;
-  make_layout(ly, L, skew, p, 8);
+  __shared__ unsigned counts[kHistBins];
+  __shared__ __align__(16) uint32_t bits_all[kSampleWarps][kBitWords], scr_all[kSampleWarps][kBitWords + 2];
+  uint32_t* bits = bits_all[threadIdx.x >> 5];
+  for (int b = threadIdx.x; b < kHistBins; b += blockDim.x) counts[b] = 0u;
+  __syncthreads();
   const int64_t warps_total = (int64_t)gridDim.x * kSampleWarps;
   for (int64_t i = (int64_t)blockIdx.x * kSampleWarps + (threadIdx.x >> 5); i < n; i += warps_total) {
-    build_start(sm.bits, L, skew != 0, ly.c, p, prefixes + (i % n_prefix) * prefix_words,
+    build_start(bits, scr_all[threadIdx.x >> 5], L, skew != 0, (L + 1) / 2, p, prefixes + (i % n_prefix) * prefix_words,
                 stream_key(seed, kPurposeThresh, (uint64_t)i, 0));
-    int E;
-    if (skew) {
-      E = build_table(sm, ly);
-    } else {
-      int e = 0;
-      for (int k = lane_id() + 1; k < L; k += 32) {
-        int c = corr_lag(sm.bits, L, k);
-        e += c * c;
-      }
-      E = warp_sum_i32(e);
-    }
+    const int E = energy_words<NW>(bits, L);
     if (lane_id() == 0) {
       E_out[i] = E;
-      atomicAdd(&hist[E >> 13], 1u);
+      atomicAdd(&counts[E >> 13], 1u);
     }
-    __syncwarp();
   }
+  __syncthreads();
+  for (int b = threadIdx.x; b < kHistBins; b += blockDim.x)
+    if (counts[b]) atomicAdd(&hist[b], counts[b]);
 }
 
-// One block: finds the bin holding `rank` in hist (kHistBins bins); sel[0] = bin, sel[1] = rank inside.
-__global__ void select_bin_kernel(const unsigned* __restrict__ hist, int64_t rank, long long* sel) {
-  __shared__ unsigned long long part[1024];
-  const int t = threadIdx.x;  // 1024 threads, 8 bins each
+// One block of 1024 threads: the bin of hist (kHistBins bins, eight a thread) that holds `rank`, and the
+// rank inside it.  Returns true on the one thread that found it.
+__device__ __forceinline__ bool find_bin(const unsigned* __restrict__ hist, unsigned long long rank, int* bin,
+                                         unsigned long long* inside) {
+  __shared__ unsigned long long warp_sum[32];
+  const int t = threadIdx.x, lane = lane_id();
+  unsigned own[8];
   unsigned long long s = 0;
-  for (int b = 0; b < 8; b++) s += hist[t * 8 + b];
-  part[t] = s;
+#pragma unroll
+  for (int b = 0; b < 8; b++) {
+    own[b] = hist[t * 8 + b];
+    s += own[b];
+  }
+  unsigned long long incl = s;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long v = __shfl_up_sync(kFull, incl, o);
+    if (lane >= o) incl += v;
+  }
+  if (lane == 31) warp_sum[t >> 5] = incl;
   __syncthreads();
-  if (t == 0) {
-    unsigned long long acc = 0;
-    int chunk = 0;
-    while (chunk < 1024 && acc + part[chunk] <= (unsigned long long)rank) acc += part[chunk++];
-    int bin = chunk * 8;
-    while (bin < chunk * 8 + 7 && acc + hist[bin] <= (unsigned long long)rank) acc += hist[bin++];
+  unsigned long long before = incl - s;
+  for (int w = 0; w < t >> 5; w++) before += warp_sum[w];
+  if (!(before <= rank && rank < before + s)) return false;
+  int b = 0;
+  while (b < 7 && before + own[b] <= rank) before += own[b++];
+  *bin = t * 8 + b;
+  *inside = rank - before;
+  return true;
+}
+
+__global__ void __launch_bounds__(1024) select_bin_kernel(const unsigned* __restrict__ hist, int64_t rank, long long* sel) {
+  int bin;
+  unsigned long long inside;
+  if (find_bin(hist, (unsigned long long)rank, &bin, &inside)) {
     sel[0] = bin;
-    sel[1] = (long long)rank - (long long)acc;
+    sel[1] = (long long)inside;
   }
 }
 
@@ -954,21 +972,30 @@ __global__ void hist_low_kernel(const int32_t* __restrict__ E, int64_t n, const 
   }
 }
 
-__global__ void finish_select_kernel(const unsigned* __restrict__ hist2, long long* sel, int32_t* E_thr_out) {
-  __shared__ unsigned long long part[1024];
-  const int t = threadIdx.x;
-  unsigned long long s = 0;
-  for (int b = 0; b < 8; b++) s += hist2[t * 8 + b];
-  part[t] = s;
-  __syncthreads();
-  if (t == 0) {
-    unsigned long long rank = (unsigned long long)sel[1], acc = 0;
-    int chunk = 0;
-    while (chunk < 1024 && acc + part[chunk] <= rank) acc += part[chunk++];
-    int low = chunk * 8;
-    while (low < chunk * 8 + 7 && acc + hist2[low] <= rank) acc += hist2[low++];
-    *E_thr_out = (int32_t)((sel[0] << 13) | low);
-  }
+__global__ void __launch_bounds__(1024) finish_select_kernel(const unsigned* __restrict__ hist2, const long long* sel,
+                                                             int32_t* E_thr_out) {
+  int low;
+  unsigned long long inside;
+  if (find_bin(hist2, (unsigned long long)sel[1], &low, &inside)) *E_thr_out = (int32_t)((sel[0] << 13) | low);
+}
+
+// The whole bound on `st`: samples into Es [n_samples], the two histograms at hist, the selected bin at sel.
+static int issue_threshold(int sms, int L, int skew, int p, const uint64_t* prefixes, int n_prefix, int prefix_words,
+                           uint64_t seed, int64_t n_samples, int64_t rank, int32_t* E_thr_out, int32_t* Es,
+                           unsigned* hist, long long* sel, cudaStream_t st) {
+  if (cudaMemsetAsync(hist, 0, sizeof(unsigned) * 2 * kHistBins, st) != cudaSuccess) return LABS_ERR_CUDA;
+  const unsigned blocks = (unsigned)std::min<int64_t>((n_samples + kSampleWarps - 1) / kSampleWarps, (int64_t)sms * 4);
+  const int s = by_words((L + 31) >> 5, [&](auto nw) {
+    sample_kernel<decltype(nw)::value>
+        <<<blocks, 32 * kSampleWarps, 0, st>>>(L, skew, p, prefixes, n_prefix, prefix_words, seed, n_samples, Es, hist);
+    return cuda_status(cudaGetLastError());
+  });
+  if (s != LABS_OK) return s;
+  select_bin_kernel<<<1, 1024, 0, st>>>(hist, rank, sel);
+  const int64_t hb = std::min<int64_t>((n_samples + 255) / 256, (int64_t)sms * 8);
+  hist_low_kernel<<<(unsigned)hb, 256, 0, st>>>(Es, n_samples, sel, hist + kHistBins);
+  finish_select_kernel<<<1, 1024, 0, st>>>(hist + kHistBins, sel, E_thr_out);
+  return cuda_status(cudaGetLastError());
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1206,15 +1233,8 @@ int launch_sample_threshold(labs_ctx* ctx, int L, int skew, int p, const uint64_
   unsigned* hist = static_cast<unsigned*>(ws_get(ctx, kWsThreshHist, sizeof(unsigned) * 2 * kHistBins + 64));
   if (!hist) return LABS_ERR_NOMEM;
   long long* sel = reinterpret_cast<long long*>(hist + 2 * kHistBins);
-  if (cudaMemsetAsync(hist, 0, sizeof(unsigned) * 2 * kHistBins, st) != cudaSuccess) return LABS_ERR_CUDA;
-  int64_t blocks = std::min<int64_t>((n_samples + kSampleWarps - 1) / kSampleWarps, (int64_t)ctx->num_sms * 8);
-  sample_kernel<<<(unsigned)blocks, 32 * kSampleWarps, 0, st>>>(L, skew, p, prefixes, n_prefix, prefix_words, seed,
-                                                                 n_samples, Es, hist);
-  select_bin_kernel<<<1, 1024, 0, st>>>(hist, rank, sel);
-  int64_t hb = std::min<int64_t>((n_samples + 255) / 256, (int64_t)ctx->num_sms * 8);
-  hist_low_kernel<<<(unsigned)hb, 256, 0, st>>>(Es, n_samples, sel, hist + kHistBins);
-  finish_select_kernel<<<1, 1024, 0, st>>>(hist + kHistBins, sel, E_thr_out);
-  return cuda_status(cudaGetLastError());
+  return issue_threshold(ctx->num_sms, L, skew, p, prefixes, n_prefix, prefix_words, seed, n_samples, rank, E_thr_out,
+                         Es, hist, sel, st);
 }
 
 int launch_skew_search(labs_ctx* ctx, const labs_walk_cfg* cfg, const uint64_t* prefixes, int n_prefix,
@@ -1458,14 +1478,7 @@ extern "C" int labs_sample_threshold_noalloc(int L, int skew, int p, const uint6
   long long* sel = reinterpret_cast<long long*>(base + kNoAllocSamplesBytes + kNoAllocHistBytes);
   cudaStream_t st = (cudaStream_t)stream;
   const int prefix_words = p > 0 ? (p + 63) / 64 : 1;
-  // the histograms keep the previous call's counts: clear them first
-  if (cudaMemsetAsync(hist, 0, kNoAllocHistBytes, st) != cudaSuccess) return LABS_ERR_CUDA;
-  int64_t blocks = std::min<int64_t>((n_samples + kSampleWarps - 1) / kSampleWarps, (int64_t)sms * 8);
-  sample_kernel<<<(unsigned)blocks, 32 * kSampleWarps, 0, st>>>(L, skew, p, prefixes, n_prefix, prefix_words, seed,
-                                                                 n_samples, Es, hist);
-  select_bin_kernel<<<1, 1024, 0, st>>>(hist, rank, sel);
-  int64_t hb = std::min<int64_t>((n_samples + 255) / 256, (int64_t)sms * 8);
-  hist_low_kernel<<<(unsigned)hb, 256, 0, st>>>(Es, n_samples, sel, hist + kHistBins);
-  finish_select_kernel<<<1, 1024, 0, st>>>(hist + kHistBins, sel, E_thr_out);
-  return cudaGetLastError() == cudaSuccess ? LABS_OK : LABS_ERR_CUDA;
+  // (the histograms keep the previous call's counts and are cleared first)
+  return issue_threshold(sms, L, skew, p, prefixes, n_prefix, prefix_words, seed, n_samples, rank, E_thr_out, Es, hist,
+                         sel, st);
 }
