@@ -56,40 +56,50 @@ __device__ __forceinline__ int count_words(X&& x) {
   }
 }
 
-// One lag group j of energy_words and those after it (compile-time recursion over j).
-template <int NW, int J, bool WITH_C>
-__device__ __forceinline__ void energy_lags(const uint32_t (&b)[NW], const uint32_t (&f)[NW], uint32_t m1, uint32_t m2,
-                                            int left, int& e, int32_t* C_out) {
+// Lag groups J, J + 1, .. of corr_words (compile-time recursion).
+template <int NW, int J, class Emit>
+__device__ __forceinline__ void corr_lags(const uint32_t (&a)[NW], const uint32_t (&f)[NW], uint32_t m1, uint32_t m2,
+                                          int left, Emit&& emit) {
   if constexpr (J < NW) {
     const int d = count_words<NW - J>([&](int w) {
-      if (w + J < NW - 2) return b[w] ^ f[w + J];
-      uint32_t x;  // (b ^ f) & m
-      asm("lop3.b32 %0, %1, %2, %3, 0x28;" : "=r"(x) : "r"(b[w]), "r"(f[w + J]), "r"(w + J == NW - 1 ? m1 : m2));
+      if (w + J < NW - 2) return a[w] ^ f[w + J];
+      uint32_t x;  // (a ^ f) & m
+      asm("lop3.b32 %0, %1, %2, %3, 0x28;" : "=r"(x) : "r"(a[w]), "r"(f[w + J]), "r"(w + J == NW - 1 ? m1 : m2));
       return x;
     });
-    const int t = left - 32 * J;  // L - k
-    const int c = max(t, 0) - 2 * d;
-    e += c * c;
-    if (WITH_C && t >= 1 && (J > 0 || lane_id() > 0)) C_out[32 * J + lane_id() - 1] = c;
-    energy_lags<NW, J + 1, WITH_C>(b, f, m1, m2, left, e, C_out);
+    emit(32 * J + lane_id(), max(left - 32 * J, 0) - 2 * d);
+    corr_lags<NW, J + 1>(a, f, m1, m2, left, emit);
   }
 }
 
-// sb: the sequence's NW 32-bit words in shared memory (16-byte aligned), bits at and above L zero,
-// 32 (NW - 1) < L <= 32 NW.  Returns E on every lane; WITH_C: C_out receives C_k at C_out[k - 1], k = 1 .. L-1.
+// emit(k, sum_{i < n-k} a_i b_{i+k}) for the lane's lags k = 32 j + lane, j < NW (0 for k >= n), of two
+// sequences of length n, 32 (NW - 1) <= n <= 32 NW, given by their NW 32-bit words in shared memory (16-byte
+// aligned), bits at and above n zero.
+template <int NW, class Emit>
+__device__ __forceinline__ void corr_words(const uint32_t* a, const uint32_t* b, int n, Emit&& emit) {
+  const int lane = lane_id();
+  uint32_t av[NW], bv[NW], f[NW];
+#pragma unroll
+  for (int w = 0; w < NW; w++) av[w] = a[w];
+#pragma unroll
+  for (int w = 0; w < NW; w++) bv[w] = b[w];
+#pragma unroll
+  for (int v = 0; v < NW; v++) f[v] = __funnelshift_r(bv[v], v + 1 < NW ? bv[v + 1] : 0u, lane);
+  // positions of the last two shifted words inside the sequence
+  auto low = [](int m) { return m >= 32 ? 0xffffffffu : (m <= 0 ? 0u : (1u << m) - 1u); };
+  const int r = n - 32 * (NW - 1) - lane;
+  corr_lags<NW, 0>(av, f, low(r), low(r + 32), n - lane, emit);
+}
+
+// E of the sequence in sb (as in corr_words, 32 (NW - 1) < L <= 32 NW), on every lane; WITH_C: C_out receives
+// C_k at C_out[k - 1], k = 1 .. L-1.
 template <int NW, bool WITH_C = false>
 __device__ __forceinline__ int energy_words(const uint32_t* sb, int L, int32_t* C_out = nullptr) {
-  const int lane = lane_id();
-  uint32_t b[NW], f[NW];
-#pragma unroll
-  for (int w = 0; w < NW; w++) b[w] = sb[w];
-#pragma unroll
-  for (int v = 0; v < NW; v++) f[v] = __funnelshift_r(b[v], v + 1 < NW ? b[v + 1] : 0u, lane);
-  // positions of the last two shifted words inside the sequence
-  auto low = [](int n) { return n >= 32 ? 0xffffffffu : (n <= 0 ? 0u : (1u << n) - 1u); };
-  const int r = L - 32 * (NW - 1) - lane;
   int e = 0;
-  energy_lags<NW, 0, WITH_C>(b, f, low(r), low(r + 32), L - lane, e, C_out);
+  corr_words<NW>(sb, sb, L, [&](int k, int c) {
+    e += c * c;
+    if (WITH_C && k >= 1 && k < L) C_out[k - 1] = c;
+  });
   return warp_sum_i32(e) - L * L;  // without k = 0
 }
 
