@@ -7,40 +7,43 @@
 // (one bin per energy, clamped at both ends of a 2^17-bin window, and a coarse level whose bins each
 // cover 256 fine bins).  The B smallest keys, or the cap smallest, are then found without ordering the pool: the
 // histogram's prefix sums give the bin where the count is reached, every entry below it is taken, and
-// only the entries of that one boundary bin are ranked (a radix select on their full (E, fp) key, so a
-// clamped bin holding several energies is still exact).  A round
-//   pop      -- the b = min(B, open, budget left) smallest keys leave the pool (one pass over it), are
-//               ranked among themselves (a 2-D grid counts, for each, the smaller keys) and become the
-//               round's pivots in key order;
-//   expand   -- one warp per pivot: its correlation table, the all-position dp4a scan and a visited-set
-//               lookup per neighbour, written to a dense [pivot][column] survivor array;
-//   dedup    -- survivors with equal (E', fp') (the same sequence) are kept once, through a hash table;
-//               the one kept is the smallest (pivot, column), as in the sequential definition;
+// only the entries of that one boundary bin are ranked (by their fingerprints' first bits, counted as they are
+// gathered, then among the few that share the boundary's; a clamped bin holding several energies takes a radix
+// select on the full key).  A round
+//   pop      -- the b = min(B, open, budget left) smallest keys leave the pool (one pass over it): the round's
+//               pivots, in any order (a sequence reached from two pivots is the same sequence);
+//   expand   -- one warp per pivot: its correlations, every neighbour's sum on the tensor cores (scan_mma.cuh),
+//               into a dense [pivot][column] array; one warp more per rotation of a pivot (MAKE_ROTATIONS,
+//               T_r > 0: columns L .. L + 2 T_r - 1);
+//   dedup    -- a visited-set lookup per child; survivors with equal (E', fp') (the same sequence) are kept once,
+//               through a hash table;
 //   best     -- strict improvement test on the smallest survivor key;
 //   cut      -- the cap smallest of (pool u survivors): entries of the pool above the cut are evicted,
 //               survivors below it are admitted into free slots and into the visited set H;
 // keeps every result identical to the sequential definition whatever order threads run in.  The seeds
-// enter through the same survivor path.  With T_r > 0 every pivot also offers its 2 T_r rotations
-// (MAKE_ROTATIONS) as survivor columns L .. L + 2 T_r - 1, after its L flips.
+// enter through the same survivor path.
+//
+// Where counts meet one address (free slots, admissions) a block adds up first, one atomic per 1,024 entries;
+// the pool's histogram after a round follows from the cut (bins below it gain the survivors', the boundary bin
+// keeps what was taken, bins above are empty), so no entry updates it.
 #include <algorithm>
 #include <new>
 
-#include "labs_core.cuh"
 #include "labs_internal.h"
+#include "scan_mma.cuh"
 
 namespace labsg {
 namespace {
 
 constexpr uint64_t kEmptyKey = ~0ull;  // free slot of the visited set (fp == ~0 is tracked by a flag)
 constexpr int kPqWarps = 4;
-constexpr int kPqM = 8;
 constexpr int kMaxProbe = 1 << 20;
 constexpr int kNB = 1 << 17;        // fine energy bins: bin = clamp(E - E_base, 0, kNB - 1)
 constexpr int kCoarse = 256;        // fine bins per coarse bin
 constexpr int kNC = kNB / kCoarse;  // coarse bins
-constexpr int kColBits = 11;        // survivor column inside a representative: width <= 576 + 128 < 2^11
-constexpr int kSortMax = 8192;      // pops per round (B <= 8192), put in key order by one block
-constexpr int kSelThreads = 1024;   // threads of the single-block select, boundary and sort kernels
+constexpr int kMaxB = 8192;         // pops per round
+constexpr int kSelThreads = 1024;   // threads of the single-block kernels
+constexpr int kFpBins = 1024;       // first bits of the boundary candidates' fingerprints
 
 // Device-side state of one refinement (every round reads and writes it; the host only polls `stop`).
 struct PqState {
@@ -48,24 +51,22 @@ struct PqState {
   long long expansions, rounds, survivors, admitted, evicted, h_size, improvements, u;
   unsigned long long best_fp;
   long long free_top;   // free pool slots (the stack holds their ids)
+  long long pop_base;   // stack slots the round's pops are freed to
   long long pop_cnt;    // entries gathered for popping this round
   long long cand_cnt;   // boundary-bin candidates gathered
   long long nU;         // unique survivors of the round
   long long n_dense;    // dense survivor entries of the round: b x width, or the seeds
-  long long sel_lt;     // entries below the boundary bin
   long long sel_need;   // entries taken from the boundary bin; 0: none; -1: no cut (everything kept)
   long long ev_round;   // evicted this round
   long long adm_round;  // admitted this round
   int b, stop, best_E, error, h_has_empty, E_base;
   int sel_bin;     // boundary fine bin
   int minE_round;  // smallest survivor energy of the round
-  int sel_E, pad0;
+  int sel_E, pmax_bin;        // pmax_bin: highest occupied bin of the pool after the pops (-1: empty pool)
   unsigned long long sel_fp;  // boundary key: a boundary-bin entry is taken iff (E, fp) <= (sel_E, sel_fp)
   unsigned long long minfp_round;
-  unsigned best_rep_round, pad1;
-  int pmax_bin;        // highest occupied bin of the pool after the pops (-1: empty pool)
-  int hist_mode;       // survivor histogram: 0 none (everything fits), 1 bins <= pmax_bin only, 2 all
   long long nU_low;    // survivors in bins <= pmax_bin
+  int grp_n, done;     // fingerprints collected by the boundary select, blocks finished with their part
 };
 
 struct PqBufs {
@@ -83,23 +84,21 @@ struct PqBufs {
   unsigned* hP2;
   unsigned* hU;       // histogram of the round's unique survivors
   unsigned* hU2;
-  int32_t* popId;     // pool ids gathered for popping [B], with their keys
+  unsigned* hF;       // [kFpBins] first fingerprint bits of the boundary candidates
+  int32_t* popId;     // pool ids of the pops [B], with their keys
   int32_t* popE;
   uint64_t* popF;
-  int32_t* pivE;      // pivots in key order [B]
-  uint64_t* pivFp;
-  uint64_t* pivSeq;   // [B][W]
+  uint64_t* pivSeq;   // [B][W]: their sequences
   int32_t* candId;    // boundary candidates: pool id >= 0, or -(u + 1) for survivor u
   int32_t* cE;        // their keys, gathered contiguously
   uint64_t* cF;
-  int32_t* popRank;   // rank of each popped entry among the pops (its pivot index)
-  int32_t* dE;        // dense survivors [pivot][column]: energy, or INT32_MAX (visited)
+  uint64_t* grp;      // fingerprints of the boundary's group
+  int32_t* dE;        // dense survivors [pivot][column]: energy, or INT32_MAX (visited, or an equal one is kept)
   uint64_t* dFp;
   uint64_t* hkey;     // dedup hash table: mixed (E, fp) key, 0 = empty
-  int32_t* hval;      // the unique survivor of a slot
-  unsigned* uRep;     // per dense entry: ~0 unless it is the unique survivor of its key, whose
-                      // representative (pivot << kColBits | column) is the smallest of the equal keys
   uint64_t* H;        // visited set (open addressing)
+  uint32_t* filter;   // its filter, 2^f_log2 bits
+  int f_log2;
   uint64_t* ztab;
   PqState* st;
   uint64_t* best_seq;
@@ -120,12 +119,21 @@ __device__ __forceinline__ void pq_child(const uint64_t* src, const PqBufs& b, i
   if (col < b.L) {
     for (int t = 0; t < b.W; t++) out[t] = src[t] ^ (t == (col >> 6) ? 1ull << (col & 63) : 0ull);
   } else {
-    const int r = rot_shift(b.L, b.Tr, col - b.L);
-    for (int t = 0; t < b.W; t++) out[t] = 0;
-    for (int i = 0; i < b.L; i++) {
-      int j = i + r;
-      if (j >= b.L) j -= b.L;
-      if ((src[j >> 6] >> (j & 63)) & 1ull) out[i >> 6] |= 1ull << (i & 63);
+    const int r = rot_shift(b.L, b.Tr, col - b.L);  // element i is element i + r (mod L)
+    for (int t = 0; t < b.W; t++) {
+      const int o = 64 * t + r, ow = o - b.L;
+      uint64_t x = 0;
+      auto window = [&](int p) {  // 64 bits from bit p on; bits at and above L are zero
+        const int w = p >> 6, sh = p & 63;
+        return (src[w] >> sh) | (sh && w + 1 < b.W ? src[w + 1] << (64 - sh) : 0ull);
+      };
+      if (o < b.L) x = window(o);
+      if (ow >= 0)  // elements past the end come from the start
+        x = window(ow);
+      else if (ow > -64)
+        x |= src[0] << -ow;
+      const int left = b.L - 64 * t;
+      out[t] = left < 64 ? x & ((1ull << left) - 1) : x;
     }
   }
   for (int t = 0; t < b.W; t++) dst[t] = out[t];
@@ -146,18 +154,25 @@ __device__ __forceinline__ bool h_contains_after(const PqBufs& b, uint64_t fp, u
   return true;
 }
 
-__device__ __forceinline__ bool h_contains(const PqBufs& b, uint64_t fp) {
-  if (fp == kEmptyKey) return b.st->h_has_empty != 0;
-  const uint64_t s = h_slot(fp, b.H_log2);
-  const uint64_t v = b.H[s];
-  if (v == fp) return true;
-  if (v == kEmptyKey) return false;
-  return h_contains_after(b, fp, s);
+// One bit per home slot of H (or per 2^k of them, at most 2^kFilterMax bits, 32 MB): a clear bit means that
+// nothing hashed there was inserted, so most lookups of new states end in L2 instead of reading H from DRAM.
+// Past kFilterFull insertions most bits are set and lookups go to H at once.
+constexpr int kFilterMax = 28;
+constexpr long long kFilterFull = 1ll << (kFilterMax - 1);
+__device__ __forceinline__ bool use_filter(const PqBufs& b) { return b.st->h_size < kFilterFull; }
+__device__ __forceinline__ uint32_t filter_bit(const PqBufs& b, uint64_t fp) {
+  return (uint32_t)((fp * kGamma) >> (64 - b.f_log2));
+}
+__device__ __forceinline__ bool filter_hit(const PqBufs& b, uint64_t fp) {
+  const uint32_t i = filter_bit(b, fp);
+  return (b.filter[i >> 5] >> (i & 31)) & 1u;
 }
 
 // Inserts fp; returns 1 when it was not there yet (the caller counts insertions into h_size in bulk).
 __device__ __forceinline__ int h_insert(const PqBufs& b, uint64_t fp) {
   if (fp == kEmptyKey) return atomicExch(&b.st->h_has_empty, 1) == 0 ? 1 : 0;
+  const uint32_t fi = filter_bit(b, fp);
+  atomicOr(&b.filter[fi >> 5], 1u << (fi & 31));
   const uint64_t mask = (1ull << b.H_log2) - 1;
   uint64_t s = h_slot(fp, b.H_log2);
   for (int it = 0; it < kMaxProbe; it++) {
@@ -182,28 +197,6 @@ __device__ __forceinline__ int e_bin(int E, int E_base) {
   const int d = E - E_base;
   return d < 0 ? 0 : (d >= kNB ? kNB - 1 : d);
 }
-
-// Adds v to *ctr once per warp (every lane of the warp calls it with its own v).
-__device__ __forceinline__ void warp_add(long long* ctr, int v) {
-  const int s = __reduce_add_sync(kFull, v);
-  if (lane_id() == 0 && s) atomicAdd(reinterpret_cast<unsigned long long*>(ctr), (unsigned long long)(long long)s);
-}
-
-// Reserves one output index per lane with pred, one atomic per warp (every lane calls it); returns the
-// lane's index, or -1.
-__device__ __forceinline__ long long warp_append(long long* ctr, bool pred) {
-  const unsigned m = __ballot_sync(kFull, pred);
-  if (!m) return -1;
-  const int leader = __ffs(m) - 1;
-  long long base = 0;
-  if (lane_id() == leader)
-    base = (long long)atomicAdd(reinterpret_cast<unsigned long long*>(ctr), (unsigned long long)__popc(m));
-  base = __shfl_sync(kFull, base, leader);
-  return pred ? base + __popc(m & ((1u << lane_id()) - 1u)) : -1;
-}
-
-// Adds the insertions of a warp to h_size (every lane calls it).
-__device__ __forceinline__ void h_count(const PqBufs& b, int inserted) { warp_add(&b.st->h_size, inserted); }
 
 // Block-wide sum added to *ctr with one atomic per block (every thread of the block calls it).
 __device__ __forceinline__ void block_add(long long* ctr, long long v) {
@@ -233,18 +226,52 @@ __device__ __forceinline__ void block_min(int* dst, int v) {
   __syncthreads();
 }
 
-// Adds delta to the fine and coarse histogram bins of every lane with bin >= 0, one atomic per distinct
-// bin of the warp (every lane calls it): the energies of a round crowd into few bins, and same-address
-// atomics from every thread would serialise there.
-__device__ __forceinline__ void hist_add(unsigned* fine, unsigned* coarse, int bin, int delta) {
-  if (!__any_sync(kFull, bin >= 0)) return;  // most warps of a pass change nothing
-  const unsigned lt = (1u << lane_id()) - 1u;
-  const unsigned pf = __match_any_sync(kFull, bin);
-  if (bin >= 0 && (pf & lt) == 0) atomicAdd(&fine[bin], (unsigned)(delta * __popc(pf)));
-  const int cb = bin >= 0 ? bin / kCoarse : -1;
-  const unsigned pc = __match_any_sync(kFull, cb);
-  if (cb >= 0 && (pc & lt) == 0) atomicAdd(&coarse[cb], (unsigned)(delta * __popc(pc)));
+// Adds sign times the block's total of n (per thread) to *ctr with one atomic (every thread calls it; two
+// barriers) and returns the counter's value before it; *before: the counts of the threads in front.
+__device__ __forceinline__ long long block_reserve(long long* ctr, int n, int sign, int* total, int* before) {
+  __shared__ int part[32];
+  __shared__ long long base;
+  int incl = n;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(kFull, incl, o);
+    if (lane_id() >= o) incl += v;
+  }
+  if (lane_id() == 31) part[threadIdx.x >> 5] = incl;
+  __syncthreads();
+  const int nw = (int)(blockDim.x >> 5);
+  int front = 0, all = 0;
+  for (int w = 0; w < nw; w++) {
+    const int v = part[w];
+    if (w < (int)(threadIdx.x >> 5)) front += v;
+    all += v;
+  }
+  if (threadIdx.x == 0)
+    base = all ? (long long)atomicAdd(reinterpret_cast<unsigned long long*>(ctr), (unsigned long long)(long long)(sign * all)) : 0;
+  __syncthreads();
+  *total = all;
+  *before = front + incl - n;
+  return base;
 }
+
+// Survivor histogram of a block: the fine bins are counted one by one in global memory (a round's energies
+// spread over some hundred), the coarse ones, few and hot, in shared memory and added once.
+struct CoarseCounts {
+  unsigned* n;  // [kNC] shared
+  __device__ __forceinline__ explicit CoarseCounts(unsigned* shared) : n(shared) {
+    for (int i = threadIdx.x; i < kNC; i += blockDim.x) n[i] = 0u;
+    __syncthreads();
+  }
+  __device__ __forceinline__ void add(unsigned* fine, int bin) {
+    atomicAdd(&fine[bin], 1u);
+    atomicAdd(&n[bin / kCoarse], 1u);
+  }
+  __device__ __forceinline__ void flush(unsigned* coarse) {
+    __syncthreads();
+    for (int i = threadIdx.x; i < kNC; i += blockDim.x)
+      if (n[i]) atomicAdd(&coarse[i], n[i]);
+  }
+};
 
 // Mixed key of (E, fp) for the dedup table; 0 marks an empty slot, so a mixed key of 0 becomes 1.
 __device__ __forceinline__ uint64_t dedup_key(int E, uint64_t fp) {
@@ -273,8 +300,8 @@ __global__ void pq_init_kernel(PqBufs b) {
     z.best_fp = ~0ull;
     z.minE_round = INT32_MAX;
     z.minfp_round = ~0ull;
-    z.best_rep_round = ~0u;
     z.pmax_bin = -1;
+    z.sel_need = -1;
     z.n_dense = b.n_seeds;
     *b.st = z;
   }
@@ -318,575 +345,622 @@ __global__ void __launch_bounds__(32 * kPqWarps) pq_seed_kernel(PqBufs b, int n_
 }
 
 // ---------------------------------------------------------------------------------------------
-// Round kernels.  SEED = true runs the survivor path on the seeds (dense = the seeds, one column each,
-// representatives are seed indices; nothing is counted as a survivor or an admission).
+// Round kernels.  SEED = true runs the survivor path on the seeds (dense = the seeds, one column each; nothing
+// is counted as a survivor or an admission).
 // ---------------------------------------------------------------------------------------------
-__global__ void pq_round_begin_kernel(PqBufs b) {
-  PqState* st = b.st;
-  if (!st->stop) {
-    if (st->error)
-      st->stop = 4;
-    else if (st->expansions >= b.max_exp)
-      st->stop = 1;
-    else if (st->nP == 0)
-      st->stop = 2;
-    else if (b.T_u > 0 && st->u >= b.T_u)
-      st->stop = 3;
-  }
-  st->pop_cnt = 0;
-  st->cand_cnt = 0;
-  st->nU = 0;
-  st->n_dense = 0;
-  st->ev_round = 0;
-  st->adm_round = 0;
-  st->minE_round = INT32_MAX;
-  st->minfp_round = ~0ull;
-  st->best_rep_round = ~0u;
-  st->nU_low = 0;
-  st->hist_mode = 0;
-  if (st->stop) {
-    st->b = 0;
-    return;
-  }
-  long long bb = min((long long)b.B, st->nP);
-  bb = min(bb, b.max_exp - st->expansions);
-  st->b = (int)bb;
-  st->n_dense = bb * b.width;
-}
 
-// One block: the fine bin where the count of entries reaches the target (POP: b over the pool; else
-// cap over the pool's rest and the survivors, or no cut when everything fits).  sel_lt = entries below
-// that bin, sel_need = entries to take from it.
-template <bool POP>
-__global__ void __launch_bounds__(kSelThreads) pq_select_kernel(PqBufs b) {
-  PqState* st = b.st;
-  __shared__ unsigned long long part[kSelThreads];
-  __shared__ long long s_target;
+// One block: the fine bin where the count of entries (hP, plus hU when CUT) reaches target > 0, into sel_bin,
+// and the entries to take from it, into sel_need.
+template <bool CUT>
+__device__ __forceinline__ void select_bin(const PqBufs& b, long long target) {
+  __shared__ unsigned long long wsum[kSelThreads / 32];
   __shared__ int s_cb;
   __shared__ unsigned long long s_before;
-  const int t = threadIdx.x;
-  if (t == 0) {
-    long long target;
-    if (POP) {
-      target = st->b;
-    } else {
-      st->cand_cnt = 0;  // the pop's candidates are done with
-      target = st->hist_mode ? b.cap : -1;
+  PqState* st = b.st;
+  const int t = threadIdx.x, lane = lane_id();
+  auto scan = [&](unsigned long long own) {  // inclusive sum over the threads in front
+    unsigned long long c = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long v = __shfl_up_sync(kFull, c, o);
+      if (lane >= o) c += v;
     }
-    s_target = target;
-    if (target <= 0) {
-      st->sel_need = target < 0 ? -1 : 0;
-      st->sel_bin = kNB;
-      st->sel_lt = 0;
-    }
-  }
-  __syncthreads();
-  const long long target = s_target;
-  if (target <= 0) return;
-  // coarse level
-  unsigned long long c = 0;
-  if (t < kNC) c = (unsigned long long)b.hP2[t] + (POP ? 0u : b.hU2[t]);
-  part[t] = c;
-  __syncthreads();
-  for (int off = 1; off < kSelThreads; off <<= 1) {  // inclusive scan
-    const unsigned long long v = t >= off ? part[t - off] : 0ull;
+    __syncthreads();  // wsum's last readers are done
+    if (lane == 31) wsum[t >> 5] = c;
     __syncthreads();
-    part[t] += v;
-    __syncthreads();
+    for (int w = 0; w < t >> 5; w++) c += wsum[w];
+    return c;
+  };
+  const unsigned long long tg = (unsigned long long)target;
+  unsigned long long own = 0;
+  if (t == 0) {  // a consistent histogram has a crossing bin
+    s_cb = 0;
+    s_before = 0;
   }
-  if (t < kNC) {
-    const unsigned long long before = t ? part[t - 1] : 0ull;
-    if (before < (unsigned long long)target && part[t] >= (unsigned long long)target) {
-      s_cb = t;
-      s_before = before;
-    }
+  if (t < kNC) own = (unsigned long long)b.hP2[t] + (CUT ? __ldcg(&b.hU2[t]) : 0u);
+  unsigned long long c = scan(own);
+  if (own && c >= tg && c - own < tg) {
+    s_cb = t;
+    s_before = c - own;
   }
   __syncthreads();
   const int cb = s_cb;
-  const unsigned long long cbefore = s_before;
-  // fine level: the coarse bin's 256 bins
-  unsigned long long f = 0;
-  if (t < kCoarse) f = (unsigned long long)b.hP[cb * kCoarse + t] + (POP ? 0u : b.hU[cb * kCoarse + t]);
+  const unsigned long long before = s_before;
+  own = 0;
+  if (t < kCoarse) own = (unsigned long long)b.hP[cb * kCoarse + t] + (CUT ? __ldcg(&b.hU[cb * kCoarse + t]) : 0u);
+  c = before + scan(own);
+  if (own && c >= tg && c - own < tg) {
+    st->sel_bin = cb * kCoarse + t;
+    st->sel_need = target - (long long)(c - own);
+  }
   __syncthreads();
-  part[t] = f;
+}
+
+// The block's list of coarse bins with entries in the pool (or, CUT, among the survivors); returns their number.
+template <bool CUT>
+__device__ __forceinline__ int occupied_coarse(const PqBufs& b, int* list) {
+  __shared__ int n;
+  const int t = threadIdx.x;
+  if (t == 0) n = 0;
   __syncthreads();
-  for (int off = 1; off < kCoarse; off <<= 1) {
-    const unsigned long long v = (t < kCoarse && t >= off) ? part[t - off] : 0ull;
+  if (t < kNC && (b.hP2[t] || (CUT && b.hU2[t]))) list[atomicAdd(&n, 1)] = t;
+  __syncthreads();
+  return n;
+}
+
+// Whether the cut needs the survivors above the pool's occupied bins counted: not when the pool's rest and the
+// survivors inside those bins reach the cap.
+__device__ __forceinline__ bool counts_all(const PqState* st, long long cap) {
+  return st->pmax_bin < 0 || st->nP - st->b + st->nU_low < cap;
+}
+
+// One block: ends the round (or the seeds): the pool's histogram after the cut, the best (a strict improvement,
+// as in Algorithm 2; for the seeds, the smallest seed) and the counters; then begins the next one: its number
+// of pops and the bin that holds the last of them.
+template <bool SEED>
+__global__ void __launch_bounds__(kSelThreads) pq_finish_kernel(PqBufs b) {
+  PqState* st = b.st;
+  __shared__ int coarse[kNC];
+  const int t = threadIdx.x, lane = lane_id();
+  if (SEED || st->b > 0) {
+    // ---- histogram: a warp per coarse bin that holds anything
+    const int nc = occupied_coarse<true>(b, coarse);
+    const bool cut = st->sel_need >= 0;
+    const int sel = cut ? st->sel_bin : kNB;
+    const unsigned need = cut ? (unsigned)st->sel_need : 0u;
+    for (int x = t >> 5; x < nc; x += kSelThreads / 32) {
+      const int cb = coarse[x];
+      unsigned u[kCoarse / 32], h[kCoarse / 32], sum = 0;
+#pragma unroll
+      for (int i = 0; i < kCoarse / 32; i++) {
+        u[i] = b.hU[cb * kCoarse + 32 * i + lane];
+        h[i] = b.hP[cb * kCoarse + 32 * i + lane];
+      }
+#pragma unroll
+      for (int i = 0; i < kCoarse / 32; i++) {
+        const int bin = cb * kCoarse + 32 * i + lane;
+        const unsigned now = bin < sel ? h[i] + u[i] : (bin == sel ? need : 0u);
+        if (now != h[i]) b.hP[bin] = now;
+        if (u[i]) b.hU[bin] = 0u;
+        sum += now;
+      }
+      sum = (unsigned)warp_sum_i32((int)sum);
+      __syncwarp();
+      if (lane == 0) {
+        b.hP2[cb] = sum;
+        b.hU2[cb] = 0u;
+      }
+    }
     __syncthreads();
-    if (t < kCoarse) part[t] += v;
+    // ---- the best: an improvement's survivor is looked up in the dense array (few rounds improve)
+    __shared__ long long s_best;
+    const bool improved = st->nU > 0 && (SEED || st->minE_round < st->best_E);
+    if (t == 0) s_best = -1;
+    __syncthreads();
+    if (improved) {
+      const int E = st->minE_round;
+      const uint64_t fp = st->minfp_round;
+      const long long n = st->n_dense, nq = (n + 3) >> 2;
+#pragma unroll 4
+      for (long long qd = t; qd < nq; qd += kSelThreads) {
+        const int4 e4 = reinterpret_cast<const int4*>(b.dE)[qd];
+        const int Ev[4] = {e4.x, e4.y, e4.z, e4.w};
+#pragma unroll
+        for (int j = 0; j < 4; j++)
+          if (Ev[j] == E && 4 * qd + j < n && b.dFp[4 * qd + j] == fp) s_best = 4 * qd + j;
+      }
+      __syncthreads();
+    }
+    if (t == 0) {
+      if (!SEED) st->survivors += st->nU;
+      if (!SEED && st->pop_cnt != st->b) st->error = 1;
+      if (improved) {
+        const int E = st->minE_round;
+        const uint64_t fp = st->minfp_round;
+        const long long i = s_best;
+        if (i < 0) {
+          st->error = 1;  // cannot happen: the smallest key is a survivor's
+        } else {
+          st->best_E = E;
+          st->best_fp = fp;
+          if (SEED) {
+            for (int w = 0; w < b.W; w++) b.best_seq[w] = b.seeds[(size_t)i * b.W + w];
+          } else {
+            pq_child(b.pivSeq + (size_t)(i / b.width) * b.W, b, (int)(i % b.width), b.best_seq);
+            st->improvements++;
+          }
+        }
+        if (!SEED) st->u = 0;
+      } else if (!SEED) {
+        st->u += st->b;
+      }
+      if (SEED) {
+        st->nP = st->adm_round;
+      } else {
+        st->nP = st->nP - st->b - st->ev_round + st->adm_round;
+        st->admitted += st->adm_round;
+        st->evicted += st->ev_round;
+        st->expansions += st->b;
+        st->rounds++;
+      }
+      const long long slots = 1ll << b.H_log2;
+      if (st->h_size * 4 > slots * 3) st->error = 1;
+    }
     __syncthreads();
   }
-  if (t < kCoarse) {
-    const unsigned long long before = cbefore + (t ? part[t - 1] : 0ull);
-    if (before < (unsigned long long)target && cbefore + part[t] >= (unsigned long long)target) {
-      st->sel_bin = cb * kCoarse + t;
-      st->sel_lt = (long long)before;
-      st->sel_need = target - (long long)before;
+  // ---- the next round
+  if (t == 0) {
+    if (!st->stop) {
+      if (st->error)
+        st->stop = 4;
+      else if (st->expansions >= b.max_exp)
+        st->stop = 1;
+      else if (st->nP == 0)
+        st->stop = 2;
+      else if (b.T_u > 0 && st->u >= b.T_u)
+        st->stop = 3;
     }
+    st->pop_cnt = 0;
+    st->cand_cnt = 0;
+    st->nU = 0;
+    st->nU_low = 0;
+    st->ev_round = 0;
+    st->adm_round = 0;
+    st->minE_round = INT32_MAX;
+    st->minfp_round = ~0ull;
+    st->sel_need = 0;
+    st->sel_bin = kNB;
+    const long long bb = st->stop ? 0 : min(min((long long)b.B, st->nP), b.max_exp - st->expansions);
+    st->b = (int)bb;
+    st->n_dense = bb * b.width;
+  }
+  for (int i = t; i < kFpBins; i += kSelThreads) b.hF[i] = 0u;
+  __syncthreads();
+  if (st->b > 0) select_bin<false>(b, st->b);
+}
+
+// Entries of a pool or survivor pass per thread: 16 consecutive ones, four 16-byte loads of their energies in
+// flight (the arrays are 256-byte aligned, their sizes rounded to whole quads), so that a pass costs a block one
+// or two reservations.
+constexpr int kPer = 16;
+__device__ __forceinline__ void load_energies(const int32_t* src, long long first, long long n, int (&E)[kPer]) {
+#pragma unroll
+  for (int v = 0; v < kPer / 4; v++) {
+    int4 e4 = make_int4(INT32_MAX, INT32_MAX, INT32_MAX, INT32_MAX);
+    if (first + 4 * v < n) e4 = reinterpret_cast<const int4*>(src + first)[v];
+    E[4 * v] = e4.x;
+    E[4 * v + 1] = first + 4 * v + 1 < n ? e4.y : INT32_MAX;
+    E[4 * v + 2] = first + 4 * v + 2 < n ? e4.z : INT32_MAX;
+    E[4 * v + 3] = first + 4 * v + 3 < n ? e4.w : INT32_MAX;
   }
 }
 
-// Pass over the pool (U = false) or the survivors (U = true): POP gathers the pool entries below the
-// boundary bin (popped) and those in it (candidates); the cut gathers the boundary bin's entries.  Each
-// thread takes four consecutive entries with one 16-byte load of their energies (the pool and the dense
-// arrays are 256-byte aligned, their sizes rounded to whole quads by the workspace layout).
-template <bool POP, bool U>
-__global__ void __launch_bounds__(256) pq_gather_kernel(PqBufs b) {
+// Appends a block's boundary candidates: the entries of the thread's mask `is`.
+__device__ __forceinline__ void append_candidates(const PqBufs& b, unsigned is, const int (&E)[kPer], long long first,
+                                                  bool survivors) {
+  if (!__syncthreads_or((int)is)) return;
+  int total, before;
+  long long o = block_reserve(&b.st->cand_cnt, __popc(is), 1, &total, &before);
+  o += before;
+#pragma unroll
+  for (int e = 0; e < kPer; e++)
+    if (is >> e & 1) {
+      if (o >= b.cand_cap) {
+        b.st->error = 1;  // the histogram bounds the count: only an inconsistent state gets here
+      } else {
+        const uint64_t fp = survivors ? b.dFp[first + e] : b.pFp[first + e];
+        b.candId[o] = survivors ? -(int32_t)(first + e) - 1 : (int32_t)(first + e);
+        b.cE[o] = E[e];
+        b.cF[o] = fp;
+        atomicAdd(&b.hF[fp >> 54], 1u);
+      }
+      o++;
+    }
+}
+
+// Pass over the pool by the first pool_blocks blocks.  POP gathers the entries below the boundary bin (popped)
+// and those in it (candidates); the cut evicts the entries above it (slot freed) and gathers those in it, and the
+// blocks behind gather the boundary bin's survivors.
+template <bool POP>
+__global__ void __launch_bounds__(256) pq_pool_kernel(PqBufs b, unsigned pool_blocks) {
   PqState* st = b.st;
   if (POP ? st->b == 0 : st->sel_need <= 0) return;
   const int sel = st->sel_bin, Eb = st->E_base;
-  const long long n = U ? st->n_dense : b.cap;
-  const long long nq = (n + 3) >> 2;
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long base = (long long)blockIdx.x * blockDim.x; base < nq; base += stride) {
-    const long long qd = base + threadIdx.x;
-    int4 e4 = make_int4(INT32_MAX, INT32_MAX, INT32_MAX, INT32_MAX);
-    uint4 r4 = make_uint4(0u, 0u, 0u, 0u);
-    if (qd < nq) {
-      e4 = reinterpret_cast<const int4*>(U ? b.dE : b.pE)[qd];
-      if (U) r4 = reinterpret_cast<const uint4*>(b.uRep)[qd];
-    }
-    const int ev[4] = {e4.x, e4.y, e4.z, e4.w};
-    const unsigned rv[4] = {r4.x, r4.y, r4.z, r4.w};
+  if (!POP && blockIdx.x >= pool_blocks) {
+    const long long n = st->n_dense;
+    const long long stride = (long long)(gridDim.x - pool_blocks) * blockDim.x * kPer;
+    for (long long base = (long long)(blockIdx.x - pool_blocks) * blockDim.x * kPer; base < n; base += stride) {
+      const long long first = base + (long long)threadIdx.x * kPer;
+      int E[kPer];
+      load_energies(b.dE, first, n, E);
+      unsigned cand = 0;
 #pragma unroll
-    for (int e = 0; e < 4; e++) {
-      const long long i = 4 * qd + e;
-      int bin = kNB;
-      int E = INT32_MAX;
-      if (i < n) {
-        E = U ? (rv[e] != ~0u ? ev[e] : INT32_MAX) : ev[e];
-        if (E != INT32_MAX) bin = e_bin(E, Eb);
-      }
-      // the histogram bounds both counts (b entries below the boundary bin at most); a count beyond a
-      // buffer can only come from an inconsistent state, which is reported instead of written
-      if (POP) {
-        const long long o = warp_append(&st->pop_cnt, bin < sel);
-        if (o >= b.B) {
-          st->error = 1;
-        } else if (o >= 0) {
-          b.popId[o] = (int32_t)i;
-          b.popE[o] = E;
-          b.popF[o] = b.pFp[i];
-        }
-      }
-      const long long o2 = warp_append(&st->cand_cnt, bin == sel);
-      if (o2 >= b.cand_cap) {
-        st->error = 1;
-      } else if (o2 >= 0) {
-        b.candId[o2] = U ? -(int32_t)i - 1 : (int32_t)i;
-        b.cE[o2] = E;
-        b.cF[o2] = U ? b.dFp[i] : b.pFp[i];
-      }
+      for (int e = 0; e < kPer; e++)
+        if (E[e] != INT32_MAX && e_bin(E[e], Eb) == sel) cand |= 1u << e;
+      append_candidates(b, cand, E, first, true);
     }
+    return;
   }
+  const long long stride = (long long)pool_blocks * blockDim.x * kPer;
+  long long freed = 0;
+  for (long long base = (long long)blockIdx.x * blockDim.x * kPer; base < b.cap; base += stride) {
+    const long long first = base + (long long)threadIdx.x * kPer;
+    int E[kPer];
+    load_energies(b.pE, first, b.cap, E);
+    unsigned take = 0, cand = 0;
+#pragma unroll
+    for (int e = 0; e < kPer; e++)
+      if (E[e] != INT32_MAX) {
+        const int bin = e_bin(E[e], Eb);
+        if (POP ? bin < sel : bin > sel) take |= 1u << e;
+        if (bin == sel) cand |= 1u << e;
+      }
+    if (__syncthreads_or((int)take)) {
+      int total, before;
+      long long o = block_reserve(POP ? &st->pop_cnt : &st->free_top, __popc(take), 1, &total, &before);
+      o += before;
+#pragma unroll
+      for (int e = 0; e < kPer; e++)
+        if (take >> e & 1) {
+          const long long i = first + e;
+          if (o >= (POP ? (long long)b.B : b.cap)) {
+            st->error = 1;  // the histogram bounds the count
+          } else if (POP) {
+            b.popId[o] = (int32_t)i;
+            b.popE[o] = E[e];
+            b.popF[o] = b.pFp[i];
+          } else {
+            b.freeIds[o] = (int32_t)i;
+            b.pE[i] = INT32_MAX;
+            freed++;
+          }
+          o++;
+        }
+    }
+    append_candidates(b, cand, E, first, false);
+  }
+  if (!POP) block_add(&st->ev_round, freed);
 }
 
-// One block: the sel_need smallest (E, fp) keys among the boundary candidates, by a most-significant-
-// digit-first radix select over the 96-bit key (four energy bytes, then eight fingerprint bytes; the
-// energy bytes are skipped when the boundary bin holds one energy, i.e. it is not clamped); keys are
-// distinct, so exactly sel_need candidates are <= the selected key.  The candidates are streamed from the
-// gather arrays until those that match the digits fixed so far fit in shared memory; they are staged
-// there and the remaining digits rank only them.  POP appends the selected candidates to the pops.
-constexpr int kCandSmem = 8192;  // candidates staged in shared memory (12 B each)
+// The sel_need smallest (E, fp) keys among the boundary candidates, whose keys are distinct.  A bin that is not
+// clamped holds one energy: the counts of the fingerprints' first ten bits give the group that holds the
+// boundary; all blocks collect that group's fingerprints (a thousandth of the candidates), and the last one to
+// finish ranks them against each other.  Otherwise (a clamped bin, or a group beyond kGroup) it does a radix
+// select over the full 96-bit key.
+constexpr int kGroup = 4096;
 template <bool POP>
 __global__ void __launch_bounds__(kSelThreads) pq_boundary_kernel(PqBufs b) {
   PqState* st = b.st;
   if (POP ? st->b == 0 : st->sel_need <= 0) return;
+  __shared__ uint64_t grp[kGroup];
+  __shared__ int s_bin, s_n, s_E, s_last;
+  __shared__ long long s_need;
+  __shared__ unsigned long long s_fp;
+  __shared__ unsigned s_hist[256];
+  __shared__ unsigned wsum[kSelThreads / 32];
+  const int t = threadIdx.x, lane = lane_id();
   const long long n = min(st->cand_cnt, b.cand_cap);
-  extern __shared__ unsigned long long sm_cand[];
-  uint64_t* sF = reinterpret_cast<uint64_t*>(sm_cand);
-  int* sE = reinterpret_cast<int*>(sm_cand + kCandSmem);
-  __shared__ unsigned hist[256];
-  __shared__ unsigned wsum[8];                     // bin-count totals of the eight warps' 32 bins
-  __shared__ unsigned long long s_pre_e, s_pre_f;  // the digits fixed so far
-  __shared__ long long s_k, s_match;               // rank still to find; candidates matching the digits
-  __shared__ int s_ns;                             // candidates staged
-  const int t = threadIdx.x;
-  const bool one_energy = st->sel_bin > 0 && st->sel_bin < kNB - 1;
+  const long long need = st->sel_need;
+  const int sel = st->sel_bin;
+  const bool one_energy = sel > 0 && sel < kNB - 1;
   if (t == 0) {
-    s_pre_e = one_energy ? (unsigned long long)(uint32_t)(st->E_base + st->sel_bin) : 0ull;
-    s_pre_f = 0;
-    s_k = st->sel_need;
-    s_match = n;
-    s_ns = 0;
+    s_n = 0;
+    s_bin = 0;
+    s_need = need;
+    s_E = st->E_base + sel;
+    s_fp = ~0ull;
+  }
+  // group of the boundary: inclusive sums of the counts
+  const unsigned own = b.hF[t];
+  unsigned c = own;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned v = __shfl_up_sync(kFull, c, o);
+    if (lane >= o) c += v;
+  }
+  if (lane == 31) wsum[t >> 5] = c;
+  __syncthreads();
+  for (int w = 0; w < t >> 5; w++) c += wsum[w];
+  if (own && (long long)c >= need && (long long)(c - own) < need) {
+    s_bin = t;
+    s_need = need - (long long)(c - own);  // rank inside the group, from 1
   }
   __syncthreads();
-  bool staged = false;
-  const int d0 = one_energy ? 4 : 0;
-  for (int d = d0; d < 12; d++) {
-    // the shared selection state is read here, behind the previous iteration's last barrier: the thread
-    // of the crossing bin rewrites it below while the others still test their bins
-    const unsigned long long pe = s_pre_e, pf = s_pre_f;
-    const long long k = s_k;
-    // does key (ue, fp) match the digits fixed before digit d?
-    auto match = [&](uint64_t ue, uint64_t fp) {
-      if (d < 4) return d == 0 || (ue >> (32 - 8 * d)) == (pe >> (32 - 8 * d));
-      return ue == pe && (d == 4 || (fp >> (64 - 8 * (d - 4))) == (pf >> (64 - 8 * (d - 4))));
-    };
-    if (!staged && s_match <= kCandSmem) {  // stage the matching candidates
-      for (long long i = t; i < n; i += kSelThreads) {
-        const uint64_t ue = (uint32_t)b.cE[i], fp = b.cF[i];
-        if (d == d0 || match(ue, fp)) {
-          const int w = atomicAdd(&s_ns, 1);
-          if (w < kCandSmem) {
-            sF[w] = fp;
-            sE[w] = (int)(uint32_t)ue;
-          }
-        }
-      }
-      staged = true;
-      __syncthreads();
-    }
-    if (t < 256) hist[t] = 0;
-    __syncthreads();
-    const long long nsel = staged ? min((long long)s_ns, (long long)kCandSmem) : n;
-    for (long long i = t; i < nsel; i += kSelThreads) {
-      const uint64_t ue = (uint32_t)(staged ? sE[i] : b.cE[i]);
-      const uint64_t fp = staged ? sF[i] : b.cF[i];
-      if (d == d0 || match(ue, fp)) {
-        const unsigned digit = d < 4 ? (unsigned)(ue >> (24 - 8 * d)) & 255u : (unsigned)(fp >> (56 - 8 * (d - 4))) & 255u;
-        atomicAdd(&hist[digit], 1u);
-      }
-    }
-    __syncthreads();
-    // the digit where the count reaches k: an inclusive scan of the 256 bins (a shuffle scan per warp of
-    // 32 bins, then the eight warp totals), then the one bin that crosses k
-    const unsigned own = t < 256 ? hist[t] : 0u;
-    unsigned c = own;
-    if (t < 256) {
+  const int gb = s_bin;
+  const bool grouped = one_energy && b.hF[gb] <= (unsigned)kGroup;
+  const long long stride = (long long)gridDim.x * kSelThreads;
+  if (grouped)
+    for (long long i0 = (long long)blockIdx.x * kSelThreads; i0 < n; i0 += 4 * stride) {
+      uint64_t f[4];
 #pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const unsigned v = __shfl_up_sync(kFull, c, off);
-        if (lane_id() >= off) c += v;
+      for (int e = 0; e < 4; e++) {
+        const long long i = i0 + e * stride + t;
+        f[e] = i < n ? b.cF[i] : 0ull;
       }
-      if (lane_id() == 31) wsum[t >> 5] = c;
-    }
-    __syncthreads();
-    if (t < 256) {
-      unsigned add = 0;
-      for (int w = 0; w < (t >> 5); w++) add += wsum[w];
-      c += add;
-      const long long before = (long long)(c - own);
-      if (before < k && (long long)c >= k) {
-        s_k = k - before;
-        s_match = own;
-        if (d < 4)
-          s_pre_e = pe | ((unsigned long long)t << (24 - 8 * d));
-        else
-          s_pre_f = pf | ((unsigned long long)t << (56 - 8 * (d - 4)));
-      }
-    }
-    __syncthreads();
-    // one candidate left with the digits fixed so far: it is the selected key, whatever its remaining
-    // digits (candidate keys are distinct)
-    if (s_match == 1 && d < 11) {
-      const unsigned long long pe2 = s_pre_e, pf2 = s_pre_f;
-      const int dn = d + 1;  // digits fixed now
-      const long long m2 = staged ? min((long long)s_ns, (long long)kCandSmem) : n;
-      for (long long i = t; i < m2; i += kSelThreads) {
-        const uint64_t ue = (uint32_t)(staged ? sE[i] : b.cE[i]);
-        const uint64_t fp = staged ? sF[i] : b.cF[i];
-        const bool hit = dn <= 4 ? (ue >> (32 - 8 * dn)) == (pe2 >> (32 - 8 * dn))
-                                 : ue == pe2 && (fp >> (64 - 8 * (dn - 4))) == (pf2 >> (64 - 8 * (dn - 4)));
-        if (hit) {
-          s_pre_e = ue;
-          s_pre_f = fp;
+#pragma unroll
+      for (int e = 0; e < 4; e++)
+        if (i0 + e * stride + t < n && (int)(f[e] >> 54) == gb) {
+          const int w = atomicAdd(&st->grp_n, 1);
+          if (w < kGroup) b.grp[w] = f[e];
         }
+    }
+  __threadfence();
+  __syncthreads();
+  if (t == 0) s_last = atomicAdd(&st->done, 1) == (int)gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  if (grouped) {
+    const int m = min(*reinterpret_cast<volatile int*>(&st->grp_n), kGroup);
+    for (int i = t; i < m; i += kSelThreads) grp[i] = *reinterpret_cast<volatile uint64_t*>(&b.grp[i]);
+    __syncthreads();
+    for (int i = t; i < m; i += kSelThreads) {
+      const uint64_t f = grp[i];
+      int r = 1;
+      for (int j = 0; j < m; j++) r += grp[j] < f ? 1 : 0;
+      if (r == (int)s_need) s_fp = f;
+    }
+    __syncthreads();
+  } else {
+    // most-significant-digit-first over the 96-bit key: four energy bytes, then eight fingerprint bytes
+    uint64_t preE = 0, preF = 0;
+    long long k = need;
+    for (int d = 0; d < 12; d++) {
+      if (t < 256) s_hist[t] = 0u;
+      __syncthreads();
+      for (long long i = t; i < n; i += kSelThreads) {
+        const uint64_t ue = (uint32_t)b.cE[i], f = b.cF[i];
+        const bool match = d < 4 ? (d == 0 || (ue >> (32 - 8 * d)) == (preE >> (32 - 8 * d)))
+                                 : ue == preE && (d == 4 || (f >> (96 - 8 * d)) == (preF >> (96 - 8 * d)));
+        if (match) atomicAdd(&s_hist[d < 4 ? (ue >> (24 - 8 * d)) & 255 : (f >> (88 - 8 * d)) & 255], 1u);
       }
       __syncthreads();
-      break;
-    }
-  }
-  const int selE = (int)(uint32_t)s_pre_e;
-  const uint64_t selF = s_pre_f;
-  if (t == 0) {
-    st->sel_E = selE;
-    st->sel_fp = selF;
-    if (s_ns > kCandSmem) st->error = 1;  // cannot happen: at most s_match <= kCandSmem are staged
-  }
-  if (POP) {
-    for (long long i = t; i < n; i += kSelThreads) {
-      if (key_le(b.cE[i], b.cF[i], selE, selF)) {
-        const long long o = (long long)atomicAdd(reinterpret_cast<unsigned long long*>(&st->pop_cnt), 1ull);
-        if (o < b.B) {
-          b.popId[o] = b.candId[i];
-          b.popE[o] = b.cE[i];
-          b.popF[o] = b.cF[i];
-        } else {
-          st->error = 1;
-        }
+      if (t == 0) {
+        long long before = 0;
+        int digit = 0;
+        while (digit < 255 && before + (long long)s_hist[digit] < k) before += s_hist[digit++];
+        s_bin = digit;
+        s_need = k - before;
       }
+      __syncthreads();
+      k = s_need;
+      if (d < 4)
+        preE |= (uint64_t)s_bin << (24 - 8 * d);
+      else
+        preF |= (uint64_t)s_bin << (88 - 8 * d);
+      __syncthreads();
     }
+    if (t == 0) {
+      s_E = (int)(uint32_t)preE;
+      s_fp = preF;
+    }
+    __syncthreads();
+  }
+  if (t == 0) {
+    st->sel_E = s_E;
+    st->sel_fp = s_fp;
+    st->grp_n = 0;  // for the next select
+    st->done = 0;
   }
 }
 
-// Grid (x: 256 popped entries per block, y: kRankChunks slices of the others): the popped entries in key
-// order.  Keys are distinct, so the number of popped keys smaller than a key is its rank; every block
-// adds its slice's count to the entry's rank.
-constexpr int kRankChunks = 16;
-__global__ void __launch_bounds__(256) pq_pop_rank_kernel(PqBufs b) {
+// The boundary candidates themselves: POP adds those up to the boundary to the pops; the cut evicts the pool's
+// beyond it.  Block 0 of POP also takes the pops out of the histogram (all below the boundary bin, sel_need of
+// it) and finds the highest occupied bin.
+template <bool POP>
+__global__ void __launch_bounds__(kSelThreads) pq_boundary_apply_kernel(PqBufs b) {
   PqState* st = b.st;
-  const int nb = st->b;
-  if (nb == 0) return;
-  if (st->pop_cnt != nb || st->error) {  // an inconsistent pop: stop the search (capacity status)
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
-      st->error = 1;
-      st->b = 0;
-      st->n_dense = 0;
+  if (POP ? st->b == 0 : st->sel_need <= 0) return;
+  const int t = threadIdx.x, lane = lane_id();
+  const long long n = min(st->cand_cnt, b.cand_cap);
+  const int selE = st->sel_E;
+  const uint64_t selF = st->sel_fp;
+  long long freed = 0;
+  for (long long i0 = (long long)blockIdx.x * kSelThreads; i0 < n; i0 += (long long)gridDim.x * kSelThreads) {
+    const long long i = i0 + t;
+    bool on = false;
+    int id = 0, E = 0;
+    uint64_t fp = 0;
+    if (i < n) {
+      id = b.candId[i];
+      E = b.cE[i];
+      fp = b.cF[i];
+      const bool in = key_le(E, fp, selE, selF);
+      on = POP ? in : (!in && id >= 0);
     }
+    if (!__syncthreads_or(on)) continue;
+    int total, before;
+    long long o = block_reserve(POP ? &st->pop_cnt : &st->free_top, on ? 1 : 0, 1, &total, &before);
+    o += before;
+    if (on) {
+      if (o >= (POP ? (long long)b.B : b.cap)) {
+        st->error = 1;
+      } else if (POP) {
+        b.popId[o] = id;
+        b.popE[o] = E;
+        b.popF[o] = fp;
+      } else {
+        b.freeIds[o] = id;
+        b.pE[id] = INT32_MAX;
+        freed++;
+      }
+    }
+  }
+  if (!POP) {
+    block_add(&st->ev_round, freed);
     return;
   }
-  __shared__ uint64_t sF[kSortMax / kRankChunks];
-  __shared__ int sE[kSortMax / kRankChunks];
-  const int per = (nb + kRankChunks - 1) / kRankChunks;
-  const int j0 = blockIdx.y * per, j1 = min(nb, j0 + per);
-  for (int j = j0 + threadIdx.x; j < j1; j += blockDim.x) {
-    sF[j - j0] = b.popF[j];
-    sE[j - j0] = b.popE[j];
-  }
+  if (blockIdx.x != 0) return;
+  __shared__ int coarse[kNC];
+  __shared__ int s_bin;
+  const int sel = st->sel_bin;
+  const unsigned need = (unsigned)st->sel_need;
+  const int nc = occupied_coarse<false>(b, coarse);
+  if (t == 0) s_bin = -1;
   __syncthreads();
-  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nb; q += gridDim.x * blockDim.x) {
-    const int E = b.popE[q];
-    const uint64_t fp = b.popF[q];
-    int r = 0;
-    for (int j = 0; j < j1 - j0; j++) r += key_lt(sE[j], sF[j], E, fp) ? 1 : 0;
-    if (r) atomicAdd(&b.popRank[q], r);
-  }
-}
-
-// Grid: the pivots' sequences leave their pool slots, which are freed (pushed on the stack) and leave
-// the histogram.
-__global__ void __launch_bounds__(256) pq_pivot_kernel(PqBufs b) {
-  PqState* st = b.st;
-  const int nb = st->b;
-  const int Eb = st->E_base;
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long base = (long long)blockIdx.x * blockDim.x; base < nb; base += stride) {
-    const long long q = base + threadIdx.x;
-    const bool on = q < nb;
-    int id = 0, bin = -1;
-    if (on) {
-      int r = b.popRank[q];  // pivot index = rank (keys are distinct, so 0 <= r < nb)
-      if (r < 0 || r >= nb) {
-        st->error = 1;
-        r = (int)q;
-      }
-      id = b.popId[q];
-      const int E = b.popE[q];
-      b.pivE[r] = E;
-      b.pivFp[r] = b.popF[q];
-      for (int w = 0; w < b.W; w++) b.pivSeq[(size_t)r * b.W + w] = b.pSeq[(size_t)id * b.W + w];
-      b.pE[id] = INT32_MAX;
-      b.popRank[q] = 0;  // cleared for the next round
-      bin = e_bin(E, Eb);
+  for (int x = t >> 5; x < nc; x += kSelThreads / 32) {
+    const int cb = coarse[x];
+    unsigned h[kCoarse / 32], left = 0;
+    int top = -1;
+#pragma unroll
+    for (int i = 0; i < kCoarse / 32; i++) h[i] = b.hP[cb * kCoarse + 32 * i + lane];
+#pragma unroll
+    for (int i = 0; i < kCoarse / 32; i++) {
+      const int bin = cb * kCoarse + 32 * i + lane;
+      const unsigned now = bin < sel ? 0u : (bin == sel ? h[i] - need : h[i]);
+      if (now != h[i]) b.hP[bin] = now;
+      left += now;
+      if (now) top = bin;
     }
-    const long long o = warp_append(&st->free_top, on);
-    if (on) b.freeIds[o] = id;
-    hist_add(b.hP, b.hP2, bin, -1);
+    left = (unsigned)warp_sum_i32((int)left);
+    top = warp_max_i32(top);
+    if (lane == 0) {
+      b.hP2[cb] = left;
+      if (top >= 0) atomicMax(&s_bin, top);
+    }
   }
-}
-
-// One block: the highest occupied bin of the pool (after the pops), -1 when it is empty.
-__global__ void __launch_bounds__(kSelThreads) pq_pmax_kernel(PqBufs b) {
-  __shared__ int s_cb, s_fb;
-  const int t = threadIdx.x;
+  __syncthreads();
   if (t == 0) {
-    s_cb = -1;
-    s_fb = -1;
+    st->pmax_bin = s_bin;
+    st->pop_base = st->free_top;
+    st->free_top += st->b;  // filled by the expansion
   }
-  __syncthreads();
-  if (t < kNC && b.hP2[t]) atomicMax(&s_cb, t);
-  __syncthreads();
-  const int cb = s_cb;
-  if (cb >= 0 && t < kCoarse && b.hP[cb * kCoarse + t]) atomicMax(&s_fb, cb * kCoarse + t);
-  __syncthreads();
-  if (t == 0) b.st->pmax_bin = cb >= 0 ? s_fb : -1;
 }
 
-// One warp per pivot: Delta E of all L single flips, visited-set test, dense survivor output.
-__global__ void __launch_bounds__(32 * kPqWarps) pq_expand_kernel(PqBufs b, Layout ly) {
-  __shared__ ScanSmem slabs[kPqWarps];
-  __shared__ uint32_t rbits_all[kPqWarps][kBitWords];
-  __shared__ int16_t P_all[kPqWarps][kMaxL];
-  __shared__ uint32_t xbits_all[kPqWarps][kBitWords];
-  ScanSmem& sm = slabs[threadIdx.x >> 5];
-  uint32_t* rbits = rbits_all[threadIdx.x >> 5];
-  int16_t* Pm = P_all[threadIdx.x >> 5];
-  uint32_t* xbits = xbits_all[threadIdx.x >> 5];
-  const int lane = lane_id();
+// Shared memory of one expanding warp, in 32-bit words from its slab's start.
+struct ExpandPlan {
+  ScanMmaPlan mma;
+  int q, x, v, words;
+};
+constexpr int kExpBits = 0, kExpClass = kBitWords, kExpRev = kExpClass + 2 * kClassWords, kExpTables = kExpRev + 2 * kClassWords;
+
+// Work items: pivot q's flips (c = 0) and its rotations (c = 1 .. 2 T_r), one warp each.  The flips' warp also
+// takes the pivot's sequence out of the pool and frees its slot.
+template <int NW>
+__global__ void __launch_bounds__(32 * kPqWarps, NW <= 8 ? 6 : 4) pq_expand_kernel(PqBufs b, ExpandPlan ep) {
+  constexpr int NT = (NW + 3) / 4;
+  extern __shared__ __align__(16) uint32_t pq_smem[];
+  uint32_t* slab = pq_smem + (size_t)(threadIdx.x >> 5) * ep.words;
+  uint32_t *bits = slab + kExpBits, *cw = slab + kExpClass, *rw = slab + kExpRev, *qt = slab + ep.q, *xt = slab + ep.x;
+  int16_t* v = reinterpret_cast<int16_t*>(slab + ep.v);
+  const int lane = lane_id(), L = b.L;
   const PqState* st = b.st;
   const int nb = st->b;
-  for (int q = blockIdx.x * kPqWarps + (threadIdx.x >> 5); q < nb; q += gridDim.x * kPqWarps) {
-    load_bits(sm, b.pivSeq + (size_t)q * b.W, b.L);
-    build_table(sm, ly);
-    const bool fast = pack_c8(sm, ly);
-    const int SC = table_sum(sm, ly);
-    build_bytes(sm, ly);
-    p_all(sm, ly, xbits, rbits, Pm);
-    const int E = b.pivE[q];
-    const uint64_t fp = b.pivFp[q];
-    for (int base = 0; base < ly.n_tiles; base += 32) {
-      const int tau = base + lane;
-      if (tau < ly.n_tiles) {
-        int cls, q0;
-        tile_of(ly, tau, cls, q0);
-        int acc[kPqM];
-        if (fast)
-          scan_tile<kPqM, false>(sm, ly, cls, q0, acc);
-        else
-          scan_tile<kPqM, true>(sm, ly, cls, q0, acc);
-        // the tile's Delta E and fingerprints, then the first visited-set probe of all of them at once
-        // (independent loads), then the rare longer probe sequences
-        int dv[kPqM], mv[kPqM];
-        uint64_t fv[kPqM], hv[kPqM];
-#pragma unroll
-        for (int j = 0; j < kPqM; j++) {
-          const SlotInfo si = slot_info(ly, cls, q0 + j);
-          mv[j] = si.active ? si.m : 0;
-          dv[j] = si.active ? finish_delta(sm, ly, cls, q0 + j, si, acc[j], SC, Pm[si.m - 1]) : 0;
-          fv[j] = si.active ? fp ^ b.ztab[si.m - 1] : kEmptyKey;
-        }
-#pragma unroll
-        for (int j = 0; j < kPqM; j++) hv[j] = (mv[j] && fv[j] != kEmptyKey) ? b.H[h_slot(fv[j], b.H_log2)] : kEmptyKey;
-#pragma unroll
-        for (int j = 0; j < kPqM; j++) {
-          if (!mv[j]) continue;
-          bool seen;
-          if (fv[j] == kEmptyKey)
-            seen = st->h_has_empty != 0;
-          else if (hv[j] == fv[j] || hv[j] == kEmptyKey)
-            seen = hv[j] == fv[j];
-          else
-            seen = h_contains_after(b, fv[j], h_slot(fv[j], b.H_log2));
-          const size_t di = (size_t)q * b.width + (mv[j] - 1);
-          b.dE[di] = seen ? INT32_MAX : E + dv[j];
-          b.dFp[di] = fv[j];
-        }
-      }
-    }
-    // MAKE_ROTATIONS of the pivot: each rotation's energy and fingerprint from scratch
-    for (int c = 0; c < 2 * b.Tr; c++) {
-      const int r = rot_shift(b.L, b.Tr, c);
-      for (int w = 0; w < kBitWords; w++) {
-        const int i = 32 * w + lane;  // 0-based position of the rotated sequence
-        int bit = 0;
-        if (i < b.L) {
-          int j = i + r;
-          if (j >= b.L) j -= b.L;
-          bit = seq_bit(sm, j + 1);
-        }
-        const unsigned word = __ballot_sync(kFull, bit);
-        if (lane == 0) rbits[w] = word;
-      }
-      __syncwarp();
-      int e = 0;
-      for (int k = lane + 1; k < b.L; k += 32) {
-        const int cv = corr_lag(rbits, b.L, k);
-        e += cv * cv;
-      }
-      e = warp_sum_i32(e);
-      uint64_t h = 0;
-      for (int i = lane; i < b.L; i += 32)
-        if (!((rbits[i >> 5] >> (i & 31)) & 1u)) h ^= b.ztab[i];
-      h = warp_xor_u64(h);
-      if (lane == 0) {
-        const size_t di = (size_t)q * b.width + b.L + c;
-        b.dE[di] = h_contains(b, h) ? INT32_MAX : e;
-        b.dFp[di] = h;
-      }
-      __syncwarp();
+  if (nb == 0 || st->pop_cnt != nb || st->error) return;  // an inconsistent pop ends the search in pq_finish_kernel
+  for (int i = lane; i < ep.words; i += 32) slab[i] = 0u;
+  __syncwarp();
+  const int per = 1 + 2 * b.Tr;
+  const uint32_t* const xs[1] = {xt};
+  for (int it = blockIdx.x * kPqWarps + (threadIdx.x >> 5); it < nb * per; it += gridDim.x * kPqWarps) {
+    // all flips first, so that a tail of short rotation items evens out the blocks
+    const int q = it < nb ? it : (it - nb) % nb, rot = it < nb ? 0 : 1 + (it - nb) / nb;
+    const int id = b.popId[q], E = b.popE[q];
+    const uint64_t* src = b.pSeq + (size_t)id * b.W;
+    __syncwarp();
+    if (lane < NW) {
+      const uint32_t w = reinterpret_cast<const uint32_t*>(src)[lane];
+      bits[lane] = lane == NW - 1 ? w & (0xffffffffu >> (32 * NW - L)) : w;
     }
     __syncwarp();
-  }
-}
-
-// Dedup, first pass: every survivor inserts its (E, fp) key; the first inserter of a key becomes the
-// key's unique survivor (marked in uRep, its representative settled by the second pass) and the table
-// slot points to its dense index.  Unique survivors stay at their dense index: nothing is compacted.
-// Each thread takes four consecutive survivors and keeps their four probes in flight together (the
-// pass is bound by the latency of the table's compare-and-swaps).
-template <bool SEED>
-__global__ void __launch_bounds__(256) pq_dedup_insert_kernel(PqBufs b) {
-  PqState* st = b.st;
-  const long long n = st->n_dense;
-  const long long nq = (n + 3) >> 2;
-  const uint64_t mask = (1ull << b.hs_log2) - 1;
-  const int Eb = st->E_base, pmax = st->pmax_bin;
-  long long fresh_n = 0, low = 0;
-  int mE = INT32_MAX;
-  for (long long qd = (long long)blockIdx.x * blockDim.x + threadIdx.x; qd < nq; qd += (long long)gridDim.x * blockDim.x) {
-    const int4 e4 = reinterpret_cast<const int4*>(b.dE)[qd];
-    const int E[4] = {e4.x, e4.y, e4.z, e4.w};
-    uint64_t k[4], s[4];
-    bool act[4], fresh[4];
-#pragma unroll
-    for (int j = 0; j < 4; j++) {
-      const long long i = 4 * qd + j;
-      act[j] = i < n && E[j] != INT32_MAX;
-      fresh[j] = false;
-      k[j] = act[j] ? dedup_key(E[j], b.dFp[i]) : 0ull;
-      s[j] = (k[j] * kGamma) >> (64 - b.hs_log2);
+    if (rot) {
+      // rotation: element i is element i + r (mod L); its energy and fingerprint from scratch
+      const int r = rot_shift(L, b.Tr, rot - 1), o = 32 * lane + r;
+      uint32_t y = 0;
+      if (lane < NW) {
+        if (o < L) y = __funnelshift_r(bits[o >> 5], bits[(o >> 5) + 1], o & 31);
+        const int ow = o - L;  // elements past the end come from the start
+        if (ow >= 0)
+          y = __funnelshift_r(bits[ow >> 5], bits[(ow >> 5) + 1], ow & 31);
+        else if (ow > -32)
+          y |= bits[0] << -ow;
+        if (lane == NW - 1) y &= 0xffffffffu >> (32 * NW - L);
+      }
+      if (lane < kBitWords) rw[lane] = y;
+      __syncwarp();
+      const int e = energy_words<NW>(rw, L);
+      uint64_t h = 0;
+      for (int i = lane; i < L; i += 32)
+        if (!((rw[i >> 5] >> (i & 31)) & 1u)) h ^= b.ztab[i];
+      h = warp_xor_u64(h);
+      if (lane == 0) {
+        const size_t di = (size_t)q * b.width + L + rot - 1;
+        b.dE[di] = e;
+        b.dFp[di] = h;
+      }
+      continue;
     }
-    for (uint64_t it = 0; it <= mask && (act[0] || act[1] || act[2] || act[3]); it++) {  // at most half full
-      unsigned long long old[4];
+    if (lane < b.W) b.pivSeq[(size_t)q * b.W + lane] = src[lane];
+    if (lane == 0) {
+      b.pE[id] = INT32_MAX;
+      b.freeIds[st->pop_base + q] = id;
+    }
+    const uint64_t fp = b.popF[q];
+    corr_words<NW>(bits, bits, L, [&](int d, int cd) {
+      if (d >= 1 && d < L) put_q(qt, ep.mma, d, cd);
+    });
+    put_x(xt, bits, L);
+    split_classes(bits, cw);
+    self_convolution<(NW + 1) / 2>(cw, rw, L, v);
+    __syncwarp();
+    float acc[1][NT][4];
+    scan_mma<1, NT>(qt, xs, ep.mma, L, acc);
+    int32_t* oe = b.dE + (size_t)q * b.width;
+    uint64_t* of = b.dFp + (size_t)q * b.width;
 #pragma unroll
-      for (int j = 0; j < 4; j++)
-        old[j] = act[j] ? atomicCAS(reinterpret_cast<unsigned long long*>(&b.hkey[s[j]]), 0ull, k[j]) : 0ull;
+    for (int T = 0; T < NT; T++) {
+      const int jl = 128 * T + 32 * (lane & 3) + (lane >> 2);
+      const uint32_t own = jl < L ? bits[jl >> 5] >> (lane >> 2) : 0u;
 #pragma unroll
-      for (int j = 0; j < 4; j++) {
-        if (!act[j]) continue;
-        if (old[j] == 0ull) {
-          fresh[j] = true;
-          b.hval[s[j]] = (int32_t)(4 * qd + j);
-          act[j] = false;
-        } else if (old[j] == k[j]) {
-          act[j] = false;
-        } else {
-          s[j] = (s[j] + 1) & mask;
+      for (int r = 0; r < 4; r++) {
+        const int o = 16 * (r & 1) + 8 * (r >> 1), m = jl + o + 1;
+        if (m <= L) {
+          const int tm = (int)acc[0][T][r];
+          oe[m - 1] = E + 4 * ((int)v[m] + (int)v[kMaxL + 1 + m] + L - 2 - ((own >> o & 1u) ? tm : -tm));
+          of[m - 1] = fp ^ b.ztab[m - 1];
         }
       }
     }
-    reinterpret_cast<uint4*>(b.uRep)[qd] = make_uint4(fresh[0] ? 0xFFFFFFFEu : ~0u, fresh[1] ? 0xFFFFFFFEu : ~0u,
-                                                       fresh[2] ? 0xFFFFFFFEu : ~0u, fresh[3] ? 0xFFFFFFFEu : ~0u);
-#pragma unroll
-    for (int j = 0; j < 4; j++)
-      if (fresh[j]) {
-        fresh_n++;
-        mE = min(mE, E[j]);
-        low += e_bin(E[j], Eb) <= pmax ? 1 : 0;
-      }
   }
-  block_add(&st->nU, fresh_n);
-  block_min(&st->minE_round, mE);
-  block_add(&st->nU_low, low);
 }
 
-// Which survivors the cut needs counted.  Everything fits: none.  The pool's rest and the survivors
-// inside its occupied bins reach the cap: the cut lies in those bins, so only they are counted.
-// Otherwise all of them.
-__device__ __forceinline__ int hist_mode_of(const PqState* st, long long cap) {
-  const long long rest = st->nP - st->b;
-  if (rest + st->nU <= cap) return 0;
-  if (st->pmax_bin >= 0 && rest + st->nU_low >= cap) return 1;
-  return 2;
-}
-
-// Dedup, second pass: each survivor finds its key's slot and lowers the representative of the key's
-// unique survivor to the smallest (pivot, column) -- the pivots are in key order, so this is the
-// sequential definition's first occurrence.  The unique survivors also enter the survivor histogram (the
-// bins the cut needs) and give the smallest fingerprint among the smallest-energy survivors.  Four
-// consecutive survivors per thread, their lookups in flight together; survivors the cut cannot reach
-// are skipped.
+// Visited set and dedup: a child found in H is dropped; every other inserts its (E, fp) key; the first inserter of a key stays the key's survivor, the
+// others are dropped from the dense array.  Which one stays does not
+// matter: equal keys are the same sequence.  Survivors inside the pool's occupied bins are counted on the way
+// (the cut lies there once the pool is full).  Each thread takes four consecutive survivors and keeps their four
+// probes in flight together (the pass is bound by the latency of the table's compare-and-swaps).
 template <bool SEED>
-__global__ void __launch_bounds__(256) pq_dedup_rep_kernel(PqBufs b) {
+__global__ void __launch_bounds__(256, 6) pq_dedup_kernel(PqBufs b) {
   PqState* st = b.st;
+  __shared__ unsigned coarse[kNC];
   const long long n = st->n_dense;
+  if (n == 0) return;
+  CoarseCounts counts(coarse);
+  const bool filter = use_filter(b);
   const long long nq = (n + 3) >> 2;
   const uint64_t mask = (1ull << b.hs_log2) - 1;
-  const int mode = hist_mode_of(st, b.cap);
-  if (blockIdx.x == 0 && threadIdx.x == 0) st->hist_mode = mode;
-  const int Eb = st->E_base, pmax = st->pmax_bin, mE = st->minE_round;
-  uint64_t mf = ~0ull;
+  const int Eb = st->E_base, pmax = SEED ? -1 : st->pmax_bin;  // the seeds' energy window is not set yet
+  long long kept = 0, low = 0;
+  int mE = INT32_MAX;
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long base = (long long)blockIdx.x * blockDim.x; base < nq; base += stride) {  // warp-uniform
     const long long qd = base + threadIdx.x;
@@ -898,53 +972,119 @@ __global__ void __launch_bounds__(256) pq_dedup_rep_kernel(PqBufs b) {
       E[2] = e4.z;
       E[3] = e4.w;
     }
-    uint64_t fp[4], k[4], s[4];
-    bool act[4];
+    uint64_t k[4], s[4];
+    bool act[4], fresh[4];
+    {
+      uint64_t fp[4], hv[4];
 #pragma unroll
-    for (int j = 0; j < 4; j++) {
-      const long long i = 4 * qd + j;
-      // with the cut inside the pool's occupied bins (mode 1), a survivor above them is never admitted
-      // nor the round's smallest (survivors inside them exist then), so its representative is not needed
-      act[j] = qd < nq && i < n && E[j] != INT32_MAX && !(mode == 1 && e_bin(E[j], Eb) > pmax);
-      fp[j] = act[j] ? b.dFp[i] : 0ull;
-      k[j] = dedup_key(E[j], fp[j]);
-      s[j] = (k[j] * kGamma) >> (64 - b.hs_log2);
-    }
-    bool look[4] = {act[0], act[1], act[2], act[3]};
-    for (uint64_t it = 0; it <= mask && (look[0] || look[1] || look[2] || look[3]); it++) {
-      uint64_t hk[4];
+      for (int j = 0; j < 4; j++) {
+        act[j] = 4 * qd + j < n;
+        fp[j] = act[j] ? b.dFp[4 * qd + j] : kEmptyKey;
+      }
+      if (!SEED) {
 #pragma unroll
-      for (int j = 0; j < 4; j++) hk[j] = look[j] ? b.hkey[s[j]] : 0ull;
+        for (int j = 0; j < 4; j++) hv[j] = fp[j] != kEmptyKey && (!filter || filter_hit(b, fp[j])) ? b.H[h_slot(fp[j], b.H_log2)] : kEmptyKey;
 #pragma unroll
-      for (int j = 0; j < 4; j++)
-        if (look[j]) {
-          if (hk[j] == k[j])
-            look[j] = false;
+        for (int j = 0; j < 4; j++) {
+          if (!act[j]) continue;
+          bool seen;
+          if (fp[j] == kEmptyKey)
+            seen = st->h_has_empty != 0;
+          else if (hv[j] == fp[j] || hv[j] == kEmptyKey)
+            seen = hv[j] == fp[j];
           else
-            s[j] = (s[j] + 1) & mask;
-        }
-    }
-    int hv[4];
-#pragma unroll
-    for (int j = 0; j < 4; j++) hv[j] = act[j] ? b.hval[s[j]] : -1;
-#pragma unroll
-    for (int j = 0; j < 4; j++) {
-      int bin = -1;
-      if (act[j]) {
-        const long long i = 4 * qd + j;
-        const unsigned rep = SEED ? (unsigned)i << kColBits
-                                  : ((unsigned)(i / b.width) << kColBits) | (unsigned)(i % b.width);
-        atomicMin(&b.uRep[hv[j]], rep);
-        if (hv[j] == (int32_t)i) {  // the key's unique survivor
-          const int eb = e_bin(E[j], Eb);
-          if (mode == 2 || (mode == 1 && eb <= pmax)) bin = eb;
-          if (E[j] == mE) mf = min(mf, fp[j]);
+            seen = h_contains_after(b, fp[j], h_slot(fp[j], b.H_log2));
+          if (seen) {
+            b.dE[4 * qd + j] = INT32_MAX;
+            act[j] = false;
+          }
         }
       }
-      if (mode) hist_add(b.hU, b.hU2, bin, 1);
+#pragma unroll
+      for (int j = 0; j < 4; j++) {
+        fresh[j] = false;
+        k[j] = act[j] ? dedup_key(E[j], fp[j]) : 0ull;
+        s[j] = (k[j] * kGamma) >> (64 - b.hs_log2);
+      }
+    }
+    for (uint64_t it = 0; it <= mask && (act[0] || act[1] || act[2] || act[3]); it++) {  // at most half full
+      unsigned long long old[4];
+#pragma unroll
+      for (int j = 0; j < 4; j++)
+        old[j] = act[j] ? atomicCAS(reinterpret_cast<unsigned long long*>(&b.hkey[s[j]]), 0ull, k[j]) : 0ull;
+#pragma unroll
+      for (int j = 0; j < 4; j++) {
+        if (!act[j]) continue;
+        if (old[j] == 0ull) {
+          fresh[j] = true;
+          act[j] = false;
+        } else if (old[j] == k[j]) {
+          act[j] = false;
+          b.dE[4 * qd + j] = INT32_MAX;
+        } else {
+          s[j] = (s[j] + 1) & mask;
+        }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+      if (fresh[j]) {
+        kept++;
+        mE = min(mE, E[j]);
+        const int bin = e_bin(E[j], Eb);
+        if (bin <= pmax) {
+          low++;
+          counts.add(b.hU, bin);
+        }
+      }
     }
   }
-  if (mf != ~0ull) atomicMin(reinterpret_cast<unsigned long long*>(&st->minfp_round), (unsigned long long)mf);
+  counts.flush(b.hU2);
+  block_add(&st->nU, kept);
+  block_min(&st->minE_round, mE);
+  block_add(&st->nU_low, low);
+}
+
+// The survivors above the pool's occupied bins are counted when the cut may lie there or nothing is cut; then the
+// last block to finish finds where the cap cuts (pool's rest u survivors), or that everything fits.
+__global__ void __launch_bounds__(kSelThreads) pq_cut_kernel(PqBufs b) {
+  PqState* st = b.st;
+  __shared__ unsigned coarse[kNC];
+  __shared__ int s_last;
+  if (counts_all(st, b.cap)) {
+    CoarseCounts counts(coarse);
+    const long long n = st->n_dense;
+    const int Eb = st->E_base, pmax = st->pmax_bin;
+    const long long stride = (long long)gridDim.x * blockDim.x * kPer;
+    for (long long first = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * kPer; first < n; first += stride) {
+      int E[kPer];
+      load_energies(b.dE, first, n, E);
+#pragma unroll
+      for (int e = 0; e < kPer; e++)
+        if (E[e] != INT32_MAX) {
+          const int bin = e_bin(E[e], Eb);
+          if (bin > pmax) counts.add(b.hU, bin);
+        }
+    }
+    counts.flush(b.hU2);
+  }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(&st->done, 1) == (int)gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  const bool fits = st->nP - st->b + st->nU <= b.cap;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    st->done = 0;
+    st->cand_cnt = 0;  // the pop's candidates are done with
+    st->sel_need = fits ? -1 : 0;
+    st->sel_bin = kNB;
+  }
+  for (int i = threadIdx.x; i < kFpBins; i += kSelThreads) b.hF[i] = 0u;
+  __syncthreads();
+  if (!fits) select_bin<true>(b, b.cap);
 }
 
 // The histogram's energy window, from the smallest seed energy (improvements stay far inside it).
@@ -953,172 +1093,75 @@ __global__ void pq_set_window_kernel(PqBufs b) {
   st->E_base = st->minE_round == INT32_MAX ? 0 : max(0, st->minE_round - kNB / 2);
 }
 
-// One thread: the best (a strict improvement, as in Algorithm 2; for the seeds, the smallest seed) and
-// the round's counters.
-template <bool SEED>
-__global__ void pq_best_kernel(PqBufs b) {
-  PqState* st = b.st;
-  if (!SEED && st->b == 0) return;
-  const unsigned rep = st->best_rep_round;
-  if (SEED) {
-    if (st->nU > 0 && (rep >> kColBits) < (unsigned)b.n_seeds) {
-      st->best_E = st->minE_round;
-      st->best_fp = st->minfp_round;
-      const int q = (int)(rep >> kColBits);
-      for (int t = 0; t < b.W; t++) b.best_seq[t] = b.seeds[(size_t)q * b.W + t];
-    }
-    return;
-  }
-  st->survivors += st->nU;
-  if (st->nU > 0 && (rep >> kColBits) >= (unsigned)st->b) {  // every survivor has a representative
-    st->error = 1;
-    return;
-  }
-  if (st->nU > 0 && st->minE_round < st->best_E) {
-    st->best_E = st->minE_round;
-    st->best_fp = st->minfp_round;
-    pq_child(b.pivSeq + (size_t)(rep >> kColBits) * b.W, b, (int)(rep & ((1u << kColBits) - 1u)), b.best_seq);
-    st->improvements++;
-    st->u = 0;
-  } else {
-    st->u += st->b;
-  }
-}
-
-// Whether a key of bin `bin` is inside the cut.
-__device__ __forceinline__ bool below_cut(const PqState* st, int bin, int E, uint64_t fp) {
-  if (st->sel_need < 0) return true;  // no cut
-  return bin < st->sel_bin || (bin == st->sel_bin && key_le(E, fp, st->sel_E, st->sel_fp));
-}
-
-// Pool pass: the entries beyond the cut are evicted (slot freed, histogram updated); four slots per
-// thread, their energies in one 16-byte load.
-__global__ void __launch_bounds__(256) pq_evict_kernel(PqBufs b) {
-  PqState* st = b.st;
-  if (st->sel_need < 0) return;
-  const int Eb = st->E_base;
-  const long long nq = (b.cap + 3) >> 2;
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long base = (long long)blockIdx.x * blockDim.x; base < nq; base += stride) {
-    const long long qd = base + threadIdx.x;
-    int4 e4 = make_int4(INT32_MAX, INT32_MAX, INT32_MAX, INT32_MAX);
-    if (qd < nq) e4 = reinterpret_cast<const int4*>(b.pE)[qd];
-    const int ev[4] = {e4.x, e4.y, e4.z, e4.w};
-#pragma unroll
-    for (int e = 0; e < 4; e++) {
-      const long long i = 4 * qd + e;
-      bool out = false;
-      int bin = 0;
-      const int E = ev[e];
-      if (i < b.cap && E != INT32_MAX) {
-        bin = e_bin(E, Eb);
-        out = bin > st->sel_bin || (bin == st->sel_bin && !key_le(E, b.pFp[i], st->sel_E, st->sel_fp));
-      }
-      const long long o = warp_append(&st->free_top, out);
-      if (out) {
-        b.freeIds[o] = (int32_t)i;
-        b.pE[i] = INT32_MAX;
-      }
-      hist_add(b.hP, b.hP2, out ? bin : -1, -1);
-      warp_add(&st->ev_round, out ? 1 : 0);
-    }
-  }
-}
-
-// Survivor pass: the survivors inside the cut take a free slot (the sequence built from the pivot, or
-// copied from the seed) and enter the visited set; the smallest survivor key's representative is noted
-// for the best.
+// Survivor pass: the survivors inside the cut take a free slot (the sequence built from the pivot, or copied
+// from the seed) and enter the visited set; the smallest fingerprint among the smallest energies is noted for
+// the best.  Four consecutive survivors per thread: a fingerprint is read only where the cut or the best test
+// needs it.
 template <bool SEED>
 __global__ void __launch_bounds__(256) pq_admit_kernel(PqBufs b) {
   PqState* st = b.st;
   const long long n = st->n_dense;
+  if (n == 0) return;
   const long long nq = (n + 3) >> 2;
   const int Eb = st->E_base;
   const bool cut = st->sel_need >= 0;
-  const int sel_bin = st->sel_bin, minE = st->minE_round;
+  const int sel_bin = st->sel_bin, minE = st->minE_round, selE = st->sel_E;
+  const uint64_t selF = st->sel_fp;
   const long long stride = (long long)gridDim.x * blockDim.x;
-  // four consecutive survivors per thread: their representatives and energies in one 16-byte load each;
-  // a fingerprint is read only where the cut or the best test needs it
-  for (long long base = (long long)blockIdx.x * blockDim.x; base < nq; base += stride) {  // warp-uniform
+  long long ins = 0, adm = 0;
+  uint64_t mf = ~0ull;
+  for (long long base = (long long)blockIdx.x * blockDim.x; base < nq; base += stride) {  // block-uniform
     const long long qd = base + threadIdx.x;
-    uint4 r4 = make_uint4(~0u, ~0u, ~0u, ~0u);
     int4 e4 = make_int4(INT32_MAX, INT32_MAX, INT32_MAX, INT32_MAX);
-    if (qd < nq) {
-      r4 = reinterpret_cast<const uint4*>(b.uRep)[qd];
-      e4 = reinterpret_cast<const int4*>(b.dE)[qd];
-    }
-    const unsigned R[4] = {r4.x, r4.y, r4.z, r4.w};
-    const int Ev[4] = {e4.x, e4.y, e4.z, e4.w};
+    if (qd < nq) e4 = reinterpret_cast<const int4*>(b.dE)[qd];
+    const int E[4] = {e4.x, e4.y, e4.z, e4.w};
+    bool in[4];
+    uint64_t fp[4];
+    int mine = 0;
 #pragma unroll
     for (int j = 0; j < 4; j++) {
       const long long u = 4 * qd + j;
-      bool in = false;
-      const int E = Ev[j];
-      int bin = 0;
-      uint64_t fp = 0;
-      if (u < n && R[j] != ~0u) {
-        bin = e_bin(E, Eb);
-        if (!cut || bin <= sel_bin || E == minE) {
-          fp = b.dFp[u];
-          in = below_cut(st, bin, E, fp);
-          if (E == minE && fp == st->minfp_round) st->best_rep_round = R[j];  // the smallest key
+      in[j] = false;
+      fp[j] = 0;
+      if (u < n && E[j] != INT32_MAX) {
+        const int bin = e_bin(E[j], Eb);
+        if (!cut || bin <= sel_bin || E[j] == minE) {
+          fp[j] = b.dFp[u];
+          in[j] = !cut || bin < sel_bin || (bin == sel_bin && key_le(E[j], fp[j], selE, selF));
+          if (E[j] == minE) mf = min(mf, fp[j]);
         }
       }
-      // free slots come off the top of the stack, one atomic per warp
-      const unsigned m = __ballot_sync(kFull, in);
-      long long top = 0;
-      if (m) {
-        const int leader = __ffs(m) - 1;
-        if (lane_id() == leader)
-          top = (long long)atomicAdd(reinterpret_cast<unsigned long long*>(&st->free_top),
-                                     (unsigned long long)(-(long long)__popc(m)));
-        top = __shfl_sync(kFull, top, leader);
-      }
-      int ins = 0;
-      const long long o = top - 1 - __popc(m & ((1u << lane_id()) - 1u));
-      if (in && o < 0) {  // more admissions than free slots: only an inconsistent state gets here
-        st->error = 1;
-        in = false;
-      }
-      const unsigned rep = in ? R[j] : 0u;
-      if (in && (rep >> kColBits) >= (unsigned)(SEED ? b.n_seeds : st->b)) {  // every survivor has one (pass 2)
-        st->error = 1;
-        in = false;
-      }
-      if (in) {
-        const int id = b.freeIds[o];
-        b.pE[id] = E;
-        b.pFp[id] = fp;
-        if (SEED) {
-          for (int t = 0; t < b.W; t++) b.pSeq[(size_t)id * b.W + t] = b.seeds[(size_t)(rep >> kColBits) * b.W + t];
-        } else {
-          pq_child(b.pivSeq + (size_t)(rep >> kColBits) * b.W, b, (int)(rep & ((1u << kColBits) - 1u)),
-                   b.pSeq + (size_t)id * b.W);
-        }
-        ins = h_insert(b, fp);
-      }
-      hist_add(b.hP, b.hP2, in ? bin : -1, 1);
-      h_count(b, ins);
-      warp_add(&st->adm_round, in ? 1 : 0);
+      mine += in[j] ? 1 : 0;
     }
+    if (!__syncthreads_or(mine)) continue;
+    int total, before;
+    // free slots come off the top of the stack, the block's share at once
+    long long o = block_reserve(&st->free_top, mine, -1, &total, &before);
+    o += before - total;
+#pragma unroll
+    for (int j = 0; j < 4; j++)
+      if (in[j]) {
+        const long long u = 4 * qd + j;
+        if (o < 0) {  // more admissions than free slots: only an inconsistent state gets here
+          st->error = 1;
+          o++;
+          continue;
+        }
+        const int id = b.freeIds[o++];
+        b.pE[id] = E[j];
+        b.pFp[id] = fp[j];
+        if (SEED) {
+          for (int t = 0; t < b.W; t++) b.pSeq[(size_t)id * b.W + t] = b.seeds[(size_t)u * b.W + t];
+        } else {
+          pq_child(b.pivSeq + (size_t)(u / b.width) * b.W, b, (int)(u % b.width), b.pSeq + (size_t)id * b.W);
+        }
+        adm++;
+        ins += h_insert(b, fp[j]);
+      }
   }
-}
-
-template <bool SEED>
-__global__ void pq_round_end_kernel(PqBufs b) {
-  PqState* st = b.st;
-  if (SEED) {
-    st->nP = st->adm_round;
-  } else {
-    if (st->b == 0) return;
-    st->nP = st->nP - st->b - st->ev_round + st->adm_round;
-    st->admitted += st->adm_round;
-    st->evicted += st->ev_round;
-    st->expansions += st->b;
-    st->rounds++;
-  }
-  const long long slots = 1ll << b.H_log2;
-  if (st->h_size * 4 > slots * 3) st->error = 1;
+  if (mf != ~0ull) atomicMin(reinterpret_cast<unsigned long long*>(&st->minfp_round), (unsigned long long)mf);
+  block_add(&st->h_size, ins);
+  block_add(&st->adm_round, adm);
 }
 
 __global__ void pq_write_stats_kernel(PqBufs b, int32_t* best_E, labs_pq_stats* out) {
@@ -1141,9 +1184,7 @@ __global__ void pq_write_stats_kernel(PqBufs b, int32_t* best_E, labs_pq_stats* 
 int launch_pq_refine(labs_ctx* ctx, const labs_pq_cfg* cfg, const uint64_t* seeds, int n_seeds, uint64_t* best_seq,
                      int32_t* best_E, labs_pq_stats* stats, cudaStream_t st) {
   const int L = cfg->L, W = (L + 63) / 64;
-  if (cfg->B > kSortMax) return LABS_ERR_INVALID_ARG;
-  Layout ly;
-  if (!make_layout(ly, L, 0, 0, kPqM)) return LABS_ERR_INVALID_ARG;
+  if (cfg->B > kMaxB) return LABS_ERR_INVALID_ARG;
   const int width = L + 2 * cfg->T_r;
   const long long n_dense = std::max<long long>((long long)cfg->B * width, n_seeds);
   int hs_log2 = 10;
@@ -1158,16 +1199,16 @@ int launch_pq_refine(labs_ctx* ctx, const labs_pq_cfg* cfg, const uint64_t* seed
   };
   const size_t opE = take(4 * ((cap + 3) & ~3ll)), opF = take(8 * cap), opS = take(8 * cap * W), ofree = take(4 * cap);
   const size_t ohP = take(4 * kNB), ohP2 = take(4 * kNC), ohU = take(4 * kNB), ohU2 = take(4 * kNC);
-  const size_t opop = take(4 * (size_t)cfg->B), opivE = take(4 * (size_t)cfg->B), opivF = take(8 * (size_t)cfg->B);
+  const size_t ohF = take(4 * kFpBins), opop = take(4 * (size_t)cfg->B);
   const size_t opopE = take(4 * (size_t)cfg->B), opopF = take(8 * (size_t)cfg->B);
   const size_t opivS = take(8 * (size_t)cfg->B * W);
   const size_t ocand = take(4 * (size_t)(cap + n_dense)), ocE = take(4 * (size_t)(cap + n_dense));
-  const size_t ocF = take(8 * (size_t)(cap + n_dense)), orank = take(4 * (size_t)cfg->B);
+  const size_t ocF = take(8 * (size_t)(cap + n_dense)), ogrp = take(8 * (size_t)kGroup);
   const size_t odE = take(4 * ((n_dense + 3) & ~3ll)), odF = take(8 * n_dense);
-  const size_t ohk = take(8ull << hs_log2), ohv = take(4ull << hs_log2);
-  const size_t ouR = take(4 * ((n_dense + 3) & ~3ll));
+  const size_t ohk = take(8ull << hs_log2);
   const size_t ozt = take(8 * L), ost = take(sizeof(PqState)), obest = take(8 * W);
-  const size_t oH = take(8ull << cfg->H_log2);
+  const int f_log2 = std::min(cfg->H_log2, kFilterMax);
+  const size_t oH = take(8ull << cfg->H_log2), ofil = take((1ull << f_log2) / 8);
   char* base = static_cast<char*>(ws_get(ctx, kWsPq0, off));
   if (!base) return LABS_ERR_NOMEM;
   PqBufs b{};
@@ -1194,71 +1235,65 @@ int launch_pq_refine(labs_ctx* ctx, const labs_pq_cfg* cfg, const uint64_t* seed
   b.popId = reinterpret_cast<int32_t*>(base + opop);
   b.popE = reinterpret_cast<int32_t*>(base + opopE);
   b.popF = reinterpret_cast<uint64_t*>(base + opopF);
-  b.pivE = reinterpret_cast<int32_t*>(base + opivE);
-  b.pivFp = reinterpret_cast<uint64_t*>(base + opivF);
+  b.hF = reinterpret_cast<unsigned*>(base + ohF);
   b.pivSeq = reinterpret_cast<uint64_t*>(base + opivS);
   b.candId = reinterpret_cast<int32_t*>(base + ocand);
   b.cE = reinterpret_cast<int32_t*>(base + ocE);
   b.cF = reinterpret_cast<uint64_t*>(base + ocF);
-  b.popRank = reinterpret_cast<int32_t*>(base + orank);
+  b.grp = reinterpret_cast<uint64_t*>(base + ogrp);
   b.dE = reinterpret_cast<int32_t*>(base + odE);
   b.dFp = reinterpret_cast<uint64_t*>(base + odF);
   b.hkey = reinterpret_cast<uint64_t*>(base + ohk);
-  b.hval = reinterpret_cast<int32_t*>(base + ohv);
-  b.uRep = reinterpret_cast<unsigned*>(base + ouR);
   b.ztab = reinterpret_cast<uint64_t*>(base + ozt);
   b.st = reinterpret_cast<PqState*>(base + ost);
   b.best_seq = reinterpret_cast<uint64_t*>(base + obest);
   b.H = reinterpret_cast<uint64_t*>(base + oH);
+  b.filter = reinterpret_cast<uint32_t*>(base + ofil);
+  b.f_log2 = f_log2;
   b.seeds = seeds;
 
-  const unsigned g_pool = (unsigned)std::max(1ll, std::min<long long>((cap + 255) / 256, (long long)ctx->num_sms * 16));
+  // a thread takes kPer entries of a pool or survivor pass a turn, four in the passes that probe hash tables
+  auto pass_blocks = [&](long long n) {
+    return (unsigned)std::max(1ll, std::min<long long>((n + 256 * kPer - 1) / (256 * kPer), (long long)ctx->num_sms * 8));
+  };
+  const unsigned g_pool = pass_blocks(cap), g_cand_dense = pass_blocks(n_dense);
   const unsigned g_dense =
-      (unsigned)std::max(1ll, std::min<long long>((n_dense + 255) / 256, (long long)ctx->num_sms * 16));
-  const size_t cand_smem = (size_t)kCandSmem * 12;
-  if (cudaFuncSetAttribute(pq_boundary_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cand_smem) !=
-          cudaSuccess ||
-      cudaFuncSetAttribute(pq_boundary_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cand_smem) !=
-          cudaSuccess)
-    return LABS_ERR_CUDA;
-  const unsigned g_piv = (unsigned)std::max(1, std::min((cfg->B + 255) / 256, ctx->num_sms * 4));
+      (unsigned)std::max(1ll, std::min<long long>((n_dense + 1023) / 1024, (long long)ctx->num_sms * 8));
 
-  // The survivor path, shared by the seeds and every round: dedup, best, cut, eviction, admission.
+  // boundary candidates: a bin's share of the pool and the survivors, a thousandth or so
+  const unsigned g_cand = (unsigned)std::max(1ll, std::min<long long>((cap + n_dense) / 65536, ctx->num_sms / 2));
+
+  // The survivor path, shared by the seeds and every round: dedup, cut, eviction, admission, best, and the next
+  // round's beginning.
   auto survivor_path = [&](bool seed, cudaStream_t s) {
     if (seed) {
-      pq_dedup_insert_kernel<true><<<g_dense, 256, 0, s>>>(b);
+      pq_dedup_kernel<true><<<g_dense, 256, 0, s>>>(b);
       pq_set_window_kernel<<<1, 1, 0, s>>>(b);
-      pq_dedup_rep_kernel<true><<<g_dense, 256, 0, s>>>(b);
     } else {
-      pq_dedup_insert_kernel<false><<<g_dense, 256, 0, s>>>(b);
-      pq_dedup_rep_kernel<false><<<g_dense, 256, 0, s>>>(b);
+      pq_dedup_kernel<false><<<g_dense, 256, 0, s>>>(b);
     }
-    pq_select_kernel<false><<<1, kSelThreads, 0, s>>>(b);
-    pq_gather_kernel<false, false><<<g_pool, 256, 0, s>>>(b);
-    pq_gather_kernel<false, true><<<g_dense, 256, 0, s>>>(b);
-    pq_boundary_kernel<false><<<1, kSelThreads, cand_smem, s>>>(b);
-    pq_evict_kernel<<<g_pool, 256, 0, s>>>(b);
+    pq_cut_kernel<<<std::max(1u, g_cand_dense / 4), kSelThreads, 0, s>>>(b);
+    pq_pool_kernel<false><<<g_pool + g_cand_dense, 256, 0, s>>>(b, g_pool);
+    pq_boundary_kernel<false><<<g_cand, kSelThreads, 0, s>>>(b);
+    pq_boundary_apply_kernel<false><<<g_cand, kSelThreads, 0, s>>>(b);
     if (seed) {
       pq_admit_kernel<true><<<g_dense, 256, 0, s>>>(b);
-      pq_best_kernel<true><<<1, 1, 0, s>>>(b);
-      pq_round_end_kernel<true><<<1, 1, 0, s>>>(b);
+      pq_finish_kernel<true><<<1, kSelThreads, 0, s>>>(b);
     } else {
       pq_admit_kernel<false><<<g_dense, 256, 0, s>>>(b);
-      pq_best_kernel<false><<<1, 1, 0, s>>>(b);
-      pq_round_end_kernel<false><<<1, 1, 0, s>>>(b);
+      pq_finish_kernel<false><<<1, kSelThreads, 0, s>>>(b);
     }
-    cudaMemsetAsync(b.hU, 0, 4 * kNB, s);
-    cudaMemsetAsync(b.hU2, 0, 4 * kNC, s);
     cudaMemsetAsync(b.hkey, 0, 8ull << hs_log2, s);  // the dedup table, for the next round
   };
 
   // ---- set-up: visited set, pool, histograms, dedup table, Zobrist keys; the seeds go through the
   // survivor path into the empty pool (equal seeds kept once, the cap smallest admitted)
-  if (cudaMemsetAsync(b.H, 0xff, 8ull << cfg->H_log2, st) != cudaSuccess) return LABS_ERR_CUDA;
+  if (cudaMemsetAsync(b.H, 0xff, 8ull << cfg->H_log2, st) != cudaSuccess ||
+      cudaMemsetAsync(b.filter, 0, (1ull << f_log2) / 8, st) != cudaSuccess)
+    return LABS_ERR_CUDA;
   if (cudaMemsetAsync(b.hP, 0, 4 * kNB, st) != cudaSuccess || cudaMemsetAsync(b.hP2, 0, 4 * kNC, st) != cudaSuccess ||
       cudaMemsetAsync(b.hU, 0, 4 * kNB, st) != cudaSuccess || cudaMemsetAsync(b.hU2, 0, 4 * kNC, st) != cudaSuccess ||
-      cudaMemsetAsync(b.hkey, 0, 8ull << hs_log2, st) != cudaSuccess ||
-      cudaMemsetAsync(b.popRank, 0, 4 * (size_t)cfg->B, st) != cudaSuccess)
+      cudaMemsetAsync(b.hkey, 0, 8ull << hs_log2, st) != cudaSuccess)
     return LABS_ERR_CUDA;
   pq_ztab_kernel<<<(L + 255) / 256, 256, 0, st>>>(b.ztab, L);
   pq_init_kernel<<<g_pool, 256, 0, st>>>(b);
@@ -1269,8 +1304,25 @@ int launch_pq_refine(labs_ctx* ctx, const labs_pq_cfg* cfg, const uint64_t* seed
 
   // ---- rounds
   const long long max_rounds = (cfg->max_expansions + cfg->B - 1) / cfg->B + 1;
-  const unsigned exp_blocks = (unsigned)std::max(1ll, std::min<long long>((cfg->B + kPqWarps - 1) / kPqWarps,
-                                                                        (long long)ctx->num_sms * 8));
+  ExpandPlan ep;
+  ep.mma = scan_mma_plan(L, 0, L - 1);
+  ep.q = kExpTables;
+  ep.x = ep.q + 2 * ep.mma.q_words;
+  ep.v = ep.x + ep.mma.x_words;
+  ep.words = (ep.v + kMaxL + 1 + 3) / 4 * 4;
+  const size_t exp_smem = sizeof(uint32_t) * (size_t)ep.words * kPqWarps;
+  void (*expand)(PqBufs, ExpandPlan) = nullptr;
+  int per_sm = 0;
+  const int es = by_words((L + 31) >> 5, [&](auto nw) {
+    expand = pq_expand_kernel<decltype(nw)::value>;
+    return cuda_status(cudaFuncSetAttribute(expand, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)exp_smem));
+  });
+  if (es != LABS_OK ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, expand, 32 * kPqWarps, exp_smem) != cudaSuccess || per_sm < 1)
+    return LABS_ERR_CUDA;
+  const long long exp_items = (long long)cfg->B * (1 + 2 * cfg->T_r);
+  const unsigned exp_blocks =
+      (unsigned)std::max(1ll, std::min<long long>((exp_items + kPqWarps - 1) / kPqWarps, (long long)ctx->num_sms * per_sm));
   // Every round issues the same launches with the same arguments (a round's sizes and stop state live
   // in device memory), so one round is captured as a CUDA graph and replayed.
   if (!ctx->capture_stream && cudaStreamCreateWithFlags(&ctx->capture_stream, cudaStreamNonBlocking) != cudaSuccess)
@@ -1278,14 +1330,10 @@ int launch_pq_refine(labs_ctx* ctx, const labs_pq_cfg* cfg, const uint64_t* seed
   if (cudaStreamBeginCapture(ctx->capture_stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return LABS_ERR_CUDA;
   {
     cudaStream_t cs = ctx->capture_stream;
-    pq_round_begin_kernel<<<1, 1, 0, cs>>>(b);
-    pq_select_kernel<true><<<1, kSelThreads, 0, cs>>>(b);
-    pq_gather_kernel<true, false><<<g_pool, 256, 0, cs>>>(b);
-    pq_boundary_kernel<true><<<1, kSelThreads, cand_smem, cs>>>(b);
-    pq_pop_rank_kernel<<<dim3((unsigned)((cfg->B + 255) / 256), kRankChunks), 256, 0, cs>>>(b);
-    pq_pivot_kernel<<<g_piv, 256, 0, cs>>>(b);
-    pq_pmax_kernel<<<1, kSelThreads, 0, cs>>>(b);
-    pq_expand_kernel<<<exp_blocks, 32 * kPqWarps, 0, cs>>>(b, ly);
+    pq_pool_kernel<true><<<g_pool, 256, 0, cs>>>(b, g_pool);
+    pq_boundary_kernel<true><<<g_cand, kSelThreads, 0, cs>>>(b);
+    pq_boundary_apply_kernel<true><<<g_cand, kSelThreads, 0, cs>>>(b);
+    expand<<<exp_blocks, 32 * kPqWarps, exp_smem, cs>>>(b, ep);
     survivor_path(false, cs);
   }
   cudaGraph_t round_graph = nullptr;
@@ -1317,8 +1365,6 @@ int launch_pq_refine(labs_ctx* ctx, const labs_pq_cfg* cfg, const uint64_t* seed
       if (*hstop) break;
     }
   }
-  // the last round may end on the budget without a following begin: settle the stop reason
-  pq_round_begin_kernel<<<1, 1, 0, st>>>(b);
   pq_write_stats_kernel<<<1, 1, 0, st>>>(b, best_E, stats);
   if (cudaMemcpyAsync(best_seq, b.best_seq, 8 * W, cudaMemcpyDeviceToDevice, st) != cudaSuccess) status = LABS_ERR_CUDA;
   if (cudaStreamSynchronize(st) != cudaSuccess) status = LABS_ERR_CUDA;
