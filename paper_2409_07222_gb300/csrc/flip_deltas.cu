@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(32 * kFdWarps, NT <= 2 ? 6 : 4) flip_deltas_ke
         const int o = 16 * (r & 1) + 8 * (r >> 1), m = jl + (lane >> 2) + o + 1;
         if (m > p && m <= L) {
           const int t = (int)acc[0][T][r];
-          out[m - 1] = 4 * ((int)v[m] + (int)v[kMaxL + 1 + m] + L - 2 - ((own >> o & 1u) ? t : -t));
+          out[m - 1] = 4 * ((int)v[m] + L - 2 - ((own >> o & 1u) ? t : -t));
         }
       }
     }
@@ -200,7 +200,7 @@ int launch_flip_deltas(labs_ctx* ctx, const uint64_t* seqs, const int32_t* C, in
           return launch_fd(ctx, flip_deltas_skew_kernel<NC, 2>, seqs, C, L, n, p, fp, dE_out, st);
       return launch_fd(ctx, flip_deltas_skew_kernel<NC, 1>, seqs, C, L, n, p, fp, dE_out, st);
     }
-    fp.words = (fp.z + kMaxL + 1 + 3) / 4 * 4;
+    fp.words = (fp.z + L / 2 + 1 + 3) / 4 * 4;  // v[1 .. L]
     constexpr int kMost = NW / 4 + 1;  // tiles when nothing is fixed
     auto run = [&](auto nt) {
       constexpr int NT = decltype(nt)::value;

@@ -884,17 +884,7 @@ __global__ void __launch_bounds__(32 * kPqWarps, NW <= 8 ? 6 : 4) pq_expand_kern
     __syncwarp();
     if (rot) {
       // rotation: element i is element i + r (mod L); its energy and fingerprint from scratch
-      const int r = rot_shift(L, b.Tr, rot - 1), o = 32 * lane + r;
-      uint32_t y = 0;
-      if (lane < NW) {
-        if (o < L) y = __funnelshift_r(bits[o >> 5], bits[(o >> 5) + 1], o & 31);
-        const int ow = o - L;  // elements past the end come from the start
-        if (ow >= 0)
-          y = __funnelshift_r(bits[ow >> 5], bits[(ow >> 5) + 1], ow & 31);
-        else if (ow > -32)
-          y |= bits[0] << -ow;
-        if (lane == NW - 1) y &= 0xffffffffu >> (32 * NW - L);
-      }
+      const uint32_t y = rotated_word<NW>(bits, L, rot_shift(L, b.Tr, rot - 1));
       if (lane < kBitWords) rw[lane] = y;
       __syncwarp();
       const int e = energy_words<NW>(rw, L);
@@ -935,7 +925,7 @@ __global__ void __launch_bounds__(32 * kPqWarps, NW <= 8 ? 6 : 4) pq_expand_kern
         const int o = 16 * (r & 1) + 8 * (r >> 1), m = jl + o + 1;
         if (m <= L) {
           const int tm = (int)acc[0][T][r];
-          oe[m - 1] = E + 4 * ((int)v[m] + (int)v[kMaxL + 1 + m] + L - 2 - ((own >> o & 1u) ? tm : -tm));
+          oe[m - 1] = E + 4 * ((int)v[m] + L - 2 - ((own >> o & 1u) ? tm : -tm));
           of[m - 1] = fp ^ b.ztab[m - 1];
         }
       }
@@ -1309,7 +1299,7 @@ int launch_pq_refine(labs_ctx* ctx, const labs_pq_cfg* cfg, const uint64_t* seed
   ep.q = kExpTables;
   ep.x = ep.q + 2 * ep.mma.q_words;
   ep.v = ep.x + ep.mma.x_words;
-  ep.words = (ep.v + kMaxL + 1 + 3) / 4 * 4;
+  ep.words = (ep.v + L / 2 + 1 + 3) / 4 * 4;  // v[1 .. L]
   const size_t exp_smem = sizeof(uint32_t) * (size_t)ep.words * kPqWarps;
   void (*expand)(PqBufs, ExpandPlan) = nullptr;
   int per_sm = 0;

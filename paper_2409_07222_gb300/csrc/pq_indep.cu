@@ -5,34 +5,41 @@
 // GB300 mapping.  One warp per candidate; a candidate's state lives in HBM:
 //   arena  -- every pushed node as a 16-byte record (E, link, fp); the survivors of one pop are appended
 //             as one run, in no particular order;
-//   runs   -- a binary heap over the runs keyed by each run's smallest (E, fp): its top is the queue
+//   runs   -- a 32-ary heap over the runs keyed by each run's smallest (E, fp): its top is the queue
 //             minimum.  A pop takes that node out of its run (the run's last node fills the gap), finds
-//             the run's new smallest by one warp-wide rescan (at most L + 2 T_r records) and sifts down;
-//             a new run is one sift-up.  Keys (E, fp) are distinct in a queue (the visited set admits a
-//             sequence once), so the pop order is that of the sequential definition;
+//             the run's new smallest by one warp-wide rescan (at most L + 2 T_r records) and sifts down, the
+//             32 children of a level read and ranked by the warp at once; a new run is one sift-up.  Keys
+//             (E, fp) are distinct in a queue (the visited set admits a sequence once), so the pop order is
+//             that of the sequential definition;
 //   pivots -- the sequence of every popped node (a node is stored as its pivot and column, and is made
-//             into a sequence only when popped), with its correlation table and P_m, so that a flip
-//             child starts from its parent's by one O(L) update;
-//   H      -- the candidate's visited set (open addressing, cleared per candidate).
-// A pop scans all L single flips (the dp4a tiles of labs_core.cuh); each neighbour is one
-// insert-if-absent into H, a survivor being one whose key was absent.  With T_r > 0 the pivot's 2 T_r
-// rotations follow the flips (a rotation equal to a flip child or to an earlier rotation finds its key in
-// H and is dropped, as the ordered dedup keeps the smaller column).  Memory per resident warp is about
-// max_expansions x ((L + 2 T_r) x 16 B + 4 L B) + 2^H_log2 x 8 B: HBM capacity, not bandwidth, is what
-// this design spends.
+//             into a sequence only when popped);
+//   H      -- the candidate's visited set (open addressing, cleared per candidate), where it is needed: without
+//             rotations every node ever pushed is the seed or a neighbour of a popped pivot, so a neighbour p^i
+//             of the pivot p was visited exactly if some earlier pivot differs from p in i and one other
+//             position, or in i alone (the seed is the first pivot).  Up to kPairPops pops the pivots
+//             themselves are compared -- a few hundred coalesced words a pop instead of L inserts at random
+//             places of a set that lies in DRAM.
+// A pop forms its correlations and every neighbour's sum from the sequence alone (scan_mma.cuh: some 2,000 warp
+// instructions, less than keeping tables per pivot would move); each neighbour is one insert-if-absent into H, a
+// survivor being one whose key was absent.  With T_r > 0 the pivot's 2 T_r rotations follow the flips (a
+// rotation equal to a flip child or to an earlier rotation finds its key in H and is dropped, as the ordered
+// dedup keeps the smaller column).  Memory per resident warp is about max_expansions x (L + 2 T_r) x 16 B, and
+// 2^H_log2 x 8 B where H is needed: HBM capacity, not bandwidth, is what this design spends.
 #include <algorithm>
 
-#include "labs_core.cuh"
 #include "labs_internal.h"
+#include "scan_mma.cuh"
 
 namespace labsg {
 namespace {
 
 constexpr int kIWarps = 4;
-constexpr int kIM = 8;
 constexpr uint64_t kEmpty = ~0ull;
 constexpr int kProbeLimit = 1 << 20;
 constexpr int kMaxTr = 64;  // rotations per side (the library's bound on T_r)
+// Pops up to which the pivots are compared pairwise: n / 2 pivots of 64 bytes a pop against L random 32-byte
+// sectors read and written, and a set that is cleared first.
+constexpr long long kPairPops = 1024;
 
 struct Node {  // one queue record: 16 bytes
   int32_t E;
@@ -60,9 +67,7 @@ struct IndepArgs {
   // per-slot workspaces (slot = resident warp)
   Node* arena;
   RunHead* heap;
-  uint64_t* pivots;
-  uint32_t* tables;  // per popped pivot: its C table (2 NG words of int16 pairs) and P_m (ceil(L/2) words)
-  int tab_words;
+  uint64_t* pivots;  // [W][max_exp] a slot
   uint64_t* H;
   const uint64_t* ztab;
   unsigned long long* counter;
@@ -134,29 +139,21 @@ __device__ __forceinline__ void flip_bits(const uint32_t* src, int col, uint32_t
   __syncwarp();
 }
 
+template <int NW>
 __device__ __forceinline__ void rotate_bits(const uint32_t* src, int L, int r, uint32_t* dst) {
-  const int lane = lane_id();
-  for (int w = 0; w < kBitWords; w++) {
-    const int i = 32 * w + lane;
-    int bit = 0;
-    if (i < L) {
-      int j = i + r;
-      if (j >= L) j -= L;
-      bit = (src[j >> 5] >> (j & 31)) & 1u;
-    }
-    const unsigned word = __ballot_sync(kFull, bit);
-    if (lane == 0) dst[w] = word;
-  }
+  const uint32_t y = rotated_word<NW>(src, L, r);
+  if (lane_id() < kBitWords) dst[lane_id()] = y;
   __syncwarp();
 }
 
-__device__ __forceinline__ void words_to_bits(const uint64_t* src, int L, uint32_t* dst) {
+// (words of a sequence `stride` apart)
+__device__ __forceinline__ void words_to_bits(const uint64_t* src, int L, uint32_t* dst, long long stride = 1) {
   const int lane = lane_id();
   if (lane < kBitWords) {
     const int W32 = (L + 31) >> 5;
     uint32_t v = 0;
     if (lane < W32) {
-      const uint64_t x = src[lane >> 1];
+      const uint64_t x = src[(lane >> 1) * stride];
       v = (lane & 1) ? (uint32_t)(x >> 32) : (uint32_t)x;
       const int rem = L - 32 * lane;
       if (rem < 32) v &= (1u << rem) - 1u;
@@ -166,18 +163,9 @@ __device__ __forceinline__ void words_to_bits(const uint64_t* src, int L, uint32
   __syncwarp();
 }
 
-__device__ __forceinline__ void bits_to_words(const uint32_t* src, int L, uint64_t* dst) {
+__device__ __forceinline__ void bits_to_words(const uint32_t* src, int L, uint64_t* dst, long long stride = 1) {
   const int lane = lane_id();
-  if (lane < ((L + 63) >> 6)) dst[lane] = (uint64_t)src[2 * lane] | ((uint64_t)src[2 * lane + 1] << 32);
-}
-
-__device__ __forceinline__ int energy_bits(const uint32_t* bits, int L) {
-  int e = 0;
-  for (int k = lane_id() + 1; k < L; k += 32) {
-    const int c = corr_lag(bits, L, k);
-    e += c * c;
-  }
-  return warp_sum_i32(e);
+  if (lane < ((L + 63) >> 6)) dst[lane * stride] = (uint64_t)src[2 * lane] | ((uint64_t)src[2 * lane + 1] << 32);
 }
 
 __device__ __forceinline__ uint64_t fp_bits(const uint32_t* bits, int L, const uint64_t* ztab) {
@@ -200,43 +188,55 @@ __device__ __forceinline__ void warp_argmin(int bE, uint64_t bf, int bi, int& E,
   idx = __shfl_sync(kFull, bi, __ffs(who) - 1);
 }
 
-// Smallest (E, fp) of arena nodes [begin, end) (non-empty, keys distinct) and its index, on every lane.
+// Smallest (E, fp) of arena nodes [begin, end) (non-empty, keys distinct) and its index, on every lane; eight
+// records a lane in flight.
 __device__ __forceinline__ void run_min(const Node* arena, int begin, int end, int& E, uint64_t& fp, int& idx) {
   int bE = INT32_MAX, bi = -1;
   uint64_t bf = ~0ull;
-  for (int i = begin + lane_id(); i < end; i += 32) {
-    const Node x = arena[i];
-    if (kless(x.E, x.fp, bE, bf)) {
-      bE = x.E;
-      bf = x.fp;
-      bi = i;
+  for (int i0 = begin + lane_id(); i0 - lane_id() < end; i0 += 256) {
+    int4 x[8];
+#pragma unroll
+    for (int j = 0; j < 8; j++)
+      x[j] = i0 + 32 * j < end ? reinterpret_cast<const int4*>(arena)[i0 + 32 * j] : make_int4(INT32_MAX, 0, -1, -1);
+#pragma unroll
+    for (int j = 0; j < 8; j++) {
+      const uint64_t f = ((uint64_t)(uint32_t)x[j].w << 32) | (uint32_t)x[j].z;
+      if (kless(x[j].x, f, bE, bf)) {
+        bE = x[j].x;
+        bf = f;
+        bi = i0 + 32 * j;
+      }
     }
   }
   warp_argmin(bE, bf, bi, E, fp, idx);
 }
 
-// Per-warp shared memory.
-struct __align__(16) IndepSmem {
-  ScanSmem s;
-  uint32_t pbits[kBitWords];  // the pivot
-  uint32_t cbits[kBitWords];  // a child
-  int16_t P[kMaxL];  // P_m of the pivot's neighbours
-  uint32_t xb[kBitWords];
-  int n_surv;
+// Shared memory of one warp, in 32-bit words from its slab's start.
+struct IndepPlan {
+  ScanMmaPlan mma;
+  int q, x, v, words;
 };
+constexpr int kInP = 0, kInC = 24, kInClass = 48, kInRev = kInClass + 2 * kClassWords, kInTables = kInRev + 2 * kClassWords;
 
-__global__ void __launch_bounds__(32 * kIWarps) pq_indep_kernel(IndepArgs a, Layout ly) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  IndepSmem& S = reinterpret_cast<IndepSmem*>(smem_raw)[threadIdx.x >> 5];
-  ScanSmem& sm = S.s;
+// Seven blocks an SM hold 28 candidates (72 registers a thread, 7.7 KB of slab a warp at L = 451).
+template <int NW, bool PAIRS>
+__global__ void __launch_bounds__(32 * kIWarps, 7) pq_indep_kernel(IndepArgs a, IndepPlan ip) {
+  constexpr int NT = (NW + 3) / 4;
+  extern __shared__ __align__(16) uint32_t in_smem[];
+  uint32_t* slab = in_smem + (size_t)(threadIdx.x >> 5) * ip.words;
+  uint32_t *pbits = slab + kInP, *cbits = slab + kInC, *cw = slab + kInClass, *rw = slab + kInRev;
+  uint32_t *qt = slab + ip.q, *xt = slab + ip.x;
+  int16_t* v = reinterpret_cast<int16_t*>(slab + ip.v);
   const int lane = lane_id();
-  const long long slot = (long long)blockIdx.x * kIWarps + (threadIdx.x >> 5);
-  Node* arena = a.arena + slot * a.arena_cap;
-  RunHead* heap = a.heap + slot * a.heap_cap;
-  uint64_t* pivots = a.pivots + slot * a.max_exp * a.W;
-  uint32_t* tables = a.tables + slot * a.max_exp * a.tab_words;
-  uint64_t* H = a.H + slot * (1ll << a.H_log2);
+  const int slot = blockIdx.x * kIWarps + (threadIdx.x >> 5);
+  Node* const arena = a.arena + slot * a.arena_cap;
+  RunHead* const heap = a.heap + slot * a.heap_cap;
+  uint64_t* const pivots = a.pivots + slot * a.max_exp * a.W;
+  uint64_t* const H = PAIRS ? nullptr : a.H + ((long long)slot << a.H_log2);
   const long long hslots = 1ll << a.H_log2;
+  const uint32_t* const xs[1] = {xt};
+  for (int i = lane; i < ip.words; i += 32) slab[i] = 0u;
+  __syncwarp();
 
   while (true) {
     unsigned long long cand = 0;
@@ -245,21 +245,23 @@ __global__ void __launch_bounds__(32 * kIWarps) pq_indep_kernel(IndepArgs a, Lay
     if ((long long)cand >= a.n) break;
     int err = 0;
     // ---- reset the visited set, seed the queue
-    for (long long t = lane; t < hslots; t += 32) H[t] = kEmpty;
+    if (!PAIRS)
+      for (long long t = lane; t < hslots / 2; t += 32) reinterpret_cast<ulonglong2*>(H)[t] = make_ulonglong2(kEmpty, kEmpty);
     __threadfence_block();
     __syncwarp();
-    words_to_bits(a.seeds + cand * a.W, a.L, S.pbits);
-    int bestE = energy_bits(S.pbits, a.L);
-    uint64_t bestfp = fp_bits(S.pbits, a.L, a.ztab);
+    words_to_bits(a.seeds + cand * a.W, a.L, pbits);
+    int bestE = energy_words<NW>(pbits, a.L);
+    uint64_t bestfp = fp_bits(pbits, a.L, a.ztab);
     bool has_empty = bestfp == kEmpty;
     if (lane == 0) {
-      if (!has_empty) hs_insert(H, a.H_log2, bestfp, &err);
+      if (!PAIRS && !has_empty) hs_insert(H, a.H_log2, bestfp, &err);
       arena[0] = Node{bestE, -1, bestfp};
       heap[0] = RunHead{bestE, 0, bestfp, 1, 0};
     }
-    bits_to_words(S.pbits, a.L, a.best_seqs + cand * a.W);
+    bits_to_words(pbits, a.L, a.best_seqs + cand * a.W);
     __syncwarp();
-    long long heap_n = 1, top = 1, exps = 0, u = 0, surv = 0, improvements = 0, h_size = 1;
+    // all counts stay below 2^31: at most 2^21 pops of 704 children
+    int heap_n = 1, top = 1, exps = 0, u = 0, improvements = 0;
     int stop = 0;
     while (true) {
       if (exps >= a.max_exp) stop = 1;
@@ -267,171 +269,168 @@ __global__ void __launch_bounds__(32 * kIWarps) pq_indep_kernel(IndepArgs a, Lay
       else if (a.T_u > 0 && u >= a.T_u) stop = 3;
       if (stop || err) break;
       // ---- pop: the top run's smallest node; the run's last node fills its place, the run's new
-      //      smallest by a rescan (warp), then the sift-down (lane 0)
+      //      smallest by a rescan, then the sift-down
       RunHead h = heap[0];
       const Node nd = arena[h.cur];
+      const Node last = arena[h.end - 1];
       const int pE = nd.E, plink = nd.link;
       const uint64_t pfp = nd.fp;
       __syncwarp();
-      if (lane == 0 && h.cur != h.end - 1) arena[h.cur] = arena[h.end - 1];
+      if (lane == 0 && h.cur != h.end - 1) arena[h.cur] = last;
       __syncwarp();
       h.end--;
-      const bool alive = h.end > h.begin;
-      if (alive) run_min(arena, h.begin, h.end, h.E, h.fp, h.cur);
-      if (lane == 0) {
-        if (!alive) {
-          heap_n--;
-          h = heap[heap_n];
-        }
-        if (heap_n > 0) {
-          long long i = 0;
-          while (true) {
-            const long long l = 2 * i + 1, r = l + 1;
-            if (l >= heap_n) break;
-            long long c = l;
-            if (r < heap_n && kless(heap[r].E, heap[r].fp, heap[l].E, heap[l].fp)) c = r;
-            if (!kless(heap[c].E, heap[c].fp, h.E, h.fp)) break;
-            heap[i] = heap[c];
-            i = c;
-          }
-          heap[i] = h;
-        }
+      if (h.end > h.begin) {
+        run_min(arena, h.begin, h.end, h.E, h.fp, h.cur);
+      } else {
+        heap_n--;
+        h = heap[heap_n];
       }
-      heap_n = __shfl_sync(kFull, heap_n, 0);
+      if (heap_n > 0) {
+        int i = 0;
+        while (true) {
+          const int c = 32 * i + 1 + lane;  // the level's children, one a lane
+          RunHead ch{INT32_MAX, 0, ~0ull, 0, 0};
+          if (c < heap_n) ch = heap[c];
+          int E;
+          uint64_t fp;
+          int who;
+          warp_argmin(ch.E, ch.fp, c < heap_n ? lane : -1, E, fp, who);
+          if (!(kless(E, fp, h.E, h.fp))) break;
+          if (lane == who) heap[i] = ch;
+          i = 32 * i + 1 + who;
+        }
+        __syncwarp();
+        if (lane == 0) heap[i] = h;
+      }
       // ---- the pivot's sequence: the seed, or the child `col` of an earlier pivot
       if (plink < 0) {
-        words_to_bits(a.seeds + cand * a.W, a.L, S.pbits);
+        words_to_bits(a.seeds + cand * a.W, a.L, pbits);
       } else {
-        words_to_bits(pivots + (long long)(plink >> 10) * a.W, a.L, S.cbits);
+        words_to_bits(pivots + (plink >> 10), a.L, cbits, a.max_exp);
         const int col = plink & 1023;
         if (col < a.L)
-          flip_bits(S.cbits, col, S.pbits);
+          flip_bits(cbits, col, pbits);
         else
-          rotate_bits(S.cbits, a.L, rshift(a.L, a.Tr, col - a.L), S.pbits);
+          rotate_bits<NW>(cbits, a.L, rshift(a.L, a.Tr, col - a.L), pbits);
       }
-      bits_to_words(S.pbits, a.L, pivots + exps * a.W);
-      // ---- the pivot's correlation table and P_m: a flip child's from its parent's (kept with every
-      //      popped pivot) by one O(L) update, the seed's and a rotation's from scratch
-      if (lane == 0) S.n_surv = 0;
-      bool fast;
-      uint32_t* ptab = tables + exps * a.tab_words;
-      const int pcol = plink & 1023;
-      if (plink >= 0 && pcol < a.L) {
-        const uint32_t* par = tables + (long long)(plink >> 10) * a.tab_words;
-        uint32_t* C16w = reinterpret_cast<uint32_t*>(sm.C16);
-        uint32_t* Pw = reinterpret_cast<uint32_t*>(S.P);
-        for (int w = lane; w < 2 * ly.NG; w += 32) C16w[w] = par[w];
-        for (int w = lane; w < (a.L + 1) / 2; w += 32) Pw[w] = par[2 * ly.NG + w];
-        for (int w = lane; w < kBitWords; w += 32) sm.bits[w] = S.cbits[w];  // the parent
+      bits_to_words(pbits, a.L, pivots + exps, a.max_exp);
+      if (PAIRS) {  // cbits: the neighbours visited before
+        if (lane < kBitWords) cbits[lane] = 0u;
         __syncwarp();
-        build_bytes(sm, ly);
-        // P_m of the child: flipping f changes the product s_f s_{2m-f} of every m != f (pads: 0)
-        const int f = pcol + 1;
-        const uint8_t* Fc = reinterpret_cast<const uint8_t*>(sm.fwd);
-        const int qf = pos_q(ly, f), sf = (int)Fc[qf] - 1;
-        for (int m = lane + 1; m <= a.L; m += 32)
-          if (m != f) S.P[m - 1] = (int16_t)(S.P[m - 1] - 2 * sf * ((int)Fc[max(2 * pos_q(ly, m) - qf, 0)] - 1));
-        __syncwarp();
-        table_update(sm, ly, f, &fast);
-        if (lane == 0) flip_position(sm, ly, f);
-        __syncwarp();
-      } else {
-        for (int w = lane; w < kBitWords; w += 32) sm.bits[w] = S.pbits[w];
-        __syncwarp();
-        build_table(sm, ly);
-        fast = pack_c8(sm, ly);
-        build_bytes(sm, ly);
-        p_all(sm, ly, S.xb, S.cbits, S.P);
-      }
-      const int SC = table_sum(sm, ly);
-      {
-        const uint32_t* C16w = reinterpret_cast<const uint32_t*>(sm.C16);
-        const uint32_t* Pw = reinterpret_cast<const uint32_t*>(S.P);
-        for (int w = lane; w < 2 * ly.NG; w += 32) ptab[w] = C16w[w];
-        for (int w = lane; w < (a.L + 1) / 2; w += 32) ptab[2 * ly.NG + w] = Pw[w];
-      }
-      Node* run = arena + top;
-      const int link0 = (int)(exps << 10);
-      int rE = INT32_MAX, ri = -1;  // this lane's smallest survivor (the run's head comes from these)
-      uint64_t rf = ~0ull;
-      for (int base = 0; base < ly.n_tiles; base += 32) {
-        const int tau = base + lane;
-        if (tau < ly.n_tiles) {
-          int cls, q0;
-          tile_of(ly, tau, cls, q0);
-          int acc[kIM];
-          if (fast)
-            scan_tile<kIM, false>(sm, ly, cls, q0, acc);
-          else
-            scan_tile<kIM, true>(sm, ly, cls, q0, acc);
-          // the tile's Delta E and fingerprints, then an insert-if-absent of each neighbour into the
-          // visited set, the first compare-and-swap of all of them in flight at once: a neighbour is a
-          // survivor when its key was absent.  Inserting while other neighbours are still tested changes
-          // none of their answers: their keys differ, and inserts only fill empty slots, which no probe
-          // sequence of a present key crosses.
-          int dv[kIM], mv[kIM];
-          uint64_t fv[kIM];
-          unsigned long long hv[kIM];
+        constexpr int W = (NW + 1) / 2;
+        for (int q0 = 0; q0 < exps; q0 += 64) {
+          uint64_t x[2][W];
 #pragma unroll
-          for (int j = 0; j < kIM; j++) {
-            const SlotInfo si = slot_info(ly, cls, q0 + j);
-            mv[j] = si.active ? si.m : 0;
-            dv[j] = si.active ? finish_delta(sm, ly, cls, q0 + j, si, acc[j], SC, S.P[si.m - 1]) : 0;
-            fv[j] = si.active ? pfp ^ a.ztab[si.m - 1] : kEmpty;
-          }
+          for (int i = 0; i < 2; i++)
 #pragma unroll
-          for (int j = 0; j < kIM; j++)
-            hv[j] = (mv[j] && fv[j] != kEmpty)
-                        ? atomicCAS(reinterpret_cast<unsigned long long*>(&H[hs_home(fv[j], a.H_log2)]),
-                                    (unsigned long long)kEmpty, fv[j])
-                        : (unsigned long long)kEmpty;
+            for (int w = 0; w < W; w++) x[i][w] = pivots[w * a.max_exp + min(q0 + 32 * i + lane, exps - 1)];
 #pragma unroll
-          for (int j = 0; j < kIM; j++) {
-            if (!mv[j]) continue;
-            bool fresh;
-            if (fv[j] == kEmpty) {
-              fresh = !has_empty;
-              has_empty = true;
-            } else if (hv[j] == kEmpty || hv[j] == fv[j]) {
-              fresh = hv[j] == kEmpty;
-            } else {
-              fresh = hs_add_from(H, a.H_log2, fv[j], hs_home(fv[j], a.H_log2), &err);
+          for (int i = 0; i < 2; i++) {
+            int d = 0;
+#pragma unroll
+            for (int w = 0; w < W; w++) {
+              x[i][w] ^= reinterpret_cast<const uint64_t*>(pbits)[w];
+              d += __popcll(x[i][w]);
             }
-            if (fresh) {
-              const int k = atomicAdd(&S.n_surv, 1);
-              run[k] = Node{pE + dv[j], link0 | (mv[j] - 1), fv[j]};
-              if (kless(pE + dv[j], fv[j], rE, rf)) {
-                rE = pE + dv[j];
-                rf = fv[j];
-                ri = (int)top + k;
+            if (d <= 2) {  // (an earlier pivot differs in one position at least)
+#pragma unroll
+              for (int w = 0; w < W; w++) {
+                if (uint32_t lo = (uint32_t)x[i][w]) atomicOr(&cbits[2 * w], lo);
+                if (uint32_t hi = (uint32_t)(x[i][w] >> 32)) atomicOr(&cbits[2 * w + 1], hi);
               }
             }
           }
+        }
+        __syncwarp();
+      }
+      // ---- correlations, V and the neighbours' sums
+      corr_words<NW>(pbits, pbits, a.L, [&](int d, int cd) {
+        if (d >= 1 && d < a.L) put_q(qt, ip.mma, d, cd);
+      });
+      put_x(xt, pbits, a.L);
+      split_classes(pbits, cw);
+      self_convolution<(NW + 1) / 2>(cw, rw, a.L, v);
+      float acc[1][NT][4];
+      scan_mma<1, NT>(qt, xs, ip.mma, a.L, acc);
+      Node* run = arena + top;
+      const int link0 = exps << 10;
+      int nu = 0;
+      int rE = INT32_MAX, ri = -1;  // this lane's smallest survivor (the run's head comes from these)
+      uint64_t rf = ~0ull;
+      // H: an insert-if-absent of each neighbour into the visited set, the first compare-and-swap of two tiles'
+      // in flight at once: a neighbour is a survivor when its key was absent.  Inserting while other
+      // neighbours are still tested changes none of their answers: their keys differ, and inserts only fill
+      // empty slots, which no probe sequence of a present key crosses.
+#pragma unroll
+      for (int T0 = 0; T0 < NT; T0 += 2) {
+        unsigned long long hv[8];
+        uint64_t fv[8];
+#pragma unroll
+        for (int i = 0; i < 8; i++) {
+          const int T = T0 + (i >> 2), m = 128 * T + 32 * (lane & 3) + (lane >> 2) + 16 * (i & 1) + 8 * ((i >> 1) & 1) + 1;
+          fv[i] = kEmpty;
+          hv[i] = kEmpty;
+          if (T < NT && m <= a.L) {
+            fv[i] = pfp ^ a.ztab[m - 1];
+            if (!PAIRS && fv[i] != kEmpty)
+              hv[i] = atomicCAS(reinterpret_cast<unsigned long long*>(&H[hs_home(fv[i], a.H_log2)]), (unsigned long long)kEmpty, fv[i]);
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < 8; i++) {
+          const int T = T0 + (i >> 2);
+          if (T >= NT) break;
+          const int jl = 128 * T + 32 * (lane & 3) + (lane >> 2) + 16 * (i & 1) + 8 * ((i >> 1) & 1), m = jl + 1;
+          bool fresh = false;
+          if (m <= a.L) {
+            if (PAIRS) {
+              fresh = !((cbits[jl >> 5] >> (jl & 31)) & 1u);
+            } else if (fv[i] == kEmpty) {
+              fresh = !has_empty;
+              has_empty = true;
+            } else if (hv[i] == kEmpty || hv[i] == fv[i]) {
+              fresh = hv[i] == kEmpty;
+            } else {
+              fresh = hs_add_from(H, a.H_log2, fv[i], hs_home(fv[i], a.H_log2), &err);
+            }
+          }
+          const unsigned who = __ballot_sync(kFull, fresh);
+          if (fresh) {
+            const int tm = (int)acc[0][T][i & 3];
+            const int E = pE + 4 * ((int)v[m] + a.L - 2 - ((pbits[jl >> 5] >> (jl & 31) & 1u) ? tm : -tm));
+            const int k = nu + __popc(who & ((1u << lane) - 1u));
+            run[k] = Node{E, link0 | jl, fv[i]};
+            if (kless(E, fv[i], rE, rf)) {
+              rE = E;
+              rf = fv[i];
+              ri = top + k;
+            }
+          }
+          nu += __popc(who);
         }
       }
       has_empty = __any_sync(kFull, has_empty);
       // ---- the rotations, after the flips: one equal to a flip child or to an earlier rotation finds
       //      its key in the visited set (the same sequence; the smaller column is kept)
-      for (int c = 0; c < 2 * a.Tr; c++) {
-        rotate_bits(S.pbits, a.L, rshift(a.L, a.Tr, c), S.cbits);
-        const int e = energy_bits(S.cbits, a.L);
-        const uint64_t hf = fp_bits(S.cbits, a.L, a.ztab);
-        if (lane == 0) {
-          if (hs_add(H, a.H_log2, hf, has_empty, &err)) {
-            const int k = S.n_surv++;
-            run[k] = Node{e, link0 | (a.L + c), hf};
-            if (kless(e, hf, rE, rf)) {
-              rE = e;
-              rf = hf;
-              ri = (int)top + k;
-            }
+      for (int c = 0; c < (PAIRS ? 0 : 2 * a.Tr); c++) {
+        rotate_bits<NW>(pbits, a.L, rshift(a.L, a.Tr, c), cbits);
+        const int e = energy_words<NW>(cbits, a.L);
+        const uint64_t hf = fp_bits(cbits, a.L, a.ztab);
+        bool fresh = false;
+        if (lane == 0 && hs_add(H, a.H_log2, hf, has_empty, &err)) {
+          fresh = true;
+          run[nu] = Node{e, link0 | (a.L + c), hf};
+          if (kless(e, hf, rE, rf)) {
+            rE = e;
+            rf = hf;
+            ri = top + nu;
           }
         }
-        __syncwarp();
+        nu += __shfl_sync(kFull, (int)fresh, 0);
       }
       has_empty = __any_sync(kFull, has_empty);
       err = __reduce_or_sync(kFull, err);
-      const int nu = S.n_surv;
+      __syncwarp();
       // ---- best, statistics, the new run
       int E0 = INT32_MAX, i0 = 0;
       uint64_t fp0 = 0;
@@ -441,43 +440,43 @@ __global__ void __launch_bounds__(32 * kIWarps) pq_indep_kernel(IndepArgs a, Lay
         bestfp = fp0;
         const int col = arena[i0].link & 1023;
         if (col < a.L)
-          flip_bits(S.pbits, col, S.cbits);
+          flip_bits(pbits, col, cbits);
         else
-          rotate_bits(S.pbits, a.L, rshift(a.L, a.Tr, col - a.L), S.cbits);
-        bits_to_words(S.cbits, a.L, a.best_seqs + cand * a.W);
+          rotate_bits<NW>(pbits, a.L, rshift(a.L, a.Tr, col - a.L), cbits);
+        bits_to_words(cbits, a.L, a.best_seqs + cand * a.W);
         improvements++;
         u = 0;
       } else {
         u++;
       }
-      if (nu > 0 && lane == 0) {  // push the run: sift up
-        const RunHead nh{E0, i0, fp0, (int)(top + nu), (int)top};
-        long long i = heap_n;
+      if (nu > 0) {  // push the run: sift up
+        const RunHead nh{E0, i0, fp0, top + nu, top};
+        int i = heap_n;
         while (i > 0) {
-          const long long pp = (i - 1) >> 1;
-          if (!kless(nh.E, nh.fp, heap[pp].E, heap[pp].fp)) break;
-          heap[i] = heap[pp];
+          const int pp = (i - 1) >> 5;
+          const RunHead par = heap[pp];
+          if (!kless(nh.E, nh.fp, par.E, par.fp)) break;
+          __syncwarp();
+          if (lane == 0) heap[i] = par;
           i = pp;
         }
-        heap[i] = nh;
+        if (lane == 0) heap[i] = nh;
+        heap_n++;
       }
-      if (nu > 0) heap_n++;
-      top += nu;
-      surv += nu;
-      h_size += nu;
+      top += nu;  // the seed and every survivor: the visited set's size
       exps++;
       __syncwarp();
-      if (h_size * 4 > hslots * 3) err = 1;  // keep the visited set below 3/4 load
+      if ((long long)top * 4 > hslots * 3) err = 1;  // keep the visited set below 3/4 load
     }
     if (lane == 0) {
       a.best_E[cand] = bestE;
       labs_pq_stats st{};
       st.expansions = exps;
       st.rounds = exps;
-      st.survivors = surv;
-      st.admitted = surv;
+      st.survivors = top - 1;
+      st.admitted = top - 1;
       st.evicted = 0;
-      st.h_size = h_size;
+      st.h_size = top;
       st.improvements = improvements;
       st.best_fp = bestfp;
       st.stop_reason = err ? 0 : stop;
@@ -499,8 +498,6 @@ int launch_pq_independent(labs_ctx* ctx, const labs_pq_indep_cfg* cfg, const uin
                           uint64_t* best_seqs, int32_t* best_E, labs_pq_stats* stats, cudaStream_t st) {
   if (n == 0) return LABS_OK;
   const int L = cfg->L, W = (L + 63) / 64;
-  Layout ly;
-  if (!make_layout(ly, L, 0, 0, kIM)) return LABS_ERR_INVALID_ARG;
   IndepArgs a{};
   a.L = L;
   a.W = W;
@@ -517,19 +514,34 @@ int launch_pq_independent(labs_ctx* ctx, const labs_pq_indep_cfg* cfg, const uin
   a.best_E = best_E;
   a.stats = stats;
   // resident warps: as many slots as the memory budget allows, at most one per candidate
-  a.tab_words = 2 * ly.NG + (L + 1) / 2;
-  const size_t per_slot = (size_t)a.arena_cap * sizeof(Node) + (size_t)a.heap_cap * sizeof(RunHead) +
-                          (size_t)a.max_exp * W * 8 + (size_t)a.max_exp * a.tab_words * 4 + (8ull << a.H_log2);
+  const bool pairs = cfg->T_r == 0 && a.max_exp <= kPairPops;
+  const size_t base_slot =
+      (size_t)a.arena_cap * sizeof(Node) + (size_t)a.heap_cap * sizeof(RunHead) + (size_t)a.max_exp * W * 8;
+  const size_t per_slot = base_slot + (pairs ? 0 : 8ull << a.H_log2);
+  // the stated need of one block (records, run heads, pivots with 4 L B of tables each, the visited set) must fit,
+  // although less is allocated
+  const size_t stated_slot = base_slot + (size_t)a.max_exp * 4 * (size_t)L + (8ull << a.H_log2);
+  const size_t budget = cfg->max_workspace_bytes > 0 ? (size_t)cfg->max_workspace_bytes : ((size_t)64 << 30);
   if (cfg->T_r > kMaxTr) return LABS_ERR_INVALID_ARG;
-  const size_t smem = sizeof(IndepSmem) * kIWarps;
-  if (cudaFuncSetAttribute(pq_indep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return LABS_ERR_CUDA;
+  if (budget / (stated_slot * kIWarps) < 1) return LABS_ERR_NOMEM;
+  IndepPlan ip;
+  ip.mma = scan_mma_plan(L, 0, L - 1);
+  ip.q = kInTables;
+  ip.x = ip.q + 2 * ip.mma.q_words;
+  ip.v = ip.x + ip.mma.x_words;
+  ip.words = (ip.v + L / 2 + 1 + 3) / 4 * 4;  // v[1 .. L]
+  const size_t smem = sizeof(uint32_t) * (size_t)ip.words * kIWarps;
+  void (*kern)(IndepArgs, IndepPlan) = nullptr;
+  const int ks = by_words((L + 31) >> 5, [&](auto nw) {
+    constexpr int NW = decltype(nw)::value;
+    kern = pairs ? pq_indep_kernel<NW, true> : pq_indep_kernel<NW, false>;
+    return cuda_status(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  });
   int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pq_indep_kernel, 32 * kIWarps, smem) != cudaSuccess ||
+  if (ks != LABS_OK || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * kIWarps, smem) != cudaSuccess ||
       per_sm < 1)
     return LABS_ERR_CUDA;
   long long blocks = std::min<long long>((long long)per_sm * ctx->num_sms, ((long long)n + kIWarps - 1) / kIWarps);
-  const size_t budget = cfg->max_workspace_bytes > 0 ? (size_t)cfg->max_workspace_bytes : ((size_t)64 << 30);
   blocks = std::min<long long>(blocks, (long long)(budget / (per_slot * kIWarps)));
   if (blocks < 1) return LABS_ERR_NOMEM;
   const size_t slots = (size_t)blocks * kIWarps;
@@ -540,8 +552,7 @@ int launch_pq_independent(labs_ctx* ctx, const labs_pq_indep_cfg* cfg, const uin
     return o;
   };
   const size_t oA = take(slots * (size_t)a.arena_cap * sizeof(Node)), oHp = take(slots * (size_t)a.heap_cap * sizeof(RunHead));
-  const size_t oP = take(slots * (size_t)a.max_exp * W * 8), oH = take(slots * (8ull << a.H_log2));
-  const size_t oT = take(slots * (size_t)a.max_exp * a.tab_words * 4);
+  const size_t oP = take(slots * (size_t)a.max_exp * W * 8), oH = take(pairs ? 0 : slots * (8ull << a.H_log2));
   const size_t oZ = take(8 * (size_t)L), oC = take(8);
   char* base = static_cast<char*>(ws_get(ctx, kWsPqIndep, off));
   if (!base) return LABS_ERR_NOMEM;
@@ -549,12 +560,11 @@ int launch_pq_independent(labs_ctx* ctx, const labs_pq_indep_cfg* cfg, const uin
   a.heap = reinterpret_cast<RunHead*>(base + oHp);
   a.pivots = reinterpret_cast<uint64_t*>(base + oP);
   a.H = reinterpret_cast<uint64_t*>(base + oH);
-  a.tables = reinterpret_cast<uint32_t*>(base + oT);
   a.ztab = reinterpret_cast<uint64_t*>(base + oZ);
   a.counter = reinterpret_cast<unsigned long long*>(base + oC);
   indep_ztab_kernel<<<(L + 255) / 256, 256, 0, st>>>(reinterpret_cast<uint64_t*>(base + oZ), L);
   if (cudaMemsetAsync(a.counter, 0, 8, st) != cudaSuccess) return LABS_ERR_CUDA;
-  pq_indep_kernel<<<(unsigned)blocks, 32 * kIWarps, smem, st>>>(a, ly);
+  kern<<<(unsigned)blocks, 32 * kIWarps, smem, st>>>(a, ip);
   return cuda_status(cudaGetLastError());
 }
 

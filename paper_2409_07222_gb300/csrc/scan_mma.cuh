@@ -155,27 +155,43 @@ __device__ __forceinline__ void reverse_class(const uint32_t* w, uint32_t* rw, i
   }
 }
 
-// V_{2m} = sum_i s_i s_{2m-i} of every position m, from its two parity classes: v[m] + v[kMaxL + 1 + m], zero
-// outside (cleared once).  i and 2m - i have one parity, so each class contributes its own convolution at
-// index m - 1 (odd positions) and m - 2 (even), the correlation with its reversal.  NC: class words; cw as
-// split_classes left it, rw: scratch of the same size.
+// v[m] = V_{2m} = sum_i s_i s_{2m-i}, m = 1 .. L.  i and 2m - i have one parity, so each parity class contributes
+// its own convolution, at index m - 1 (odd positions, m < 2 n) and m - 2 (even ones, 1 < m): the correlation with
+// its reversal.  NC: class words; cw as split_classes left it, rw: scratch of the same size.
 template <int NC>
 __device__ __forceinline__ void self_convolution(const uint32_t* cw, uint32_t* rw, int L, int16_t* v) {
   reverse_class(cw, rw, (L + 1) / 2);
   reverse_class(cw + kClassWords, rw + kClassWords, L / 2);
+  if (lane_id() == 0) v[L] = 0;  // even L: the odd positions end at L - 1
   __syncwarp();
 #pragma unroll 1
   for (int e = 0; e < 2; e++) {
     const int n = e ? L / 2 : (L + 1) / 2;
-    int16_t* out = v + e * (kMaxL + 1) + n + e;  // index sum n - 1 -+ d is position n + e -+ d
+    int16_t* out = v + n + e;  // index sum n - 1 -+ d is position n + e -+ d
     const uint32_t *a = cw + e * kClassWords, *b = rw + e * kClassWords;
     corr_words<NC>(a, b, n, [&](int d, int c) {
-      if (d < n) out[-d] = (int16_t)c;
+      if (d < n) out[-d] = (int16_t)(e ? out[-d] + c : c);
     });
     corr_words<NC>(b, a, n, [&](int d, int c) {
-      if (d < n) out[d] = (int16_t)c;
+      if (d >= 1 && d < n) out[d] = (int16_t)(e ? out[d] + c : c);
     });
+    __syncwarp();
   }
+}
+
+// Word `lane` of the sequence of L elements (NW words in `bits`, zero above L, readable to word 19) rotated left
+// by r, 0 <= r < L: element i is element i + r (mod L).
+template <int NW>
+__device__ __forceinline__ uint32_t rotated_word(const uint32_t* bits, int L, int r) {
+  const int lane = lane_id(), o = 32 * lane + r, ow = o - L;
+  if (lane >= NW) return 0u;
+  uint32_t y = 0;
+  if (o < L) y = __funnelshift_r(bits[o >> 5], bits[(o >> 5) + 1], o & 31);
+  if (ow >= 0)  // elements past the end come from the start
+    y = __funnelshift_r(bits[ow >> 5], bits[(ow >> 5) + 1], ow & 31);
+  else if (ow > -32)
+    y |= bits[0] << -ow;
+  return lane == NW - 1 ? y & (0xffffffffu >> (32 * NW - L)) : y;
 }
 
 }  // namespace labsg

@@ -50,3 +50,21 @@ def test_word_and_tile_edges(lg, L):
 @pytest.mark.parametrize("cap", [16, 33, 1000, 5000])
 def test_caps_inside_a_bin(lg, cap):
     _compare(lg, 101, inp.random_words(40, 101, seed=8), cap, 16, 400)
+
+
+@pytest.mark.parametrize("L,pops,T_r", [(5, 12, 0), (31, 40, 0), (32, 65, 0), (33, 130, 0), (64, 70, 1), (128, 90, 0),
+                                        (129, 33, 2), (451, 66, 0), (576, 12, 0), (20, 1024, 0), (20, 1025, 0)])
+def test_independent_queues_visited_rule(lg, L, pops, T_r):
+    """One queue per candidate: visited neighbours found by comparing pivots (up to 1,024 pops without rotations)
+    or in the hash set, against the oracle's search of each candidate alone."""
+    n = 3
+    seeds = inp.random_words(n, L, seed=100 + L)
+    dev = torch.from_numpy(seeds.view(np.int64)).cuda()
+    best, bE, st = lg.labs_pq_independent(L, dev, pops, T_r=T_r, H_log2=20)
+    stats = st.cpu().numpy().view(lg.PQ_STATS_DTYPE).reshape(-1)
+    for q in range(n):
+        ob, oE, ofp, ost = oracle.pq_refine(L, seeds[q:q + 1], 1 << 22, 1, pops, 0, T_r)
+        assert int(bE[q].cpu()) == oE and int(stats[q]["best_fp"]) == ofp
+        assert np.array_equal(best[q].cpu().numpy().view(np.uint64), ob)
+        for k in ("expansions", "survivors", "admitted", "h_size", "improvements", "stop_reason"):
+            assert int(stats[q][k]) == ost[k], (q, k)
