@@ -11,8 +11,8 @@
 //       i0-4 .. i0+131 are staged once; the A operand of tap t is the same tile started t rows
 //       (16 t bytes) later, so the 36 MMAs (M 128, N 64, K 16) of a tile read one 17.5 KB tile.  The
 //       whole weight image (9 x 64 x 64 BF16, 72 KB) stays in shared memory; CTAs are persistent.
-//   dense_tc_kernel -- Linear(64 L -> 256) + bias + ReLU: 128 samples x 256 outputs per CTA, K in
-//       stages of 64 with two shared-memory stages, so the loads of stage k+1 overlap the MMAs of k.
+//   dense_tc_kernel -- Linear(64 L -> 256) + bias + ReLU: 256 samples x 256 outputs per CTA, K in
+//       stages of 64 with three shared-memory stages, fetched and multiplied by different warps.
 //
 // One thread issues the MMAs; tcgen05.commit arrives on an mbarrier that the CTA waits on with an
 // iteration limit (on expiry the kernel records an error, stops issuing work and still frees its
@@ -23,6 +23,7 @@
 #include <cstdint>
 
 #include "labs_internal.h"
+#include "fma2.cuh"
 #include "policy_tc.h"
 
 namespace labsg {
@@ -51,10 +52,6 @@ __device__ __forceinline__ void tmem_alloc(uint32_t* dst, int ncols) {
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, int ncols) {
   asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols));
 }
-__device__ __forceinline__ void mbar_init(uint64_t* bar) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar)));
-  asm volatile("fence.mbarrier_init.release.cluster;");
-}
 __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accum) {
   asm volatile(
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
@@ -77,19 +74,6 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;"); }
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;"); }
 __device__ __forceinline__ void fence_smem_to_async() { asm volatile("fence.proxy.async.shared::cta;"); }
-
-// 16 consecutive FP32 columns of this thread's TMEM lane.
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-  uint32_t r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;");
-#pragma unroll
-  for (int j = 0; j < 16; j++) v[j] = __uint_as_float(r[j]);
-}
 
 // 64 consecutive FP32 columns of this thread's TMEM lane, one load and one wait.
 __device__ __forceinline__ void tmem_ld64(uint32_t taddr, float (&v)[64]) {
@@ -121,7 +105,6 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
 __device__ __forceinline__ void cp16(void* dst, const void* src, bool valid) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(valid ? 16 : 0));
 }
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;"); }
 template <int N>
 __device__ __forceinline__ void cp_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N));
@@ -272,98 +255,130 @@ __global__ void __launch_bounds__(kConvThreads, 2) conv64_tc_kernel(const __nv_b
 
 // ------------------------------------------------------------------------------------------------
 // Linear(K -> 256): partial sums part[split][q][j] = sum over the split's K range of A[q][k] B[j][k].
-// K in stages of 64 (4 MMAs of M 128, N 256, K 16), three shared-memory stages filled by cp.async two
-// stages ahead.  The splits of K spread the 64 L-long rows over the SMs; dense_reduce_kernel adds the
-// partial sums in split order (deterministic), the bias and the ReLU.
+// K in stages of 64.  Bound: the operands' way from L2: a CTA takes 256 samples x 256 outputs (two accumulators of
+// 128 x 256, all of TMEM), so the weights come once per 256 samples; its stage is 65 KB and three are in flight.
+// The weights are laid out as the image of a stage, 32 KB that one bulk copy brings; the activations come by cp.async.
+// Warps 0-7 fetch and, at the end, read the accumulators out; one lane of warp 8 issues the weights' copies and the
+// MMAs.  Per stage buffer: full (256 arrivals of the fetching threads, one of the bulk copy) and used (commit).
+// The splits of K spread the 64 L-long rows over the SMs; dense_reduce_kernel adds the partial sums in split order
+// (deterministic), the bias and the ReLU.  8,192 samples of L = 451: 166 us (442 us with 128 samples a CTA and all
+// copies by the threads that also waited for the MMAs), 5.7 TB/s of operands.
 // ------------------------------------------------------------------------------------------------
-constexpr int kDLboA = 128 * 16 + 16;  // 2,064 B
-constexpr int kDLboB = 256 * 16 + 16;  // 4,112 B
-constexpr int kDStageA = 8 * kDLboA;   // 16,512 B
-constexpr int kDStageB = 8 * kDLboB;   // 32,896 B
+constexpr int kDRows = 256;
+constexpr int kDLboA = kDRows * 16 + 16;  // 4,112 B
+constexpr int kDLboB = 256 * 16;          // 4,096 B
+constexpr int kDStageA = 8 * kDLboA;      // 32,896 B
+constexpr int kDStageB = 8 * kDLboB;      // 32,768 B
 constexpr int kDStage = kDStageA + kDStageB;
 constexpr int kDStages = 3;
+constexpr int kDThreads = 288;
 constexpr int kDenseSmem = kDStages * kDStage + 1024;
 
-__global__ void __launch_bounds__(128, 1) dense_tc_kernel(const __nv_bfloat16* __restrict__ A,
-                                                          const __nv_bfloat16* __restrict__ B, float* __restrict__ part,
-                                                          long long n, int K, int kb_per_split, int* err) {
+__global__ void __launch_bounds__(kDThreads, 1) dense_tc_kernel(const __nv_bfloat16* __restrict__ A,
+                                                                const __nv_bfloat16* __restrict__ Bimg,
+                                                                float* __restrict__ part, long long n, int K,
+                                                                int kb_per_split, int* err) {
   extern __shared__ __align__(1024) unsigned char dsm[];
   unsigned char* base = dsm + ((1024 - (smem_u32(dsm) & 1023)) & 1023);
   __shared__ uint32_t tmem_base;
-  __shared__ __align__(8) uint64_t bar[kDStages];
+  __shared__ __align__(8) uint64_t full[kDStages], used[kDStages];
+  __shared__ int fail;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const long long m0 = (long long)blockIdx.x * 128;
+  const long long m0 = (long long)blockIdx.x * kDRows;
   const int nk = K / 64;
   const int kb0 = blockIdx.y * kb_per_split;
   const int nkb = max(0, min(nk, kb0 + kb_per_split) - kb0);
-  auto load = [&](int i) {
-    unsigned char* As = base + (i % kDStages) * kDStage;
-    unsigned char* Bs = As + kDStageA;
-    const long long k0 = (long long)(kb0 + i) * 64;
-    for (int e = tid; e < 128 * 8; e += 128) {
-      const int r = e >> 3, c8 = e & 7;
-      const bool ok = m0 + r < n;
-      cp16(As + c8 * kDLboA + r * 16, ok ? A + (m0 + r) * (long long)K + k0 + c8 * 8 : A, ok);
+  if (warp == 0) tmem_alloc(&tmem_base, 512);
+  if (tid == 0) {
+    for (int b = 0; b < kDStages; b++) {
+      mbar_init_n(&full[b], 257);
+      mbar_init_n(&used[b], 1);
     }
-    for (int e = tid; e < 256 * 8; e += 128) {
-      const int r = e >> 3, c8 = e & 7;
-      cp16(Bs + c8 * kDLboB + r * 16, B + (long long)r * K + k0 + c8 * 8, true);
-    }
-  };
-  if (nkb > 0) load(0);
-  cp_commit();
-  if (nkb > 1) load(1);
-  cp_commit();
-  if (warp == 0) tmem_alloc(&tmem_base, 256);
-  if (tid == 0)
-    for (int b = 0; b < kDStages; b++) mbar_init(&bar[b]);
-  const uint32_t idesc = idesc_bf16(128, 256);
-  uint32_t phase[kDStages] = {0u, 0u, 0u};
-  bool failed = false;
-  for (int i = 0; i < nkb; i++) {
-    const int st = i % kDStages;
-    cp_wait<1>();  // stage i has landed (only the most recent group may still be in flight)
-    fence_smem_to_async();
-    fence_before();
-    __syncthreads();
-    fence_after();
-    if (tid == 0) {
-      const uint32_t a0 = smem_u32(base + st * kDStage), b0 = a0 + kDStageA;
-#pragma unroll
-      for (int c = 0; c < 4; c++)
-        mma_bf16(tmem_base, sdesc(a0 + 2 * c * kDLboA, kDLboA, 128), sdesc(b0 + 2 * c * kDLboB, kDLboB, 128), idesc,
-                 (i | c) ? 1u : 0u);
-      mma_commit(&bar[st]);
-    }
-    if (i >= 1) {  // the MMAs of stage i-1 are done: its buffer takes stage i+2
-      const int sp = (i - 1) % kDStages;
-      const bool ok = mbar_wait(&bar[sp], phase[sp]);
-      phase[sp] ^= 1u;
-      if (__syncthreads_or(!ok)) {
-        failed = true;
+    fail = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;");
+  }
+  fence_before();
+  __syncthreads();
+  fence_after();
+  // use u of a buffer: its `full` completes with parity u & 1, its `used` likewise
+  if (warp < 8) {
+    for (int i = 0; i < nkb; i++) {
+      const int st = i % kDStages, u = i / kDStages;
+      if (u && !mbar_wait(&used[st], (uint32_t)((u - 1) & 1))) {
+        atomicExch(&fail, 1);
         break;
       }
+      unsigned char* As = base + st * kDStage;
+      const __nv_bfloat16* src = A + (long long)(kb0 + i) * 64;
+#pragma unroll
+      for (int j = 0; j < kDRows * 8 / 256; j++) {
+        const int e = tid + 256 * j, r = e >> 3, c8 = e & 7;
+        const bool ok = m0 + r < n;
+        cp16(As + c8 * kDLboA + r * 16, ok ? src + (m0 + r) * (long long)K + c8 * 8 : A, ok);
+      }
+      cp_arrive(&full[st]);
     }
-    if (i + 2 < nkb) load(i + 2);
-    cp_commit();
+  } else if (lane == 0) {
+    const uint32_t idesc = idesc_bf16(128, 256);
+    auto weights = [&](int i) {
+      const int st = i % kDStages;
+      const uint32_t bar = smem_u32(&full[st]), dst = smem_u32(base + st * kDStage + kDStageA);
+      asm volatile("{\n .reg .b64 t;\n mbarrier.arrive.expect_tx.shared::cta.b64 t, [%0], %1;\n}\n" ::"r"(bar),
+                   "r"(kDStageB));
+      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+                   "l"(Bimg + (long long)(kb0 + i) * (kDStageB / 2)), "r"(kDStageB), "r"(bar)
+                   : "memory");
+    };
+    for (int i = 0; i < min(nkb, kDStages); i++) weights(i);
+    bool ok = true;
+    int started = min(nkb, kDStages), landed = 0;  // the weights' copies
+    for (int i = 0; i < nkb && ok; i++) {
+      const int st = i % kDStages, u = i / kDStages;
+      ok = mbar_wait(&full[st], (uint32_t)(u & 1));
+      if (!ok) break;
+      landed = i + 1;
+      fence_smem_to_async();
+      fence_after();
+      const uint32_t a0 = smem_u32(base + st * kDStage), b0 = a0 + kDStageA;
+#pragma unroll
+      for (int h = 0; h < 2; h++)
+#pragma unroll
+        for (int c = 0; c < 4; c++)
+          mma_bf16(tmem_base + 256 * h, sdesc(a0 + 2048 * h + 2 * c * kDLboA, kDLboA, 128),
+                   sdesc(b0 + 2 * c * kDLboB, kDLboB, 128), idesc, (i | c) ? 1u : 0u);
+      mma_commit(&used[st]);
+      // the buffer of stage i - 1 takes stage i + 2 once its MMAs are done
+      if (i >= 1 && i - 1 + kDStages < nkb) {
+        ok = mbar_wait(&used[(i - 1) % kDStages], (uint32_t)(((i - 1) / kDStages) & 1));
+        if (ok) {
+          weights(i - 1 + kDStages);
+          started++;
+        }
+      }
+    }
+    if (!ok) {
+      // the copies that were started must land before shared memory is given up
+      atomicExch(&fail, 1);
+      for (int i = landed; i < started; i++) mbar_wait(&full[i % kDStages], (uint32_t)((i / kDStages) & 1));
+    }
   }
-  if (!failed && nkb > 0) {
-    const int sl = (nkb - 1) % kDStages;
-    const bool ok = mbar_wait(&bar[sl], phase[sl]);
-    if (__syncthreads_or(!ok)) failed = true;
+  bool done = true;
+  if (warp < 8) {
+    cp_wait<0>();
+    if (nkb > 0) done = mbar_wait(&used[(nkb - 1) % kDStages], (uint32_t)(((nkb - 1) / kDStages) & 1));
   }
-  cp_wait<0>();
-  if (failed) {
+  if (__syncthreads_or(!done || *reinterpret_cast<volatile int*>(&fail))) {
     if (tid == 0) atomicExch(err, 1);
-  } else {
+  } else if (warp < 8) {
     fence_after();
-    const long long q = m0 + warp * 32 + lane;
+    const long long q = m0 + tid;  // rows 0 .. 127: the first accumulator, warps 0 .. 3; then the second
+    const uint32_t acc = tmem_base + 256u * (uint32_t)(warp >> 2) + ((uint32_t)((warp & 3) * 32) << 16);
     float* dst = part + ((long long)blockIdx.y * n + q) * 256;
 #pragma unroll 1
     for (int c0 = 0; c0 < 256; c0 += 64) {
       float v[64];
       if (nkb > 0) {
-        tmem_ld64(tmem_base + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
+        tmem_ld64(acc + (uint32_t)c0, v);
       } else {
 #pragma unroll
         for (int j = 0; j < 64; j++) v[j] = 0.f;
@@ -378,7 +393,7 @@ __global__ void __launch_bounds__(128, 1) dense_tc_kernel(const __nv_bfloat16* _
   fence_before();
   __syncthreads();
   fence_after();
-  if (warp == 0) tmem_dealloc(tmem_base, 256);
+  if (warp == 0) tmem_dealloc(tmem_base, 512);
 }
 
 // out[q][j] = relu(bias[j] + sum over splits of part[s][q][j]), splits added in order.
@@ -398,20 +413,21 @@ __global__ void dense_reduce_kernel(const float* __restrict__ part, const float*
 // ------------------------------------------------------------------------------------------------
 // One block per (sample, 128 positions), 256 threads: thread (cp, g) keeps the 36 weights of output
 // channels 2cp, 2cp+1 in registers and slides over positions i0 + 16g .. i0 + 16g + 15 of the two input
-// channels staged in shared memory; a warp's 32 channel pairs write one 128-byte position row.
+// channels staged in shared memory; a warp's 32 channel pairs write one 128-byte position row.  Bound: FP32
+// FMA, two an instruction; four positions a turn share a window of twelve inputs (six 16-byte broadcasts for
+// 72 two-wide FMAs, where a load per operand took one for two).
 __global__ void __launch_bounds__(256) conv1_cl_kernel(const float* __restrict__ x, const __nv_bfloat16* __restrict__ w,
                                                        const float* __restrict__ bias, __nv_bfloat16* __restrict__ out,
                                                        int L, long long n) {
-  __shared__ float xs[2][136];
+  __shared__ __align__(16) float xs[2][136];
   const int cp = threadIdx.x & 31, g = threadIdx.x >> 5;
-  float wr[2][2][9];
+  uint64_t wr[2][9];  // of both output channels
 #pragma unroll
-  for (int o = 0; o < 2; o++)
+  for (int ci = 0; ci < 2; ci++)
 #pragma unroll
-    for (int ci = 0; ci < 2; ci++)
-#pragma unroll
-      for (int t = 0; t < 9; t++) wr[o][ci][t] = __bfloat162float(w[((2 * cp + o) * 2 + ci) * 9 + t]);
-  const float b0 = bias[2 * cp], b1 = bias[2 * cp + 1];
+    for (int t = 0; t < 9; t++)
+      wr[ci][t] = pack2(__bfloat162float(w[(2 * cp * 2 + ci) * 9 + t]), __bfloat162float(w[((2 * cp + 1) * 2 + ci) * 9 + t]));
+  const uint64_t b01 = pack2(bias[2 * cp], bias[2 * cp + 1]);
   const int tps = (L + 127) / 128;
   for (long long tile = blockIdx.x; tile < n * tps; tile += gridDim.x) {
     const long long s = tile / tps;
@@ -423,18 +439,30 @@ __global__ void __launch_bounds__(256) conv1_cl_kernel(const float* __restrict__
     }
     __syncthreads();
     uint32_t* dst = reinterpret_cast<uint32_t*>(out + (s * L + i0 + 16 * g) * 64) + cp;
-#pragma unroll 4
-    for (int k = 0; k < 16; k++) {
-      float a0 = b0, a1 = b1;
+#pragma unroll 1
+    for (int k = 0; k < 16; k += 4) {
+      uint64_t acc[4] = {b01, b01, b01, b01};
 #pragma unroll
-      for (int ci = 0; ci < 2; ci++)
+      for (int ci = 0; ci < 2; ci++) {
+        uint64_t xv[12];
 #pragma unroll
-        for (int t = 0; t < 9; t++) {
-          const float xv = xs[ci][16 * g + k + t];
-          a0 = fmaf(wr[0][ci][t], xv, a0);
-          a1 = fmaf(wr[1][ci][t], xv, a1);
+        for (int v = 0; v < 3; v++) {
+          const float4 q = *reinterpret_cast<const float4*>(&xs[ci][16 * g + k + 4 * v]);
+          xv[4 * v] = pack2(q.x, q.x);
+          xv[4 * v + 1] = pack2(q.y, q.y);
+          xv[4 * v + 2] = pack2(q.z, q.z);
+          xv[4 * v + 3] = pack2(q.w, q.w);
         }
-      if (i0 + 16 * g + k < L) dst[k * 32] = pack_bf16(fmaxf(a0, 0.f), fmaxf(a1, 0.f));
+#pragma unroll
+        for (int t = 0; t < 9; t++)
+#pragma unroll
+          for (int j = 0; j < 4; j++) ffma2(acc[j], wr[ci][t], xv[j + t]);
+      }
+#pragma unroll
+      for (int j = 0; j < 4; j++) {
+        const float2 a = unpack2(acc[j]);
+        if (i0 + 16 * g + k + j < L) dst[(k + j) * 32] = pack_bf16(fmaxf(a.x, 0.f), fmaxf(a.y, 0.f));
+      }
     }
   }
 }
@@ -449,13 +477,14 @@ __global__ void conv_image_kernel(const float* __restrict__ w, __nv_bfloat16* __
   }
 }
 
-// The dense layer's weights in channels-last input order: Bp[j][i * 64 + c] = W4[j][c * L + i].
-__global__ void dense_perm_kernel(const float* __restrict__ W4, __nv_bfloat16* __restrict__ Bp, int L) {
+// The dense layer's weights in channels-last input order, k = i * 64 + c of W4[j][c * L + i], as the images of its
+// stages of 64 k: stage, eight k, output j, k.
+__global__ void dense_perm_kernel(const float* __restrict__ W4, __nv_bfloat16* __restrict__ Bimg, int L) {
   const long long K = 64ll * L;
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < 256 * K; e += (long long)gridDim.x * blockDim.x) {
-    const long long j = e / K, k = e % K;
-    const long long i = k / 64, c = k % 64;
-    Bp[e] = __float2bfloat16_rn(W4[j * K + c * L + i]);
+    const long long i = e >> 14;
+    const int c = (int)(e >> 11 & 7) * 8 + (int)(e & 7), j = (int)(e >> 3 & 255);
+    Bimg[e] = __float2bfloat16_rn(W4[j * K + c * L + i]);
   }
 }
 
@@ -497,9 +526,9 @@ int tc_conv64(const __nv_bfloat16* in, const __nv_bfloat16* img, const float* bi
   return cuda_status(cudaGetLastError());
 }
 
-// Splits of K: a function of K alone (about 64 stages each, at most 8), so a sample's logits do not
-// depend on the batch it is evaluated in.
-int tc_dense_splits(int K) { return std::max(1, std::min(8, (K / 64) / 64)); }
+// Splits of K: a function of K alone, so a sample's logits do not depend on the batch it is evaluated in: about 48
+// stages each, at most 9 (with the 32 row blocks of 8,192 samples, two rounds of CTAs).
+int tc_dense_splits(int K) { return std::max(1, std::min(9, (K / 64) / 48)); }
 
 int tc_dense(const __nv_bfloat16* A, const __nv_bfloat16* Bp, const float* bias, float* part, float* out, long long n,
              int K, int num_sms, int* err, cudaStream_t st) {
@@ -514,7 +543,7 @@ int tc_dense(const __nv_bfloat16* A, const __nv_bfloat16* Bp, const float* bias,
   if (K % 64 || n <= 0) return n == 0 ? LABS_OK : LABS_ERR_INVALID_ARG;
   const int splits = tc_dense_splits(K);
   const int nk = K / 64, per = (nk + splits - 1) / splits;
-  dense_tc_kernel<<<dim3((unsigned)((n + 127) / 128), (unsigned)splits), 128, kDenseSmem, st>>>(A, Bp, part, n, K, per, err);
+  dense_tc_kernel<<<dim3((unsigned)((n + kDRows - 1) / kDRows), (unsigned)splits), kDThreads, kDenseSmem, st>>>(A, Bp, part, n, K, per, err);
   dense_reduce_kernel<<<(unsigned)std::min<long long>((n * 256 + 255) / 256, (long long)num_sms * 16), 256, 0, st>>>(
       part, bias, out, n, splits);
   return cuda_status(cudaGetLastError());
