@@ -186,9 +186,6 @@ __device__ __forceinline__ int h_insert(const PqBufs& b, uint64_t fp) {
   return 0;
 }
 
-__device__ __forceinline__ bool key_lt(int Ea, uint64_t fa, int Eb, uint64_t fb) {
-  return Ea < Eb || (Ea == Eb && fa < fb);
-}
 __device__ __forceinline__ bool key_le(int Ea, uint64_t fa, int Eb, uint64_t fb) {
   return Ea < Eb || (Ea == Eb && fa <= fb);
 }
