@@ -81,6 +81,20 @@ def terms_per_flip(L, p):
     return (k - p + 1) * ((L - 1) // 2)  # free neighbours x even lags
 
 
+def flip_ops(L, p):
+    """Integer operations that a flip cannot do without: it changes one product pair of every lag and, of every
+    neighbour's energy change, one second difference (four table values, a product, the sum).  Skew walks (odd L)
+    keep k-p+1 neighbours and (L-1)/2 even lags, unrestricted ones L and L-1."""
+    k = (L - 1) // 2
+    return 8 * ((k - p + 1) + k) if L % 2 else 8 * (L + L - 1)
+
+
+def energy_words(L):
+    """Words of 32 products over all lags.  Each takes a funnel shift and, in a carry-save adder (which the XOR of
+    its products is merged into), two three-input logic operations: three half-rate instructions."""
+    return sum(-(-(L - k) // 32) for k in range(1, L))
+
+
 def kernel_source_hash():
     h = hashlib.sha256()
     for f in KERNEL_SOURCES:
@@ -89,17 +103,31 @@ def kernel_source_hash():
     return h.hexdigest()[:16]
 
 
-def traffic_per_launch(n_walks):
-    """DRAM bytes of one walk-kernel launch, scaled by walks from the committed ncu capture of a smaller
-    launch (its traffic is the per-walk candidate records and statistics); None if the kernel changed."""
+def walk_profile():
+    """The committed ncu figures of the walk kernel; None if the kernel changed since."""
     try:
         with open(PROFILE_TRAFFIC) as f:
             d = json.load(f)
     except (OSError, ValueError):
         return None
-    if d.get("source_hash") != kernel_source_hash():
+    return d if d.get("source_hash") == kernel_source_hash() else None
+
+
+def walk_issue(flips_per_s):
+    """Share of the issue slots (4 a clock and SM) that the walk kernel's own instructions take."""
+    d = walk_profile()
+    if not d:
         return None
-    return d["dram_bytes_per_walk"] * n_walks
+    peak = SMS * 4 * SM_MAX_MHZ * 1e6
+    return {"warp_instructions_per_flip": d["warp_instructions_per_flip"], "peak_Ginst_s": peak / 1e9,
+            "frac": d["warp_instructions_per_flip"] * flips_per_s / peak}
+
+
+def traffic_per_launch(n_walks):
+    """DRAM bytes of one walk-kernel launch, scaled by walks from the committed ncu capture of a smaller
+    launch (its traffic is the per-walk candidate records and statistics); None if the kernel changed."""
+    d = walk_profile()
+    return d["dram_bytes_per_walk"] * n_walks if d else None
 
 
 class ClockSampler:
@@ -192,14 +220,6 @@ def run_reference(args, ws, rank):
     return 0
 
 
-def unit_terms(L, p):
-    """Neighbour-lag multiply-adds of one flip: skew walks scan k-p+1 neighbours over (L-1)/2 even lags,
-    unrestricted walks L neighbours over L-1 lags."""
-    if L % 2:
-        return terms_per_flip(L, p)
-    return L * (L - 1)
-
-
 def run_mixed(args, ws, rank, local):
     """Batched step 1 over L = 450..527: per-length sieve bounds + one persistent walk launch, replayed
     from a CUDA graph; walks per length uniform in {1024..16384} (seed 2410), 10^4 flips each."""
@@ -222,7 +242,7 @@ def run_mixed(args, ws, rank, local):
                             n_thresh_samples=W1["n_thresh_samples"], thresh_rank=W1["thresh_rank"], use_graph=True)
     flush = torch.empty(256 * 1024 * 1024, dtype=torch.uint8, device=dev)
     t0 = time.perf_counter()
-    out = lg.labs_batched_search(cfg, lengths, walks, pre, walk_stats=False)  # autotune + capture
+    out = lg.labs_batched_search(cfg, lengths, walks, pre, walk_stats=False)  # capture
     torch.cuda.synchronize()
     first_s = time.perf_counter() - t0
     for _ in range(max(0, args.warmup - 1)):
@@ -246,7 +266,7 @@ def run_mixed(args, ws, rank, local):
     clk = clocks.stop()
     total_ms = sum(step_ms)
     flips = args.steps * sum(walks) * budget
-    terms = sum(w * budget * unit_terms(L, p) for L, w in zip(lengths, walks))
+    terms = sum(w * budget * flip_ops(L, p) for L, w in zip(lengths, walks))
     peak = SMS * LANES_PER_SM * SM_MAX_MHZ * 1e6 / 1e9
     achieved = terms / (statistics.mean(step_ms) * 1e-3) / 1e9
     line = {"metric": METRIC, "value": flips / (total_ms * 1e-3), "unit": METRIC, "n_gpus": 1, "steps": args.steps,
@@ -254,12 +274,13 @@ def run_mixed(args, ws, rank, local):
             "scaling": "weak", "vs_baseline": None, "dtype": "int32", "data": "synthetic",
             "config": {"workload": "mixed_L450-527_walks_U1024-16384_1e4flips", "lengths": len(lengths),
                        "walks": sum(walks), "flips_per_walk": budget, "p_odd": p, "graph": True,
-                       "first_call_s_incl_autotune_and_capture": first_s,
+                       "first_call_s_incl_capture": first_s,
                        "l2": "flushed between timed steps (256 MB write)"},
             "gpu_launches": (4 * len(lengths) + 2) * args.steps, "clocks": clk,
             "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Gop/s", "frac": achieved / peak,
                          "traffic": None, "kernel": "walk_kernel (one launch, all lengths) + 78 sieve bounds",
-                         "work": "per flip: (k-p+1)(L-1)/2 terms (odd L, skew) or L(L-1) terms (even L)"}}
+                         "work": "per flip 8 x (neighbours + lags) integer operations: k-p+1 and (L-1)/2 (odd L, "
+                                 "skew) or L and L-1 (even L)"}}
     print(json.dumps(line))
     return 0
 
@@ -303,7 +324,7 @@ def run_pq(args, ws, rank, local):
     t = statistics.mean(times[-args.steps:])
     s2 = lg.pq_stats_numpy(st)
     exps = int(s2["expansions"])
-    terms = exps * L * (L - 1)
+    terms = exps * 8 * (2 * L - 1)
     peak = SMS * LANES_PER_SM * SM_MAX_MHZ * 1e6 / 1e9
     line = {"metric": "expansions/s", "value": exps / t, "unit": "expansions/s", "n_gpus": 1, "steps": args.steps,
             "warmup": max(1, args.warmup), "ms_per_step": t * 1e3, "higher_is_better": True, "scaling": "weak",
@@ -317,7 +338,8 @@ def run_pq(args, ws, rank, local):
             "neighbour_evaluations_per_s": exps * L / t,
             "roofline": {"bound": "alu", "achieved": terms / t / 1e9, "peak": peak, "unit": "Gop/s",
                          "frac": terms / t / 1e9 / peak, "traffic": None,
-                         "work": "per expansion L(L-1) neighbour-lag multiply-adds (whole step timed, host-driven)"}}
+                         "work": "per expansion 8 x (L neighbours + L-1 lags) integer operations, as a flip "
+                                 "(whole step timed, host-driven)"}}
     print(json.dumps(line))
     return 0
 
@@ -468,8 +490,8 @@ def network_roofline(lg, L, n, local):
 
 def run_operators(args, ws, rank, local):
     """The end-element operators at L=451 on 2^20 sequences (the four L+1 and two L-1 results with their
-    exact energies), as results per second.  The work is the six energies: one popcount per 32 products,
-    sum over k of ceil((L'-k)/32) per result; POPC issues at 16 lanes per clock per SM on this part."""
+    exact energies), as results per second.  The work is the six energies: three half-rate operations per 32
+    products, sum over k of ceil((L'-k)/32) words per result."""
     import torch
 
     import paper_2409_07222_gb300 as lg
@@ -490,20 +512,17 @@ def run_operators(args, ws, rank, local):
     e1.record(st)
     st.synchronize()
     ms = e0.elapsed_time(e1) / reps
-    def popc_per_energy(Lv):  # one popcount per 32 products of each lag
-        return sum(-(-(Lv - k) // 32) for k in range(1, Lv))
-
-    popc = 4 * popc_per_energy(L + 1) + 2 * popc_per_energy(L - 1)
-    ach = popc * n / (ms * 1e-3) / 1e9
-    peak = SMS * 16 * SM_MAX_MHZ * 1e6 / 1e9
+    ops = 3 * (4 * energy_words(L + 1) + 2 * energy_words(L - 1))
+    ach = ops * n / (ms * 1e-3) / 1e9
+    peak = SMS * 64 * SM_MAX_MHZ * 1e6 / 1e9
     line = {"metric": "operator results/s", "value": 6 * n / (ms * 1e-3), "unit": "results/s", "n_gpus": 1,
             "steps": reps, "warmup": 3, "ms_per_step": ms, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": "int32", "data": "synthetic",
             "config": {"workload": "sequence_operators_L451_2^20seq", "L": L, "n": n},
-            "roofline": {"bound": "alu", "achieved": ach, "peak": peak, "unit": "Gpopc/s", "frac": ach / peak,
+            "roofline": {"bound": "alu", "achieved": ach, "peak": peak, "unit": "Gop/s", "frac": ach / peak,
                          "traffic": None, "kernel": "operators_kernel",
-                         "work": "6 energies per sequence: sum_k ceil((L'-k)/32) popcounts each; "
-                                 "peak = 152 SMs x 16 POPC/clk x 2070 MHz"}}
+                         "work": "6 energies per sequence: 3 half-rate operations per word of 32 products; "
+                                 "peak = 152 SMs x 64 lanes/clk x 2070 MHz"}}
     print(json.dumps(line))
     return 0
 
@@ -525,7 +544,7 @@ def _time_calls(fn, reps=10, warm=3):
 
 def run_energy(args, ws, rank, local):
     """labs_energy_batch on 2^22 random sequences of L = 451 (the sieve sample's shape, 4x larger): all
-    C_k and E; one popcount per 32 products of each lag, 268 MB of sequences read per call."""
+    C_k and E; three half-rate operations per 32 products of each lag, 268 MB of sequences read per call."""
     import torch
 
     import paper_2409_07222_gb300 as lg
@@ -535,14 +554,14 @@ def run_energy(args, ws, rank, local):
     L, n = W1["L"], 1 << 22
     w = torch.from_numpy(inp.random_words(n, L, seed=21).view(np.int64)).to(torch.device("cuda", local))
     t = _time_calls(lambda: lg.labs_energy_batch(w, L))
-    popc = n * sum(-(-(L - k) // 32) for k in range(1, L))
-    peak = SMS * 16 * SM_MAX_MHZ * 1e6 / 1e9
+    ops = 3 * n * energy_words(L)
+    peak = SMS * 64 * SM_MAX_MHZ * 1e6 / 1e9
     line = {"metric": "energies/s", "value": n / t, "unit": "energies/s", "n_gpus": 1, "steps": 10, "warmup": 3,
             "ms_per_step": t * 1e3, "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "int32",
             "data": "synthetic", "config": {"workload": "energy_batch_L451_2^22seq", "L": L, "n": n},
-            "roofline": {"bound": "alu", "achieved": popc / t / 1e9, "peak": peak, "unit": "Gpopc/s",
-                         "frac": popc / t / 1e9 / peak, "traffic": None, "kernel": "energy_batch_kernel",
-                         "work": "sum_k ceil((L-k)/32) popcounts per sequence; input %.0f MB per call, "
+            "roofline": {"bound": "alu", "achieved": ops / t / 1e9, "peak": peak, "unit": "Gop/s",
+                         "frac": ops / t / 1e9 / peak, "traffic": None, "kernel": "energy_batch_kernel",
+                         "work": "3 half-rate operations per word of 32 products (64 lanes/clk/SM); input %.0f MB per call, "
                                  "%.2f TB/s" % (n * 64 / 1e6, n * 64 / t / 1e12)}}
     print(json.dumps(line))
     return 0
@@ -567,14 +586,15 @@ def run_deltas(args, ws, rank, local):
     seqs = torch.from_numpy(np.ascontiguousarray(cand["seq"][:, :W]).view(np.int64)).to(torch.device("cuda", local))
     t = _time_calls(lambda: lg.labs_flip_deltas(seqs, L, skew=True, p=p))
     terms = n * terms_per_flip(L, p)
-    peak = SMS * LANES_PER_SM * SM_MAX_MHZ * 1e6 / 1e9
+    peak = SMS * 1012 * SM_MAX_MHZ * 1e6 / 1e9  # measured f16 mma.sync rate
     line = {"metric": "neighbour evaluations/s", "value": n * 202 / t, "unit": "evaluations/s", "n_gpus": 1,
             "steps": 10, "warmup": 3, "ms_per_step": t * 1e3, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": "int32", "data": "synthetic",
             "config": {"workload": "flip_deltas_skew_L451_p24_2^16seq", "L": L, "p": p, "n": n},
-            "roofline": {"bound": "alu", "achieved": terms / t / 1e9, "peak": peak, "unit": "Gop/s",
-                         "frac": terms / t / 1e9 / peak, "traffic": None, "kernel": "flip_deltas_kernel",
-                         "work": "45450 neighbour-lag multiply-adds per sequence (as the walk's step)"}}
+            "roofline": {"bound": "tensor", "achieved": terms / t / 1e9, "peak": peak, "unit": "Gop/s",
+                         "frac": terms / t / 1e9 / peak, "traffic": None, "kernel": "flip_deltas_skew_kernel",
+                         "work": "45450 neighbour-lag multiply-adds per sequence; peak = 152 SMs x 1012 f16 "
+                                 "mma.sync multiply-adds/clk x 2070 MHz"}}
     print(json.dumps(line))
     return 0
 
@@ -659,7 +679,7 @@ def run_pq_indep(args, ws, rank, local):
     t = statistics.mean(times[-args.steps:])
     stn = st.cpu().numpy().view(lg.PQ_STATS_DTYPE).reshape(-1)
     exps = int(stn["expansions"].sum())
-    terms = exps * L * (L - 1)
+    terms = exps * 8 * (2 * L - 1)
     peak = SMS * LANES_PER_SM * SM_MAX_MHZ * 1e6 / 1e9
     line = {"metric": "expansions/s", "value": exps / t, "unit": "expansions/s", "n_gpus": 1, "steps": args.steps,
             "warmup": max(1, args.warmup), "ms_per_step": t * 1e3, "higher_is_better": True, "scaling": "weak",
@@ -672,14 +692,15 @@ def run_pq_indep(args, ws, rank, local):
             "neighbour_evaluations_per_s": exps * L / t,
             "roofline": {"bound": "alu", "achieved": terms / t / 1e9, "peak": peak, "unit": "Gop/s",
                          "frac": terms / t / 1e9 / peak, "traffic": None,
-                         "work": "per expansion L(L-1) neighbour-lag multiply-adds (whole refinement timed)"}}
+                         "work": "per expansion 8 x (L neighbours + L-1 lags) integer operations, as a flip "
+                                 "(whole refinement timed)"}}
     print(json.dumps(line))
     return 0
 
 
 def run_legendre(args, ws, rank, local):
     """Legendre seeds: the construction's throughput (every rotation of every prime with up to 30%
-    appended, L = 450..527, exact energies on the device) with its POPC roofline; then, at the lengths of
+    appended, L = 450..527, exact energies on the device) with its roofline; then, at the lengths of
     Table 2, the (0.20, 0.24, 0.1) family and step 2 (Algorithm 2, B = 4,096, open set 2^22) from all of
     its seeds, with the best constructed and refined merit factors per length (Table 2 prints 6.1976 /
     6.3088, 6.2332 / 6.2998, 6.4292 / 6.4292, 6.3240 / 6.3240: context from the paper's own search)."""
@@ -704,7 +725,7 @@ def run_legendre(args, ws, rank, local):
     torch.cuda.synchronize()
     t_con = e0.elapsed_time(e1) * 1e-3
     n_tot = sum(int(f.shape[0]) for _, f in fams)
-    popc_tot = sum(int(f.shape[0]) * sum(-(-(L - k) // 32) for k in range(1, L)) for L, f in fams)
+    ops_tot = sum(3 * int(f.shape[0]) * energy_words(L) for L, f in fams)
     # Table 2 lengths: the (0.20, 0.24, 0.1) family, then step 2 from all of its seeds
     per_L = []
     for L in (450, 471, 491, 526):
@@ -721,16 +742,17 @@ def run_legendre(args, ws, rank, local):
         per_L.append({"L": L, "seeds": int(n), "F_construct": round(L * L / (2.0 * int(E.min())), 4),
                       "F_refined": round(L * L / (2.0 * int(bE.cpu()[0])), 4), "expansions": int(s2["expansions"]),
                       "refine_s": t_pq})
-    peak = SMS * 16 * SM_MAX_MHZ * 1e6 / 1e9
-    ach = popc_tot / t_con / 1e9
+    peak = SMS * 64 * SM_MAX_MHZ * 1e6 / 1e9
+    ach = ops_tot / t_con / 1e9
     line = {"metric": "seeds/s", "value": n_tot / t_con, "unit": "seeds/s", "n_gpus": 1, "steps": 1, "warmup": 2,
             "ms_per_step": t_con * 1e3, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
             "dtype": "int32", "data": "synthetic",
             "config": {"workload": "legendre_seeds_L450-527_all_rotations", "seeds": n_tot,
                        "table2_family": "r 0.20..0.24 of L, t <= 0.1 p", "max_expansions": args.pq_expansions},
-            "roofline": {"bound": "alu", "achieved": ach, "peak": peak, "unit": "Gpopc/s", "frac": ach / peak,
+            "roofline": {"bound": "alu", "achieved": ach, "peak": peak, "unit": "Gop/s", "frac": ach / peak,
                          "traffic": None, "kernel": "legendre_kernel",
-                         "work": "sum_k ceil((L-k)/32) popcounts per seed; peak = 152 SMs x 16 POPC/clk x 2070 MHz"},
+                         "work": "3 half-rate operations per word of 32 products of a seed's energy; peak = 152 SMs x "
+                                 "64 lanes/clk x 2070 MHz"},
             "per_length": per_L}
     print(json.dumps(line))
     return 0
@@ -912,7 +934,7 @@ def main():
         return 0
 
     flips_per_launch = n_walks * budget
-    terms = flips_per_launch * terms_per_flip(L, p)
+    terms = flips_per_launch * flip_ops(L, p)
     walk_s = statistics.mean(walk_ms) * 1e-3
     achieved = terms / walk_s / 1e9
     peak = SMS * LANES_PER_SM * SM_MAX_MHZ * 1e6 / 1e9
@@ -934,14 +956,10 @@ def main():
         "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Gop/s", "frac": achieved / peak,
                      "traffic": traffic_per_launch(n_walks),
                      "kernel": "walk_kernel", "walk_kernel_ms": walk_s * 1e3,
-                     "work": "%d neighbour-lag terms per flip (202 free x 225 even lags), one int32 multiply-add "
-                             "each; peak = 152 SMs x 128 lanes x 2070 MHz (issue slots)" % terms_per_flip(L, p),
-                     "measured_lanes_per_clk_per_sm": rates,
-                     "dp4a_pipe": {"peak": SMS * rates["DP4A"] * 4 * SM_MAX_MHZ * 1e6 / 1e9,
-                                   "frac": achieved / (SMS * rates["DP4A"] * 4 * SM_MAX_MHZ * 1e6 / 1e9),
-                                   "unit": "Gop/s",
-                                   "basis": "measured DP4A lane rate x 4 multiply-adds per DP4A x 152 SMs x "
-                                            "2070 MHz: the ceiling of a scan made of DP4A alone"}},
+                     "work": "%d integer operations per flip: 8 x (202 free neighbours + 225 even lags); peak = "
+                             "152 SMs x 128 lanes x 2070 MHz (issue slots)" % flip_ops(L, p),
+                     "issue": walk_issue(flips_per_launch / walk_s),
+                     "measured_lanes_per_clk_per_sm": rates},
     }
     if ws == 1 and not args.no_cpu_baseline:
         line["cpu_baseline"] = cpu_baseline(args.cpu_walks, args.cpu_flips)

@@ -262,8 +262,8 @@ typedef struct {
  * the device until a stop condition holds.  The host drives the rounds and polls a device flag, so the
  * call returns after `stream` has finished the refinement.
  *   seeds [n_seeds][W] uint64 DEVICE; best_seq [W] uint64 DEVICE; best_E int32 DEVICE; stats DEVICE.
- *   Workspace: two open-set buffers (cap * (12 + 8W) bytes each), the visited set (8 * 2^H_log2 bytes),
- *   survivor and sort buffers (about 60 * B * L bytes).
+ *   Workspace: the open-set pool (about cap * (32 + 8W) bytes), the visited set (8 * 2^H_log2 bytes) and its
+ *   filter (at most 32 MB), survivor and selection buffers (about 60 * B * L bytes).
  * Errors: LABS_ERR_INVALID_ARG on a bad configuration, LABS_ERR_NOMEM if the
  * workspace cannot be allocated.
  */
@@ -277,10 +277,11 @@ int labs_pq_refine(labs_ctx* ctx, const labs_pq_cfg* cfg, const uint64_t* seeds,
  * without improvement.  Equivalent to labs_pq_refine with one seed, B = 1 and a cap never reached
  * (rotations included when T_r > 0).
  *   seeds [n][W] uint64, best_seqs [n][W] uint64, best_E [n] int32, stats [n] labs_pq_stats -- device.
- *   Memory: each resident warp holds max_expansions x (L + 2 T_r) x 16 B of queue records, 24 B per pop
- *   of run heads, 8 W B per pop of pivots, about 4 L B per pop of pivot tables (C_k and P_m) and
- *   2^H_log2 x 8 B of visited set; as many warps run as fit in max_workspace_bytes (0: 64 GiB) and the
- *   occupancy limit, the rest of the candidates wait for a warp.
+ *   Memory: each resident warp is counted with max_expansions x (L + 2 T_r) x 16 B of queue records, 24 B
+ *   per pop of run heads, 8 W B per pop of pivots, about 4 L B per pop of pivot tables and 2^H_log2 x 8 B of
+ *   visited set (an upper bound: no tables are kept, and the visited set is allocated with T_r > 0 or more
+ *   than 1,024 pops only); as many warps run as fit in max_workspace_bytes (0: 64 GiB) and the occupancy
+ *   limit, the rest of the candidates wait for a warp.
  * Errors: LABS_ERR_INVALID_ARG on a bad configuration; per candidate, stats.status = LABS_ERR_CAPACITY if
  * its visited set passed 3/4 load (raise H_log2).
  */
