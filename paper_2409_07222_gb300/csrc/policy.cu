@@ -17,7 +17,7 @@
 // weights); an outer-product kernel for the weight gradient; a 128x128-tile GEMM with strided operands for
 // the two dense layers and their gradients, its K split over blocks where the output has few tiles.  A
 // training step on 512 samples of L = 451 takes 3.11 ms (8.56 ms with one shared load an operand and unsplit tiles); the
-// FMAs alone, 62 G, take 1.67 ms at one a lane and clock.
+// FMAs alone, 63 G, take 1.57 ms at one a lane and clock.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -99,8 +99,9 @@ constexpr int kCT = 8;  // input channels staged at a time
 // chunk is padded) and all 64 output channels, a thread 8 channels x one chunk: its window of sixteen inputs (four
 // 16-byte loads a channel) serves all nine taps, and its eight weights of a tap are two 16-byte broadcasts: 22 shared
 // loads for 288 two-wide FMAs.  (With 4 positions a thread it is 21 for 144, and the loads' 512 bytes each are the
-// bound.)  512 samples of L = 451: 328 us a layer (26 TFMA/s of 37; 488 us before).  The sum runs over channels, then taps, as one chain per output.  The windows lie 20 floats apart: eight
-// threads' 16-byte reads fall into different banks.  The results go through shared memory to leave in whole lines.
+// bound.)  512 samples of L = 451: 328 us a layer (26 TFMA/s of 40; 488 us before).  The sum runs over channels, then
+// taps, as one chain per output.  The windows lie 20 floats apart: eight threads' 16-byte reads fall into different
+// banks.  The results go through shared memory to leave in whole lines.
 constexpr int kConvThreads = 128, kChunks = 16, kWin = 20;
 
 template <int CIN>
