@@ -342,7 +342,7 @@ __global__ void flip_transpose_kernel(const float* __restrict__ w, __nv_bfloat16
 // outputs a thread (four 16-byte shared loads for 64 FMAs), the next tile's operands loaded while this one is
 // multiplied, two buffers and one barrier a tile.  An output of few tiles (fc2 and its gradients) gets its K split over blocks, whose partial
 // sums splitk_reduce_kernel adds in order (deterministic).  512 samples, L = 451: W4's gradient 172 us, h3's 206 us
-// (64 x 64 tiles of 4 x 4 a thread: 0.6 ms each).
+// (322 and 439 us in 64 x 64 tiles of 4 x 4 a thread).
 // ---------------------------------------------------------------------------------------------
 template <typename T>
 __device__ __forceinline__ float ld_as_float(const T* p, long long i);
@@ -488,7 +488,7 @@ void gemm(cudaStream_t st, int M, int N, long long K, const TA* A, long long am,
 // gradients, so it is not split as the other long sums are.  512 samples have eight 128 x 128 tiles: here a block
 // takes 32 samples x 32 outputs, a thread 2 x 4 of them, which is what the FMA pipe needs to be busy in all of an SM
 // and what bounds the kernel by its shared reads instead (eight 16-byte reads for 64 FMAs, the weights kept BF16).
-// Chunks of 64 k (K is a multiple) through three cp.async buffers.  L = 451: 345 us for 512 samples (2.6 ms in the
+// Chunks of 64 k (K is a multiple) through three cp.async buffers.  L = 451: 345 us for 512 samples (3.81 ms in the
 // former 64 x 64 tiles), 2.99 ms for 6,112.  gemm_kernel takes 4.47 ms for anything up to one tile an SM (9,728
 // samples), where fc1_kernel would take 4.8 ms: the line lies there.
 constexpr int kFT = 32, kFK = 64, kFStages = 3;
