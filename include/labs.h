@@ -350,7 +350,7 @@ int labs_policy_train_step(labs_policy* policy, const uint64_t* seqs, const int3
  * counterpart: this is the library's learned proposal.
  *   Arguments as in labs_skew_search, plus (all nullable, DEVICE, n_chunks = ceil(flip_budget / chunk)):
  *   logits_log [n_chunks][n_walks][L] FP32: the logits each chunk used;
- *   state_log  [n_chunks][n_walks][W] uint64: every walk's sequence when its chunk began;
+ *   state_log  [n_chunks][n_walks][W] uint64 (of any alignment): every walk's sequence when its chunk began;
  *   move_log   [n_chunks][n_walks][2] int32: the chunk's first move (position, Delta E), (-1, 0) if none.
  *   Workspace with a policy: about 8 KB per walk (up to 11 KB at L = 576).  With a policy the call synchronises `stream` at its end and returns
  *   LABS_ERR_TIMEOUT if a tensor-core wait of the network expired.

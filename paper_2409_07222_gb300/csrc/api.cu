@@ -204,7 +204,7 @@ int labs_chunked_search(labs_ctx* ctx, const labs_walk_cfg* cfg, labs_policy* po
   if (!cfg->E_thr_dev && cfg->E_thr == LABS_AUTO_THRESHOLD &&
       (cfg->n_thresh_samples < 1 || cfg->thresh_rank < 0 || cfg->thresh_rank >= cfg->n_thresh_samples))
     return LABS_ERR_INVALID_ARG;
-  if (!stats || !aligned8(stats) || (cfg->n_walks > 0 && (!out || !aligned8(out))))
+  if (!stats || !aligned8(stats) || (cfg->n_walks > 0 && (!out || !aligned8(out))) || (move_log && !aligned4(move_log)))
     return LABS_ERR_INVALID_ARG;
   if (policy && labsg::policy_length(policy) != cfg->L) return LABS_ERR_INVALID_ARG;
   s = set_device(ctx);

@@ -1266,8 +1266,16 @@ int launch_chunked_search(labs_ctx* ctx, const labs_walk_cfg* cfg, labs_policy* 
   fill_params(*P, lens, cfg->bloom_log2, &ln);
   const long long n = cfg->n_walks;
   const int L = cfg->L, W = (L + 63) / 64;
+  const long long n_chunks = chunk > 0 ? (cfg->flip_budget + chunk - 1) / chunk : 0;
   unsigned char* state = nullptr;
   uint64_t* seqbuf = nullptr;
+  // the kernel logs whole words: a log that is not aligned for them is written in workspace and copied
+  uint64_t* log = state_log;
+  const size_t log_bytes = 8 * (size_t)n_chunks * (size_t)n * W;
+  if (!policy && reinterpret_cast<uintptr_t>(state_log) & 7u) {
+    log = static_cast<uint64_t*>(ws_get(ctx, kWsChunkIo, log_bytes));
+    if (!log) return LABS_ERR_NOMEM;
+  }
   float* logits = nullptr;
   if (policy) {
     P->state_stride = P->slab.bytes + 128 * walk_slots(ln.mode, ln.ns, ln.nu);
@@ -1295,11 +1303,13 @@ int launch_chunked_search(labs_ctx* ctx, const labs_walk_cfg* cfg, labs_policy* 
   if (s != LABS_OK) return s;
   if (!policy) {
     P->log_chunk = state_log || move_log ? chunk : 0;
-    P->state_log = state_log;
+    P->state_log = log;
     P->move_log = move_log;
-    return n > 0 ? run_walks(*P, ln, st) : LABS_OK;
+    s = n > 0 ? run_walks(*P, ln, st) : LABS_OK;
+    if (s == LABS_OK && log != state_log && log_bytes)
+      s = cuda_status(cudaMemcpyAsync(state_log, log, log_bytes, cudaMemcpyDeviceToDevice, st));
+    return s;
   }
-  const long long n_chunks = (cfg->flip_budget + chunk - 1) / chunk;
   P->state = state;
   P->seq_out = seqbuf;
   P->chunk = -1;  // set-up launch: every walk's first state

@@ -1,0 +1,70 @@
+/* A stand-in for the CUDA runtime, preloaded into a child process on a machine without a GPU: device memory is host
+ * memory that nothing touches, kernels do not run.  Every allocation, release and device-to-device copy is written
+ * to FAKE_CUDART_LOG; a release of something that is not live is written as "bad-free".  Allocations of more than
+ * FAKE_CUDART_LIMIT bytes fail. */
+#include <stddef.h>
+#include <stdint.h>
+#include <stdio.h>
+#include <stdlib.h>
+#include <string.h>
+
+typedef int err_t;
+enum { kMax = 4096 };
+static uintptr_t live[kMax];
+static uintptr_t next_addr = 0x100000000ull;
+
+static void note(const char* what, uintptr_t a, uintptr_t b, size_t n) {
+  const char* path = getenv("FAKE_CUDART_LOG");
+  FILE* f = path ? fopen(path, "a") : NULL;
+  if (!f) return;
+  fprintf(f, "%s %llu %llu %llu\n", what, (unsigned long long)a, (unsigned long long)b, (unsigned long long)n);
+  fclose(f);
+}
+
+err_t cudaGetDeviceCount(int* n) { *n = 1; return 0; }
+err_t cudaSetDevice(int d) { (void)d; return 0; }
+err_t cudaGetDevice(int* d) { *d = 0; return 0; }
+err_t cudaDeviceGetAttribute(int* v, int attr, int d) { (void)d; *v = attr == 97 ? 232448 : 152; return 0; }
+err_t cudaDeviceSynchronize(void) { return 0; }
+err_t cudaStreamSynchronize(void* s) { (void)s; return 0; }
+err_t cudaGetLastError(void) { return 0; }
+err_t cudaFuncSetAttribute(const void* f, int a, int v) { (void)f; (void)a; (void)v; return 0; }
+err_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void* f, int t, size_t s, unsigned g) {
+  (void)f; (void)t; (void)s; (void)g;
+  *n = 1;
+  return 0;
+}
+err_t cudaMalloc(void** p, size_t n) {
+  const char* lim = getenv("FAKE_CUDART_LIMIT");
+  *p = NULL;
+  if (lim && n > strtoull(lim, NULL, 10)) { note("no-memory", 0, 0, n); return 2; }
+  for (int i = 0; i < kMax; i++)
+    if (!live[i]) {
+      live[i] = next_addr;
+      next_addr += (n + 511) / 256 * 256;
+      *p = (void*)live[i];
+      note("malloc", live[i], 0, n);
+      return 0;
+    }
+  return 2;
+}
+err_t cudaFree(void* p) {
+  if (!p) return 0;
+  for (int i = 0; i < kMax; i++)
+    if (live[i] == (uintptr_t)p) {
+      live[i] = 0;
+      note("free", (uintptr_t)p, 0, 0);
+      return 0;
+    }
+  note("bad-free", (uintptr_t)p, 0, 0);
+  return 1;
+}
+err_t cudaMemset(void* p, int v, size_t n) { (void)p; (void)v; (void)n; return 0; }
+err_t cudaMemsetAsync(void* p, int v, size_t n, void* s) { (void)p; (void)v; (void)n; (void)s; return 0; }
+err_t cudaMemcpyAsync(void* d, const void* s, size_t n, int kind, void* st) {
+  (void)kind; (void)st;
+  note("copy", (uintptr_t)d, (uintptr_t)s, n);
+  return 0;
+}
+err_t cudaLaunchKernel(const void* f, ...) { (void)f; return 0; }
+err_t __cudaLaunchKernel(const void* f, ...) { (void)f; return 0; }
