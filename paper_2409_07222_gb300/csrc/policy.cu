@@ -743,13 +743,10 @@ int ensure_acts(labs_policy* P, long long n) {
                        kPartFloats};
   float** dst[] = {&P->x, &P->h1, &P->h2, &P->h3, &P->a, &P->logits, &P->d_logits, &P->da, &P->dh_a, &P->dh_b,
                    &P->lossv, &P->wpart, &P->kpart};
-  for (int i = 0; i < 13; i++) {
-    *dst[i] = nullptr;
-    if (cudaMalloc(dst[i], sizeof(float) * sz[i]) != cudaSuccess) {
-      P->cap_n = 0;
-      return LABS_ERR_NOMEM;
-    }
-  }
+  for (float** d : dst) *d = nullptr;  // none is left dangling where one of the allocations fails
+  P->cap_n = 0;
+  for (int i = 0; i < 13; i++)
+    if (cudaMalloc(dst[i], sizeof(float) * sz[i]) != cudaSuccess) return LABS_ERR_NOMEM;
   P->cap_n = n;
   return LABS_OK;
 }

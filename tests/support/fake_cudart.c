@@ -1,7 +1,7 @@
 /* A stand-in for the CUDA runtime, preloaded into a child process on a machine without a GPU: device memory is host
  * memory that nothing touches, kernels do not run.  Every allocation, release and device-to-device copy is written
- * to FAKE_CUDART_LOG; a release of something that is not live is written as "bad-free".  Allocations of more than
- * FAKE_CUDART_LIMIT bytes fail. */
+ * to FAKE_CUDART_LOG; a release of something that is not live is written as "bad-free".  Allocation number
+ * FAKE_CUDART_FAIL (from 1) fails. */
 #include <stddef.h>
 #include <stdint.h>
 #include <stdio.h>
@@ -35,9 +35,10 @@ err_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void*
   return 0;
 }
 err_t cudaMalloc(void** p, size_t n) {
-  const char* lim = getenv("FAKE_CUDART_LIMIT");
+  static int count;
+  const char* fail = getenv("FAKE_CUDART_FAIL");
   *p = NULL;
-  if (lim && n > strtoull(lim, NULL, 10)) { note("no-memory", 0, 0, n); return 2; }
+  if (fail && ++count == atoi(fail)) { note("no-memory", 0, 0, n); return 2; }
   for (int i = 0; i < kMax; i++)
     if (!live[i]) {
       live[i] = next_addr;
