@@ -195,6 +195,9 @@ __device__ __forceinline__ int e_bin(int E, int E_base) {
   return d < 0 ? 0 : (d >= kNB ? kNB - 1 : d);
 }
 
+// Whether a bin holds one energy only: not the window's end bins.
+__device__ __forceinline__ bool one_energy(int bin) { return bin > 0 && bin < kNB - 1; }
+
 // Block-wide sum added to *ctr with one atomic per block (every thread of the block calls it).
 __device__ __forceinline__ void block_add(long long* ctr, long long v) {
   __shared__ long long part[32];
@@ -252,19 +255,41 @@ __device__ __forceinline__ long long block_reserve(long long* ctr, int n, int si
 }
 
 // Survivor histogram of a block: the fine bins are counted one by one in global memory (a round's energies
-// spread over some hundred), the coarse ones, few and hot, in shared memory and added once.
+// spread over some hundred), the coarse ones, few and hot, in shared memory and added once.  The window's two end
+// bins hold every energy beyond it, a round's survivors all together where a search has left the window: a thread
+// counts those itself (low half: bin 0, high half: the last), and a block adds them once.
 struct CoarseCounts {
   unsigned* n;  // [kNC] shared
-  __device__ __forceinline__ explicit CoarseCounts(unsigned* shared) : n(shared) {
+  unsigned ends;
+  __device__ __forceinline__ explicit CoarseCounts(unsigned* shared) : n(shared), ends(0) {
     for (int i = threadIdx.x; i < kNC; i += blockDim.x) n[i] = 0u;
     __syncthreads();
   }
   __device__ __forceinline__ void add(unsigned* fine, int bin) {
-    atomicAdd(&fine[bin], 1u);
-    atomicAdd(&n[bin / kCoarse], 1u);
+    if (one_energy(bin)) {
+      atomicAdd(&fine[bin], 1u);
+      atomicAdd(&n[bin / kCoarse], 1u);
+    } else {
+      ends += bin ? 0x10000u : 1u;  // (a thread sees some ten entries a round)
+    }
   }
-  __device__ __forceinline__ void flush(unsigned* coarse) {
-    __syncthreads();
+  __device__ __forceinline__ void flush(unsigned* fine, unsigned* coarse) {
+    if (__syncthreads_or((int)ends)) {
+      __shared__ unsigned both[2];
+      if (threadIdx.x < 2) both[threadIdx.x] = 0u;
+      __syncthreads();
+      const unsigned lo = __reduce_add_sync(kFull, ends & 0xffffu), hi = __reduce_add_sync(kFull, ends >> 16);
+      if (lane_id() == 0) {
+        if (lo) atomicAdd(&both[0], lo);
+        if (hi) atomicAdd(&both[1], hi);
+      }
+      __syncthreads();
+      if (threadIdx.x < 2 && both[threadIdx.x]) {
+        atomicAdd(&fine[threadIdx.x ? kNB - 1 : 0], both[threadIdx.x]);
+        atomicAdd(&n[threadIdx.x ? kNC - 1 : 0], both[threadIdx.x]);
+      }
+      __syncthreads();
+    }
     for (int i = threadIdx.x; i < kNC; i += blockDim.x)
       if (n[i]) atomicAdd(&coarse[i], n[i]);
   }
@@ -556,6 +581,7 @@ __device__ __forceinline__ void load_energies(const int32_t* src, long long firs
 __device__ __forceinline__ void append_candidates(const PqBufs& b, unsigned is, const int (&E)[kPer], long long first,
                                                   bool survivors) {
   if (!__syncthreads_or((int)is)) return;
+  const bool grouped = one_energy(b.st->sel_bin);
   int total, before;
   long long o = block_reserve(&b.st->cand_cnt, __popc(is), 1, &total, &before);
   o += before;
@@ -569,7 +595,7 @@ __device__ __forceinline__ void append_candidates(const PqBufs& b, unsigned is, 
         b.candId[o] = survivors ? -(int32_t)(first + e) - 1 : (int32_t)(first + e);
         b.cE[o] = E[e];
         b.cF[o] = fp;
-        atomicAdd(&b.hF[fp >> 54], 1u);
+        if (grouped) atomicAdd(&b.hF[fp >> 54], 1u);
       }
       o++;
     }
@@ -642,9 +668,14 @@ __global__ void __launch_bounds__(256) pq_pool_kernel(PqBufs b, unsigned pool_bl
 // The sel_need smallest (E, fp) keys among the boundary candidates, whose keys are distinct.  A bin that is not
 // clamped holds one energy: the counts of the fingerprints' first ten bits give the group that holds the
 // boundary; all blocks collect that group's fingerprints (a thousandth of the candidates), and the last one to
-// finish ranks them against each other.  Otherwise (a clamped bin, or a group beyond kGroup) it does a radix
-// select over the full 96-bit key.
+// finish ranks them against each other.  Otherwise (a clamped bin, or a group beyond kGroup) the last block narrows
+// the 96-bit key down, eleven bits a pass over the candidates, and ranks those that share the boundary's bits as
+// soon as they fit in shared memory: one pass and the gathering one where the energies are spread.  Measured on 4
+// random seeds of L = 527 (4,000 pops of 64 a round, cap 65,536: 30,000 candidates a select): 10.5 ms in all; 24.3 ms
+// with twelve passes of a byte each, one global atomic per survivor of the end bin and one block to apply the cut,
+// and 15.7 ms with a full pass per byte until 8,192 were left.
 constexpr int kGroup = 4096;
+constexpr int kDigit = 11, kStage = 2048;  // bits a pass; candidates ranked in shared memory
 template <bool POP>
 __global__ void __launch_bounds__(kSelThreads) pq_boundary_kernel(PqBufs b) {
   PqState* st = b.st;
@@ -653,13 +684,12 @@ __global__ void __launch_bounds__(kSelThreads) pq_boundary_kernel(PqBufs b) {
   __shared__ int s_bin, s_n, s_E, s_last;
   __shared__ long long s_need;
   __shared__ unsigned long long s_fp;
-  __shared__ unsigned s_hist[256];
+  __shared__ unsigned s_hist[1 << kDigit];
   __shared__ unsigned wsum[kSelThreads / 32];
   const int t = threadIdx.x, lane = lane_id();
   const long long n = min(st->cand_cnt, b.cand_cap);
   const long long need = st->sel_need;
   const int sel = st->sel_bin;
-  const bool one_energy = sel > 0 && sel < kNB - 1;
   if (t == 0) {
     s_n = 0;
     s_bin = 0;
@@ -684,7 +714,7 @@ __global__ void __launch_bounds__(kSelThreads) pq_boundary_kernel(PqBufs b) {
   }
   __syncthreads();
   const int gb = s_bin;
-  const bool grouped = one_energy && b.hF[gb] <= (unsigned)kGroup;
+  const bool grouped = one_energy(sel) && b.hF[gb] <= (unsigned)kGroup;
   const long long stride = (long long)gridDim.x * kSelThreads;
   if (grouped)
     for (long long i0 = (long long)blockIdx.x * kSelThreads; i0 < n; i0 += 4 * stride) {
@@ -719,37 +749,95 @@ __global__ void __launch_bounds__(kSelThreads) pq_boundary_kernel(PqBufs b) {
     }
     __syncthreads();
   } else {
-    // most-significant-digit-first over the 96-bit key: four energy bytes, then eight fingerprint bytes
-    uint64_t preE = 0, preF = 0;
-    long long k = need;
-    for (int d = 0; d < 12; d++) {
-      if (t < 256) s_hist[t] = 0u;
-      __syncthreads();
-      for (long long i = t; i < n; i += kSelThreads) {
-        const uint64_t ue = (uint32_t)b.cE[i], f = b.cF[i];
-        const bool match = d < 4 ? (d == 0 || (ue >> (32 - 8 * d)) == (preE >> (32 - 8 * d)))
-                                 : ue == preE && (d == 4 || (f >> (96 - 8 * d)) == (preF >> (96 - 8 * d)));
-        if (match) atomicAdd(&s_hist[d < 4 ? (ue >> (24 - 8 * d)) & 255 : (f >> (88 - 8 * d)) & 255], 1u);
+    // Keys that agree with (preE, preF) in all bits from (sE, sF) up are still in question; the boundary is the k-th
+    // of them.  Energies of the lower end bin are at most E_base, all below 2^26.
+    uint64_t preF = 0;
+    uint32_t preE = one_energy(sel) ? (uint32_t)s_E : 0u;
+    int sE = one_energy(sel) ? 0 : (sel == 0 ? 32 - __clz(st->E_base) : 26), sF = 64;
+    long long k = need, left = n;
+    auto in_question = [&](uint32_t e, uint64_t f) {
+      return e >> sE == preE >> sE && (sF == 64 || (f >> sF) == (preF >> sF));
+    };
+    auto each = [&](auto&& fn) {  // fn(candidate, energy); a thread's quads are loaded four at a time
+      const long long nq = (n + 3) >> 2;
+#pragma unroll 4
+      for (long long q = t; q < nq; q += kSelThreads) {
+        const int4 e4 = reinterpret_cast<const int4*>(b.cE)[q];
+        const uint32_t e[4] = {(uint32_t)e4.x, (uint32_t)e4.y, (uint32_t)e4.z, (uint32_t)e4.w};
+#pragma unroll
+        for (int j = 0; j < 4; j++)
+          if (4 * q + j < n) fn(4 * q + j, e[j]);
       }
+    };
+    while (left > kStage && sE + sF > 0) {
+      // the next bits: of the energy, then of the fingerprint
+      const int nE = sE ? max(sE - kDigit, 0) : 0, nF = sE ? 64 : max(sF - kDigit, 0);
+      const bool fp_bits = sE == 0;
+      for (int i = t; i < 1 << kDigit; i += kSelThreads) s_hist[i] = 0u;
       __syncthreads();
-      if (t == 0) {
-        long long before = 0;
-        int digit = 0;
-        while (digit < 255 && before + (long long)s_hist[digit] < k) before += s_hist[digit++];
-        s_bin = digit;
-        s_need = k - before;
+      each([&](long long i, uint32_t e) {
+        const uint64_t f = fp_bits ? b.cF[i] : 0ull;
+        if (in_question(e, f)) {
+          const unsigned digit = fp_bits ? (unsigned)(f >> nF) : e >> nE;
+          atomicAdd(&s_hist[digit & ((1u << kDigit) - 1u)], 1u);
+        }
+      });
+      __syncthreads();
+      // the digit where the count reaches k: two bins a thread
+      const unsigned own0 = s_hist[2 * t], own1 = s_hist[2 * t + 1];
+      unsigned c = own0 + own1;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned v = __shfl_up_sync(kFull, c, o);
+        if (lane >= o) c += v;
+      }
+      if (lane == 31) wsum[t >> 5] = c;
+      __syncthreads();
+      for (int w = 0; w < t >> 5; w++) c += wsum[w];
+      const long long before = (long long)c - own0 - own1;
+      if (before < k && (long long)c >= k) {
+        const bool second = before + own0 < k;
+        s_bin = 2 * t + (second ? 1 : 0);
+        s_need = k - before - (second ? own0 : 0u);
+        s_n = (int)(second ? own1 : own0);
       }
       __syncthreads();
       k = s_need;
-      if (d < 4)
-        preE |= (uint64_t)s_bin << (24 - 8 * d);
+      left = s_n;
+      if (fp_bits)
+        preF |= (uint64_t)s_bin << nF;
       else
-        preF |= (uint64_t)s_bin << (88 - 8 * d);
+        preE |= (uint32_t)s_bin << nE;
+      sE = nE;
+      sF = nF;
       __syncthreads();
     }
-    if (t == 0) {
-      s_E = (int)(uint32_t)preE;
-      s_fp = preF;
+    // the candidates left, ranked against each other (grp: their fingerprints, behind them their energies)
+    int* grpE = reinterpret_cast<int*>(grp + kStage);
+    if (t == 0) s_n = 0;
+    __syncthreads();
+    each([&](long long i, uint32_t e) {
+      if (e >> sE != preE >> sE) return;
+      const uint64_t f = b.cF[i];
+      if (in_question(e, f)) {
+        const int w = atomicAdd(&s_n, 1);
+        if (w < kStage) {
+          grp[w] = f;
+          grpE[w] = (int)e;
+        }
+      }
+    });
+    __syncthreads();
+    const int m = min(s_n, kStage);
+    for (int i = t; i < m; i += kSelThreads) {
+      const uint64_t f = grp[i];
+      const int e = grpE[i];
+      int r = 0;
+      for (int j = 0; j < m; j++) r += key_le(grpE[j], grp[j], e, f) ? 1 : 0;
+      if (r == (int)k) {
+        s_E = e;
+        s_fp = f;
+      }
     }
     __syncthreads();
   }
@@ -1026,7 +1114,7 @@ __global__ void __launch_bounds__(256, 6) pq_dedup_kernel(PqBufs b) {
       }
     }
   }
-  counts.flush(b.hU2);
+  counts.flush(b.hU, b.hU2);
   block_add(&st->nU, kept);
   block_min(&st->minE_round, mE);
   block_add(&st->nU_low, low);
@@ -1053,7 +1141,7 @@ __global__ void __launch_bounds__(kSelThreads) pq_cut_kernel(PqBufs b) {
           if (bin > pmax) counts.add(b.hU, bin);
         }
     }
-    counts.flush(b.hU2);
+    counts.flush(b.hU, b.hU2);
   }
   __threadfence();
   __syncthreads();
@@ -1074,7 +1162,9 @@ __global__ void __launch_bounds__(kSelThreads) pq_cut_kernel(PqBufs b) {
   if (!fits) select_bin<true>(b, b.cap);
 }
 
-// The histogram's energy window, from the smallest seed energy (improvements stay far inside it).
+// The histogram's energy window, from the smallest seed energy: 65,536 below it and above it.  From sieved seeds a
+// search stays inside; from random ones at L = 527 the best is below after some thirty rounds, and from then on most
+// entries lie in bin 0 (from constant ones in either end bin).
 __global__ void pq_set_window_kernel(PqBufs b) {
   PqState* st = b.st;
   st->E_base = st->minE_round == INT32_MAX ? 0 : max(0, st->minE_round - kNB / 2);
@@ -1247,8 +1337,11 @@ int launch_pq_refine(labs_ctx* ctx, const labs_pq_cfg* cfg, const uint64_t* seed
   const unsigned g_dense =
       (unsigned)std::max(1ll, std::min<long long>((n_dense + 1023) / 1024, (long long)ctx->num_sms * 8));
 
-  // boundary candidates: a bin's share of the pool and the survivors, a thousandth or so
+  // boundary candidates: a bin's share of the pool and the survivors, a thousandth or so (collected by g_cand
+  // blocks), but all of them where they lie in an end bin of the window (applied by g_apply blocks, a barrier for
+  // every 1,024 of them)
   const unsigned g_cand = (unsigned)std::max(1ll, std::min<long long>((cap + n_dense) / 65536, ctx->num_sms / 2));
+  const unsigned g_apply = (unsigned)std::max(1ll, std::min<long long>((cap + n_dense) / 4096, ctx->num_sms));
 
   // The survivor path, shared by the seeds and every round: dedup, cut, eviction, admission, best, and the next
   // round's beginning.
@@ -1262,7 +1355,7 @@ int launch_pq_refine(labs_ctx* ctx, const labs_pq_cfg* cfg, const uint64_t* seed
     pq_cut_kernel<<<std::max(1u, g_cand_dense / 4), kSelThreads, 0, s>>>(b);
     pq_pool_kernel<false><<<g_pool + g_cand_dense, 256, 0, s>>>(b, g_pool);
     pq_boundary_kernel<false><<<g_cand, kSelThreads, 0, s>>>(b);
-    pq_boundary_apply_kernel<false><<<g_cand, kSelThreads, 0, s>>>(b);
+    pq_boundary_apply_kernel<false><<<g_apply, kSelThreads, 0, s>>>(b);
     if (seed) {
       pq_admit_kernel<true><<<g_dense, 256, 0, s>>>(b);
       pq_finish_kernel<true><<<1, kSelThreads, 0, s>>>(b);
@@ -1319,7 +1412,7 @@ int launch_pq_refine(labs_ctx* ctx, const labs_pq_cfg* cfg, const uint64_t* seed
     cudaStream_t cs = ctx->capture_stream;
     pq_pool_kernel<true><<<g_pool, 256, 0, cs>>>(b, g_pool);
     pq_boundary_kernel<true><<<g_cand, kSelThreads, 0, cs>>>(b);
-    pq_boundary_apply_kernel<true><<<g_cand, kSelThreads, 0, cs>>>(b);
+    pq_boundary_apply_kernel<true><<<g_apply, kSelThreads, 0, cs>>>(b);
     expand<<<exp_blocks, 32 * kPqWarps, exp_smem, cs>>>(b, ep);
     survivor_path(false, cs);
   }
