@@ -70,7 +70,8 @@ int labs_energy_batch(labs_ctx* ctx, const uint64_t* seqs, int L, int64_t n, int
  *             s_m and its mirror s_{L+1-m} (the centre k+1 alone); dE[q][m-1] holds its Delta E.
  *   Entries outside the free range are INT32_MAX.  dE is [n][L] int32, device.
  *   C      nullable; [n][L-1] int32 correlation tables as written by labs_energy_batch.  When given,
- *          the kernel uses them instead of rebuilding them (results are identical when they match).
+ *          the results are formed from them (the low 16 bits of each entry, exactly), which are the
+ *          sequence's own when they match; other tables are slower.
  * Errors: LABS_ERR_INVALID_ARG for L outside [2, 576], odd/even mismatch with `skew`, p out of range.
  */
 int labs_flip_deltas(labs_ctx* ctx, const uint64_t* seqs, const int32_t* C, int L, int64_t n, int skew, int p,

@@ -25,10 +25,43 @@ struct FdPlan {
   ScanMmaPlan mma;
   int q, x, z, words;  // q: two copies; x: class sequences; z: int16 tables; bits, classes in front
 };
-constexpr int kFdBits = 0, kFdClass = kBitWords, kFdRev = kFdClass + 2 * kClassWords, kFdTables = kFdRev + 2 * kClassWords;
+constexpr int kFdBits = 0, kFdClass = kBitWords, kFdRev = kFdClass + 2 * kClassWords,
+              kFdOdd = kFdRev + 2 * kClassWords, kFdTables = kFdOdd + 4;  // kFdOdd: the warp met such a table
 
-// NC: 32-bit words of the longer parity class; NT: tiles of 128 neighbours per class.
-template <int NC, int NT>
+// Entries of a table of up to these bits (and a sign) are exact as FP16 operands: a sequence's own are (|C| <= 575).
+constexpr int kHalfBits = 11;
+
+// A caller's table is used as it is given (16 bits of every entry).  A warp that met one that the kernels' fast way
+// does not serve goes over its sequences once more: Delta E of the neighbours p + 1 .. last by plain loops over the
+// lags that are multiples of lam (2: skew pairs; their mirror's product drops out).  No table of a sequence's own
+// correlations comes here, so this is small rather than fast, and behind the loop that needs the registers: inside
+// it, 8,192 unrestricted sequences of L = 576 took 44.5 us with a table, behind it 42.3 (41.4 without the check).
+__device__ __forceinline__ void odd_tables(const uint64_t* seqs, const int32_t* Cin, int L, int64_t n, int lam, int p,
+                                           int last, uint32_t* bits, int32_t* dE) {
+  const int W = (L + 63) >> 6, lane = lane_id();
+  const int64_t warps_total = (int64_t)gridDim.x * kFdWarps;
+  auto s_at = [&](int i) { return i < 1 || i > L ? 0 : ((bits[(i - 1) >> 5] >> ((i - 1) & 31)) & 1u) ? 1 : -1; };
+  for (int64_t s = (int64_t)blockIdx.x * kFdWarps + (threadIdx.x >> 5); s < n; s += warps_total) {
+    const int32_t* C = Cin + s * (L - 1);
+    if (lane < (L + 31) >> 5) bits[lane] = reinterpret_cast<const uint32_t*>(seqs + s * W)[lane];
+    __syncwarp();
+    for (int m = p + 1 + lane; m <= last; m += 32) {
+      const int mirror = lam == 2 && 2 * m != L + 1 ? L + 1 - m : 0, alpha = mirror ? 4 : 2;
+      const int sm = s_at(m);
+      int linear = 0, square = 0;  // C_k changes by - alpha s_m y
+      for (int k = lam; k < L; k += lam) {
+        const int y = (m + k == mirror ? 0 : s_at(m + k)) + s_at(m - k);
+        linear += (int16_t)C[k - 1] * y;
+        square += y * y;
+      }
+      dE[s * L + m - 1] = alpha * (alpha * square - 2 * sm * linear);
+    }
+    __syncwarp();
+  }
+}
+
+// NC: 32-bit words of the longer parity class; NT: tiles of 128 neighbours per class; GIVEN: with a caller's table.
+template <int NC, int NT, bool GIVEN>
 __global__ void __launch_bounds__(32 * kFdWarps, NT == 1 ? 6 : 5) flip_deltas_skew_kernel(const uint64_t* __restrict__ seqs,
                                                                           const int32_t* __restrict__ Cin, int L, int64_t n,
                                                                           int p, FdPlan fp, int32_t* __restrict__ dE) {
@@ -58,17 +91,19 @@ __global__ void __launch_bounds__(32 * kFdWarps, NT == 1 ? 6 : 5) flip_deltas_sk
     // class correlations at lag g (twice the class index): positions of one parity are one class of distances
     int16_t* zo = e_odd ? z1 : z0;
     int16_t* ze = e_odd ? z0 : z1;
+    int odd = 0;  // whether the given table differs from the sequence's own, which the sums below are formed from
     corr_words<NC>(cw, cw, n_odd, [&](int g, int r) { zo[g] = (int16_t)r; });
     corr_words<NC>(cw + kClassWords, cw + kClassWords, n_even, [&](int g, int r) {
       const int r_odd = zo[g];  // the lane's own
-      int cg = r_odd + r;
-      if (Cin && g >= 1 && g <= k) cg = Cin[s * (L - 1) + 2 * g - 1];
+      const int cg = r_odd + r;
+      if (GIVEN && g >= 1 && g <= k) odd |= Cin[s * (L - 1) + 2 * g - 1] ^ cg;
       zo[g] = (int16_t)(2 * r_odd + cg);
       ze[g] = (int16_t)(2 * r + cg);
       if (g >= 1 && g <= k) put_q(q, fp.mma, g, cg);
     });
     put_x(slab + fp.x, cw, n_odd);
     put_x(slab + fp.x + fp.mma.x_words, cw + kClassWords, n_even);
+    if (GIVEN && odd) slab[kFdOdd] = 1u;
     __syncwarp();
     float acc[2][NT][4];
     scan_mma<2, NT>(q, xs, fp.mma, n_odd, acc);
@@ -102,10 +137,11 @@ __global__ void __launch_bounds__(32 * kFdWarps, NT == 1 ? 6 : 5) flip_deltas_sk
     }
     __syncwarp();
   }
+  if (GIVEN && slab[kFdOdd]) odd_tables(seqs, Cin, L, n, 2, p, c, bits, dE);
 }
 
-// NW: 32-bit words of the sequence; NT: tiles of 128 neighbours.
-template <int NW, int NT>
+// NW: 32-bit words of the sequence; NT: tiles of 128 neighbours; GIVEN: with a caller's table.
+template <int NW, int NT, bool GIVEN>
 __global__ void __launch_bounds__(32 * kFdWarps, NT <= 2 ? 6 : 4) flip_deltas_kernel(const uint64_t* __restrict__ seqs,
                                                                      const int32_t* __restrict__ Cin, int L, int64_t n,
                                                                      int p, FdPlan fp, int32_t* __restrict__ dE) {
@@ -126,8 +162,14 @@ __global__ void __launch_bounds__(32 * kFdWarps, NT <= 2 ? 6 : 4) flip_deltas_ke
       bits[lane] = rem < 32 ? w & ((1u << rem) - 1u) : w;
     }
     __syncwarp();
-    if (Cin) {
-      for (int d = lane + 1; d < L; d += 32) put_q(q, fp.mma, d, Cin[s * (L - 1) + d - 1]);
+    if constexpr (GIVEN) {
+      int odd = 0;  // ones above kHalfBits where an entry has more bits
+      for (int d = lane + 1; d < L; d += 32) {
+        const int cd = Cin[s * (L - 1) + d - 1];
+        odd |= cd ^ (cd >> 31);
+        put_q(q, fp.mma, d, cd);
+      }
+      if (odd >> kHalfBits) slab[kFdOdd] = 1u;
     } else {
       corr_words<NW>(bits, bits, L, [&](int d, int cd) {
         if (d >= 1 && d < L) put_q(q, fp.mma, d, cd);
@@ -156,6 +198,7 @@ __global__ void __launch_bounds__(32 * kFdWarps, NT <= 2 ? 6 : 4) flip_deltas_ke
     }
     __syncwarp();
   }
+  if (GIVEN && slab[kFdOdd]) odd_tables(seqs, Cin, L, n, 1, p, L, bits, dE);
 }
 
 template <class Kernel>
@@ -197,14 +240,18 @@ int launch_flip_deltas(labs_ctx* ctx, const uint64_t* seqs, const int32_t* C, in
       constexpr int kMost = (16 * NW / 2 + 63 + 128) / 128;  // tiles when nothing is fixed, j0 rounded down
       if constexpr (kMost >= 2)
         if (fp.mma.nt == 2)
-          return launch_fd(ctx, flip_deltas_skew_kernel<NC, 2>, seqs, C, L, n, p, fp, dE_out, st);
-      return launch_fd(ctx, flip_deltas_skew_kernel<NC, 1>, seqs, C, L, n, p, fp, dE_out, st);
+          return launch_fd(ctx, C ? flip_deltas_skew_kernel<NC, 2, true> : flip_deltas_skew_kernel<NC, 2, false>, seqs, C, L,
+                           n, p, fp, dE_out, st);
+      return launch_fd(ctx, C ? flip_deltas_skew_kernel<NC, 1, true> : flip_deltas_skew_kernel<NC, 1, false>, seqs, C, L, n,
+                       p, fp, dE_out, st);
     }
     fp.words = (fp.z + L / 2 + 1 + 3) / 4 * 4;  // v[1 .. L]
     constexpr int kMost = NW / 4 + 1;  // tiles when nothing is fixed
     auto run = [&](auto nt) {
       constexpr int NT = decltype(nt)::value;
-      if constexpr (NT <= kMost) return launch_fd(ctx, flip_deltas_kernel<NW, NT>, seqs, C, L, n, p, fp, dE_out, st);
+      if constexpr (NT <= kMost)
+        return launch_fd(ctx, C ? flip_deltas_kernel<NW, NT, true> : flip_deltas_kernel<NW, NT, false>, seqs, C, L, n, p, fp,
+                         dE_out, st);
       return (int)LABS_ERR_INVALID_ARG;
     };
     switch (fp.mma.nt) {
