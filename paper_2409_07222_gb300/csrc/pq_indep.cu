@@ -218,15 +218,19 @@ struct IndepPlan {
 };
 constexpr int kInP = 0, kInC = 24, kInClass = 48, kInRev = kInClass + 2 * kClassWords, kInTables = kInRev + 2 * kClassWords;
 
-// Seven blocks an SM hold 28 candidates (72 registers a thread, 7.7 KB of slab a warp at L = 451).
-template <int NW, bool PAIRS>
-__global__ void __launch_bounds__(32 * kIWarps, 7) pq_indep_kernel(IndepArgs a, IndepPlan ip) {
+// Seven blocks an SM hold 28 candidates (72 registers a thread, 7.7 KB of slab a warp at L = 451), 4,256 on the chip.
+// Beyond 512 positions the slab leaves room for six blocks (80 registers), 3,648 candidates.  V_IN_Q (compiled there): V is formed
+// first, where the table of q comes to lie, and a lane keeps its outputs' values in registers, so that seven blocks
+// fit again; a pop takes longer (more registers saved).
+template <int NW, bool PAIRS, bool V_IN_Q>
+__global__ void __launch_bounds__(32 * kIWarps, NW > 16 && !V_IN_Q ? 6 : 7) pq_indep_kernel(IndepArgs a, IndepPlan ip) {
   constexpr int NT = (NW + 3) / 4;
   extern __shared__ __align__(16) uint32_t in_smem[];
   uint32_t* slab = in_smem + (size_t)(threadIdx.x >> 5) * ip.words;
   uint32_t *pbits = slab + kInP, *cbits = slab + kInC, *cw = slab + kInClass, *rw = slab + kInRev;
   uint32_t *qt = slab + ip.q, *xt = slab + ip.x;
-  int16_t* v = reinterpret_cast<int16_t*>(slab + ip.v);
+  // v[1 .. L]; in q: its elements at distances -(L - 1) .. 0, all of which but q(0) = 0 are written for every pivot
+  int16_t* v = V_IN_Q ? reinterpret_cast<int16_t*>(qt) + ip.mma.off - a.L : reinterpret_cast<int16_t*>(slab + ip.v);
   const int lane = lane_id();
   const int slot = blockIdx.x * kIWarps + (threadIdx.x >> 5);
   Node* const arena = a.arena + slot * a.arena_cap;
@@ -344,12 +348,29 @@ __global__ void __launch_bounds__(32 * kIWarps, 7) pq_indep_kernel(IndepArgs a, 
         __syncwarp();
       }
       // ---- correlations, V and the neighbours' sums
+      auto output = [&](int T, int r) { return 128 * T + 32 * (lane & 3) + (lane >> 2) + 16 * (r & 1) + 8 * (r >> 1) + 1; };
+      uint32_t vr[V_IN_Q ? 2 * NT : 1];  // V of the lane's outputs, two a word
+      if constexpr (V_IN_Q) {
+        split_classes(pbits, cw);
+        self_convolution<(NW + 1) / 2>(cw, rw, a.L, v);
+#pragma unroll
+        for (int i = 0; i < 2 * NT; i++) {
+          const int m0 = output(i >> 1, 2 * (i & 1)), m1 = output(i >> 1, 2 * (i & 1) + 1);
+          vr[i] = (m0 <= a.L ? (uint32_t)(uint16_t)v[m0] : 0u) | (m1 <= a.L ? (uint32_t)(uint16_t)v[m1] << 16 : 0u);
+        }
+        __syncwarp();
+        if (lane == 0) v[a.L] = 0;  // q(0)
+      }
       corr_words<NW>(pbits, pbits, a.L, [&](int d, int cd) {
         if (d >= 1 && d < a.L) put_q(qt, ip.mma, d, cd);
       });
       put_x(xt, pbits, a.L);
-      split_classes(pbits, cw);
-      self_convolution<(NW + 1) / 2>(cw, rw, a.L, v);
+      if constexpr (!V_IN_Q) {
+        split_classes(pbits, cw);
+        self_convolution<(NW + 1) / 2>(cw, rw, a.L, v);
+      } else {
+        __syncwarp();
+      }
       float acc[1][NT][4];
       scan_mma<1, NT>(qt, xs, ip.mma, a.L, acc);
       Node* run = arena + top;
@@ -367,7 +388,7 @@ __global__ void __launch_bounds__(32 * kIWarps, 7) pq_indep_kernel(IndepArgs a, 
         uint64_t fv[8];
 #pragma unroll
         for (int i = 0; i < 8; i++) {
-          const int T = T0 + (i >> 2), m = 128 * T + 32 * (lane & 3) + (lane >> 2) + 16 * (i & 1) + 8 * ((i >> 1) & 1) + 1;
+          const int T = T0 + (i >> 2), m = output(T, i & 3);
           fv[i] = kEmpty;
           hv[i] = kEmpty;
           if (T < NT && m <= a.L) {
@@ -380,7 +401,7 @@ __global__ void __launch_bounds__(32 * kIWarps, 7) pq_indep_kernel(IndepArgs a, 
         for (int i = 0; i < 8; i++) {
           const int T = T0 + (i >> 2);
           if (T >= NT) break;
-          const int jl = 128 * T + 32 * (lane & 3) + (lane >> 2) + 16 * (i & 1) + 8 * ((i >> 1) & 1), m = jl + 1;
+          const int m = output(T, i & 3), jl = m - 1;
           bool fresh = false;
           if (m <= a.L) {
             if (PAIRS) {
@@ -397,7 +418,8 @@ __global__ void __launch_bounds__(32 * kIWarps, 7) pq_indep_kernel(IndepArgs a, 
           const unsigned who = __ballot_sync(kFull, fresh);
           if (fresh) {
             const int tm = (int)acc[0][T][i & 3];
-            const int E = pE + 4 * ((int)v[m] + a.L - 2 - ((pbits[jl >> 5] >> (jl & 31) & 1u) ? tm : -tm));
+            const int vm = V_IN_Q ? (int)(int16_t)(vr[V_IN_Q ? 2 * T + ((i & 3) >> 1) : 0] >> (16 * (i & 1))) : (int)v[m];
+            const int E = pE + 4 * (vm + a.L - 2 - ((pbits[jl >> 5] >> (jl & 31) & 1u) ? tm : -tm));
             const int k = nu + __popc(who & ((1u << lane) - 1u));
             run[k] = Node{E, link0 | jl, fv[i]};
             if (kless(E, fv[i], rE, rf)) {
@@ -529,21 +551,39 @@ int launch_pq_independent(labs_ctx* ctx, const labs_pq_indep_cfg* cfg, const uin
   ip.q = kInTables;
   ip.x = ip.q + 2 * ip.mma.q_words;
   ip.v = ip.x + ip.mma.x_words;
-  ip.words = (ip.v + L / 2 + 1 + 3) / 4 * 4;  // v[1 .. L]
-  const size_t smem = sizeof(uint32_t) * (size_t)ip.words * kIWarps;
   void (*kern)(IndepArgs, IndepPlan) = nullptr;
-  const int ks = by_words((L + 31) >> 5, [&](auto nw) {
-    constexpr int NW = decltype(nw)::value;
-    kern = pairs ? pq_indep_kernel<NW, true> : pq_indep_kernel<NW, false>;
-    return cuda_status(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  });
-  int per_sm = 0;
-  if (ks != LABS_OK || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * kIWarps, smem) != cudaSuccess ||
-      per_sm < 1)
-    return LABS_ERR_CUDA;
-  long long blocks = std::min<long long>((long long)per_sm * ctx->num_sms, ((long long)n + kIWarps - 1) / kIWarps);
-  blocks = std::min<long long>(blocks, (long long)(budget / (per_slot * kIWarps)));
-  if (blocks < 1) return LABS_ERR_NOMEM;
+  size_t smem = 0;
+  long long blocks = 0, rounds = 0;
+  // the plain form, or with V in q where that lets all candidates run in fewer rounds (4,096 of L = 527, T_r = 4, 64
+  // pops: 35 ms in two rounds, 24.4 ms in one; 3,600, one round either way: 20.4 and 22.5 ms)
+  for (int v_in_q = 0; v_in_q < 2; v_in_q++) {
+    const int words = ip.v + (v_in_q ? 0 : L / 2 + 1);  // v[1 .. L]
+    const size_t bytes = sizeof(uint32_t) * (size_t)((words + 3) / 4 * 4) * kIWarps;
+    void (*k)(IndepArgs, IndepPlan) = nullptr;
+    const int ks = by_words((L + 31) >> 5, [&](auto nw) {
+      constexpr int NW = decltype(nw)::value;
+      if constexpr (NW > 16)
+        if (v_in_q) k = pairs ? pq_indep_kernel<NW, true, true> : pq_indep_kernel<NW, false, true>;
+      if (!v_in_q) k = pairs ? pq_indep_kernel<NW, true, false> : pq_indep_kernel<NW, false, false>;
+      return k ? cuda_status(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) : LABS_OK;
+    });
+    if (!k && ks == LABS_OK) break;  // compiled in the plain form only
+    int per_sm = 0;
+    if (ks != LABS_OK || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 32 * kIWarps, bytes) != cudaSuccess ||
+        per_sm < 1)
+      return LABS_ERR_CUDA;
+    long long b = std::min<long long>((long long)per_sm * ctx->num_sms, ((long long)n + kIWarps - 1) / kIWarps);
+    b = std::min<long long>(b, (long long)(budget / (per_slot * kIWarps)));
+    if (b < 1) return LABS_ERR_NOMEM;
+    const long long r = ((long long)n + b * kIWarps - 1) / (b * kIWarps);
+    if (kern && r >= rounds) break;
+    kern = k;
+    smem = bytes;
+    blocks = b;
+    rounds = r;
+    ip.words = (int)(bytes / sizeof(uint32_t)) / kIWarps;
+    if (r == 1) break;
+  }
   const size_t slots = (size_t)blocks * kIWarps;
   size_t off = 0;
   auto take = [&](size_t bytes) {
