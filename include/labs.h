@@ -168,7 +168,9 @@ typedef struct {
   int64_t thresh_rank;      /* per-length sieve bound: 0-based rank */
   int32_t E_target;         /* per-walk first flip reaching E <= E_target (walk_stats[5]); INT32_MIN = off */
   int32_t tile_m;           /* as in labs_walk_cfg */
-  int32_t warps_per_cta;    /* 0: chosen by the library; 1..8 */
+  int32_t warps_per_cta;    /* 0: autotuned (a timed trial on the first use of a length set and its walk counts,
+                               which waits for the stream; kept in the context; none for a search shorter than
+                               the trial, some 10^7 flips, or while `stream` is being captured); 1..8 */
   int32_t use_graph;        /* 1: capture the step into a CUDA graph on first use and replay it */
 } labs_batch_cfg;
 

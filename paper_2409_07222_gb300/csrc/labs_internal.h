@@ -20,6 +20,7 @@ struct LabsTraceRange {
 #define LABS_TRACE(name) LabsTraceRange labs_trace_range_(name)
 
 constexpr int kWorkspaces = 9;
+constexpr int kMaxTuned = 64;  // batched length sets whose walks per block are kept (the oldest is replaced)
 
 struct labs_ctx {
   int device;
@@ -32,6 +33,10 @@ struct labs_ctx {
   cudaGraphExec_t graph_exec;
   uint64_t graph_key;
   cudaStream_t capture_stream;
+  // walks per block of a batched length set, from its timed trial
+  uint64_t tuned_key[kMaxTuned];
+  int tuned_warps[kMaxTuned];
+  int n_tuned;
 };
 
 namespace labsg {

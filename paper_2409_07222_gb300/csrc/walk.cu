@@ -1357,6 +1357,65 @@ int issue_batch(labs_ctx* ctx, const labs_batch_cfg* cfg, const std::vector<LenS
   return s;
 }
 
+// Whether `st` is being captured (or cannot be asked for it now).
+bool capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &status) == cudaSuccess) return status != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return true;
+}
+
+// Walks per block of a batch by a timed trial: the number that plan_launch chose against the next two multiples of
+// four below (an SM has four schedulers), each with a proportional part of the walks that fills its blocks kTrialRounds
+// times, for kTrialFlips flips, the sieve closed.  How many walks an SM should hold depends on the lengths in the
+// launch: L = 450 .. 527, 42,000 walks x 500 flips: 33.4 ms with 23 (as many as fit), 30.7 with 20, 33.1 with 16; L =
+// 500 .. 576: 38.2 with 22, 39.6 and 37.2; L = 64 .. 141: 13.6 with 32, 14.8 with 24.  Slots a lane need no trial: the
+// smallest number that holds the lengths is the fastest (one step more: 8 to 100% slower).  Candidates of the trial go
+// to `out`, which the search then overwrites.
+constexpr int kTrialFlips = 256, kTrialRounds = 3;
+int trial_warps(labs_ctx* ctx, const labs_batch_cfg* cfg, const std::vector<LenSpec>& lens, const WalkParams& P,
+                const Launch& ln, cudaStream_t st, int* warps) {
+  std::unique_ptr<WalkParams> Q(new (std::nothrow) WalkParams(P));
+  if (!Q) return LABS_ERR_NOMEM;
+  Q->flip_budget = std::min<int64_t>(cfg->flip_budget, kTrialFlips);
+  Q->walk_stats = nullptr;
+  Q->E_thr_dev = nullptr;
+  cudaEvent_t e0 = nullptr, e1 = nullptr;
+  if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
+    if (e0) cudaEventDestroy(e0);
+    return LABS_ERR_CUDA;
+  }
+  double best = 0;
+  int s = LABS_OK;
+  for (int turn = -1; turn < 3 && s == LABS_OK; turn++) {  // turn -1: untimed
+    const int w = turn < 1 ? ln.warps : (ln.warps - 1) / 4 * 4 - 4 * (turn - 1);
+    if (w < 4) break;
+    std::vector<LenSpec> part = lens;
+    const double share = std::min(1.0, (double)kTrialRounds * w * ctx->num_sms / (double)P.n_items);
+    for (LenSpec& e : part) e.walks = e.walks > 0 ? std::max<int64_t>(1, (int64_t)(share * (double)e.walks)) : 0;
+    Launch q;
+    fill_params(*Q, part, cfg->bloom_log2, &q);
+    for (int i = 0; i < Q->n_len; i++) Q->len[i].E_thr_value = INT32_MIN;
+    s = plan_launch(ctx, *Q, w, false, &q);
+    if (s == LABS_OK) s = run_init(*Q, st);
+    if (s == LABS_OK && cudaEventRecord(e0, st) != cudaSuccess) s = LABS_ERR_CUDA;
+    if (s == LABS_OK) s = run_walks(*Q, q, st);
+    float ms = 0.f;
+    if (s == LABS_OK && (cudaEventRecord(e1, st) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
+                         cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess))
+      s = LABS_ERR_CUDA;
+    if (s != LABS_OK || turn < 0) continue;
+    const double per_walk = (double)ms / (double)Q->n_items;
+    if (turn == 0 || per_walk < 0.98 * best) {  // fewer walks only where that is clearly faster
+      best = per_walk;
+      *warps = w;
+    }
+  }
+  cudaEventDestroy(e0);
+  cudaEventDestroy(e1);
+  return s;
+}
+
 }  // namespace
 
 int launch_batched_search(labs_ctx* ctx, const labs_batch_cfg* cfg, const int32_t* lengths, const int64_t* walks,
@@ -1387,6 +1446,26 @@ int launch_batched_search(labs_ctx* ctx, const labs_batch_cfg* cfg, const int32_
   // kernel attributes and grid size before any capture
   int s = plan_launch(ctx, *P, cfg->warps_per_cta, false, &ln);
   if (s != LABS_OK) return s;
+  // (a search shorter than its trial is left to plan_launch)
+  const double trial_flips = 4.0 * kTrialRounds * ln.warps * ctx->num_sms * kTrialFlips;
+  if (cfg->warps_per_cta == 0 && ln.warps >= 8 && (double)P->n_items * (double)cfg->flip_budget >= trial_flips &&
+      !capturing(st)) {
+    uint64_t tkey = mix_key((uint64_t)ctx->num_sms,
+                            ((uint64_t)cfg->bloom_log2 << 32) ^ ((uint64_t)cfg->bloom_k << 16) ^ (uint64_t)cfg->R);
+    for (const LenSpec& e : lens) tkey = mix_key(tkey, ((uint64_t)e.L << 50) ^ ((uint64_t)e.p << 40) ^ (uint64_t)e.walks);
+    int warps = 0;
+    for (int i = 0; i < std::min(ctx->n_tuned, kMaxTuned); i++)
+      if (ctx->tuned_key[i] == tkey) warps = ctx->tuned_warps[i];
+    if (!warps) {
+      s = trial_warps(ctx, cfg, lens, *P, ln, st, &warps);
+      if (s != LABS_OK) return s;
+      ctx->tuned_key[ctx->n_tuned % kMaxTuned] = tkey;
+      ctx->tuned_warps[ctx->n_tuned % kMaxTuned] = warps;
+      ctx->n_tuned++;
+    }
+    s = plan_launch(ctx, *P, warps, false, &ln);  // (the trial left the kernel set up for its last launch)
+    if (s != LABS_OK) return s;
+  }
   if (!cfg->use_graph) return issue_batch(ctx, cfg, lens, *P, ln, thr, st);
 
   // ---- CUDA graph: capture once per (configuration, buffers), replay afterwards

@@ -1,6 +1,6 @@
 /* A stand-in for the CUDA runtime, preloaded into a child process on a machine without a GPU: device memory is host
- * memory that nothing touches, kernels do not run.  Every allocation, release and device-to-device copy is written
- * to FAKE_CUDART_LOG; a release of something that is not live is written as "bad-free".  Allocation number
+ * memory that nothing touches, kernels do not run.  Every allocation, release, device-to-device copy and
+ * launch is written to FAKE_CUDART_LOG; a release of something that is not live is written as "bad-free".  Allocation number
  * FAKE_CUDART_FAIL (from 1) fails. */
 #include <stddef.h>
 #include <stdint.h>
@@ -65,6 +65,47 @@ err_t cudaMemsetAsync(void* p, int v, size_t n, void* s) { (void)p; (void)v; (vo
 err_t cudaMemcpyAsync(void* d, const void* s, size_t n, int kind, void* st) {
   (void)kind; (void)st;
   note("copy", (uintptr_t)d, (uintptr_t)s, n);
+  return 0;
+}
+err_t cudaStreamIsCapturing(void* s, int* status) {
+  (void)s;
+  *status = getenv("FAKE_CUDART_CAPTURING") ? 1 : 0;
+  return 0;
+}
+err_t cudaEventCreate(void** e) { *e = (void*)1; return 0; }
+err_t cudaEventDestroy(void* e) { (void)e; return 0; }
+err_t cudaEventRecord(void* e, void* s) { (void)e; (void)s; return 0; }
+err_t cudaEventSynchronize(void* e) { (void)e; return 0; }
+err_t cudaEventElapsedTime(float* ms, void* a, void* b) { /* the times of FAKE_CUDART_MS, a comma-separated list */
+  static int turn;
+  const char* t = getenv("FAKE_CUDART_MS");
+  (void)a; (void)b;
+  for (int i = 0; t && i < turn; i++) {
+    t = strchr(t, ',');
+    if (t) t++;
+  }
+  turn++;
+  *ms = t ? (float)atof(t) : 1.f;
+  note("elapsed", 0, 0, (size_t)turn);
+  return 0;
+}
+typedef struct { unsigned x, y, z; } dim3_t;
+static dim3_t last_grid, last_block;
+static size_t last_smem;
+static void* last_stream;
+unsigned __cudaPushCallConfiguration(dim3_t grid, dim3_t block, size_t smem, void* stream) {
+  last_grid = grid;
+  last_block = block;
+  last_smem = smem;
+  last_stream = stream;
+  note("launch", grid.x, block.x, smem);
+  return 0;
+}
+err_t __cudaPopCallConfiguration(dim3_t* grid, dim3_t* block, size_t* smem, void* stream) {
+  *grid = last_grid;
+  *block = last_block;
+  *smem = last_smem;
+  *(void**)stream = last_stream;
   return 0;
 }
 err_t cudaLaunchKernel(const void* f, ...) { (void)f; return 0; }

@@ -22,15 +22,14 @@ assert lib.labs_ctx_create(c.byref(ctx), 0) == 0
 """ % LIB
 
 
-def _run(tmp_path, code, fail=None):
+def _run(tmp_path, code, **fake):
     """Runs code in a child on the stand-in; returns the log's lines as tuples (what, a, b, bytes)."""
     so = tmp_path / "libfake_cudart.so"
     subprocess.run(["gcc", "-shared", "-fPIC", "-O1", "-o", str(so),
                     os.path.join(ROOT, "tests", "support", "fake_cudart.c")], check=True)
     log = tmp_path / "calls.log"
     env = dict(os.environ, LD_PRELOAD=str(so), FAKE_CUDART_LOG=str(log))
-    if fail is not None:
-        env["FAKE_CUDART_FAIL"] = str(fail)
+    env.update(("FAKE_CUDART_" + k.upper(), str(v)) for k, v in fake.items())
     subprocess.run([sys.executable, "-c", HEAD + code], check=True, env=env, cwd=ROOT, timeout=120)
     rows = [l.split() for l in log.read_text().splitlines()]
     return [(r[0], int(r[1]), int(r[2]), int(r[3])) for r in rows]
@@ -106,3 +105,50 @@ lib.labs_ctx_destroy(ctx)
     assert what.count("no-memory") == 1
     assert what.count("bad-free") == 0
     assert what.count("malloc") == what.count("free") == 26 + which + 13
+
+
+BATCH = """
+class Cfg(c.Structure):
+    _fields_ = %s
+cfg = Cfg()
+cfg.n_len, cfg.p, cfg.flip_budget, cfg.R, cfg.bloom_log2, cfg.bloom_k = 2, 0, %d, 4, 15, 4
+cfg.n_thresh_samples, cfg.warps_per_cta = 10, %d
+lens, walks = (c.c_int32 * 2)(100, 101), (c.c_int64 * 2)(5000, 4000)
+for turn in range(2):
+    open(%r, "a").write("call 0 0 0\\n")
+    rc = lib.labs_batched_search(ctx, c.byref(cfg), lens, walks, P(0x1000), 1, P(0x2000), None, None, P(0x3000), None)
+    assert rc == 0, rc
+"""
+
+
+@pytest.mark.parametrize("times,best", [("9,3.0,1.0,2.0", 1), ("9,1,1,1", 0), ("9,3,2,1", 2), ("0.1,3,2.99,2.99", 0)])
+def test_batched_search_takes_the_walks_per_block_of_its_timed_trial(tmp_path, times, best):
+    """The first call of a length set times three numbers of walks per block (after an untimed turn) and runs with the
+    fastest, later calls without a trial.  (Every turn takes all walks of this batch, so the times compare.)"""
+    from paper_2409_07222_gb300 import _lib
+
+    fields = "[" + ", ".join("(%r, c.%s)" % (n, t.__name__) for n, t in _lib.BatchCfg._fields_) + "]"
+    log = str(tmp_path / "calls.log")
+    rows = _run(tmp_path, BATCH % (fields, 100000, 0, log), ms=times)
+    calls = [i for i, r in enumerate(rows) if r[0] == "call"]
+    # the walk kernel is the last launch of a call, and of every turn of the trial
+    first, second = rows[calls[0]:calls[1]], rows[calls[1]:]
+    turns = [first[i - 1] for i, r in enumerate(first) if r[0] == "elapsed"]
+    assert len(turns) == 4 and all(r[0] == "launch" for r in turns)
+    tried = [r[2] // 32 for r in turns][1:]
+    assert tried[0] > tried[1] > tried[2] and tried[1] % 4 == 0 and tried[2] == tried[1] - 4
+    assert first[-1][0] == second[-1][0] == "launch"
+    assert first[-1][2] == second[-1][2] == 32 * tried[best]
+    assert not [r for r in second if r[0] == "elapsed"]
+
+
+@pytest.mark.parametrize("flips,warps,fake", [(100000, 4, {}), (50, 0, {}), (100000, 0, {"capturing": 1})])
+def test_batched_search_without_a_trial(tmp_path, flips, warps, fake):
+    """No trial where the caller gives the walks per block, for a search shorter than the trial, or under capture."""
+    from paper_2409_07222_gb300 import _lib
+
+    fields = "[" + ", ".join("(%r, c.%s)" % (n, t.__name__) for n, t in _lib.BatchCfg._fields_) + "]"
+    rows = _run(tmp_path, BATCH % (fields, flips, warps, str(tmp_path / "calls.log")), **fake)
+    assert not [r for r in rows if r[0] == "elapsed"]
+    if warps:
+        assert rows[-1][2] == 32 * warps
