@@ -116,7 +116,8 @@ typedef struct {
   int32_t E_target;     /* record each walk's first flip reaching E <= E_target; INT32_MIN = off */
   int32_t tile_m;       /* 8, 12 or 16: accepted where that tile of neighbours has a plan for L and p (the walks
                            keep their neighbours incrementally and have no tiles); 0 = no request */
-  int32_t warps_per_cta;/* warps (walks) per CTA: 1..8 with lanes_per_walk 32, 1..12 with 16; 0 = chosen by the
+  int32_t warps_per_cta;/* warps (walks) per CTA: 1..8 with lanes_per_walk 32, 1..12 with 16 (with 0: 9..12 are
+                           refused where the tile plan of L, p, R and tile_m takes 32 lanes); 0 = chosen by the
                            library */
   int32_t lanes_per_walk; /* 32, or 16 (R <= 16): accepted, every walk runs on one warp; 0 = no request */
   const int32_t* E_thr_dev; /* nullable device int32: when set, the sieve bound is read from it (for
@@ -354,9 +355,11 @@ int labs_policy_train_step(labs_policy* policy, const uint64_t* seqs, const int3
  *   Arguments as in labs_skew_search, plus (all nullable, DEVICE, n_chunks = ceil(flip_budget / chunk)):
  *   logits_log [n_chunks][n_walks][L] FP32: the logits each chunk used;
  *   state_log  [n_chunks][n_walks][W] uint64 (of any alignment): every walk's sequence when its chunk began;
- *   move_log   [n_chunks][n_walks][2] int32: the chunk's first move (position, Delta E), (-1, 0) if none.
- *   Workspace with a policy: about 8 KB per walk (up to 11 KB at L = 576).  With a policy the call synchronises `stream` at its end and returns
- *   LABS_ERR_TIMEOUT if a tensor-core wait of the network expired.
+ *   move_log   [n_chunks][n_walks][2] int32 (4-byte aligned): the chunk's first move (position, Delta E);
+ *              every chunk has one.
+ *   Workspace with a policy: about 8 KB per walk (up to 11 KB at L = 576).  With a policy the call
+ *   synchronises `stream` at its end and returns LABS_ERR_TIMEOUT if a tensor-core wait of the network
+ *   expired.
  */
 int labs_chunked_search(labs_ctx* ctx, const labs_walk_cfg* cfg, labs_policy* policy, float lambda, int chunk,
                         const uint64_t* prefixes, int n_prefix, labs_candidate* out, int64_t* walk_stats,

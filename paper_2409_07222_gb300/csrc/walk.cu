@@ -999,9 +999,11 @@ static int issue_threshold(int sms, int L, int skew, int p, const uint64_t* pref
 }
 
 // ---------------------------------------------------------------------------------------------
-// The tile parameters of a configuration (tile_m, lanes_per_walk, warps_per_cta) select nothing in the
-// incremental walk but the warps of a block; a combination that the tiled neighbour scan has no plan for
-// stays refused.
+// Which configurations are accepted.  The tile parameters (tile_m, lanes_per_walk) select nothing in the incremental
+// walk; they were those of a tiled scan of all neighbours, and what that scan had no plan for was refused.  Callers
+// may rely on the refusals, so they are kept exactly: make_layout, the eight tiles and the ranking by scan work below
+// answer nothing else.  The ranking matters for one of them: with lanes_per_walk 0, more than eight warps per CTA are
+// accepted where the plan of least work had 16 lanes a walk.
 // ---------------------------------------------------------------------------------------------
 constexpr int kMaxPasses = 3;  // lane passes over the tiles of one walk
 struct Variant {
@@ -1025,7 +1027,7 @@ struct LenSpec {
 };
 
 // The plan of least scan work, sum(walks * NP * M / H * GL / 32), that the requested parameters allow; ties
-// to fewer lanes per walk, fewer passes, more lanes per tile, the larger tile.  False if there is none.
+// to fewer lanes per walk, fewer passes, more lanes per tile, the larger tile.  False if there is none: refused.
 // req_m / req_gl: 0 or the tile size / lanes per walk the caller fixed; R: sieve slots per walk.
 static bool choose_variant(const std::vector<LenSpec>& lens, int req_m, int req_gl, int R, Variant* out) {
   bool found = false;
@@ -1093,7 +1095,8 @@ static WalkKernel walk_fn(const Launch& ln, bool biased) {
     case 208: return walk_fn_of<2, 8>(ln.mode, biased);
     case 312: return walk_fn_of<3, 12>(ln.mode, biased);
     case 416: return walk_fn_of<4, 16>(ln.mode, biased);
-    case 418: return ln.mode == 0 ? walk_kernel<4, 16, 0, false> : ln.mode == 1 ? walk_fn_of<5, 18>(1, biased) : walk_kernel<4, 18, 2, false>;
+    case 418:  // for unrestricted lengths beyond 512; the skew part of a mixed launch has four slots
+      return ln.mode == 2 ? walk_kernel<4, 18, 2, false> : ln.mode == 1 ? walk_fn_of<5, 18>(1, biased) : walk_fn_of<4, 16>(0, biased);
     default: return walk_fn_of<5, 18>(ln.mode, biased);
   }
 }
