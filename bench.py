@@ -114,7 +114,8 @@ def walk_profile():
 
 
 def walk_issue(flips_per_s):
-    """Share of the issue slots (4 a clock and SM) that the walk kernel's own instructions take."""
+    """Share of the issue slots (4 a clock and SM) that the walk kernel's own instructions take: those of ten whole
+    segments, their starts included, as a long run has them."""
     d = walk_profile()
     if not d:
         return None
@@ -242,7 +243,7 @@ def run_mixed(args, ws, rank, local):
                             n_thresh_samples=W1["n_thresh_samples"], thresh_rank=W1["thresh_rank"], use_graph=True)
     flush = torch.empty(256 * 1024 * 1024, dtype=torch.uint8, device=dev)
     t0 = time.perf_counter()
-    out = lg.labs_batched_search(cfg, lengths, walks, pre, walk_stats=False)  # capture
+    out = lg.labs_batched_search(cfg, lengths, walks, pre, walk_stats=False)  # trial of the walks per block, capture
     torch.cuda.synchronize()
     first_s = time.perf_counter() - t0
     for _ in range(max(0, args.warmup - 1)):
@@ -274,7 +275,7 @@ def run_mixed(args, ws, rank, local):
             "scaling": "weak", "vs_baseline": None, "dtype": "int32", "data": "synthetic",
             "config": {"workload": "mixed_L450-527_walks_U1024-16384_1e4flips", "lengths": len(lengths),
                        "walks": sum(walks), "flips_per_walk": budget, "p_odd": p, "graph": True,
-                       "first_call_s_incl_capture": first_s,
+                       "first_call_s_incl_trial_and_capture": first_s,
                        "l2": "flushed between timed steps (256 MB write)"},
             "gpu_launches": (4 * len(lengths) + 2) * args.steps, "clocks": clk,
             "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Gop/s", "frac": achieved / peak,

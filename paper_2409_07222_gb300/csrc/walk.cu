@@ -12,7 +12,7 @@
 //             fingerprint; on a hit the owner lane looks for its next smallest (same result as testing all),
 //   apply  -- the flip, the O(L) tables, then every neighbour's sum from them,
 //   sieve  -- the walk's R best distinct (E, fp) states with E <= E_thr.
-// Measured (L = 451, p = 24, 65,536 walks x 2,000 flips, sieve bound of 10^6 samples included): 78.8 ms, where
+// Measured (L = 451, p = 24, 65,536 walks x 2,000 flips, sieve bound of 10^6 samples included): 77.6 ms, where
 // the scan of every neighbour took 337 ms; 256 walks x 8,192 flips 11.3 ms (74.6 ms: its blocks filled 11 SMs).
 #include <algorithm>
 #include <cstring>
@@ -29,7 +29,11 @@ namespace {
 constexpr int kMaxLens = 96;  // lengths in one launch (kernel parameter table)
 
 // Slots (values of T) a lane of a walk kernel holds, and the threads per block it is compiled for (one block
-// per SM): 32 walks of up to 10 slots a lane (64 registers a thread), 24 walks of up to 18 slots (80).
+// per SM): 32 walks of up to 10 slots a lane (64 registers a thread), 24 walks of up to 18 slots (80).  Every
+// instantiation spills some registers: 104 bytes a thread at <4, 16, 0>, the slots of L = 451, 276 to 380 at <4, 16, 1>,
+// <4, 18, 2>, <5, 18, 1> and <5, 18, 2>.  Measured with 24 walks (80 registers, 48 bytes) in place of 32 for <4, 16, 0>:
+// 65,536 walks x 2,000 flips 76.4 ms against 77.6, 256 walks x 8,192 flips 10.3 against 11.4; learned, 8,192 walks in
+// chunks of 64, 8.55 against 8.33.  The 32 were chosen for what an SM holds, not for these times.
 __host__ __device__ constexpr int walk_slots(int mode, int ns, int nu) {
   return mode == 0 ? 2 * ns : (mode == 1 || nu > 2 * ns ? nu : 2 * ns);
 }
@@ -178,8 +182,9 @@ __device__ __forceinline__ int corr_bits(const uint32_t* a, const uint32_t* b, i
 // unrestricted one.  MODE 0: a launch of one skew length, 1: one unrestricted length, 2: several lengths of
 // either kind; BIASED: the choice key is the proposal score of WalkParams::bias.
 //
-// Bound (L = 451, skew): issue slots and shared-memory instructions -- a flip is about 75 shared-memory
-// accesses and a few hundred warp instructions, where scanning every neighbour took 2,285.
+// Bound (L = 451, skew): issue slots (88% used) and shared-memory instructions -- a flip is about 75 shared-memory
+// accesses and 608 warp instructions (623 with its share of a segment's start), where scanning every neighbour took
+// 2,285.
 template <int NS, int NU, int MODE, bool BIASED>
 __global__ void __launch_bounds__(walk_block_threads(MODE, NS, NU), 1)
     walk_kernel(const __grid_constant__ WalkParams P) {
@@ -1167,7 +1172,7 @@ static void fill_params(WalkParams& P, const std::vector<LenSpec>& lens, int blo
 
 // Sets the kernel's shared-memory limit and sizes the persistent grid.  A block is one SM's walks: as many
 // warps as its registers and shared memory hold, fewer when the launch has fewer walks than that per SM (a
-// few walks then spread over all SMs instead of filling some).
+// few walks then spread over all SMs instead of filling some).  A batch times that number against fewer (trial_warps).
 static int plan_launch(labs_ctx* ctx, const WalkParams& P, int requested_warps, bool biased, Launch* ln) {
   int warps = walk_block_threads(ln->mode, ln->ns, ln->nu) / 32;
   if (requested_warps > 0) {
