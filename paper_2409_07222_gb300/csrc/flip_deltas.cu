@@ -205,7 +205,7 @@ template <class Kernel>
 int launch_fd(labs_ctx* ctx, Kernel* kern, const uint64_t* seqs, const int32_t* C, int L, int64_t n, int p, const FdPlan& fp,
               int32_t* dE, cudaStream_t st) {
   const size_t smem = sizeof(uint32_t) * (size_t)fp.words * kFdWarps;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return LABS_ERR_CUDA;
+  if (allow_smem(ctx, kern) != cudaSuccess) return LABS_ERR_CUDA;
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * kFdWarps, smem) != cudaSuccess || per_sm < 1)
     return LABS_ERR_CUDA;

@@ -69,6 +69,13 @@ int by_words(int n, Fn&& fn) {
   }
 }
 
+// Lets `kernel` take all the dynamic shared memory that a block can have, whatever a launch asks for: the limit belongs
+// to the function, so one set by a launch's own size would be in the way of another thread's launch of another length.
+template <class Kernel>
+cudaError_t allow_smem(const labs_ctx* ctx, Kernel* kernel) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ctx->smem_optin);
+}
+
 inline int cuda_status(cudaError_t e) { return e == cudaSuccess ? LABS_OK : LABS_ERR_CUDA; }
 
 // Shape of a walk or a sieve sample (Algorithm 1): length, mode, prefix length (Eq. 3) and the prefix

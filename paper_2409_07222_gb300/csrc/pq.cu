@@ -1397,7 +1397,7 @@ int launch_pq_refine(labs_ctx* ctx, const labs_pq_cfg* cfg, const uint64_t* seed
   int per_sm = 0;
   const int es = by_words((L + 31) >> 5, [&](auto nw) {
     expand = pq_expand_kernel<decltype(nw)::value>;
-    return cuda_status(cudaFuncSetAttribute(expand, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)exp_smem));
+    return cuda_status(allow_smem(ctx, expand));
   });
   if (es != LABS_OK ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, expand, 32 * kPqWarps, exp_smem) != cudaSuccess || per_sm < 1)

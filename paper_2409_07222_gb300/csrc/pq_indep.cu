@@ -565,7 +565,7 @@ int launch_pq_independent(labs_ctx* ctx, const labs_pq_indep_cfg* cfg, const uin
       if constexpr (NW > 16)
         if (v_in_q) k = pairs ? pq_indep_kernel<NW, true, true> : pq_indep_kernel<NW, false, true>;
       if (!v_in_q) k = pairs ? pq_indep_kernel<NW, true, false> : pq_indep_kernel<NW, false, false>;
-      return k ? cuda_status(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) : LABS_OK;
+      return k ? cuda_status(allow_smem(ctx, k)) : LABS_OK;
     });
     if (!k && ks == LABS_OK) break;  // compiled in the plain form only
     int per_sm = 0;

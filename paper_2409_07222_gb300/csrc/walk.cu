@@ -1170,7 +1170,7 @@ static void fill_params(WalkParams& P, const std::vector<LenSpec>& lens, int blo
   sp.bytes = sp.off_bloom + up16(std::max(kScratch, (1 << bloom_log2) / 8));
 }
 
-// Sets the kernel's shared-memory limit and sizes the persistent grid.  A block is one SM's walks: as many
+// Lets the kernel have its shared memory and sizes the persistent grid.  A block is one SM's walks: as many
 // warps as its registers and shared memory hold, fewer when the launch has fewer walks than that per SM (a
 // few walks then spread over all SMs instead of filling some).  A batch times that number against fewer (trial_warps).
 static int plan_launch(labs_ctx* ctx, const WalkParams& P, int requested_warps, bool biased, Launch* ln) {
@@ -1185,8 +1185,7 @@ static int plan_launch(labs_ctx* ctx, const WalkParams& P, int requested_warps, 
   ln->warps = warps;
   ln->smem = (size_t)P.slab.bytes * warps;
   WalkKernel kern = walk_fn(*ln, biased);
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ln->smem) != cudaSuccess)
-    return LABS_ERR_CUDA;
+  if (allow_smem(ctx, kern) != cudaSuccess) return LABS_ERR_CUDA;
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * warps, ln->smem) != cudaSuccess || per_sm < 1)
     return LABS_ERR_CUDA;
@@ -1471,7 +1470,7 @@ int launch_batched_search(labs_ctx* ctx, const labs_batch_cfg* cfg, const int32_
       ctx->tuned_warps[ctx->n_tuned % kMaxTuned] = warps;
       ctx->n_tuned++;
     }
-    s = plan_launch(ctx, *P, warps, false, &ln);  // (the trial left the kernel set up for its last launch)
+    s = plan_launch(ctx, *P, warps, false, &ln);
     if (s != LABS_OK) return s;
   }
   if (!cfg->use_graph) return issue_batch(ctx, cfg, lens, *P, ln, thr, st);

@@ -1,6 +1,6 @@
 /* A stand-in for the CUDA runtime, preloaded into a child process on a machine without a GPU: device memory is host
- * memory that nothing touches, kernels do not run.  Every allocation, release, device-to-device copy and
- * launch is written to FAKE_CUDART_LOG; a release of something that is not live is written as "bad-free".  Allocation number
+ * memory that nothing touches, kernels do not run.  Every allocation, release, device-to-device copy,
+ * function attribute and launch is written to FAKE_CUDART_LOG; a release of something that is not live is written as "bad-free".  Allocation number
  * FAKE_CUDART_FAIL (from 1) fails. */
 #include <stddef.h>
 #include <stdint.h>
@@ -28,7 +28,10 @@ err_t cudaDeviceGetAttribute(int* v, int attr, int d) { (void)d; *v = attr == 97
 err_t cudaDeviceSynchronize(void) { return 0; }
 err_t cudaStreamSynchronize(void* s) { (void)s; return 0; }
 err_t cudaGetLastError(void) { return 0; }
-err_t cudaFuncSetAttribute(const void* f, int a, int v) { (void)f; (void)a; (void)v; return 0; }
+err_t cudaFuncSetAttribute(const void* f, int a, int v) {
+  note("attribute", (uintptr_t)f, (uintptr_t)a, (size_t)v);
+  return 0;
+}
 err_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void* f, int t, size_t s, unsigned g) {
   (void)f; (void)t; (void)s; (void)g;
   *n = 1;
@@ -108,5 +111,14 @@ err_t __cudaPopCallConfiguration(dim3_t* grid, dim3_t* block, size_t* smem, void
   *(void**)stream = last_stream;
   return 0;
 }
+err_t cudaHostAlloc(void** p, size_t n, unsigned flags) { (void)flags; *p = calloc(1, n); return 0; }
+err_t cudaFreeHost(void* p) { free(p); return 0; }
+err_t cudaStreamCreateWithFlags(void** s, unsigned f) { (void)f; *s = (void*)1; return 0; }
+err_t cudaStreamBeginCapture(void* s, int mode) { (void)s; (void)mode; return 0; }
+err_t cudaStreamEndCapture(void* s, void** g) { (void)s; *g = (void*)1; return 0; }
+err_t cudaGraphInstantiate(void** x, void* g, unsigned long long f) { (void)g; (void)f; *x = (void*)1; return 0; }
+err_t cudaGraphLaunch(void* x, void* s) { (void)x; (void)s; return 0; }
+err_t cudaGraphDestroy(void* g) { (void)g; return 0; }
+err_t cudaGraphExecDestroy(void* x) { (void)x; return 0; }
 err_t cudaLaunchKernel(const void* f, ...) { (void)f; return 0; }
 err_t __cudaLaunchKernel(const void* f, ...) { (void)f; return 0; }

@@ -152,3 +152,41 @@ def test_batched_search_without_a_trial(tmp_path, flips, warps, fake):
     assert not [r for r in rows if r[0] == "elapsed"]
     if warps:
         assert rows[-1][2] == 32 * warps
+
+
+def test_shared_memory_limit_of_a_kernel_does_not_depend_on_the_launch(tmp_path):
+    """The limit belongs to the function: set by a launch's own size, it would be too small for another thread's launch
+    of another length of the same instantiation in between."""
+    from paper_2409_07222_gb300 import _lib
+
+    def fields(t):
+        return "[" + ", ".join("(%r, c.%s)" % (n, x.__name__) for n, x in t._fields_) + "]"
+
+    rows = _run(tmp_path, """
+class Pq(c.Structure):
+    _fields_ = %s
+class Indep(c.Structure):
+    _fields_ = %s
+class Walk(c.Structure):
+    _fields_ = %s
+i64 = c.c_int64
+for L in (449, 455, 480, 513, 515, 543):
+    for skew in (0, L %% 2):
+        for C in (None, P(0x3000)):
+            assert lib.labs_flip_deltas(ctx, P(0x1000), C, L, i64(10), skew, 0, P(0x2000), None) == 0
+    pq = Pq()
+    pq.L, pq.B, pq.cap, pq.H_log2, pq.max_expansions = L, 4, 64, 12, 8
+    assert lib.labs_pq_refine(ctx, c.byref(pq), P(0x1000), 1, P(0x2000), P(0x3000), P(0x4000), None) == 0
+    for T_r in (0, 2):
+        ind = Indep()
+        ind.L, ind.T_r, ind.H_log2, ind.max_expansions = L, T_r, 12, 8
+        assert lib.labs_pq_independent(ctx, c.byref(ind), P(0x1000), 5000, P(0x2000), P(0x3000), P(0x4000), None) == 0
+    w = Walk()
+    w.L, w.skew, w.n_walks, w.flip_budget, w.R, w.bloom_log2, w.bloom_k, w.E_thr = L, L %% 2, 9999, 10, 4, 15, 4, 1
+    assert lib.labs_skew_search(ctx, c.byref(w), P(0x1000), 1, P(0x2000), None, P(0x3000), None) == 0
+""" % (fields(_lib.PqCfg), fields(_lib.PqIndepCfg), fields(_lib.WalkCfg)))
+    limits = {}
+    for r in rows:
+        if r[0] == "attribute":
+            limits.setdefault(r[1], set()).add(r[3])
+    assert len(limits) > 10 and all(len(v) == 1 for v in limits.values()), limits
