@@ -7,9 +7,9 @@
 // the self-convolution V.
 //
 // Measured against the dp4a scan of all neighbours x lags (one lane per tile of eight neighbours): 32,768 skew
-// sequences of L = 451, p = 24: 217 -> 77 us; 8,192 unrestricted ones of L = 452: 123 -> 38 us, of L = 576: 191
-// -> 46 us.  Bound: issue slots (1,720 warp instructions a skew sequence, 67% busy at 20 warps an SM), the
-// tensor cores 15% busy.
+// sequences of L = 451, p = 24: 217 -> 72 us; 8,192 unrestricted ones of L = 452: 123 -> 38 us, of L = 576: 191
+// -> 46 us.  Bound: issue slots (1,646 warp instructions a skew sequence, 67% busy at 20 warps an SM), the
+// tensor cores 16% busy.
 #include <algorithm>
 
 #include "labs_internal.h"

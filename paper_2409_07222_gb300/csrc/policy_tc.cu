@@ -526,8 +526,9 @@ int tc_conv64(const __nv_bfloat16* in, const __nv_bfloat16* img, const float* bi
   return cuda_status(cudaGetLastError());
 }
 
-// Splits of K: a function of K alone, so a sample's logits do not depend on the batch it is evaluated in: about 48
-// stages each, at most 9 (with the 32 row blocks of 8,192 samples, two rounds of CTAs).
+// Splits of K: a function of K alone, so a sample's logits do not depend on the batch it is evaluated in: 48 stages or
+// more each, so that a CTA's set-up and its partial sums (read and added by dense_reduce_kernel) stay small beside them,
+// and at most 9, which bounds that scratch to 9 KB a sample.  A small batch then still has nine CTAs from L = 432 on.
 int tc_dense_splits(int K) { return std::max(1, std::min(9, (K / 64) / 48)); }
 
 int tc_dense(const __nv_bfloat16* A, const __nv_bfloat16* Bp, const float* bias, float* part, float* out, long long n,

@@ -221,7 +221,9 @@ constexpr int kInP = 0, kInC = 24, kInClass = 48, kInRev = kInClass + 2 * kClass
 // Seven blocks an SM hold 28 candidates (72 registers a thread, 7.7 KB of slab a warp at L = 451), 4,256 on the chip.
 // Beyond 512 positions the slab leaves room for six blocks (80 registers), 3,648 candidates.  V_IN_Q (compiled there): V is formed
 // first, where the table of q comes to lie, and a lane keeps its outputs' values in registers, so that seven blocks
-// fit again; a pop takes longer (more registers saved).
+// fit again; a pop takes longer (more registers saved).  The 72 registers cost spills (92 bytes a thread at L = 451, 232
+// with a visited set, 212 to 400 in the V_IN_Q forms); with six blocks of 80 registers, 4,096 candidates of L = 451 x 256
+// pops take 11.3 ms, with seven 10.5 ms.
 template <int NW, bool PAIRS, bool V_IN_Q>
 __global__ void __launch_bounds__(32 * kIWarps, NW > 16 && !V_IN_Q ? 6 : 7) pq_indep_kernel(IndepArgs a, IndepPlan ip) {
   constexpr int NT = (NW + 3) / 4;
